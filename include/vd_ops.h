@@ -96,7 +96,7 @@ typedef struct {
     int32_t ksize;              /* 1 or 3 (zero padding ksize/2, stride 1) */
     int32_t upsample;           /* 1: nearest-2x upsample folded into the addressing; output is 2*in_h x 2*in_w.
                                    2: the same result phase-collapsed (four 2x2 convolutions of the source with
-                                   pre-summed weights; tensor-core kernel only, 3x3, c_out % 128 == 0, no residual) */
+                                   pre-summed weights; 3x3, no residual; c_out % 128 == 0, or fp32 in and out and c_out % 32 == 0) */
     int32_t silu;               /* 1: SiLU after the scale/shift prologue */
     int32_t in_dtype;           /* vd_dtype of x */
     int32_t out_dtype;          /* vd_dtype of y */

@@ -24,7 +24,9 @@ struct Step {
     AttnArgs attn;
     IngestArgs ing;
     ConvTcPlan tc;
+    ConvF32Plan f32;             // valid: the layer runs on conv_f32.cu
     AttnTcPlan attn_tc;
+    bool skip;                   // statistics that the consuming layer merges from its producer's records: no launch
     // batch-dependent pointers are rebased per call: strides per frame
     bool has_residual;
 };
@@ -127,11 +129,11 @@ class Planner {
     struct ConvW { size_t w_off, b_off; bool tc; };
 
     // registers the repack of a conv weight (possibly a stack of several source tensors along Cout)
-    ConvW conv_weight(const std::vector<std::string>& names, int Cout_each, int Cin, int taps, bool tc, bool phase = false) {
+    ConvW conv_weight(const std::vector<std::string>& names, int Cout_each, int Cin, int taps, bool tc, bool phase) {
         const int Cout = Cout_each * (int)names.size();
         ConvW r;
         r.tc = tc;
-        const size_t wbytes = tc ? conv_tc_packed_bytes(Cout, Cin, taps, phase) : (size_t)taps * Cin * Cout * 4;
+        const size_t wbytes = tc ? conv_tc_packed_bytes(Cout, Cin, taps, phase) : (size_t)(phase ? 16 : taps) * Cin * Cout * 4;
         r.w_off = alloc(wbytes);
         r.b_off = alloc((size_t)Cout * 4);
         for (size_t i = 0; i < names.size(); ++i) {
@@ -179,6 +181,10 @@ class Planner {
                       ptr<float>(b_off), ptr<float>(scale_off_), ptr<float>(shift_off_), ptr<float>(partial_off_),
                       ptr<unsigned int>(partial_off_ + gn_partial_bytes(cfg_.max_batch, cfg_.norm_groups)),
                       pending(x_off) != kNone ? ptr<float>(pending(x_off)) : nullptr};
+        if (rec_.count(x_off) && pending(x_off) == kNone && rec_groups_ok(C, cfg_.norm_groups)) {
+            s.gn.rec = ptr<float4>(rec_[x_off].off);
+            s.gn.slots = rec_[x_off].slots;
+        }
         fill_info(s, name, 0, C, C, 0, 0, H, W, C, VD_F32, 0, -1);
         s.info.launches = 1;
         s.info.bytes_per_frame = (double)H * W * C * elt(dtype);
@@ -217,6 +223,15 @@ class Planner {
         }
         if (phase) a.upsample = 2;
         const bool tc = tc_on && conv_tc_supported(probe);
+        // fp32 layers: the direct kernel remains for the bf16 layout's cross-check path (and the 9-tap upsampling form)
+        bool f32 = false;
+        if (!tc && !(bf16() && (cfg_.flags & VD_FLAG_FORCE_SIMT))) {
+            probe.B = cfg_.max_batch;
+            probe.upsample = upsample ? ((cfg_.flags & VD_FLAG_UPSAMPLE_9TAP) ? 1 : 2) : 0;
+            f32 = conv_f32_choose(probe, &s.f32);
+            if (f32 && upsample) { phase = true; a.upsample = 2; }
+        }
+        s.f32.valid = f32 ? 1 : 0;
         ConvW cw = conv_weight(wnames, Cout_each, Cin, ksize * ksize, tc, phase);
         a.w = ptr<void>(cw.w_off);
         a.bias = ptr<float>(cw.b_off);
@@ -262,6 +277,30 @@ class Planner {
                 if (pres != kNone) pending_[y_off] = pres;      // accumulated in place: what was pending stays pending
                 else pending_.erase(y_off);
             }
+        }
+        // ---- statistics as records (conv_cluster.cuh): where there are few, this layer merges them itself and the step
+        // just planned needs no launch
+        if (f32 && prologue) {
+            Step& g = h_->steps.back();
+            if (g.kind == VD_STEP_GN_STATS && g.gn.rec && g.gn.slots <= kRecMergeSlots) {
+                a.in_rec = g.gn.rec; a.in_slots = g.gn.slots;
+                a.in_gamma = g.gn.gamma; a.in_beta = g.gn.beta; a.in_G = g.gn.G; a.in_eps = g.gn.eps;
+                a.scale = a.shift = nullptr;
+                g.skip = true;
+                g.info.launches = 0;
+            }
+        }
+        if (!y_is_frames) rec_.erase(y_off);
+        const bool records = !no_records_;
+        no_records_ = false;
+        if (f32 && records && !y_is_frames && rec_groups_ok(Cout, cfg_.norm_groups)) {
+            const int slots = conv_f32_slots(probe, s.f32, cfg_.norm_groups);
+            rec_toggle_ ^= 1;
+            a.out_rec = ptr<float4>(rec_buf_[rec_toggle_]);
+            a.out_slots = slots;
+            a.out_G = cfg_.norm_groups;
+            rec_[y_off] = {rec_buf_[rec_toggle_], slots};
+            max_slots_ = std::max(max_slots_, slots);
         }
         s.conv = a;
         s.use_tc = tc;
@@ -317,6 +356,7 @@ class Planner {
             add_conv(p + ".conv2", {p + ".conv2"}, Cout, hbuf_, act_dtype(), H, W, Cout, 3, false, true, true, -1, y,
                      VD_F32, false, false, p + ".shortcut", x, Cin);
         } else {
+            no_records_ = true;          // conv2 accumulates into this layer's output and leaves the records
             add_conv(p + ".shortcut", {p + ".shortcut"}, Cout, x, VD_F32, H, W, Cin, 1, false, false, false, -1, y, VD_F32,
                      false, false);
             defer_ = true;
@@ -355,7 +395,16 @@ class Planner {
         cur_x_ ^= 1;
     }
 
+    // Laid out twice: how much room the statistics records need is known once every layer has its kernel.
     vd_status plan() {
+        vd_handle_s scratch;
+        scratch.cfg = cfg_;
+        Planner first(&scratch, nullptr);
+        first.layout(0);
+        return layout(first.max_slots_);
+    }
+
+    vd_status layout(int rec_slots) {
         const int h = cfg_.latent_h, w = cfg_.latent_w, B = cfg_.max_batch;
         const int lc = cfg_.latent_channels;
         const size_t P0 = (size_t)h * w;
@@ -401,6 +450,7 @@ class Planner {
         stat_off_ = alloc(conv_stat_scratch_bytes(B, cfg_.norm_groups));
         h_->stat_off = stat_off_;
         h_->stat_bytes = conv_stat_scratch_bytes(B, cfg_.norm_groups);
+        for (int i = 0; i < 2; ++i) rec_buf_[i] = alloc((size_t)B * cfg_.norm_groups * rec_slots * sizeof(float4));
         zbuf_ = alloc((size_t)B * P0 * lc * 4);
         xs_[0] = alloc((size_t)B * max_x * 4);
         xs_[1] = alloc((size_t)B * max_x * 4);
@@ -479,6 +529,11 @@ class Planner {
     size_t stat_off_ = 0;
     std::map<size_t, size_t> pending_;   // tensor offset -> offset of its pending-bias vector
     size_t pending(size_t off) const { auto it = pending_.find(off); return it == pending_.end() ? kNone : it->second; }
+    struct Records { size_t off; int slots; };
+    std::map<size_t, Records> rec_;      // tensor offset -> the statistics records its producing layer leaves
+    size_t rec_buf_[2] = {0, 0};         // written alternately: a layer reads one while it writes the other
+    int rec_toggle_ = 0, max_slots_ = 0;
+    bool no_records_ = false;            // set by the caller of add_conv: nothing normalises this layer's output as it is
     bool defer_ = false;                 // set by the caller of add_conv: this layer's bias may be left pending
     size_t ones_off_ = kNone;
     int max_c_ = 0;
@@ -525,6 +580,7 @@ const vd_tensor* find_tensor(const vd_tensor* t, int n, const std::string& name)
 cudaError_t launch_step(const vd_handle_s* h, const Step& st, int B, const void* latents, const void* v_prev,
                         float lambda, void* z_out, void* v_out, void* frames, cudaStream_t s) {
     unsigned int* status = (unsigned int*)(h->ws + h->status_off);
+    if (st.skip) return cudaSuccess;
     switch (st.kind) {
         case VD_STEP_INGEST: {
             IngestArgs a = st.ing;
@@ -534,12 +590,13 @@ cudaError_t launch_step(const vd_handle_s* h, const Step& st, int B, const void*
         case VD_STEP_GN_STATS: {
             GnArgs a = st.gn;
             a.B = B;
-            return launch_gn_stats(a, s);
+            return a.rec ? launch_gn_merge(a, s) : launch_gn_stats(a, s);
         }
         case VD_STEP_CONV: {
             ConvArgs a = st.conv;
             a.B = B;
             if (!a.y) a.y = frames;
+            if (st.f32.valid) return launch_conv_f32(a, st.f32, status, s);
             return st.use_tc ? launch_conv_tc(a, st.tc, status, s) : launch_conv_simt(a, s);
         }
         case VD_STEP_ATTENTION: {
@@ -675,6 +732,8 @@ vd_status vd_create(const vd_config* cfg, const vd_tensor* weights, int32_t n_we
             e = launch_to_f32(t->dptr, t->dtype, (float*)(h->ws + j.dst_off), j.kind == 1 ? j.Cout : (int64_t)j.Cout * j.Cin, s);
         } else if (j.tc) {
             e = launch_pack_weight_tc(t->dptr, t->dtype, h->ws + j.dst_off, j.Cout, j.Cin, j.taps, j.cout_total, j.cout_offset, j.phase, s);
+        } else if (j.phase) {
+            e = launch_pack_weight_f32_phase(t->dptr, t->dtype, (float*)(h->ws + j.dst_off), j.Cout, j.Cin, s);
         } else {
             e = launch_pack_weight_simt(t->dptr, t->dtype, (float*)(h->ws + j.dst_off), j.Cout, j.Cin, j.taps, j.cout_total, j.cout_offset, s);
         }
@@ -690,6 +749,10 @@ vd_status vd_create(const vd_config* cfg, const vd_tensor* weights, int32_t n_we
         if (e != cudaSuccess) { delete h; return cuda_fail(nullptr, e, "bias rows"); }
     }
     for (Step& st : h->steps) {
+        if (st.kind == VD_STEP_CONV && st.f32.valid) {
+            e = conv_f32_prepare(st.conv, &st.f32);
+            if (e != cudaSuccess) { delete h; return cuda_fail(nullptr, e, "weight tensor map"); }
+        }
         if (st.kind == VD_STEP_CONV && st.use_tc) {
             ConvArgs pa = st.conv;
             pa.B = cfg->max_batch;
@@ -926,7 +989,7 @@ static vd_status resolve_impl(const vd_conv_desc* d, const ConvArgs& a, bool* tc
     const bool can = a.bf16_operands && conv_tc_supported(probe);
     if (d->impl == VD_IMPL_TC && !can) return fail(nullptr, VD_ERR_UNSUPPORTED, "the tensor-core convolution does not support this shape");
     *tc = d->impl == VD_IMPL_TC || (d->impl == VD_IMPL_AUTO && can);
-    if (!*tc && a.upsample == 2) return fail(nullptr, VD_ERR_UNSUPPORTED, "the phase-collapsed upsampling form exists in the tensor-core kernel only");
+    if (!*tc && a.upsample == 2 && !conv_f32_supported(a)) return fail(nullptr, VD_ERR_UNSUPPORTED, "this layer has no phase-collapsed upsampling form");
     return VD_OK;
 }
 
@@ -938,7 +1001,7 @@ vd_status vd_conv_packed_weight_bytes(const vd_conv_desc* d, size_t* bytes) {
     st = resolve_impl(d, conv_args_from_desc(d), &tc);
     if (st != VD_OK) return st;
     const int taps = d->ksize * d->ksize;
-    *bytes = tc ? conv_tc_packed_bytes(d->c_out, d->c_in, taps, d->upsample == 2) : (size_t)taps * d->c_in * d->c_out * 4;
+    *bytes = tc ? conv_tc_packed_bytes(d->c_out, d->c_in, taps, d->upsample == 2) : (size_t)(d->upsample == 2 ? 16 : taps) * d->c_in * d->c_out * 4;
     return VD_OK;
 }
 
@@ -952,6 +1015,7 @@ vd_status vd_conv_pack_weight(const vd_conv_desc* d, const void* w_oihw, int32_t
     if (st != VD_OK) return st;
     const int taps = d->ksize * d->ksize;
     cudaError_t e = tc ? launch_pack_weight_tc(w_oihw, w_dtype, packed, d->c_out, d->c_in, taps, d->c_out, 0, d->upsample == 2, (cudaStream_t)cuda_stream)
+                       : d->upsample == 2 ? launch_pack_weight_f32_phase(w_oihw, w_dtype, (float*)packed, d->c_out, d->c_in, (cudaStream_t)cuda_stream)
                        : launch_pack_weight_simt(w_oihw, w_dtype, (float*)packed, d->c_out, d->c_in, taps, d->c_out, 0, (cudaStream_t)cuda_stream);
     return e == cudaSuccess ? VD_OK : cuda_fail(nullptr, e, "vd_conv_pack_weight");
 }
@@ -982,7 +1046,13 @@ vd_status vd_op_conv2d(const vd_conv_desc* d, const void* x, const void* w_packe
         e = conv_tc_prepare(a, &plan);
         if (e == cudaSuccess) e = launch_conv_tc(a, plan, nullptr, (cudaStream_t)cuda_stream);
     } else {
-        e = launch_conv_simt(a, (cudaStream_t)cuda_stream);
+        ConvF32Plan plan{};
+        if (conv_f32_choose(a, &plan)) {
+            e = conv_f32_prepare(a, &plan);
+            if (e == cudaSuccess) e = launch_conv_f32(a, plan, nullptr, (cudaStream_t)cuda_stream);
+        } else {
+            e = launch_conv_simt(a, (cudaStream_t)cuda_stream);
+        }
     }
     return e == cudaSuccess ? VD_OK : cuda_fail(nullptr, e, "vd_op_conv2d");
 }

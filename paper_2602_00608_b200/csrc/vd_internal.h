@@ -43,6 +43,16 @@ struct ConvArgs {
     float* stat_shift;           // [B,Cout]
     int stat_G;
     float stat_eps;
+    // optional (conv_f32.cu, conv_split.cu): the input's GroupNorm statistics as records of its producing layer's CTAs
+    // instead of scale / shift, and the records of this layer's output: [B][G][slots] of (count, mean, sum of squared
+    // deviations, -)
+    const float4* in_rec;        // or null
+    const float* in_gamma;       // [Cin]
+    const float* in_beta;        // [Cin]
+    int in_slots, in_G;
+    float in_eps;
+    float4* out_rec;             // or null
+    int out_slots, out_G;
     // tensor-core kernel: ceil(2^32 / d) for the divisors of its tile numbering (tiles per image, channel
     // blocks, tiles per row), filled in by its launcher; 0 stands for d = 1
     unsigned int div_tiles, div_nblk, div_tx;
@@ -65,6 +75,8 @@ struct GnArgs {
     unsigned int* counters; // [B] arrival counters, zero before the launch; the kernel leaves them zero
     const float* offset;    // [C] or null: the statistics are those of x + offset[c] (a bias the tensor's producer
                             // left out), and shift takes scale * offset in, so scale * x + shift normalises x + offset
+    const float4* rec;      // or the producing layer's statistics records [B][G][slots] (launch_gn_merge)
+    int slots;
 };
 constexpr int kGnMaxChunks = 296;      // two blocks per SM on a 148-SM device
 // bytes of the partial records / of the whole scratch (records, then the arrival counters)
@@ -138,6 +150,31 @@ struct alignas(64) ConvTcPlan {
 };
 cudaError_t conv_tc_prepare(const ConvArgs& a, ConvTcPlan* plan);      // a.w must be the final packed-weight address
 cudaError_t launch_conv_tc(const ConvArgs& a, const ConvTcPlan& plan, unsigned int* status_word, cudaStream_t s);
+// ---- layers whose CTAs divide K among a cluster and leave statistics records (conv_cluster.cuh)
+constexpr int kSplitSmemMax = (228 * 1024 - 2 * 1024) / 2;     // two CTAs share an SM
+constexpr int kRecMergeSlots = 64;                             // up to here the consuming layer's CTAs merge the records themselves
+inline bool rec_groups_ok(int channels, int groups) {          // records of such groups can be written and merged
+    const int cpg = groups > 0 ? channels / groups : 0;
+    return groups > 0 && channels % groups == 0 && (cpg == 4 || cpg == 8 || cpg == 16);
+}
+cudaError_t launch_gn_merge(const GnArgs& a, cudaStream_t s);  // a.rec -> a.scale, a.shift
+
+// ---- single-precision convolution (conv_f32.cu)
+struct alignas(64) ConvF32Plan {
+    unsigned char tmap[128];    // weights, fp32 [tap][Cin][Cout]
+    int th, bn;                 // tile height, output channels per CTA (4: frame head)
+    int splits;                 // CTAs that share K (the cluster)
+    int n_w;                    // weight stages
+    int valid;
+};
+bool conv_f32_supported(const ConvArgs& a);
+bool conv_f32_choose(const ConvArgs& a, ConvF32Plan* plan);    // a.B = the handle's batch
+int conv_f32_slots(const ConvArgs& a, const ConvF32Plan& plan, int groups);
+cudaError_t conv_f32_prepare(const ConvArgs& a, ConvF32Plan* plan);
+cudaError_t launch_conv_f32(const ConvArgs& a, const ConvF32Plan& plan, unsigned int* status_word, cudaStream_t s);
+// OIHW 3x3 -> the sixteen pre-summed 2x2 taps of the phase-collapsed upsampling form, fp32 [16][Cin][Cout]
+cudaError_t launch_pack_weight_f32_phase(const void* w, int w_dtype, float* packed, int Cout, int Cin, cudaStream_t s);
+
 bool attn_tc_supported(const AttnArgs& a);
 size_t attn_tc_scratch_bytes(int B, int T, int C);
 // Launch-invariant state of the tensor-core attention: the TMA descriptors of q, k and the transposed v.
