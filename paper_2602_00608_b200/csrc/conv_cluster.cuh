@@ -1,9 +1,11 @@
 // Shared by the convolution kernels whose CTAs divide K among a thread-block cluster (conv_f32.cu, conv_split.cu):
 // the exchange of partial sums through distributed shared memory, and GroupNorm statistics as records.
 //
-//   * A CTA adds up and writes 1/S of its cluster's output rows (row = pixel of the tile).  Every CTA stores its partial
-//     of a row into the owner's exchange buffer with st.async, which counts the bytes on the owner's barrier: one
-//     wait, no cluster-wide barrier on the way.  The owner adds the partials in a fixed order (bitwise reproducible).
+//   * A CTA adds up and writes 1/S of its cluster's output rows (row = pixel of the tile).  Every CTA lays its partials
+//     out in its own shared memory, and one bulk copy per owner carries an owner's rows there and counts the bytes on the
+//     owner's barrier: one wait, no cluster-wide barrier on the way.  (16-byte st.async stores straight from registers
+//     took 2.3-3.7 us of a 12 us layer: 2048 packets per CTA.)  The owner adds the partials in a fixed order (bitwise
+//     reproducible).
 //   * While it writes its rows a CTA takes their statistics, and leaves one record (count, mean, sum of squared
 //     deviations) per group and warp share.  The CTAs of the layer that normalises merge the records of their own input
 //     channels (Chan's formula, a fixed order), or a small launch does where there are many.  The normalisation then
@@ -31,10 +33,11 @@ __device__ __forceinline__ uint32_t peer_addr(uint32_t smem_addr, uint32_t cta) 
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_addr), "r"(cta));
     return r;
 }
-// 16 bytes into a CTA of the cluster; their arrival is counted on that CTA's barrier `bar`
-__device__ __forceinline__ void st_peer_v4(uint32_t addr, uint32_t bar, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
-    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%2, %3, %4, %5}, [%1];"
-                 ::"r"(addr), "r"(bar), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
+// `bytes` (a multiple of 16) from this CTA's shared memory into another CTA's (cluster addresses); their arrival is
+// counted on that CTA's barrier `bar`
+__device__ __forceinline__ void copy_to_peer(uint32_t dst, uint32_t src, uint32_t bytes, uint32_t bar) {
+    asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                 ::"r"(dst), "r"(src), "r"(bytes), "r"(bar) : "memory");
 }
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
@@ -55,46 +58,91 @@ __device__ __forceinline__ bool wait_cluster(uint32_t bar, uint32_t parity, vola
     return true;
 }
 
-// Statistics of one group from its records: lanes of `L` (8 or 32, the same for the whole warp) share a group.
-// Deviations are from the first record's mean, so one round of loads and one of shuffles suffice.
-__device__ __forceinline__ void merge_group(const float4* rec, int slots, int l, int L, float eps, float& mean, float& rstd) {
-    const float ref = __ldcg(&rec->y);
-    float n = 0.f, s = 0.f, q = 0.f;
-#pragma unroll 4
-    for (int i = l; i < slots; i += L) {
-        const float4 r = __ldcg(rec + i);
-        const float d = r.y - ref, nd = r.x * d;
-        n += r.x;
-        s += nd;
-        q += fmaf(nd, d, r.z);
+// Statistics of one group from its records (count, mean, sum of squared deviations), for the whole warp the same number L
+// (8 or 32) of lanes to a group.  Deviations are from the first record's mean, so one round of loads and one of shuffles
+// suffice; a lane's first two records are loaded by `load`, so that they are on their way before other loads.
+struct GroupRecords {
+    float4 r0, r1;
+    float ref;
+    __device__ __forceinline__ void load(const float4* rec, int slots, int l, int L) {
+        ref = __ldcg(&rec->y);
+        r0 = r1 = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (l < slots) r0 = __ldcg(rec + l);
+        if (l + L < slots) r1 = __ldcg(rec + l + L);
     }
-    for (int d = L >> 1; d > 0; d >>= 1) {
-        n += __shfl_xor_sync(0xffffffffu, n, d);
-        s += __shfl_xor_sync(0xffffffffu, s, d);
-        q += __shfl_xor_sync(0xffffffffu, q, d);
+    __device__ __forceinline__ void merge(const float4* rec, int slots, int l, int L, float inv_n, float eps, float& mean, float& rstd) const {
+        const float d0 = r0.y - ref, d1 = r1.y - ref, n0 = r0.x * d0, n1 = r1.x * d1;
+        float s = n0 + n1, q = fmaf(n0, d0, r0.z) + fmaf(n1, d1, r1.z);
+        for (int i = l + 2 * L; i < slots; i += L) {
+            const float4 r = __ldcg(rec + i);
+            const float d = r.y - ref, nd = r.x * d;
+            s += nd;
+            q += fmaf(nd, d, r.z);
+        }
+        for (int d = L >> 1; d > 0; d >>= 1) {
+            s += __shfl_xor_sync(0xffffffffu, s, d);
+            q += __shfl_xor_sync(0xffffffffu, q, d);
+        }
+        const float dm = s * inv_n;
+        mean = ref + dm;
+        rstd = 1.f / sqrtf(fmaxf(fmaf(-dm, dm, q * inv_n), 0.f) + eps);
     }
-    const float inv_n = 1.f / n, dm = s * inv_n;
-    mean = ref + dm;
-    rstd = 1.f / sqrtf(fmaxf(fmaf(-dm, dm, q * inv_n), 0.f) + eps);
-}
+};
 
 // half * scale and half * shift of the input channels [c0, c0 + nch) of `frame`, from the producing layer's records, by
-// eight warps (w = 0..7); c0 and nch are multiples of the group size
-__device__ __forceinline__ void merge_input_stats(const ConvArgs& a, int frame, int c0, int nch, float half, float* s_scale,
-                                                  float* s_shift, int w, int lane) {
-    const int cpg = a.Cin / a.in_G, L = a.in_slots <= 16 ? 8 : 32, per = 32 / L, l = lane & (L - 1), ng = nch / cpg;
-    for (int g0 = w * per; g0 < ng; g0 += 8 * per) {
-        const int g = min(g0 + lane / L, ng - 1);            // (all lanes take part in the shuffles)
-        float mean, rstd;
-        merge_group(a.in_rec + ((size_t)frame * a.in_G + c0 / cpg + g) * a.in_slots, a.in_slots, l, L, a.in_eps, mean, rstd);
-        for (int i = l; i < cpg; i += L) {
-            const int c = g * cpg + i;
-            const float sc = __ldg(a.in_gamma + c0 + c) * rstd;
-            s_scale[c] = sc * half;
-            s_shift[c] = (__ldg(a.in_beta + c0 + c) - mean * sc) * half;
+// eight warps (w = 0..7); c0 and nch are multiples of the group size.  Everything but the records is ready before
+// the kernel before has finished: set up with `prepare`, then `load`, then (other loads issued) `finish`.
+struct InputStats {
+    const float4* rec;
+    int cpg, L, l, g, ng;
+    float inv_n, gamma[2], beta[2];
+    GroupRecords gr;
+    __device__ __forceinline__ void prepare(const ConvArgs& a, int frame, int c0, int nch, int w, int lane) {
+        cpg = a.Cin / a.in_G;
+        L = a.in_slots <= 16 ? 8 : 32;
+        l = lane & (L - 1);
+        ng = nch / cpg;
+        g = w * (32 / L) + lane / L;
+        inv_n = 1.f / ((float)a.in_pixels * (float)cpg);
+        rec = a.in_rec + ((size_t)frame * a.in_G + c0 / cpg + min(g, ng - 1)) * a.in_slots;
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            const int c = c0 + min(g, ng - 1) * cpg + l + i * L;
+            const bool on = l + i * L < cpg;
+            gamma[i] = on ? __ldg(a.in_gamma + c) : 0.f;
+            beta[i] = on ? __ldg(a.in_beta + c) : 0.f;
         }
     }
-}
+    __device__ __forceinline__ void load(const ConvArgs& a) { gr.load(rec, a.in_slots, l, L); }
+    __device__ __forceinline__ void finish(const ConvArgs& a, int c0, float half, float* s_scale, float* s_shift) {
+        const int step = 8 * (32 / L);
+        for (;;) {
+            float mean, rstd;
+            gr.merge(rec, a.in_slots, l, L, inv_n, a.in_eps, mean, rstd);
+            if (g < ng) {
+#pragma unroll
+                for (int i = 0; i < 2; ++i)
+                    if (l + i * L < cpg) {
+                        const float sc = gamma[i] * rstd;
+                        s_scale[g * cpg + l + i * L] = sc * half;
+                        s_shift[g * cpg + l + i * L] = (beta[i] - mean * sc) * half;
+                    }
+            }
+            if (g - (int)(threadIdx.x & 31) / L + step >= ng) break;     // (the same for the whole warp)
+            g += step;
+            rec += (size_t)step * a.in_slots;
+            const int gg = min(g, ng - 1);
+            rec -= (size_t)(g - gg) * a.in_slots;
+            gr.load(rec, a.in_slots, l, L);
+#pragma unroll
+            for (int i = 0; i < 2; ++i)
+                if (l + i * L < cpg) {
+                    gamma[i] = __ldg(a.in_gamma + c0 + gg * cpg + l + i * L);
+                    beta[i] = __ldg(a.in_beta + c0 + gg * cpg + l + i * L);
+                }
+        }
+    }
+};
 
 // The eight warps that write a CTA's rows: a warp has CPW four-channel columns of the BN channels (two at least: whole
 // 32-byte sectors), WC warps lie side by side and WR below one another.
@@ -142,21 +190,25 @@ __device__ __forceinline__ void finish_rows(const ConvArgs& a, float* rx, int np
     };
     load_residual(rg);
     ready();
-    float sum = 0.f, cnt = 0.f;
+    // statistics: deviations from a value of the group (the first one inside the image that this warp holds)
+    const int cpg = !HEAD && a.out_rec ? a.Cout / a.out_G : 4, lpg = min(cpg >> 2, CPW);        // four-channel columns of a group in this warp
+    const uint32_t peers = (lpg * RL >= 32 ? 0xffffffffu : ((1u << (lpg * RL & 31)) - 1u)) << (lane / (lpg * RL) * (lpg * RL));
+    float sum = 0.f, sq = 0.f, cnt = 0.f, pivot = 0.f;
 #pragma unroll 1
-    for (int l0 = rg; l0 < rpo; l0 += PRE * RSTEP) {
-        if (l0 != rg) load_residual(l0);
+    for (int l0 = rg - lane % RL; l0 < rpo; l0 += PRE * RSTEP) {
+        const int first = l0 + lane % RL;
+        if (first != rg) load_residual(first);
 #pragma unroll
         for (int i = 0; i < PRE; ++i) {
-            const int local = l0 + i * RSTEP;
-            if (local >= rpo) break;
-            int oy, ox;
-            const bool valid = locate(local, oy, ox);
+            const int local = first + i * RSTEP;
+            int oy = 0, ox = 0;
+            const bool on = local < rpo, valid = on && locate(local, oy, ox);
             const size_t pixel = ((size_t)frame * OH + oy) * OW + ox;
             float4 v = bias;
-            float* q = rx + local * RXS + cg * 4;
+            const float* q = rx + local * RXS + cg * 4;
 #pragma unroll 4
             for (int s = 0; s < nparts; ++s) {
+                if (!on) break;
                 const float4 p = *(const float4*)(q + (size_t)s * rpo * RXS);
                 v.x += p.x; v.y += p.y; v.z += p.z; v.w += p.w;
             }
@@ -180,38 +232,32 @@ __device__ __forceinline__ void finish_rows(const ConvArgs& a, float* rx, int np
                     v.x += res[i].x; v.y += res[i].y; v.z += res[i].z; v.w += res[i].w;
                     *(float4*)((float*)a.y + pixel * a.Cout + co) = v;
                 }
-                sum += (v.x + v.y) + (v.z + v.w);
-                cnt += 4.f;
             }
-            if (!HEAD && a.out_rec) *(float4*)q = v;         // for the second pass (this thread's own entry)
+            if (!HEAD && a.out_rec) {
+                if (l0 + i * RSTEP < RSTEP) {                // the warp's first rows
+                    const uint32_t m = __ballot_sync(0xffffffffu, valid) & peers;
+                    pivot = __shfl_sync(0xffffffffu, v.x, m ? __ffs(m) - 1 : lane);
+                }
+                if (valid) {
+                    const float d0 = v.x - pivot, d1 = v.y - pivot, d2 = v.z - pivot, d3 = v.w - pivot;
+                    sum += (d0 + d1) + (d2 + d3);
+                    sq += fmaf(d0, d0, d1 * d1) + fmaf(d2, d2, d3 * d3);
+                    cnt += 4.f;
+                }
+            }
         }
     }
     if (!HEAD && a.out_rec) {
-        const int cpg = a.Cout / a.out_G, lpg = min(cpg >> 2, CPW);                  // four-channel columns of a group in this warp
-        auto reduce = [&](float v) {
-#pragma unroll
-            for (int d = 1; d < RL; d <<= 1) v += __shfl_xor_sync(0xffffffffu, v, d);
-            if (lpg > 1) v += __shfl_xor_sync(0xffffffffu, v, RL);
-            if (CPW == 4 && lpg > 2) v += __shfl_xor_sync(0xffffffffu, v, 2 * RL);
-            return v;
-        };
-        sum = reduce(sum);
-        cnt = reduce(cnt);
-        const float mean = cnt > 0.f ? sum / cnt : 0.f;
-        float m2 = 0.f;
-#pragma unroll 2
-        for (int local = rg; local < rpo; local += RSTEP) {
-            int oy, ox;
-            if (locate(local, oy, ox)) {
-                const float4 v = *(const float4*)(rx + local * RXS + cg * 4);
-                const float d0 = v.x - mean, d1 = v.y - mean, d2 = v.z - mean, d3 = v.w - mean;
-                m2 += fmaf(d0, d0, d1 * d1) + fmaf(d2, d2, d3 * d3);
-            }
+        for (int d = 1; d < lpg * RL; d <<= 1) {
+            sum += __shfl_xor_sync(0xffffffffu, sum, d);
+            sq += __shfl_xor_sync(0xffffffffu, sq, d);
+            cnt += __shfl_xor_sync(0xffffffffu, cnt, d);
         }
-        m2 = reduce(m2);
-        if (lane % RL == 0 && (lane / RL) % lpg == 0) {
+        if ((lane & (lpg * RL - 1)) == 0) {
             const int side = max(cpg / (4 * CPW), 1), part = (w / WC) * side + (w % WC) % side;
-            a.out_rec[((size_t)frame * a.out_G + co / cpg) * a.out_slots + slot0 * (side * (8 / WC)) + part] = make_float4(cnt, mean, m2, 0.f);
+            const float dm = cnt > 0.f ? sum / cnt : 0.f;
+            a.out_rec[((size_t)frame * a.out_G + co / cpg) * a.out_slots + slot0 * (side * (8 / WC)) + part] =
+                make_float4(cnt, pivot + dm, fmaxf(fmaf(-dm, sum, sq), 0.f), 0.f);
         }
     }
 }

@@ -76,15 +76,16 @@ constexpr int kFTail = 2 * kMaxSlice * 4 + 128;              // scale / shift of
 
 template <int TH, int BN, int KIND>
 __global__ void __launch_bounds__(kThreads, 2)
-conv_f32_kernel(const ConvArgs a, const int S, const int n_w, const __grid_constant__ CUtensorMap tm_w, unsigned int* status) {
+conv_f32_kernel(const ConvArgs a, const int S, const int n_w, const int ops_floats, const __grid_constant__ CUtensorMap tm_w, unsigned int* status) {
     using C = FCfg<TH, BN, KIND>;
     constexpr bool HEAD = BN < 32;
     constexpr int KH = C::KH, CS = C::CS, KT = C::KT;
     extern __shared__ uint8_t smem_raw[];
     float* s_in = (float*)(((uintptr_t)smem_raw + 127) & ~(uintptr_t)127);           // two input chunks
     float* s_w = s_in + (2 * C::IN_FLOATS + 31) / 32 * 32;                           // n_w weight stages (head: the whole slice)
-    float* rx = s_w + n_w * C::W_FLOATS;
-    float* s_scale = rx + C::RX_FLOATS;
+    float* rx = s_in + ops_floats;                                                   // partials of this CTA's rows
+    float* part = s_in;                                                              // this CTA's partials, once every thread is done with its operands
+    float* s_scale = s_in + ops_floats + C::RX_FLOATS;
     float* s_shift = s_scale + kMaxSlice;
     FBars* bars = (FBars*)(s_shift + kMaxSlice);
     volatile uint32_t* abort_flag = &bars->abort_flag;
@@ -117,7 +118,7 @@ conv_f32_kernel(const ConvArgs a, const int S, const int n_w, const __grid_const
         bars->abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         fence_proxy_async_smem();
-        mbar_arrive_expect_tx(smem_u32(&bars->rx_full), KT * TH * kTW * BN * 4);     // this CTA's rows from all S * KT partials
+        mbar_arrive_expect_tx(smem_u32(&bars->rx_full), C::RX_FLOATS * 4);           // this CTA's rows from all S * KT partials
         if (!HEAD)
             for (int u = 0; u < min(units, n_w); ++u) load_weights(u);
     }
@@ -131,9 +132,8 @@ conv_f32_kernel(const ConvArgs a, const int S, const int n_w, const __grid_const
         }
     }
     __syncthreads();
-    cluster_arrive();                                        // (waited for before anything is sent to another CTA)
+    if (S > 1) cluster_arrive();                             // (waited for before anything is sent to another CTA)
     griddep_launch();
-    griddep_wait();
 
     // ---- input: entry e of a thread is (pixel, four channels) of the tile
     constexpr int NE = (C::RH * C::RW * (kChunk / 4) + kThreads - 1) / kThreads;
@@ -158,9 +158,13 @@ conv_f32_kernel(const ConvArgs a, const int S, const int n_w, const __grid_const
             if (on && (vm >> e & 1u)) raw[e] = __ldg((const float4*)(src[e] + u * kChunk));
         }
     };
+    InputStats st;
+    if (a.in_rec) st.prepare(a, frame, c_first, nch, tid >> 5, lane);
+    griddep_wait();                                          // everything above is arithmetic, weights and parameters
+    if (a.in_rec) st.load(a);
     fetch(0);
     if (prologue) {
-        if (a.in_rec) merge_input_stats(a, frame, c_first, nch, 1.f, s_scale, s_shift, tid >> 5, lane);
+        if (a.in_rec) st.finish(a, c_first, 1.f, s_scale, s_shift);
         else
             for (int c = tid; c < nch; c += kThreads) {
                 s_scale[c] = __ldg(a.scale + (size_t)frame * a.Cin + c_first + c);
@@ -239,21 +243,27 @@ conv_f32_kernel(const ConvArgs a, const int S, const int n_w, const __grid_const
     }
 
     // ---- partials to the CTA that owns the row (row R of the tile's TH x 8 belongs to CTA R / rpo)
-    __syncwarp();
-    cluster_wait();
     const int rpo = TH * kTW / S;
-    {
-        const uint32_t rx0 = smem_u32(rx), bar0 = smem_u32(&bars->rx_full);
+    __syncthreads();                                         // every thread is done with the operands
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const int R = row * kTW + i, owner = R / rpo, local = R - owner * rpo;
-            const float2 lo = halves(acc[i][0]), hi = halves(acc[i][1]);
-            st_peer_v4(peer_addr(rx0 + (uint32_t)((((rank * KT + kt) * rpo + local) * C::RXS + cg * 4) * 4), (uint32_t)owner), peer_addr(bar0, (uint32_t)owner),
-                       __float_as_uint(lo.x), __float_as_uint(lo.y), __float_as_uint(hi.x), __float_as_uint(hi.y));
-        }
+    for (int i = 0; i < 8; ++i) {
+        const float2 lo = halves(acc[i][0]), hi = halves(acc[i][1]);
+        *(float4*)(part + ((kt * TH + row) * kTW + i) * C::RXS + cg * 4) = make_float4(lo.x, lo.y, hi.x, hi.y);
     }
-    __syncwarp();
-    cluster_arrive();
+    if (S > 1) {
+        fence_proxy_async_smem();
+        __syncthreads();
+        cluster_wait();
+        if (tid < S * KT) {
+            const int owner = tid / KT, q = tid % KT;
+            copy_to_peer(peer_addr(smem_u32(rx + (rank * KT + q) * rpo * C::RXS), (uint32_t)owner), smem_u32(part + (q * TH * kTW + owner * rpo) * C::RXS),
+                         (uint32_t)(rpo * C::RXS * 4), peer_addr(smem_u32(&bars->rx_full), (uint32_t)owner));
+        }
+        __syncwarp();
+    } else {
+        rx = part;
+        __syncthreads();
+    }
     finish_rows<BN>(a, rx, S * KT, rpo, tid, frame, n0, KIND == KPHASE ? 2 * H : H, KIND == KPHASE ? 2 * W : W,
                     (KIND == KPHASE ? tile * 4 + par : tile) * S + rank,
                     [&](int local, int& oy, int& ox) -> bool {
@@ -264,15 +274,23 @@ conv_f32_kernel(const ConvArgs a, const int S, const int n_w, const __grid_const
                         if (KIND == KPHASE) { oy = 2 * oy + (par >> 1); ox = 2 * ox + (par & 1); }
                         return valid;
                     },
-                    [&] { (void)wait_cluster(smem_u32(&bars->rx_full), 0, abort_flag); });
+                    [&] {
+                        if (S > 1) {
+                            (void)wait_cluster(smem_u32(&bars->rx_full), 0, abort_flag);
+                            __syncwarp();
+                            cluster_arrive();                // what is sent to this CTA has landed
+                        }
+                    });
     if (tid == 0 && bars->abort_flag && status) {
         if (atomicCAS(status, 0u, kStatusConvTimeout) == 0u) {
             status[1] = blockIdx.x;
             status[2] = (uint32_t)BN;
         }
     }
-    __syncwarp();
-    cluster_wait();                                          // every CTA has sent all it sends
+    if (S > 1) {                                             // the sources of this CTA's copies may go
+        __syncwarp();
+        cluster_wait();
+    }
 }
 
 // [16 taps][Cin][Cout]: parity * 4 + dy * 2 + dx, each the sum of the 3x3 taps that read the same source pixel (see conv_tc.cu)
@@ -297,9 +315,14 @@ constexpr int kMaxDevices = 64;
 std::mutex g_mu;
 
 template <int TH, int BN, int KIND>
+int ops_floats(int n_w) {                                    // operand stages; the partials lie over them
+    using C = FCfg<TH, BN, KIND>;
+    return std::max((2 * C::IN_FLOATS + 31) / 32 * 32 + n_w * C::W_FLOATS, C::RX_FLOATS);
+}
+template <int TH, int BN, int KIND>
 int smem_bytes(int n_w) {
     using C = FCfg<TH, BN, KIND>;
-    return ((2 * C::IN_FLOATS + 31) / 32 * 32 + n_w * C::W_FLOATS + C::RX_FLOATS) * 4 + kFTail + 128;
+    return (ops_floats<TH, BN, KIND>(n_w) + C::RX_FLOATS) * 4 + kFTail + 128;
 }
 
 template <int TH, int BN, int KIND>
@@ -338,7 +361,7 @@ cudaError_t launch_one(const ConvArgs& a, const ConvF32Plan& p, unsigned int* st
     }
     cfg.attrs = attr;
     cfg.numAttrs = na;
-    return cudaLaunchKernelEx(&cfg, kern, a, p.splits, p.n_w, *(const CUtensorMap*)p.tmap, status);
+    return cudaLaunchKernelEx(&cfg, kern, a, p.splits, p.n_w, ops_floats<TH, BN, KIND>(p.n_w), *(const CUtensorMap*)p.tmap, status);
 }
 
 int kind_of(const ConvArgs& a) { return a.upsample == 2 ? KPHASE : (a.ksize == 1 ? K1X1 : K3X3); }
@@ -439,8 +462,11 @@ __global__ void __launch_bounds__(256) gn_merge_kernel(GnArgs a) {
     const int g = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31, n = blockIdx.y;
     if (g >= a.G) return;
     const int cpg = a.C / a.G;
+    const float4* rec = a.rec + ((size_t)n * a.G + g) * a.slots;
+    GroupRecords gr;
     float mean, rstd;
-    merge_group(a.rec + ((size_t)n * a.G + g) * a.slots, a.slots, lane, 32, a.eps, mean, rstd);
+    gr.load(rec, a.slots, lane, 32);
+    gr.merge(rec, a.slots, lane, 32, 1.f / ((float)a.P * (float)cpg), a.eps, mean, rstd);
     for (int i = lane; i < cpg; i += 32) {
         const int c = g * cpg + i;
         const float sc = __ldg(a.gamma + c) * rstd;

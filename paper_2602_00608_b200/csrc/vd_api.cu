@@ -24,6 +24,7 @@ struct Step {
     AttnArgs attn;
     IngestArgs ing;
     ConvTcPlan tc;
+    ConvSplitPlan split;         // valid: the layer runs on conv_split.cu
     ConvF32Plan f32;             // valid: the layer runs on conv_f32.cu
     AttnTcPlan attn_tc;
     bool skip;                   // statistics that the consuming layer merges from its producer's records: no launch
@@ -224,9 +225,12 @@ class Planner {
         if (phase) a.upsample = 2;
         const bool tc = tc_on && conv_tc_supported(probe);
         // fp32 layers: the direct kernel remains for the bf16 layout's cross-check path (and the 9-tap upsampling form)
+        probe.B = cfg_.max_batch;
+        probe.upsample = a.upsample;
+        const bool split = tc && !(cfg_.flags & VD_FLAG_FUSED_STATS) && conv_split_choose(probe, &s.split);
+        s.split.valid = split ? 1 : 0;
         bool f32 = false;
         if (!tc && !(bf16() && (cfg_.flags & VD_FLAG_FORCE_SIMT))) {
-            probe.B = cfg_.max_batch;
             probe.upsample = upsample ? ((cfg_.flags & VD_FLAG_UPSAMPLE_9TAP) ? 1 : 2) : 0;
             f32 = conv_f32_choose(probe, &s.f32);
             if (f32 && upsample) { phase = true; a.upsample = 2; }
@@ -262,7 +266,7 @@ class Planner {
         const size_t b2_off = a.bias2 ? (size_t)((const char*)a.bias2 - base_) : kNone;
         const size_t w2_off = a.w2 ? (size_t)((const char*)a.w2 - base_) : kNone;
         if (!y_is_frames) {
-            if (tc && want_defer && !(cfg_.flags & VD_FLAG_FUSED_STATS)) {
+            if (tc && want_defer && !split && !(cfg_.flags & VD_FLAG_FUSED_STATS)) {
                 const size_t v = alloc((size_t)Cout * 4);
                 h_->folds.push_back({v, pres, cw.b_off, b2_off, px2 != kNone ? w2_off : kNone, px2, Cin2, Cout});
                 a.bias = nullptr;
@@ -280,10 +284,10 @@ class Planner {
         }
         // ---- statistics as records (conv_cluster.cuh): where there are few, this layer merges them itself and the step
         // just planned needs no launch
-        if (f32 && prologue) {
+        if ((f32 || split) && prologue) {
             Step& g = h_->steps.back();
             if (g.kind == VD_STEP_GN_STATS && g.gn.rec && g.gn.slots <= kRecMergeSlots) {
-                a.in_rec = g.gn.rec; a.in_slots = g.gn.slots;
+                a.in_rec = g.gn.rec; a.in_slots = g.gn.slots; a.in_pixels = g.gn.P;
                 a.in_gamma = g.gn.gamma; a.in_beta = g.gn.beta; a.in_G = g.gn.G; a.in_eps = g.gn.eps;
                 a.scale = a.shift = nullptr;
                 g.skip = true;
@@ -293,8 +297,8 @@ class Planner {
         if (!y_is_frames) rec_.erase(y_off);
         const bool records = !no_records_;
         no_records_ = false;
-        if (f32 && records && !y_is_frames && rec_groups_ok(Cout, cfg_.norm_groups)) {
-            const int slots = conv_f32_slots(probe, s.f32, cfg_.norm_groups);
+        if ((f32 || split) && records && !y_is_frames && rec_groups_ok(Cout, cfg_.norm_groups)) {
+            const int slots = split ? conv_split_slots(probe, s.split, cfg_.norm_groups) : conv_f32_slots(probe, s.f32, cfg_.norm_groups);
             rec_toggle_ ^= 1;
             a.out_rec = ptr<float4>(rec_buf_[rec_toggle_]);
             a.out_slots = slots;
@@ -596,6 +600,7 @@ cudaError_t launch_step(const vd_handle_s* h, const Step& st, int B, const void*
             ConvArgs a = st.conv;
             a.B = B;
             if (!a.y) a.y = frames;
+            if (st.split.valid) return launch_conv_split(a, st.split, status, s);
             if (st.f32.valid) return launch_conv_f32(a, st.f32, status, s);
             return st.use_tc ? launch_conv_tc(a, st.tc, status, s) : launch_conv_simt(a, s);
         }
@@ -756,7 +761,7 @@ vd_status vd_create(const vd_config* cfg, const vd_tensor* weights, int32_t n_we
         if (st.kind == VD_STEP_CONV && st.use_tc) {
             ConvArgs pa = st.conv;
             pa.B = cfg->max_batch;
-            e = conv_tc_prepare(pa, &st.tc);
+            e = st.split.valid ? conv_split_prepare(pa, &st.split) : conv_tc_prepare(pa, &st.tc);
             if (e == cudaErrorInvalidConfiguration && pa.upsample == 2) {
                 delete h;
                 return fail(nullptr, VD_ERR_UNSUPPORTED, "this device cannot co-schedule the CTA pairs of the phase-collapsed "

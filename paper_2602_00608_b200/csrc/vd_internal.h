@@ -49,7 +49,7 @@ struct ConvArgs {
     const float4* in_rec;        // or null
     const float* in_gamma;       // [Cin]
     const float* in_beta;        // [Cin]
-    int in_slots, in_G;
+    int in_slots, in_G, in_pixels;   // in_pixels: pixels the statistics are over
     float in_eps;
     float4* out_rec;             // or null
     int out_slots, out_G;
@@ -174,6 +174,26 @@ cudaError_t conv_f32_prepare(const ConvArgs& a, ConvF32Plan* plan);
 cudaError_t launch_conv_f32(const ConvArgs& a, const ConvF32Plan& plan, unsigned int* status_word, cudaStream_t s);
 // OIHW 3x3 -> the sixteen pre-summed 2x2 taps of the phase-collapsed upsampling form, fp32 [16][Cin][Cout]
 cudaError_t launch_pack_weight_f32_phase(const void* w, int w_dtype, float* packed, int Cout, int Cin, cudaStream_t s);
+
+// ---- tcgen05 convolution divided along K for small images (conv_split.cu)
+struct ConvSplitShape {
+    int splits;                 // CTAs that share K (the cluster)
+    int n_a, n_b;               // operand and weight stages
+    int tail_off;               // shared-memory offset of what follows the stages
+    int w_rows;                 // packed weight rows per tap
+};
+struct alignas(64) ConvSplitPlan {
+    unsigned char tmap[128];    // packed weights
+    unsigned char tmap2[128];   // weights of the fused shortcut
+    unsigned char tmap_x2[128]; // input of the fused shortcut
+    ConvSplitShape shape;
+    int bn, smem, batch, valid;
+};
+bool conv_split_supported(const ConvArgs& a);
+bool conv_split_choose(const ConvArgs& a, ConvSplitPlan* plan);   // a.B = the handle's batch; false: conv_tc.cu is the faster one
+int conv_split_slots(const ConvArgs& a, const ConvSplitPlan& plan, int groups);
+cudaError_t conv_split_prepare(const ConvArgs& a, ConvSplitPlan* plan);
+cudaError_t launch_conv_split(const ConvArgs& a, const ConvSplitPlan& plan, unsigned int* status_word, cudaStream_t s);
 
 bool attn_tc_supported(const AttnArgs& a);
 size_t attn_tc_scratch_bytes(int B, int T, int C);
