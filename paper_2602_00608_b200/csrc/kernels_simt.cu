@@ -243,6 +243,93 @@ __global__ void __launch_bounds__(kGnThreads, 2) gn_stats_kernel(GnArgs a, int c
     if (threadIdx.x == 0) a.counters[n] = 0u;        // ready for the next launch
 }
 
+// The same statistics for tensors small enough that the pass above is mostly its own latency: a cluster of eight CTAs
+// takes 16 channels (one, two or four groups) of one sample, an eighth of its pixels each; the eight sums meet in the first
+// CTA's shared memory, and that CTA writes scale and shift: no records in memory, no arrival counter, no second reading
+// phase.  Sums are of (x - K) with the reference value K of the pass above.
+constexpr int kGnSplit = 8;
+template <typename T, int SPG>                       // SPG: four-channel slots per group (1, 2, 4)
+__global__ void __cluster_dims__(kGnSplit, 1, 1) __launch_bounds__(1024 / SPG) gn_cluster_kernel(GnArgs a) {
+    constexpr int THREADS = 1024 / SPG, NG = 4 / SPG, ROWS = THREADS / 4, U = 8;
+    __shared__ float2 s_warp[THREADS / 32][NG], s_all[NG][kGnSplit];
+    griddep_launch();
+    const int rank = blockIdx.x % kGnSplit, n = blockIdx.y, lane = threadIdx.x & 31;
+    const int slot = threadIdx.x & 3, row = threadIdx.x >> 2, c0 = (int)blockIdx.x / kGnSplit * 16, cg = c0 + slot / SPG * (SPG * 4);
+    const int p0 = (int)((long long)a.P * rank / kGnSplit), p1 = (int)((long long)a.P * (rank + 1) / kGnSplit);
+    const T* x = (const T*)a.x + (size_t)n * a.P * a.C;
+    float off_k = 0.f;
+    float4 off_c = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (a.offset) {
+        const float4 og = __ldg((const float4*)(a.offset + cg));
+        off_k = 0.25f * ((og.x + og.y) + (og.z + og.w));
+        off_c = __ldg((const float4*)(a.offset + c0 + slot * 4));
+    }
+    griddep_wait();
+    float kv[4];
+    load4<T>(x + (size_t)(a.P / 2) * a.C + cg, kv);
+    const T* q = x + (size_t)(p0 + row) * a.C + c0 + slot * 4;
+    const size_t step = (size_t)ROWS * a.C;
+    float s = 0.f, ss = 0.f, k = 0.f, ko[4] = {0.f, 0.f, 0.f, 0.f};
+    bool first = true;
+    for (int p = p0 + row; p < p1; p += U * ROWS, q += U * step) {
+        float u[U][4];
+#pragma unroll
+        for (int j = 0; j < U; ++j) {
+            u[j][0] = u[j][1] = u[j][2] = u[j][3] = 0.f;
+            if (p + j * ROWS < p1) load4<T>(q + j * step, u[j]);
+        }
+        if (first) {                                 // (its load is in flight together with the first of the others)
+            k = 0.25f * ((kv[0] + kv[1]) + (kv[2] + kv[3])) + off_k;
+            ko[0] = k - off_c.x; ko[1] = k - off_c.y; ko[2] = k - off_c.z; ko[3] = k - off_c.w;
+            first = false;
+        }
+#pragma unroll
+        for (int j = 0; j < U; ++j)
+            if (p + j * ROWS < p1)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const float d = u[j][e] - ko[e];
+                    s += d;
+                    ss = fmaf(d, d, ss);
+                }
+    }
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) {
+        if (d >= 4 || d < SPG) {                     // (lane bits 0 and 1 are the slot)
+            s += __shfl_xor_sync(0xffffffffu, s, d);
+            ss += __shfl_xor_sync(0xffffffffu, ss, d);
+        }
+    }
+    if (lane < 4 && lane % SPG == 0) s_warp[threadIdx.x / 32][lane / SPG] = make_float2(s, ss);
+    __syncthreads();
+    if (threadIdx.x < NG) {
+        float2 t = s_warp[0][threadIdx.x];
+#pragma unroll 8
+        for (int w = 1; w < THREADS / 32; ++w) { t.x += s_warp[w][threadIdx.x].x; t.y += s_warp[w][threadIdx.x].y; }
+        uint32_t dst;
+        asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(dst) : "r"((uint32_t)__cvta_generic_to_shared(&s_all[threadIdx.x][rank])));
+        asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(dst), "f"(t.x), "f"(t.y) : "memory");
+    }
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    if (rank != 0 || threadIdx.x >= 16) return;
+    const int g = threadIdx.x / (SPG * 4), c = c0 + threadIdx.x;
+    float2 t = s_all[g][0];
+#pragma unroll
+    for (int r = 1; r < kGnSplit; ++r) { t.x += s_all[g][r].x; t.y += s_all[g][r].y; }
+    load4<T>(x + (size_t)(a.P / 2) * a.C + c0 + g * SPG * 4, kv);
+    float kk = 0.25f * ((kv[0] + kv[1]) + (kv[2] + kv[3]));
+    if (a.offset) {
+        const float4 og = __ldg((const float4*)(a.offset + c0 + g * SPG * 4));
+        kk += 0.25f * ((og.x + og.y) + (og.z + og.w));
+    }
+    const float inv_n = 1.f / ((float)a.P * (float)(SPG * 4));
+    const float md = t.x * inv_n, var = fmaxf(fmaf(-md, md, t.y * inv_n), 0.f);
+    const float sc = __ldg(a.gamma + c) * (1.f / sqrtf(var + a.eps));
+    a.scale[(size_t)n * a.C + c] = sc;
+    a.shift[(size_t)n * a.C + c] = __ldg(a.beta + c) - (kk + md - (a.offset ? __ldg(a.offset + c) : 0.f)) * sc;
+}
+
 // ------------------------------------------------------------------------------- direct conv
 // Block = TH x TW output pixels x CT output channels; input channels are consumed KC at a time
 // through shared memory (the transformed input tile with its halo, and the weight slice).
@@ -464,6 +551,20 @@ cudaError_t launch_ingest(const IngestArgs& a, cudaStream_t s) {
 
 cudaError_t launch_gn_stats(const GnArgs& a, cudaStream_t s) {
     if (a.C % 4 != 0 || a.C / 4 > kGnThreads || a.G > kGnThreads || (a.C / a.G) % 4 != 0) return cudaErrorInvalidValue;
+    const int spg = a.C / a.G / 4;
+    // Up to here the clusters' few CTAs read a sample faster than the other kernel's phases run (the line depends on the
+    // sample size only, like everything below).  Measured by itself, one sample, us, other kernel -> this one, a 2 us memset
+    // included in both: 512 channels 32x32 10.3 -> 6.3, 60x90 10.4 -> 8.2; 256 channels 128x128 12.2 -> 8.6, bf16 240x360
+    // 14.5 -> 20.7; 128 channels 296x424 14.5 -> 16.5.  Whole decodes: 424x296 1565 -> 1536 us with the line at 3 million
+    // elements, 1567 at 12 million and 1666 at 20 million (the next layer's lines leave L2 later).
+    if (a.C % 16 == 0 && (spg == 1 || spg == 2 || spg == 4) && (long long)a.P * a.C <= 3000000) {
+        const dim3 grid(a.C / 16 * kGnSplit, a.B), block(1024 / spg);
+        if (a.dtype == VD_BF16)
+            return spg == 4 ? launch_pdl(gn_cluster_kernel<__nv_bfloat16, 4>, grid, block, 0, s, a)
+                 : spg == 2 ? launch_pdl(gn_cluster_kernel<__nv_bfloat16, 2>, grid, block, 0, s, a) : launch_pdl(gn_cluster_kernel<__nv_bfloat16, 1>, grid, block, 0, s, a);
+        return spg == 4 ? launch_pdl(gn_cluster_kernel<float, 4>, grid, block, 0, s, a)
+             : spg == 2 ? launch_pdl(gn_cluster_kernel<float, 2>, grid, block, 0, s, a) : launch_pdl(gn_cluster_kernel<float, 1>, grid, block, 0, s, a);
+    }
     // chunks per sample depend on the sample size only (so a frame's statistics, and with them
     // the frame, do not depend on the batch it is decoded in): at least 32 pixels per chunk
     int ppc = max(32, (a.P + kGnMaxChunks - 1) / kGnMaxChunks);
