@@ -90,9 +90,9 @@ struct GroupRecords {
 };
 
 // half * scale and half * shift of the input channels [c0, c0 + nch) of `frame`, from the producing layer's records, by
-// eight warps (w = 0..7); c0 and nch are multiples of the group size.  Everything but the records is ready before
+// NW warps (w = 0..NW - 1); c0 and nch are multiples of the group size.  Everything but the records is ready before
 // the kernel before has finished: set up with `prepare`, then `load`, then (other loads issued) `finish`.
-struct InputStats {
+template <int NW> struct InputStatsOf {
     const float4* rec;
     int cpg, L, l, g, ng;
     float inv_n, gamma[2], beta[2];
@@ -115,7 +115,7 @@ struct InputStats {
     }
     __device__ __forceinline__ void load(const ConvArgs& a) { gr.load(rec, a.in_slots, l, L); }
     __device__ __forceinline__ void finish(const ConvArgs& a, int c0, float half, float* s_scale, float* s_shift) {
-        const int step = 8 * (32 / L);
+        const int step = NW * (32 / L);
         for (;;) {
             float mean, rstd;
             gr.merge(rec, a.in_slots, l, L, inv_n, a.in_eps, mean, rstd);
@@ -144,6 +144,8 @@ struct InputStats {
     }
 };
 
+using InputStats = InputStatsOf<8>;
+
 // The eight warps that write a CTA's rows: a warp has CPW four-channel columns of the BN channels (two at least: whole
 // 32-byte sectors), WC warps lie side by side and WR below one another.
 template <int BN> struct Split8 {
@@ -156,14 +158,13 @@ inline int rec_parts(int bn, int cpg) {
 }
 
 // Adds up the `nparts` partials of this CTA's `rpo` rows, adds bias and residual, writes the output and the statistics
-// records.  rx: [nparts][rpo][BN + 4] floats (head: BN).  ptid: 0..255.  locate(local row, oy, ox) gives the row's output pixel and
+// records.  rx: [nparts][rpo][RXS] floats, 16-byte piece c of a row at c ^ swizzle(row).  ptid: 0..255.  locate(local row, oy, ox) gives the row's output pixel and
 // whether it exists; ready() returns when the partials have arrived (the residual is on its way by then).
 // A thread takes four channels (cg) of every RSTEP-th row, so a warp's share of a group comes from shuffles alone.  BN < 32: the frame head (planes or packed pixels of a.Cout channels).
-template <int BN, class Locate, class Ready>
+template <int BN, int RXS, class Locate, class Swizzle, class Ready>
 __device__ __forceinline__ void finish_rows(const ConvArgs& a, float* rx, int nparts, int rpo, int ptid, int frame, int n0, int OH, int OW,
-                                            int slot0, Locate locate, Ready ready) {
+                                            int slot0, Locate locate, Swizzle swizzle, Ready ready) {
     constexpr bool HEAD = BN < 32;
-    constexpr int RXS = HEAD ? BN : BN + 4;
     constexpr int CPW = HEAD ? 1 : Split8<HEAD ? 64 : BN>::CPW, WC = HEAD ? 1 : Split8<HEAD ? 64 : BN>::WC, RL = 32 / CPW;
     constexpr int RSTEP = HEAD ? kFinishThreads / (BN / 4) : RL * (8 / WC);
     const int w = ptid >> 5, lane = ptid & 31;
@@ -205,7 +206,7 @@ __device__ __forceinline__ void finish_rows(const ConvArgs& a, float* rx, int np
             const bool on = local < rpo, valid = on && locate(local, oy, ox);
             const size_t pixel = ((size_t)frame * OH + oy) * OW + ox;
             float4 v = bias;
-            const float* q = rx + local * RXS + cg * 4;
+            const float* q = rx + local * RXS + (cg ^ swizzle(local)) * 4;
 #pragma unroll 4
             for (int s = 0; s < nparts; ++s) {
                 if (!on) break;

@@ -53,6 +53,11 @@ __device__ __forceinline__ void tma_load_3d(uint32_t dst, const void* tmap, int 
                  ::"r"(dst), "l"(tmap), "r"(x), "r"(y), "r"(z), "r"(bar) : "memory");
 }
 
+__device__ __forceinline__ unsigned long long pair(float x, float y) {
+    unsigned long long d;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(x), "f"(y));
+    return d;
+}
 struct FBars {
     uint64_t w_full[kMaxW];
     uint64_t rx_full;
@@ -67,12 +72,16 @@ template <int TH, int BN, int KIND> struct FCfg {
     static constexpr int KT = kThreads / (TH * (BN / 4));                // thread groups along K
     static constexpr int IN_FLOATS = kChunk * CS;
     static constexpr int W_FLOATS = TAPS * kChunk * BN;
-    static constexpr int RXS = BN < 32 ? BN : BN + 4;                    // floats per row of the exchange buffer
-    static constexpr int RX_FLOATS = KT * TH * kTW * RXS;
-    static_assert(KT >= 1 && kThreads % (TH * (BN / 4)) == 0 && CS % 4 == 0, "thread layout");
+    static constexpr int RX_FLOATS = TH * kTW * BN;                      // one partial of the tile
+    static constexpr int PART_FLOATS = KT / 2 * RX_FLOATS;               // partials of half the K groups at a time
+    static_assert(KT >= 2 && kThreads % (TH * (BN / 4)) == 0 && CS % 4 == 0, "thread layout");
 };
 constexpr int kMaxSlice = 512;                               // input channels of one CTA
 constexpr int kFTail = 2 * kMaxSlice * 4 + 128;              // scale / shift of the slice, barriers
+
+// A partial lies in memory as rows (pixels) of BN floats whose 16-byte pieces are permuted by the row, so that neither the
+// threads that write it (eight tile rows side by side) nor those that read it (eight pixels of a row) meet on a bank.
+template <int BN> __device__ __forceinline__ int piece(int R) { return BN < 32 ? 0 : (R ^ (R >> 3)) & 7; }
 
 template <int TH, int BN, int KIND>
 __global__ void __launch_bounds__(kThreads, 2)
@@ -85,7 +94,7 @@ conv_f32_kernel(const ConvArgs a, const int S, const int n_w, const int ops_floa
     float* s_w = s_in + (2 * C::IN_FLOATS + 31) / 32 * 32;                           // n_w weight stages (head: the whole slice)
     float* rx = s_in + ops_floats;                                                   // partials of this CTA's rows
     float* part = s_in;                                                              // this CTA's partials, once every thread is done with its operands
-    float* s_scale = s_in + ops_floats + C::RX_FLOATS;
+    float* s_scale = s_in + ops_floats + (S > 1 ? C::RX_FLOATS : 0);
     float* s_shift = s_scale + kMaxSlice;
     FBars* bars = (FBars*)(s_shift + kMaxSlice);
     volatile uint32_t* abort_flag = &bars->abort_flag;
@@ -242,45 +251,66 @@ conv_f32_kernel(const ConvArgs a, const int S, const int n_w, const int ops_floa
         }
     }
 
-    // ---- partials to the CTA that owns the row (row R of the tile's TH x 8 belongs to CTA R / rpo)
-    const int rpo = TH * kTW / S;
-    __syncthreads();                                         // every thread is done with the operands
+    // ---- the K groups' partials are added in halves (a fixed order); the first group keeps the sum
+    auto at = [&](int slab, int i) -> float4* {
+        const int R = row * kTW + i;
+        return (float4*)(part + (slab * TH * kTW + R) * BN + (cg ^ piece<BN>(R)) * 4);
+    };
+    auto put = [&](int slab) {
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        const float2 lo = halves(acc[i][0]), hi = halves(acc[i][1]);
-        *(float4*)(part + ((kt * TH + row) * kTW + i) * C::RXS + cg * 4) = make_float4(lo.x, lo.y, hi.x, hi.y);
+        for (int i = 0; i < 8; ++i) {
+            const float2 lo = halves(acc[i][0]), hi = halves(acc[i][1]);
+            *at(slab, i) = make_float4(lo.x, lo.y, hi.x, hi.y);
+        }
+    };
+#pragma unroll 1
+    for (int half = KT / 2; half >= 1; half >>= 1) {
+        __syncthreads();                                     // every thread is done with the operands / with the slabs before
+        if (kt >= half && kt < 2 * half) put(kt - half);
+        __syncthreads();
+        if (kt < half) {
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const float4 v = *at(kt, i);
+                const float2 lo = halves(acc[i][0]), hi = halves(acc[i][1]);
+                acc[i][0] = pair(lo.x + v.x, lo.y + v.y);
+                acc[i][1] = pair(hi.x + v.z, hi.y + v.w);
+            }
+        }
     }
+    if (kt == 0) put(0);                                     // (where it has just read itself)
+    // ---- row R of the tile's TH x 8 belongs to CTA R / rpo of the cluster
+    const int rpo = TH * kTW / S;
     if (S > 1) {
-        fence_proxy_async_smem();
+        if (kt == 0) fence_proxy_async_smem();
         __syncthreads();
         cluster_wait();
-        if (tid < S * KT) {
-            const int owner = tid / KT, q = tid % KT;
-            copy_to_peer(peer_addr(smem_u32(rx + (rank * KT + q) * rpo * C::RXS), (uint32_t)owner), smem_u32(part + (q * TH * kTW + owner * rpo) * C::RXS),
-                         (uint32_t)(rpo * C::RXS * 4), peer_addr(smem_u32(&bars->rx_full), (uint32_t)owner));
-        }
+        if (tid < S)
+            copy_to_peer(peer_addr(smem_u32(rx + rank * rpo * BN), (uint32_t)tid), smem_u32(part + tid * rpo * BN), (uint32_t)(rpo * BN * 4),
+                         peer_addr(smem_u32(&bars->rx_full), (uint32_t)tid));
         __syncwarp();
     } else {
         rx = part;
         __syncthreads();
     }
-    finish_rows<BN>(a, rx, S * KT, rpo, tid, frame, n0, KIND == KPHASE ? 2 * H : H, KIND == KPHASE ? 2 * W : W,
-                    (KIND == KPHASE ? tile * 4 + par : tile) * S + rank,
-                    [&](int local, int& oy, int& ox) -> bool {
-                        const int R = rank * rpo + local;
-                        oy = ty + R / kTW;
-                        ox = tx + R % kTW;
-                        const bool valid = oy < H && ox < W;
-                        if (KIND == KPHASE) { oy = 2 * oy + (par >> 1); ox = 2 * ox + (par & 1); }
-                        return valid;
-                    },
-                    [&] {
-                        if (S > 1) {
-                            (void)wait_cluster(smem_u32(&bars->rx_full), 0, abort_flag);
-                            __syncwarp();
-                            cluster_arrive();                // what is sent to this CTA has landed
-                        }
-                    });
+    finish_rows<BN, BN>(a, rx, S, rpo, tid, frame, n0, KIND == KPHASE ? 2 * H : H, KIND == KPHASE ? 2 * W : W,
+                        (KIND == KPHASE ? tile * 4 + par : tile) * S + rank,
+                        [&](int local, int& oy, int& ox) -> bool {
+                            const int R = rank * rpo + local;
+                            oy = ty + R / kTW;
+                            ox = tx + R % kTW;
+                            const bool valid = oy < H && ox < W;
+                            if (KIND == KPHASE) { oy = 2 * oy + (par >> 1); ox = 2 * ox + (par & 1); }
+                            return valid;
+                        },
+                        [&](int local) { return piece<BN>(rank * rpo + local); },
+                        [&] {
+                            if (S > 1) {
+                                (void)wait_cluster(smem_u32(&bars->rx_full), 0, abort_flag);
+                                __syncwarp();
+                                cluster_arrive();            // what is sent to this CTA has landed
+                            }
+                        });
     if (tid == 0 && bars->abort_flag && status) {
         if (atomicCAS(status, 0u, kStatusConvTimeout) == 0u) {
             status[1] = blockIdx.x;
@@ -317,12 +347,12 @@ std::mutex g_mu;
 template <int TH, int BN, int KIND>
 int ops_floats(int n_w) {                                    // operand stages; the partials lie over them
     using C = FCfg<TH, BN, KIND>;
-    return std::max((2 * C::IN_FLOATS + 31) / 32 * 32 + n_w * C::W_FLOATS, C::RX_FLOATS);
+    return std::max((2 * C::IN_FLOATS + 31) / 32 * 32 + n_w * C::W_FLOATS, C::PART_FLOATS);
 }
 template <int TH, int BN, int KIND>
-int smem_bytes(int n_w) {
+int smem_bytes(int n_w, int splits) {
     using C = FCfg<TH, BN, KIND>;
-    return (ops_floats<TH, BN, KIND>(n_w) + C::RX_FLOATS) * 4 + kFTail + 128;
+    return (ops_floats<TH, BN, KIND>(n_w) + (splits > 1 ? C::RX_FLOATS : 0)) * 4 + kFTail + 128;
 }
 
 template <int TH, int BN, int KIND>
@@ -347,7 +377,7 @@ cudaError_t launch_one(const ConvArgs& a, const ConvF32Plan& p, unsigned int* st
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)grid);
     cfg.blockDim = dim3(kThreads);
-    cfg.dynamicSmemBytes = (size_t)smem_bytes<TH, BN, KIND>(p.n_w);
+    cfg.dynamicSmemBytes = (size_t)smem_bytes<TH, BN, KIND>(p.n_w, p.splits);
     cfg.stream = s;
     cudaLaunchAttribute attr[2];
     int na = 0;
@@ -399,13 +429,13 @@ bool conv_f32_choose(const ConvArgs& a, ConvF32Plan* p) {
     auto fit = [&](int base, int stage) { return std::min(std::min(units, kMaxW), (kSplitSmemMax - base) / stage); };
     if (head) p->n_w = units;
     else if (p->th == 16) {
-        p->n_w = kind == K3X3 ? fit(smem_bytes<16, 32, K3X3>(0), FCfg<16, 32, K3X3>::W_FLOATS * 4)
-                 : kind == K1X1 ? fit(smem_bytes<16, 32, K1X1>(0), FCfg<16, 32, K1X1>::W_FLOATS * 4)
-                                : fit(smem_bytes<16, 32, KPHASE>(0), FCfg<16, 32, KPHASE>::W_FLOATS * 4);
+        p->n_w = kind == K3X3 ? fit(smem_bytes<16, 32, K3X3>(0, s), FCfg<16, 32, K3X3>::W_FLOATS * 4)
+                 : kind == K1X1 ? fit(smem_bytes<16, 32, K1X1>(0, s), FCfg<16, 32, K1X1>::W_FLOATS * 4)
+                                : fit(smem_bytes<16, 32, KPHASE>(0, s), FCfg<16, 32, KPHASE>::W_FLOATS * 4);
     } else {
-        p->n_w = kind == K3X3 ? fit(smem_bytes<8, 32, K3X3>(0), FCfg<8, 32, K3X3>::W_FLOATS * 4)
-                 : kind == K1X1 ? fit(smem_bytes<8, 32, K1X1>(0), FCfg<8, 32, K1X1>::W_FLOATS * 4)
-                                : fit(smem_bytes<8, 32, KPHASE>(0), FCfg<8, 32, KPHASE>::W_FLOATS * 4);
+        p->n_w = kind == K3X3 ? fit(smem_bytes<8, 32, K3X3>(0, s), FCfg<8, 32, K3X3>::W_FLOATS * 4)
+                 : kind == K1X1 ? fit(smem_bytes<8, 32, K1X1>(0, s), FCfg<8, 32, K1X1>::W_FLOATS * 4)
+                                : fit(smem_bytes<8, 32, KPHASE>(0, s), FCfg<8, 32, KPHASE>::W_FLOATS * 4);
     }
     return p->n_w >= 1;
 }

@@ -350,7 +350,7 @@ conv_split_kernel(const ConvArgs a, const ConvSplitShape sh, const __grid_consta
             __syncwarp();
             cluster_arrive();                                // what is sent to this CTA has landed
         };
-        finish_rows<BN>(a, rx, S, rpo, ptid, frame, n0, KIND == KPHASE ? 2 * H : H, KIND == KPHASE ? 2 * W : W,
+        finish_rows<BN, RXS>(a, rx, S, rpo, ptid, frame, n0, KIND == KPHASE ? 2 * H : H, KIND == KPHASE ? 2 * W : W,
                         (KIND == KPHASE ? tile * 4 + par : tile) * S + rank,
                         [&](int local, int& oy, int& ox) -> bool {
                             const int R = rank * rpo + local;
@@ -360,7 +360,7 @@ conv_split_kernel(const ConvArgs a, const ConvSplitShape sh, const __grid_consta
                             if (KIND == KPHASE) { oy = 2 * oy + (par >> 1); ox = 2 * ox + (par & 1); }
                             return valid;
                         },
-                        exchange);
+                        [](int) { return 0; }, exchange);
     }
     __syncwarp();
     if (warp < kProd0) cluster_arrive();
