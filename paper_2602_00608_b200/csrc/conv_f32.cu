@@ -483,30 +483,52 @@ cudaError_t launch_pack_weight_f32_phase(const void* w, int w_dtype, float* pack
     return cudaGetLastError();
 }
 
-// One warp per (group, frame) merges a layer's records into scale and shift: where there are too many for every CTA of
-// the consuming layer to merge for itself.
+// One block per (group, frame) merges a layer's records into scale and shift: where there are too many for every CTA of
+// the consuming layer to merge for itself, or the consumer cannot.
 namespace {
-__global__ void __launch_bounds__(256) gn_merge_kernel(GnArgs a) {
+constexpr int kMergeThreads = 512;
+__global__ void __launch_bounds__(kMergeThreads) gn_merge_kernel(GnArgs a) {
+    __shared__ float2 s_part[kMergeThreads / 32];
     griddep_launch();
-    griddep_wait();
-    const int g = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31, n = blockIdx.y;
-    if (g >= a.G) return;
-    const int cpg = a.C / a.G;
+    const int g = blockIdx.x, n = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, cpg = a.C / a.G, c = g * cpg + threadIdx.x;
+    const bool mine = threadIdx.x < cpg;
+    const float gamma = mine ? __ldg(a.gamma + c) : 0.f, beta = mine ? __ldg(a.beta + c) : 0.f, off = mine && a.offset ? __ldg(a.offset + c) : 0.f;
     const float4* rec = a.rec + ((size_t)n * a.G + g) * a.slots;
-    GroupRecords gr;
-    float mean, rstd;
-    gr.load(rec, a.slots, lane, 32);
-    gr.merge(rec, a.slots, lane, 32, 1.f / ((float)a.P * (float)cpg), a.eps, mean, rstd);
-    for (int i = lane; i < cpg; i += 32) {
-        const int c = g * cpg + i;
-        const float sc = __ldg(a.gamma + c) * rstd;
-        a.scale[(size_t)n * a.C + c] = sc;
-        a.shift[(size_t)n * a.C + c] = __ldg(a.beta + c) - mean * sc;
+    griddep_wait();
+    const float ref = __ldcg(&rec->y);
+    float s = 0.f, q = 0.f;
+    constexpr int U = 8;                                     // records of a thread on their way at a time
+    for (int i0 = threadIdx.x; i0 < a.slots; i0 += U * kMergeThreads) {
+        float4 r[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) r[u] = i0 + u * kMergeThreads < a.slots ? __ldcg(rec + i0 + u * kMergeThreads) : make_float4(0.f, ref, 0.f, 0.f);
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const float d = r[u].y - ref, nd = r[u].x * d;
+            s += nd;
+            q += fmaf(nd, d, r[u].z);
+        }
     }
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) {
+        s += __shfl_xor_sync(0xffffffffu, s, d);
+        q += __shfl_xor_sync(0xffffffffu, q, d);
+    }
+    if (lane == 0) s_part[warp] = make_float2(s, q);
+    __syncthreads();
+    if (!mine) return;
+    float2 t = s_part[0];
+#pragma unroll
+    for (int w = 1; w < kMergeThreads / 32; ++w) { t.x += s_part[w].x; t.y += s_part[w].y; }
+    const float inv_n = 1.f / ((float)a.P * (float)cpg), dm = t.x * inv_n;
+    const float sc = gamma * (1.f / sqrtf(fmaxf(fmaf(-dm, dm, t.y * inv_n), 0.f) + a.eps));
+    a.scale[(size_t)n * a.C + c] = sc;
+    a.shift[(size_t)n * a.C + c] = beta - (ref + dm - off) * sc;
 }
 }  // namespace
 cudaError_t launch_gn_merge(const GnArgs& a, cudaStream_t s) {
-    return launch_pdl(gn_merge_kernel, dim3((a.G + 7) / 8, a.B), dim3(256), 0, s, a);
+    if (a.C / a.G > kMergeThreads) return cudaErrorInvalidValue;
+    return launch_pdl(gn_merge_kernel, dim3(a.G, a.B), dim3(kMergeThreads), 0, s, a);
 }
 
 }  // namespace vd

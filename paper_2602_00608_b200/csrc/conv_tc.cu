@@ -127,6 +127,9 @@ struct Bars {                    // lives in shared memory
     uint32_t abort_flag;
     uint32_t stat_last;          // this CTA is the last to finish (it folds the statistics records)
 };
+// REC builds (they have no bias copies: these take the last warp's place): [epilogue warp][slice number & 3]: slice written /
+// read by its statistics warp
+struct RecBars { uint64_t ready[4][4], free[4][4]; };
 
 // Tiles are numbered (frame, channel block, tile row, tile column), column fastest.  Every CTA
 // owns a contiguous, balanced range of tile numbers and walks it in items of `pair` tiles (one
@@ -335,6 +338,153 @@ __device__ void stat_finalize(const ConvArgs& a, int tid, void* smem_scratch) {
     }
 }
 
+// REC builds: the statistics warps.  Warp j reads the slices of epilogue warp j (the last one those of warps 2 and 3): a lane holds
+// one 16-byte piece (4 fp32 or 8 bf16 channels) of every fourth row, its slice is handed back as soon as the loads have landed,
+// and one record per (tile, warp, group) is written: the result does not depend on how tiles are divided among CTAs.
+// They sit on sub-partition 0 with the MMA warp; at some 70 packed instructions per 32 x 32 slice they take a tenth to a
+// fifth of its issue slots.
+constexpr int REC_WARP0 = 8, REC_WARP1 = 12, REC_WARP2 = 20, REC_WARPS = 3;
+// output slice buffers of a CTA's last item, in the then idle weight stages (statistics: the barriers' ring has four)
+template <class Cfg> __host__ __device__ constexpr int tail_bufs(bool rec) {
+    const int n = Cfg::SMEM_B / (4 * WARP_SLICE_BYTES) >= 2 ? Cfg::SMEM_B / (4 * WARP_SLICE_BYTES) : 2;
+    return rec && n > 4 ? 4 : n;
+}
+__device__ __forceinline__ unsigned long long add2(unsigned long long a, unsigned long long b) {
+    unsigned long long r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ unsigned long long sqacc2(unsigned long long d, unsigned long long q) {
+    unsigned long long r;
+    asm("fma.rn.f32x2 %0, %1, %1, %2;" : "=l"(r) : "l"(d), "l"(q));
+    return r;
+}
+__device__ __forceinline__ unsigned long long pack2(float x, float y) {
+    unsigned long long r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
+    return r;
+}
+__device__ __forceinline__ float sum2(unsigned long long v) {
+    float x, y;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(v));
+    return x + y;
+}
+template <class Cfg, int BN, bool OUT_BF16>
+__device__ __forceinline__ void rec_warp(const ConvArgs& a, const Sched& sched, Bars* bars, RecBars* rbars, const uint8_t* smem_out, const uint8_t* smem_b,
+                                         float* s_pend, int j, int lane) {
+    constexpr int NH = OUT_BF16 ? 2 : 1, CS = OUT_BF16 ? 64 : 32, NSL = BN / CS, TAIL = tail_bufs<Cfg>(true);
+    volatile uint32_t* abort_flag = &bars->abort_flag;
+    float* pend = s_pend + j * BN;                           // what the stored values lack (see the planner), this warp's copy
+    const int cpg = a.Cout / a.out_G, piece = lane & 7, r0 = lane >> 3;
+    const int e_n = j == 2 ? 2 : 1;                          // epilogue warps j .. j + e_n - 1
+    int pend_n0 = -1;
+    uint32_t k = 0;                                          // slices of one epilogue warp so far
+    griddep_wait();
+    for (int t = sched.begin; t < sched.end;) {
+        const int n = sched.count(t);
+        const bool last_item = t + n >= sched.end && Cfg::SMEM_B >= 8 * WARP_SLICE_BYTES;
+        for (int slot = 0; slot < n; ++slot) {
+            const Tile tl = sched.get(t + slot, BN);
+            if (tl.n0 != pend_n0) {
+                __syncwarp();
+                for (int i = lane; i < BN; i += 32) pend[i] = a.out_pending ? __ldg(a.out_pending + tl.n0 + i) : 0.f;
+                pend_n0 = tl.n0;
+                __syncwarp();
+            }
+            const bool inside = tl.ty0 + TILE_H <= a.H && tl.tx0 + TILE_W <= a.W;
+            const int cols = min(max(a.W - tl.tx0, 0), TILE_W);
+            int pixels = 0;
+            for (int e = 0; e < e_n; ++e) pixels += min(max(a.H - (tl.ty0 + 4 * (j + e)), 0), 4) * cols;
+            const int rec_slot = ((tl.ty0 / TILE_H) * sched.tiles_x + tl.tx0 / TILE_W) * REC_WARPS + j;
+#pragma unroll 1
+            for (int sl = 0; sl < NSL; ++sl) {
+                unsigned long long s[NH][2], q[NH][2], ko[NH][2];
+                float pivot[NH];
+#pragma unroll
+                for (int h = 0; h < NH; ++h) { s[h][0] = s[h][1] = q[h][0] = q[h][1] = ko[h][0] = ko[h][1] = 0ull; pivot[h] = 0.f; }
+#pragma unroll 1
+                for (int e = 0; e < e_n; ++e) {
+                    const int ew = j + e;
+                    const uint32_t kk = k + sl;
+                    if (!mbar_wait(smem_u32(&rbars->ready[ew][kk & 3]), (kk >> 2) & 1, abort_flag)) return;
+                    __syncwarp();
+                    const uint8_t* buf = last_item ? smem_b + (ew * TAIL + (int)(kk % TAIL)) * WARP_SLICE_BYTES
+                                                   : smem_out + (ew * Cfg::OUT_BUFS + (int)(kk % Cfg::OUT_BUFS)) * WARP_SLICE_BYTES;
+                    uint4 v[8];
+#pragma unroll
+                    for (int it = 0; it < 8; ++it) {
+                        const int r = it * 4 + r0;
+                        v[it] = lds_u4(smem_u32(buf) + (uint32_t)(r * 128 + ((piece ^ (r & 7)) << 4)));
+                    }
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(smem_u32(&rbars->free[ew][kk & 3]));
+                    if (e == 0) {
+                        // deviations from the first pixel's first channel of the group (it lies in the image if any of the warp's does)
+                        const float4 p0 = *(const float4*)(pend + sl * CS + piece * (4 * NH));
+                        const float f0 = OUT_BF16 ? __uint_as_float(v[0].x << 16) : __uint_as_float(v[0].x);
+                        const int lead = OUT_BF16 ? (cpg == 16 ? piece & 6 : piece) : piece & ~((cpg >> 2) - 1);
+                        pivot[0] = __shfl_sync(0xffffffffu, f0 + p0.x, lead);
+                        ko[0][0] = pack2(p0.x - pivot[0], p0.y - pivot[0]);
+                        ko[0][1] = pack2(p0.z - pivot[0], p0.w - pivot[0]);
+                        if (NH == 2) {
+                            const float4 p1 = *(const float4*)(pend + sl * CS + piece * 8 + 4);
+                            const float f1 = __shfl_sync(0xffffffffu, __uint_as_float(v[0].z << 16) + p1.x, lead);
+                            pivot[NH - 1] = cpg == 4 ? f1 : pivot[0];
+                            ko[NH - 1][0] = pack2(p1.x - pivot[NH - 1], p1.y - pivot[NH - 1]);
+                            ko[NH - 1][1] = pack2(p1.z - pivot[NH - 1], p1.w - pivot[NH - 1]);
+                        }
+                    }
+#pragma unroll
+                    for (int it = 0; it < 8; ++it) {
+                        const int r = it * 4 + r0;
+                        if (!inside && (tl.ty0 + 4 * ew + (r >> 3) >= a.H || tl.tx0 + (r & 7) >= a.W)) continue;
+#pragma unroll
+                        for (int h = 0; h < NH; ++h) {
+                            const uint32_t w0 = h ? v[it].z : v[it].x, w1 = h ? v[it].w : v[it].y;
+                            const unsigned long long x0 = OUT_BF16 ? pack2(__uint_as_float(w0 << 16), __uint_as_float(w0 & 0xffff0000u))
+                                                                   : pack2(__uint_as_float(v[it].x), __uint_as_float(v[it].y));
+                            const unsigned long long x1 = OUT_BF16 ? pack2(__uint_as_float(w1 << 16), __uint_as_float(w1 & 0xffff0000u))
+                                                                   : pack2(__uint_as_float(v[it].z), __uint_as_float(v[it].w));
+                            const unsigned long long d0 = add2(x0, ko[h][0]), d1 = add2(x1, ko[h][1]);
+                            s[h][0] = add2(s[h][0], d0); s[h][1] = add2(s[h][1], d1);
+                            q[h][0] = sqacc2(d0, q[h][0]); q[h][1] = sqacc2(d1, q[h][1]);
+                        }
+                    }
+                }
+                float fs[NH], fq[NH];
+#pragma unroll
+                for (int h = 0; h < NH; ++h) { fs[h] = sum2(add2(s[h][0], s[h][1])); fq[h] = sum2(add2(q[h][0], q[h][1])); }
+                const bool both = NH == 2 && cpg >= 8;       // the lane's two halves are one group
+                if (both) { fs[0] += fs[NH - 1]; fq[0] += fq[NH - 1]; }
+                auto cross = [&](int d) {
+#pragma unroll
+                    for (int h = 0; h < NH; ++h) {
+                        fs[h] += __shfl_xor_sync(0xffffffffu, fs[h], d);
+                        fq[h] += __shfl_xor_sync(0xffffffffu, fq[h], d);
+                    }
+                };
+                cross(8);
+                cross(16);
+                const int lanes = max(cpg / (4 * NH), 1);    // lanes of a group: 1, 2 or 4
+                if (lanes > 1) cross(1);
+                if (lanes > 2) cross(2);
+                if (r0 == 0 && (piece & (lanes - 1)) == 0) {
+                    const float cntf = (float)(pixels * cpg), inv = pixels > 0 ? 1.f / cntf : 0.f;
+                    float4* o = a.out_rec + ((size_t)tl.b * a.out_G + (tl.n0 + sl * CS + piece * 4 * NH) / cpg) * a.out_slots + rec_slot;
+#pragma unroll
+                    for (int h = 0; h < NH; ++h) {
+                        if (h > 0 && both) break;
+                        const float dm = fs[h] * inv;
+                        o[(size_t)h * a.out_slots] = make_float4(cntf, pivot[h] + dm, fmaxf(fmaf(-dm, fs[h], fq[h]), 0.f), 0.f);
+                    }
+                }
+            }
+            k += NSL;
+        }
+        t += n;
+    }
+}
+
 // OUT_MODE: 0 = fp32 NHWC, 1 = bf16 NHWC (both through shared memory and TMA stores),
 //           2 = NCHW frame written directly (dtype from a.out_dtype)
 // STATS: the epilogue also takes the GroupNorm statistics of the output (a build of its own: compiled in but switched
@@ -343,7 +493,10 @@ __device__ void stat_finalize(const ConvArgs& a, int tid, void* smem_scratch) {
 // additions and the bias loads are more than half of a pass's instructions)
 // X2: the layer has a second input (the fused 1x1 shortcut); the other builds carry none of its code
 // KS: kernel size, 3 or 1 (the 1x1 layers take the centre view of the halo tile only)
-template <int BN, bool IN_BF16, int OUT_MODE, int CG = 1, bool PH = false, bool STATS = false, bool BIAS = true, bool X2 = false, int KS = 3>
+// REC: three otherwise idle warps read the output slices on their way out through shared memory and leave statistics records
+//      (conv_cluster.cuh) for the normalisation that follows: no pass over the tensor, and nothing added to the epilogue
+//      warps but a barrier arrival per slice
+template <int BN, bool IN_BF16, int OUT_MODE, int CG = 1, bool PH = false, bool STATS = false, bool BIAS = true, bool X2 = false, int KS = 3, bool REC = false>
 __global__ void __launch_bounds__(NUM_THREADS, 1)
 conv_tc_kernel(const ConvArgs a, const __grid_constant__ CUtensorMap tmap, const __grid_constant__ CUtensorMap tmap2,
                const __grid_constant__ CUtensorMap tmap_y, const __grid_constant__ CUtensorMap tmap_x2, unsigned int* status) {
@@ -360,6 +513,8 @@ conv_tc_kernel(const ConvArgs a, const __grid_constant__ CUtensorMap tmap, const
     static_assert(Cfg::SMEM_TOTAL <= 232448, "shared memory of one CTA");
     uint8_t* smem_stage = smem_bias + Cfg::SMEM_BIAS + Cfg::SMEM_BARS;  // raw input of the next unit (two-tile items only)
     volatile uint32_t* abort_flag = &bars->abort_flag;
+    RecBars* rbars = (RecBars*)(smem_bias + 3 * BN * 4);
+    static_assert(!REC || (BN * 4 >= (int)sizeof(RecBars) && !BIAS && OUT_MODE != 2 && CG == 1), "statistics barriers");
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     constexpr int taps = KS * KS;
@@ -393,6 +548,8 @@ conv_tc_kernel(const ConvArgs a, const __grid_constant__ CUtensorMap tmap, const
         for (int i = 0; i < Cfg::A_STAGES; ++i) { mbar_init(smem_u32(&bars->a_full[i]), CG * NUM_PRODUCER_WARPS); mbar_init(smem_u32(&bars->a_empty[i]), 1); }
         for (int i = 0; i < Cfg::B_STAGES; ++i) { mbar_init(smem_u32(&bars->b_full[i]), CG); mbar_init(smem_u32(&bars->b_empty[i]), 1); }
         for (int i = 0; i < 4; ++i) { mbar_init(smem_u32(&bars->acc_full[i]), 1); mbar_init(smem_u32(&bars->acc_empty[i]), 4 * CG); }
+        if (REC)
+            for (int i = 0; i < 16; ++i) { mbar_init(smem_u32(&rbars->ready[0][0] + i), 1); mbar_init(smem_u32(&rbars->free[0][0] + i), 1); }
         bars->abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         fence_proxy_async_smem();
@@ -804,7 +961,7 @@ conv_tc_kernel(const ConvArgs a, const __grid_constant__ CUtensorMap tmap, const
 #pragma unroll
             for (int p = 0; p < NPS; ++p) sacc[p] = 0;
             int stat_b = -1, stat_n0 = 0;
-            constexpr int TAIL_BUFS = Cfg::SMEM_B / (4 * WARP_SLICE_BYTES) >= 2 ? Cfg::SMEM_B / (4 * WARP_SLICE_BYTES) : 2;
+            constexpr int TAIL_BUFS = tail_bufs<Cfg>(REC);
             for (int t = sched.begin; t < sched.end && ok; ++n_item) {
                 const int n = sched.count(t);
                 const int cnt = sched.mine(n);
@@ -879,6 +1036,10 @@ conv_tc_kernel(const ConvArgs a, const __grid_constant__ CUtensorMap tmap, const
                             if (lane == 0) {                              // the store that last read this buffer is done
                                 if (last_item) bulk_wait_group_read<TAIL_BUFS - 1>();
                                 else bulk_wait_group_read<Cfg::OUT_BUFS - 1>();
+                                if constexpr (REC) {                      // and its statistics have been taken
+                                    const uint32_t bufs = last_item ? TAIL_BUFS : Cfg::OUT_BUFS, k = n_slice + sl;
+                                    if (k >= bufs) (void)mbar_wait(smem_u32(&rbars->free[ew][(k - bufs) & 3]), ((k - bufs) >> 2) & 1, abort_flag);
+                                }
                             }
                             __syncwarp();
                         }
@@ -953,6 +1114,7 @@ conv_tc_kernel(const ConvArgs a, const __grid_constant__ CUtensorMap tmap, const
                                 else if (reduce_add) tma_reduce_add_4d(&tmap_y, smem_u32(obuf), tl.n0 + sl * CS, tl.tx0, tl.ty0 + 4 * ew, tl.b, pol_out);
                                 else tma_store_4d(&tmap_y, smem_u32(obuf), tl.n0 + sl * CS, tl.tx0, tl.ty0 + 4 * ew, tl.b, pol_out);
                                 bulk_commit_group();
+                                if constexpr (REC) mbar_arrive(smem_u32(&rbars->ready[ew][(n_slice + sl) & 3]));
                             }
                         }
                     }
@@ -964,6 +1126,8 @@ conv_tc_kernel(const ConvArgs a, const __grid_constant__ CUtensorMap tmap, const
             if (stats) __threadfence();
             if (lane == 0) bulk_wait_group<0>();             // all stores have landed before the CTA retires
         }
+    } else if (REC && (warp == REC_WARP0 || warp == REC_WARP1 || warp == REC_WARP2)) {
+        if constexpr (REC) rec_warp<Cfg, BN, OUT_MODE == 1>(a, sched, bars, rbars, smem_out, smem_b, (float*)smem_bias, warp == REC_WARP0 ? 0 : (warp == REC_WARP1 ? 1 : 2), lane);
     } else if (warp == TMA_WARP) {
         // ------------------------------------------------ weight loads (TMA)
         if (lane == 0) {
@@ -1444,9 +1608,9 @@ cudaError_t kernel_state(K kern, int smem, int cg, KernelState& st, int* pairs, 
     return cudaSuccess;
 }
 
-template <int BN, bool IB, int OM, int CG, bool PH = false, bool STATS = false, bool BIAS = true, bool X2 = false, int KS = 3>
+template <int BN, bool IB, int OM, int CG, bool PH = false, bool STATS = false, bool BIAS = true, bool X2 = false, int KS = 3, bool REC = false>
 cudaError_t launch_one(const ConvArgs& a, const ConvTcPlan& plan, unsigned int* status, cudaStream_t s) {
-    auto kern = conv_tc_kernel<BN, IB, OM, CG, PH, STATS, BIAS, X2, KS>;
+    auto kern = conv_tc_kernel<BN, IB, OM, CG, PH, STATS, BIAS, X2, KS, REC>;
     constexpr int SMEM = TileCfg<BN, CG, PH, IB>::SMEM_TOTAL;
     static KernelState state = {};
     int pairs = 0, sms = 0;
@@ -1525,6 +1689,23 @@ bool conv_tc_stats_supported(const ConvArgs& a, int groups) {
     const int cpg = a.Cout / groups;
     return cpg == 4 || cpg == 8 || cpg == 16;
 }
+
+// Layers that leave statistics records: the stored values are final but for a pending bias, and the epilogue warps have time
+// for the hand-over of every slice: 256-channel blocks (a tile's MMAs take twice their time) and the layers with a fused
+// shortcut.  Measured, layer + normalisation, us, without -> with: 512->512 at 60x90 39.6 + 14.4 -> 45.0 + 6.1, at 120x180
+// 94 + 17 -> 97 + 8; 256->256 at 240x360 81 + 19.4 -> 87 + 10.2; with shortcut 512->256 at 240x360 163 + 24 -> 168 + 12, 256->128 at
+// 480x720 230 + 38 -> 236 + 21.  Where the epilogue paces the layer it loses: 128->128 at 480x720 109 + 27 -> 172 + 20, phase
+// form 256->256 to 480x720 186 + 64 -> 337 + 21.
+static bool rec_layer(const ConvArgs& a) {
+    if (!conv_tc_supported(a) || a.Cout % 128 != 0 || a.residual || a.bias || a.bias2 || a.ksize != 3 || a.upsample) return false;
+    if (!a.x2) return a.Cout % 256 == 0 && a.in_dtype == VD_F32 && a.out_dtype == VD_BF16;
+    return true;                                              // fused shortcut: bf16 in, fp32 out
+}
+// Below 6 million output elements (all frames of the handle's batch) the hand-over costs as much as the normalisation's own
+// pass, which overlaps its neighbours there: 256x256 frame 1049 us without, 1073 with, 424x296 1539 / 1571; four 256x256
+// frames 2772 / 2673.
+bool conv_tc_records_supported(const ConvArgs& a) { return rec_layer(a) && (double)a.H * a.W * a.Cout * a.B >= 6e6; }
+int conv_tc_slots(const ConvArgs& a) { return ((a.W + TILE_W - 1) / TILE_W) * ((a.H + TILE_H - 1) / TILE_H) * REC_WARPS; }
 
 bool conv_tc_pairs_available() { return pairs_available(); }
 
@@ -1655,6 +1836,12 @@ cudaError_t launch_conv_tc(const ConvArgs& a, const ConvTcPlan& plan, unsigned i
     const bool ib = a.in_dtype == VD_BF16, ob = a.out_dtype == VD_BF16;
     const bool hb = a.bias != nullptr || a.bias2 != nullptr;
     const bool k1 = a.ksize == 1;
+    if (a.out_rec) {
+        if (!rec_layer(a) || !rec_groups_ok(a.Cout, a.out_G) || a.out_slots != conv_tc_slots(a) || a.stat_sum) return cudaErrorInvalidValue;
+        if (a.x2) return plan.bn == 256 ? launch_one<256, true, 0, 1, false, false, false, true, 3, true>(a, plan, status, s)
+                                        : launch_one<128, true, 0, 1, false, false, false, true, 3, true>(a, plan, status, s);
+        return launch_one<256, false, 1, 1, false, false, false, false, 3, true>(a, plan, status, s);
+    }
     if (a.stat_sum) {          // bf16 output with the statistics of the following GroupNorm (checked above)
         if (plan.bn == 256 && plan.cg == 2) return ib ? launch_one<256, true, 1, 2, false, true>(a, plan, status, s) : launch_one<256, false, 1, 2, false, true>(a, plan, status, s);
         if (plan.bn == 256) {

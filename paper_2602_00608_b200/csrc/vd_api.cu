@@ -182,7 +182,7 @@ class Planner {
                       ptr<float>(b_off), ptr<float>(scale_off_), ptr<float>(shift_off_), ptr<float>(partial_off_),
                       ptr<unsigned int>(partial_off_ + gn_partial_bytes(cfg_.max_batch, cfg_.norm_groups)),
                       pending(x_off) != kNone ? ptr<float>(pending(x_off)) : nullptr};
-        if (rec_.count(x_off) && pending(x_off) == kNone && rec_groups_ok(C, cfg_.norm_groups)) {
+        if (rec_.count(x_off) && rec_groups_ok(C, cfg_.norm_groups)) {
             s.gn.rec = ptr<float4>(rec_[x_off].off);
             s.gn.slots = rec_[x_off].slots;
         }
@@ -286,7 +286,7 @@ class Planner {
         // just planned needs no launch
         if ((f32 || split) && prologue) {
             Step& g = h_->steps.back();
-            if (g.kind == VD_STEP_GN_STATS && g.gn.rec && g.gn.slots <= kRecMergeSlots) {
+            if (g.kind == VD_STEP_GN_STATS && g.gn.rec && !g.gn.offset && g.gn.slots <= kRecMergeSlots) {
                 a.in_rec = g.gn.rec; a.in_slots = g.gn.slots; a.in_pixels = g.gn.P;
                 a.in_gamma = g.gn.gamma; a.in_beta = g.gn.beta; a.in_G = g.gn.G; a.in_eps = g.gn.eps;
                 a.scale = a.shift = nullptr;
@@ -297,11 +297,15 @@ class Planner {
         if (!y_is_frames) rec_.erase(y_off);
         const bool records = !no_records_;
         no_records_ = false;
-        if ((f32 || split) && records && !y_is_frames && rec_groups_ok(Cout, cfg_.norm_groups)) {
-            const int slots = split ? conv_split_slots(probe, s.split, cfg_.norm_groups) : conv_f32_slots(probe, s.f32, cfg_.norm_groups);
+        ConvArgs whole = a;
+        whole.B = cfg_.max_batch;
+        const bool tc_rec = tc && !split && !(cfg_.flags & VD_FLAG_FUSED_STATS) && !y_is_frames && conv_tc_records_supported(whole);
+        if ((f32 || split || tc_rec) && records && !y_is_frames && rec_groups_ok(Cout, cfg_.norm_groups)) {
+            const int slots = tc_rec ? conv_tc_slots(a) : split ? conv_split_slots(probe, s.split, cfg_.norm_groups) : conv_f32_slots(probe, s.f32, cfg_.norm_groups);
             rec_toggle_ ^= 1;
             a.out_rec = ptr<float4>(rec_buf_[rec_toggle_]);
             a.out_slots = slots;
+            a.out_pending = tc_rec && pending(y_off) != kNone ? ptr<float>(pending(y_off)) : nullptr;
             a.out_G = cfg_.norm_groups;
             rec_[y_off] = {rec_buf_[rec_toggle_], slots};
             max_slots_ = std::max(max_slots_, slots);

@@ -51,7 +51,8 @@ struct ConvArgs {
     const float* in_beta;        // [Cin]
     int in_slots, in_G, in_pixels;   // in_pixels: pixels the statistics are over
     float in_eps;
-    float4* out_rec;             // or null
+    float4* out_rec;             // or null (conv_tc.cu too)
+    const float* out_pending;    // conv_tc.cu: the records are those of y + out_pending[c] (null: of y)
     int out_slots, out_G;
     // tensor-core kernel: ceil(2^32 / d) for the divisors of its tile numbering (tiles per image, channel
     // blocks, tiles per row), filled in by its launcher; 0 stands for d = 1
@@ -128,6 +129,8 @@ cudaError_t launch_fill_rows(float* dst, const float* src, int C, int B, cudaStr
 // ---- tcgen05 kernels (conv_tc.cu, attn_tc.cu)
 bool conv_tc_supported(const ConvArgs& a);
 bool conv_tc_stats_supported(const ConvArgs& a, int groups);   // the epilogue can take the next GroupNorm's statistics
+bool conv_tc_records_supported(const ConvArgs& a);             // the kernel can leave statistics records of this layer's output
+int conv_tc_slots(const ConvArgs& a);
 bool conv_tc_pairs_available();          // can the current device co-schedule the kernels' CTA pairs?
 size_t conv_tc_packed_bytes(int Cout, int Cin, int taps, bool phase);
 // OIHW weight (bf16) -> bf16 [tap][Cout_pad][Cin] (K-major rows for the B operand); phase: the sixteen
@@ -152,7 +155,7 @@ cudaError_t conv_tc_prepare(const ConvArgs& a, ConvTcPlan* plan);      // a.w mu
 cudaError_t launch_conv_tc(const ConvArgs& a, const ConvTcPlan& plan, unsigned int* status_word, cudaStream_t s);
 // ---- layers whose CTAs divide K among a cluster and leave statistics records (conv_cluster.cuh)
 constexpr int kSplitSmemMax = (228 * 1024 - 2 * 1024) / 2;     // two CTAs share an SM
-constexpr int kRecMergeSlots = 64;                             // up to here the consuming layer's CTAs merge the records themselves
+constexpr int kRecMergeSlots = 128;                             // up to here the consuming layer's CTAs merge the records themselves
 inline bool rec_groups_ok(int channels, int groups) {          // records of such groups can be written and merged
     const int cpg = groups > 0 ? channels / groups : 0;
     return groups > 0 && channels % groups == 0 && (cpg == 4 || cpg == 8 || cpg == 16);
