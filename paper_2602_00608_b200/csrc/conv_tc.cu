@@ -1696,6 +1696,14 @@ bool conv_tc_stats_supported(const ConvArgs& a, int groups) {
 // 94 + 17 -> 97 + 8; 256->256 at 240x360 81 + 19.4 -> 87 + 10.2; with shortcut 512->256 at 240x360 163 + 24 -> 168 + 12, 256->128 at
 // 480x720 230 + 38 -> 236 + 21.  Where the epilogue paces the layer it loses: 128->128 at 480x720 109 + 27 -> 172 + 20, phase
 // form 256->256 to 480x720 186 + 64 -> 337 + 21.
+// 3x3 layers of 256-channel blocks with ten tiles or more per SM run as CTA pairs: the chip is at its power limit there, and a
+// pair reads each weight from L2 once instead of twice.  Eight 720x480 frames per decode 26.34 -> 25.80 ms, two 1280x720
+// frames 18.20 -> 17.85; smaller layers lose more to the signals between the two CTAs than they gain (one 720x480 frame,
+// whose layers have 96 to 675 tiles: 3.57 -> 3.64 ms).
+static bool wide_layer(const ConvArgs& a) {
+    if (a.Cout % 256 != 0 || a.ksize != 3 || a.upsample || a.x2 || a.out_nchw || a.out_u8) return false;
+    return (long long)((a.H + TILE_H - 1) / TILE_H) * ((a.W + TILE_W - 1) / TILE_W) * a.B * (a.Cout / 256) >= 1500;
+}
 static bool rec_layer(const ConvArgs& a) {
     if (!conv_tc_supported(a) || a.Cout % 128 != 0 || a.residual || a.bias || a.bias2 || a.ksize != 3 || a.upsample) return false;
     if (!a.x2) return a.Cout % 256 == 0 && a.in_dtype == VD_F32 && a.out_dtype == VD_BF16;
@@ -1704,7 +1712,8 @@ static bool rec_layer(const ConvArgs& a) {
 // Below 6 million output elements (all frames of the handle's batch) the hand-over costs as much as the normalisation's own
 // pass, which overlaps its neighbours there: 256x256 frame 1049 us without, 1073 with, 424x296 1539 / 1571; four 256x256
 // frames 2772 / 2673.
-bool conv_tc_records_supported(const ConvArgs& a) { return rec_layer(a) && (double)a.H * a.W * a.Cout * a.B >= 6e6; }
+// On CTA pairs the hand-over costs more than it saves (two 1280x720 frames 17.85 ms without, 18.00 with).
+bool conv_tc_records_supported(const ConvArgs& a) { return rec_layer(a) && !wide_layer(a) && (double)a.H * a.W * a.Cout * a.B >= 6e6; }
 int conv_tc_slots(const ConvArgs& a) { return ((a.W + TILE_W - 1) / TILE_W) * ((a.H + TILE_H - 1) / TILE_H) * REC_WARPS; }
 
 bool conv_tc_pairs_available() { return pairs_available(); }
@@ -1744,7 +1753,8 @@ cudaError_t conv_tc_prepare(const ConvArgs& a, ConvTcPlan* plan) {
     const int bn = phase ? 128 : pick_bn(a.Cout);
     // 256-channel blocks of the folded upsampling form and the phase form run as two-CTA pairs (each CTA loads
     // half of the rows of a weight tile); the device must be able to co-schedule such pairs
-    int cg = (phase || (bn == 256 && a.upsample)) ? 2 : 1;
+    // So do the other 3x3 layers of 256-channel blocks that are large enough (wide_layer).
+    int cg = (phase || (bn == 256 && a.upsample) || wide_layer(a)) ? 2 : 1;
     if (cg == 2 && !pairs_available()) {
         if (phase) return cudaErrorInvalidConfiguration;     // the phase form has no one-CTA variant
         cg = 1;
