@@ -58,93 +58,76 @@ __device__ __forceinline__ bool wait_cluster(uint32_t bar, uint32_t parity, vola
     return true;
 }
 
-// Statistics of one group from its records (count, mean, sum of squared deviations), for the whole warp the same number L
-// (8 or 32) of lanes to a group.  Deviations are from the first record's mean, so one round of loads and one of shuffles
-// suffice; a lane's first two records are loaded by `load`, so that they are on their way before other loads.
-struct GroupRecords {
-    float4 r0, r1;
-    float ref;
-    __device__ __forceinline__ void load(const float4* rec, int slots, int l, int L) {
-        ref = __ldcg(&rec->y);
-        r0 = r1 = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (l < slots) r0 = __ldcg(rec + l);
-        if (l + L < slots) r1 = __ldcg(rec + l + L);
-    }
-    __device__ __forceinline__ void merge(const float4* rec, int slots, int l, int L, float inv_n, float eps, float& mean, float& rstd) const {
-        const float d0 = r0.y - ref, d1 = r1.y - ref, n0 = r0.x * d0, n1 = r1.x * d1;
-        float s = n0 + n1, q = fmaf(n0, d0, r0.z) + fmaf(n1, d1, r1.z);
-        for (int i = l + 2 * L; i < slots; i += L) {
-            const float4 r = __ldcg(rec + i);
-            const float d = r.y - ref, nd = r.x * d;
-            s += nd;
-            q += fmaf(nd, d, r.z);
-        }
-        for (int d = L >> 1; d > 0; d >>= 1) {
-            s += __shfl_xor_sync(0xffffffffu, s, d);
-            q += __shfl_xor_sync(0xffffffffu, q, d);
-        }
-        const float dm = s * inv_n;
-        mean = ref + dm;
-        rstd = 1.f / sqrtf(fmaxf(fmaf(-dm, dm, q * inv_n), 0.f) + eps);
-    }
-};
-
 // half * scale and half * shift of the input channels [c0, c0 + nch) of `frame`, from the producing layer's records, by
-// NW warps (w = 0..NW - 1); c0 and nch are multiples of the group size.  Everything but the records is ready before
-// the kernel before has finished: set up with `prepare`, then `load`, then (other loads issued) `finish`.
-template <int NW> struct InputStatsOf {
+// eight warps (w = 0..7); c0 and nch are multiples of the group size.  A group has 8 lanes of a warp (32 where there are more
+// than 16 records); a lane's first two records are loaded by `load`, so that they are on their way before other loads, and
+// `finish` merges.  Deviations are from the first record's mean, so one round of loads and one of shuffles suffice.
+// Everything that does not need the kernel before is done ahead by `prepare`, gamma and beta into s_scale and s_shift
+// included (a lane reads back what it has put there itself); what stays in registers across the loads is kept small, since
+// a loaded value that is spilled has to be waited for.
+struct InputStats {
     const float4* rec;
-    int cpg, L, l, g, ng;
-    float inv_n, gamma[2], beta[2];
-    GroupRecords gr;
-    __device__ __forceinline__ void prepare(const ConvArgs& a, int frame, int c0, int nch, int w, int lane) {
-        cpg = a.Cin / a.in_G;
-        L = a.in_slots <= 16 ? 8 : 32;
-        l = lane & (L - 1);
-        ng = nch / cpg;
-        g = w * (32 / L) + lane / L;
-        inv_n = 1.f / ((float)a.in_pixels * (float)cpg);
-        rec = a.in_rec + ((size_t)frame * a.in_G + c0 / cpg + min(g, ng - 1)) * a.in_slots;
-#pragma unroll
-        for (int i = 0; i < 2; ++i) {
-            const int c = c0 + min(g, ng - 1) * cpg + l + i * L;
-            const bool on = l + i * L < cpg;
-            gamma[i] = on ? __ldg(a.in_gamma + c) : 0.f;
-            beta[i] = on ? __ldg(a.in_beta + c) : 0.f;
-        }
-    }
-    __device__ __forceinline__ void load(const ConvArgs& a) { gr.load(rec, a.in_slots, l, L); }
-    __device__ __forceinline__ void finish(const ConvArgs& a, int c0, float half, float* s_scale, float* s_shift) {
-        const int step = NW * (32 / L);
-        for (;;) {
-            float mean, rstd;
-            gr.merge(rec, a.in_slots, l, L, inv_n, a.in_eps, mean, rstd);
-            if (g < ng) {
-#pragma unroll
-                for (int i = 0; i < 2; ++i)
-                    if (l + i * L < cpg) {
-                        const float sc = gamma[i] * rstd;
-                        s_scale[g * cpg + l + i * L] = sc * half;
-                        s_shift[g * cpg + l + i * L] = (beta[i] - mean * sc) * half;
-                    }
+    float4 r0, r1;
+    int g;                                                   // this lane's group of the slice
+    static __device__ __forceinline__ int lanes_log2(const ConvArgs& a) { return a.in_slots <= 16 ? 3 : 5; }
+    __device__ __forceinline__ void prepare(const ConvArgs& a, int frame, int c0, int nch, int w, int lane, float* s_scale, float* s_shift) {
+        const int ll = lanes_log2(a), L = 1 << ll, l = lane & (L - 1), ng = nch >> a.in_shift;
+        g = (w << (5 - ll)) + (lane >> ll);
+        rec = a.in_rec + ((size_t)frame * a.in_G + (c0 >> a.in_shift) + min(g, ng - 1)) * a.in_slots;
+#pragma unroll 1
+        for (int gg = g; gg < ng; gg += 8 << (5 - ll))
+            for (int i = l; i < 1 << a.in_shift; i += L) {
+                const int c = (gg << a.in_shift) + i;
+                s_scale[c] = __ldg(a.in_gamma + c0 + c);
+                s_shift[c] = __ldg(a.in_beta + c0 + c);
             }
-            if (g - (int)(threadIdx.x & 31) / L + step >= ng) break;     // (the same for the whole warp)
-            g += step;
-            rec += (size_t)step * a.in_slots;
-            const int gg = min(g, ng - 1);
-            rec -= (size_t)(g - gg) * a.in_slots;
-            gr.load(rec, a.in_slots, l, L);
+    }
+    __device__ __forceinline__ void load(const ConvArgs& a, int lane) {
+        const int ll = lanes_log2(a), L = 1 << ll, l = lane & (L - 1);
+        r0 = r1 = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (l < a.in_slots) r0 = __ldcg(rec + l);
+        if (l + L < a.in_slots) r1 = __ldcg(rec + l + L);
+    }
+    __device__ __forceinline__ void finish(const ConvArgs& a, int nch, int lane, float half, float* s_scale, float* s_shift) {
+        const int ll = lanes_log2(a), L = 1 << ll, l = lane & (L - 1), ng = nch >> a.in_shift;
+#pragma unroll 1
+        for (;;) {
+            const float ref = __shfl_sync(0xffffffffu, r0.y, lane & ~(L - 1));
+            const float d0 = r0.y - ref, d1 = r1.y - ref, n0 = r0.x * d0, n1 = r1.x * d1;
+            float s = n0 + n1, q = fmaf(n0, d0, r0.z) + fmaf(n1, d1, r1.z);
+#pragma unroll 1
+            for (int i = l + 2 * L; i < a.in_slots; i += L) {
+                const float4 r = __ldcg(rec + i);
+                const float d = r.y - ref, nd = r.x * d;
+                s += nd;
+                q += fmaf(nd, d, r.z);
+            }
+            if (ll == 5) {
+                s += __shfl_xor_sync(0xffffffffu, s, 16); q += __shfl_xor_sync(0xffffffffu, q, 16);
+                s += __shfl_xor_sync(0xffffffffu, s, 8); q += __shfl_xor_sync(0xffffffffu, q, 8);
+            }
 #pragma unroll
-            for (int i = 0; i < 2; ++i)
-                if (l + i * L < cpg) {
-                    gamma[i] = __ldg(a.in_gamma + c0 + gg * cpg + l + i * L);
-                    beta[i] = __ldg(a.in_beta + c0 + gg * cpg + l + i * L);
+            for (int d = 4; d > 0; d >>= 1) {
+                s += __shfl_xor_sync(0xffffffffu, s, d);
+                q += __shfl_xor_sync(0xffffffffu, q, d);
+            }
+            const float dm = s * a.in_inv_n, mean = ref + dm;
+            const float rstd = 1.f / sqrtf(fmaxf(fmaf(-dm, dm, q * a.in_inv_n), 0.f) + a.in_eps);
+            if (g < ng)
+                for (int i = l; i < 1 << a.in_shift; i += L) {
+                    const int c = (g << a.in_shift) + i;
+                    const float sc = s_scale[c] * rstd;
+                    s_scale[c] = sc * half;
+                    s_shift[c] = (s_shift[c] - mean * sc) * half;
                 }
+            const int step = 8 << (5 - ll);
+            if (g - (lane >> ll) + step >= ng) break;        // (the same for the whole warp)
+            rec += (size_t)(min(g + step, ng - 1) - min(g, ng - 1)) * a.in_slots;
+            g += step;
+            load(a, lane);
         }
     }
 };
-
-using InputStats = InputStatsOf<8>;
 
 // The eight warps that write a CTA's rows: a warp has CPW four-channel columns of the BN channels (two at least: whole
 // 32-byte sectors), WC warps lie side by side and WR below one another.
@@ -158,15 +141,18 @@ inline int rec_parts(int bn, int cpg) {
 }
 
 // Adds up the `nparts` partials of this CTA's `rpo` rows, adds bias and residual, writes the output and the statistics
-// records.  rx: [nparts][rpo][RXS] floats, 16-byte piece c of a row at c ^ swizzle(row).  ptid: 0..255.  locate(local row, oy, ox) gives the row's output pixel and
-// whether it exists; ready() returns when the partials have arrived (the residual is on its way by then).
-// A thread takes four channels (cg) of every RSTEP-th row, so a warp's share of a group comes from shuffles alone.  BN < 32: the frame head (planes or packed pixels of a.Cout channels).
+// records.  rx: [nparts][rpo][RXS] floats, 16-byte piece c of a row at c ^ swizzle(row).  ptid: 0..255.  locate(local row,
+// oy, ox) gives the row's output pixel and whether it exists; ready() returns when the partials have arrived.  The first
+// rows' addresses and residual and the record's address are made before that (the empty asm keeps them there).
+// A thread takes four channels (cg) of every RSTEP-th row, so a warp's share of a group comes from shuffles alone.  BN < 32:
+// the frame head (planes or packed pixels of a.Cout channels).
 template <int BN, int RXS, class Locate, class Swizzle, class Ready>
-__device__ __forceinline__ void finish_rows(const ConvArgs& a, float* rx, int nparts, int rpo, int ptid, int frame, int n0, int OH, int OW,
+__device__ __forceinline__ void finish_rows(const ConvArgs& a, const float* rx, int nparts, int rpo, int ptid, int frame, int n0, int OH, int OW,
                                             int slot0, Locate locate, Swizzle swizzle, Ready ready) {
     constexpr bool HEAD = BN < 32;
     constexpr int CPW = HEAD ? 1 : Split8<HEAD ? 64 : BN>::CPW, WC = HEAD ? 1 : Split8<HEAD ? 64 : BN>::WC, RL = 32 / CPW;
-    constexpr int RSTEP = HEAD ? kFinishThreads / (BN / 4) : RL * (8 / WC);
+    constexpr int RSTEP = HEAD ? kFinishThreads / (BN / 4) : RL * (8 / WC), CPW_LOG2 = CPW == 4 ? 2 : CPW - 1;
+    static_assert(CPW == 1 || CPW == 2 || CPW == 4, "columns of a warp");
     const int w = ptid >> 5, lane = ptid & 31;
     const int cg = HEAD ? ptid % (BN / 4) : (w % WC) * CPW + lane / RL, rg = HEAD ? ptid / (BN / 4) : (w / WC) * RL + lane % RL;
     const int co = n0 + cg * 4;
@@ -178,87 +164,91 @@ __device__ __forceinline__ void finish_rows(const ConvArgs& a, float* rx, int np
             bias.x += t.x; bias.y += t.y; bias.z += t.z; bias.w += t.w;
         }
     }
-    constexpr int PRE = 2;                                   // residual rows on their way at a time
+    constexpr int PRE = 2;                                   // rows on their way at a time
     float4 res[PRE];
-    auto load_residual = [&](int l0) {
+    size_t off[PRE];                                         // element of y (head: pixel of the frame)
+    bool valid[PRE];
+    auto place = [&](int first) {
 #pragma unroll
         for (int i = 0; i < PRE; ++i) {
             res[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-            int oy, ox;
-            if (!HEAD && a.residual && l0 + i * RSTEP < rpo && locate(l0 + i * RSTEP, oy, ox))
-                res[i] = __ldcg((const float4*)(a.residual + (((size_t)frame * OH + oy) * OW + ox) * a.Cout + co));
+            int oy = 0, ox = 0;
+            valid[i] = first + i * RSTEP < rpo && locate(first + i * RSTEP, oy, ox);
+            off[i] = HEAD ? (size_t)oy * OW + ox : (((size_t)frame * OH + oy) * OW + ox) * a.Cout + co;
+            asm volatile("" : "+l"(off[i]));
+            if (!HEAD && a.residual && valid[i]) res[i] = __ldcg((const float4*)(a.residual + off[i]));
         }
     };
-    load_residual(rg);
-    ready();
+    place(rg);
     // statistics: deviations from a value of the group (the first one inside the image that this warp holds)
-    const int cpg = !HEAD && a.out_rec ? a.Cout / a.out_G : 4, lpg = min(cpg >> 2, CPW);        // four-channel columns of a group in this warp
-    const uint32_t peers = (lpg * RL >= 32 ? 0xffffffffu : ((1u << (lpg * RL & 31)) - 1u)) << (lane / (lpg * RL) * (lpg * RL));
-    float sum = 0.f, sq = 0.f, cnt = 0.f, pivot = 0.f;
+    const int side_log2 = max(a.out_shift - 2 - CPW_LOG2, 0), part = ((w / WC) << side_log2) + ((w % WC) & ((1 << side_log2) - 1));
+    const int peer_lanes = RL << min(max(a.out_shift - 2, 0), CPW_LOG2);
+    uint32_t peers = (0xffffffffu >> (32 - peer_lanes)) << (lane & -peer_lanes & 31);
+    float4* rec = a.out_rec + ((size_t)frame * a.out_G + (co >> a.out_shift)) * a.out_slots + ((slot0 * (8 / WC)) << side_log2) + part;
+    asm volatile("" : "+l"(rec), "+r"(peers));
+    ready();
+    float sum = 0.f, sq = 0.f, pivot = 0.f;
+    int cnt = 0;
 #pragma unroll 1
     for (int l0 = rg - lane % RL; l0 < rpo; l0 += PRE * RSTEP) {
         const int first = l0 + lane % RL;
-        if (first != rg) load_residual(first);
+        if (first != rg) place(first);
 #pragma unroll
         for (int i = 0; i < PRE; ++i) {
             const int local = first + i * RSTEP;
-            int oy = 0, ox = 0;
-            const bool on = local < rpo, valid = on && locate(local, oy, ox);
-            const size_t pixel = ((size_t)frame * OH + oy) * OW + ox;
             float4 v = bias;
-            const float* q = rx + local * RXS + (cg ^ swizzle(local)) * 4;
+            if (valid[i]) {
+                const float* q = rx + local * RXS + (cg ^ swizzle(local)) * 4;
 #pragma unroll 4
-            for (int s = 0; s < nparts; ++s) {
-                if (!on) break;
-                const float4 p = *(const float4*)(q + (size_t)s * rpo * RXS);
-                v.x += p.x; v.y += p.y; v.z += p.z; v.w += p.w;
-            }
-            if (valid) {
+                for (int s = 0; s < nparts; ++s, q += rpo * RXS) {
+                    const float4 p = *(const float4*)q;
+                    v.x += p.x; v.y += p.y; v.z += p.z; v.w += p.w;
+                }
                 if (HEAD) {
                     const float f[4] = {v.x, v.y, v.z, v.w};
+                    const size_t plane = (size_t)OH * OW;
 #pragma unroll
                     for (int e = 0; e < 4; ++e) {
                         if (co + e >= a.Cout) break;
                         const float x = f[e] + (a.bias ? __ldg(a.bias + co + e) : 0.f);
-                        const size_t o = (((size_t)frame * a.Cout + co + e) * OH + oy) * OW + ox;
-                        if (a.out_u8) ((unsigned char*)a.y)[pixel * a.Cout + co + e] = pack_u8(x);
+                        const size_t o = ((size_t)frame * a.Cout + co + e) * plane + off[i];
+                        if (a.out_u8) ((unsigned char*)a.y)[(frame * plane + off[i]) * a.Cout + co + e] = pack_u8(x);
                         else if (a.out_dtype == VD_BF16) ((__nv_bfloat16*)a.y)[o] = __float2bfloat16_rn(x);
                         else ((float*)a.y)[o] = x;
                     }
                 } else if (a.out_dtype == VD_BF16) {
                     const uint32_t lo = tc::pack_bf16(v.x, v.y), hi = tc::pack_bf16(v.z, v.w);
-                    *(uint2*)((__nv_bfloat16*)a.y + pixel * a.Cout + co) = make_uint2(lo, hi);
+                    *(uint2*)((__nv_bfloat16*)a.y + off[i]) = make_uint2(lo, hi);
                     v = make_float4(__uint_as_float(lo << 16), __uint_as_float(lo & 0xffff0000u), __uint_as_float(hi << 16), __uint_as_float(hi & 0xffff0000u));
                 } else {
                     v.x += res[i].x; v.y += res[i].y; v.z += res[i].z; v.w += res[i].w;
-                    *(float4*)((float*)a.y + pixel * a.Cout + co) = v;
+                    *(float4*)((float*)a.y + off[i]) = v;
                 }
             }
             if (!HEAD && a.out_rec) {
-                if (l0 + i * RSTEP < RSTEP) {                // the warp's first rows
-                    const uint32_t m = __ballot_sync(0xffffffffu, valid) & peers;
+                const uint32_t m = __ballot_sync(0xffffffffu, valid[i]) & peers;
+                if (l0 + i * RSTEP < RSTEP)                  // the warp's first rows
                     pivot = __shfl_sync(0xffffffffu, v.x, m ? __ffs(m) - 1 : lane);
-                }
-                if (valid) {
+                cnt += __popc(m);
+                if (valid[i]) {
                     const float d0 = v.x - pivot, d1 = v.y - pivot, d2 = v.z - pivot, d3 = v.w - pivot;
                     sum += (d0 + d1) + (d2 + d3);
                     sq += fmaf(d0, d0, d1 * d1) + fmaf(d2, d2, d3 * d3);
-                    cnt += 4.f;
                 }
             }
         }
     }
     if (!HEAD && a.out_rec) {
-        for (int d = 1; d < lpg * RL; d <<= 1) {
-            sum += __shfl_xor_sync(0xffffffffu, sum, d);
-            sq += __shfl_xor_sync(0xffffffffu, sq, d);
-            cnt += __shfl_xor_sync(0xffffffffu, cnt, d);
-        }
-        if ((lane & (lpg * RL - 1)) == 0) {
-            const int side = max(cpg / (4 * CPW), 1), part = (w / WC) * side + (w % WC) % side;
-            const float dm = cnt > 0.f ? sum / cnt : 0.f;
-            a.out_rec[((size_t)frame * a.out_G + co / cpg) * a.out_slots + slot0 * (side * (8 / WC)) + part] =
-                make_float4(cnt, pivot + dm, fmaxf(fmaf(-dm, sum, sq), 0.f), 0.f);
+        const float n = (float)(cnt * 4), inv = cnt ? 1.f / n : 0.f;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1)
+            if (d < RL || d < peer_lanes) {
+                sum += __shfl_xor_sync(0xffffffffu, sum, d);
+                sq += __shfl_xor_sync(0xffffffffu, sq, d);
+            }
+        if ((lane & (peer_lanes - 1)) == 0) {
+            const float dm = sum * inv;
+            *rec = make_float4(n, pivot + dm, fmaxf(fmaf(-dm, sum, sq), 0.f), 0.f);
         }
     }
 }

@@ -164,16 +164,16 @@ conv_f32_kernel(const ConvArgs a, const int S, const int n_w, const int ops_floa
 #pragma unroll
         for (int e = 0; e < NE; ++e) {
             raw[e] = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (on && (vm >> e & 1u)) raw[e] = __ldg((const float4*)(src[e] + u * kChunk));
+            if (on && (vm >> e & 1u)) raw[e] = __ldcg((const float4*)(src[e] + u * kChunk));
         }
     };
     InputStats st;
-    if (a.in_rec) st.prepare(a, frame, c_first, nch, tid >> 5, lane);
+    if (a.in_rec) st.prepare(a, frame, c_first, nch, tid >> 5, lane, s_scale, s_shift);
     griddep_wait();                                          // everything above is arithmetic, weights and parameters
-    if (a.in_rec) st.load(a);
+    if (a.in_rec) st.load(a, lane);
     fetch(0);
     if (prologue) {
-        if (a.in_rec) st.finish(a, c_first, 1.f, s_scale, s_shift);
+        if (a.in_rec) st.finish(a, nch, lane, 1.f, s_scale, s_shift);
         else
             for (int c = tid; c < nch; c += kThreads) {
                 s_scale[c] = __ldg(a.scale + (size_t)frame * a.Cin + c_first + c);

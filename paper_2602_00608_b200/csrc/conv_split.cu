@@ -32,11 +32,8 @@ using convtile::A_TILE_BYTES;
 using convtile::ITEMS;
 using convtile::NPIX;
 using convtile::PW;
-using convtile::Raw8;
 using convtile::TILE_H;
 using convtile::TILE_W;
-using convtile::load_raw_at;
-using convtile::unpack_raw;
 
 constexpr int kWarps = 10, kThreads = kWarps * 32;           // MMA, weights, eight producer / epilogue warps
 constexpr int kProd0 = 2, kProd = 8 * 32;
@@ -224,7 +221,9 @@ conv_split_kernel(const ConvArgs a, const ConvSplitShape sh, const __grid_consta
         const float half = silu ? 0.5f : 1.0f;               // SiLU is evaluated as h + h * tanh(h), h = v / 2
         // what depends on the thread alone, before the kernel before has to be done
         int goff[kBatch];                                    // byte offset of the entry's source pixel
-        uint32_t soff[kBatch];                               // where its operand goes
+        // where its operand goes (entry e is kProd / 8 pixels, a multiple of the swizzle's eight rows, after entry 0)
+        const int pix0 = ptid >> 3;
+        const uint32_t soff = (uint32_t)(pix0 * 128) + (IN_BF16 ? (uint32_t)((j ^ (pix0 & 7)) << 4) : (uint32_t)((((j >> 1) ^ (pix0 & 7)) << 4) + (j & 1) * 8));
         uint32_t vm = 0u;                                    // entries inside the image
 #pragma unroll
         for (int e = 0; e < kBatch; ++e) {
@@ -234,27 +233,31 @@ conv_split_kernel(const ConvArgs a, const ConvSplitShape sh, const __grid_consta
             if (KIND == K1X1) v = v && py >= 1 && py <= TILE_H && px >= 1 && px <= TILE_W;
             vm |= (v ? 1u : 0u) << e;
             goff[e] = v ? (oy * W + ox) * a.Cin * ESZ : 0;
-            soff[e] = IN_BF16 ? (uint32_t)(pix * 128 + ((j ^ (pix & 7)) << 4)) : (uint32_t)(pix * 128 + (((j >> 1) ^ (pix & 7)) << 4) + (j & 1) * 8);
         }
         InputStats stats;
-        if (a.in_rec) stats.prepare(a, frame, k0 * 64, nch, pw, lane);
+        if (a.in_rec) stats.prepare(a, frame, k0 * 64, nch, pw, lane, s_scale, s_shift);
         const char* xb = (const char*)a.x + ((size_t)frame * H * W * a.Cin + k0 * 64 + (IN_BF16 ? j * 8 : j * 4)) * ESZ;
         griddep_wait();
-        if (a.in_rec) stats.load(a);
+        if (a.in_rec) stats.load(a, lane);
         uint32_t as = 0, aph = 0;
         bool ok = true;
+        // An entry's registers take the next chunk's values as soon as they have been read: 515 -> 465 us for one 64x64 frame,
+        // most of whose layers give a CTA two chunks.  fp32 input: 4 channels from the chunk's first half, 4 from its second.
+        constexpr int HALVES = IN_BF16 ? 1 : 2, NV = 8 / HALVES;
+        uint4 raw[HALVES][kBatch];
+        auto load = [&](int u, int h, int e) {
+            if (vm >> e & 1u) raw[h][e] = convtile::ldg_stream(xb + (size_t)u * (64 * ESZ) + goff[e] + h * 128);
+        };
+#pragma unroll
+        for (int h = 0; h < HALVES; ++h)
+#pragma unroll
+            for (int e = 0; e < kBatch; ++e) load(0, h, e);
 #pragma unroll 1
         for (int u = 0; u < units; ++u) {
             const bool second = BN == 64 && KIND == K3X3 && u >= nk;
             uint8_t* dst = smem_a + as * A_TILE_BYTES;
-            Raw8 raw[kBatch];
-            if (!second) {
-#pragma unroll
-                for (int e = 0; e < kBatch; ++e)
-                    if (vm >> e & 1u) load_raw_at(IN_BF16, xb + (size_t)u * (64 * ESZ) + goff[e], raw[e]);
-            }
             if (u == 0 && prologue) {
-                if (a.in_rec) stats.finish(a, k0 * 64, half, s_scale, s_shift);
+                if (a.in_rec) stats.finish(a, nch, lane, half, s_scale, s_shift);
                 else
                     for (int c = ptid; c < nch; c += kProd) {
                         s_scale[c] = __ldg(a.scale + (size_t)frame * a.Cin + k0 * 64 + c) * half;
@@ -272,35 +275,44 @@ conv_split_kernel(const ConvArgs a, const ConvSplitShape sh, const __grid_consta
                     tma_load_4d(smem_u32(dst), &tm_x2, (q0 + u - nk) * 32, tx, ty, frame, smem_u32(&bars->a_full[as]));
                 }
             } else {
-                float sc[8], sf[8];
-                if (prologue) {
-                    const int ca = u * 64 + (IN_BF16 ? j * 8 : j * 4), cb = IN_BF16 ? ca + 4 : ca + 32;
-                    *(float4*)&sc[0] = *(const float4*)(s_scale + ca); *(float4*)&sc[4] = *(const float4*)(s_scale + cb);
-                    *(float4*)&sf[0] = *(const float4*)(s_shift + ca); *(float4*)&sf[4] = *(const float4*)(s_shift + cb);
-                }
 #pragma unroll
-                for (int e = 0; e < kBatch; ++e) {
-                    if (e == kBatch - 1 && ((e * kProd + ptid) >> 3) >= NPIX) break;
-                    uint32_t o0 = 0u, o1 = 0u, o2 = 0u, o3 = 0u;
-                    if (vm >> e & 1u) {
-                        float v[8];
-                        unpack_raw(IN_BF16, raw[e], v);
-                        if (prologue) {
+                for (int h = 0; h < HALVES; ++h) {
+                    float sc[NV], sf[NV];
+                    if (prologue) {
+                        const int c = u * 64 + j * NV + h * 32;
 #pragma unroll
-                            for (int i = 0; i < 8; ++i) v[i] = fmaf(v[i], sc[i], sf[i]);
-                            if (silu) {
-#pragma unroll
-                                for (int i = 0; i < 8; ++i) v[i] = fmaf(v[i], tanh_fast(v[i]), v[i]);
-                            }
+                        for (int i = 0; i < NV; i += 4) {
+                            *(float4*)&sc[i] = *(const float4*)(s_scale + c + i);
+                            *(float4*)&sf[i] = *(const float4*)(s_shift + c + i);
                         }
-                        if (KIND == KPHASE) { o0 = pack_f16(v[0], v[1]); o1 = pack_f16(v[2], v[3]); o2 = pack_f16(v[4], v[5]); o3 = pack_f16(v[6], v[7]); }
-                        else { o0 = pack_bf16(v[0], v[1]); o1 = pack_bf16(v[2], v[3]); o2 = pack_bf16(v[4], v[5]); o3 = pack_bf16(v[6], v[7]); }
                     }
-                    if (IN_BF16) {
-                        *(uint4*)(dst + soff[e]) = make_uint4(o0, o1, o2, o3);
-                    } else {
-                        *(uint2*)(dst + soff[e]) = make_uint2(o0, o1);
-                        *(uint2*)(dst + (soff[e] ^ 64u)) = make_uint2(o2, o3);
+#pragma unroll
+                    for (int e = 0; e < kBatch; ++e) {
+                        if (e == kBatch - 1 && ((e * kProd + ptid) >> 3) >= NPIX) break;
+                        uint32_t o[NV / 2];
+#pragma unroll
+                        for (int i = 0; i < NV / 2; ++i) o[i] = 0u;
+                        if (vm >> e & 1u) {
+                            float v[NV];
+                            const uint32_t r[4] = {raw[h][e].x, raw[h][e].y, raw[h][e].z, raw[h][e].w};
+#pragma unroll
+                            for (int i = 0; i < NV; ++i)
+                                v[i] = __uint_as_float(!IN_BF16 ? r[i & 3] : (i & 1) ? r[i >> 1] & 0xffff0000u : r[i >> 1] << 16);
+                            if (u + 1 < nk) load(u + 1, h, e);
+                            if (prologue) {
+#pragma unroll
+                                for (int i = 0; i < NV; ++i) v[i] = fmaf(v[i], sc[i], sf[i]);
+                                if (silu) {
+#pragma unroll
+                                    for (int i = 0; i < NV; ++i) v[i] = fmaf(v[i], tanh_fast(v[i]), v[i]);
+                                }
+                            }
+#pragma unroll
+                            for (int i = 0; i < NV / 2; ++i) o[i] = KIND == KPHASE ? pack_f16(v[2 * i], v[2 * i + 1]) : pack_bf16(v[2 * i], v[2 * i + 1]);
+                        }
+                        uint8_t* d = dst + (h ? soff ^ 64u : soff) + e * (kProd * 16);
+                        if constexpr (IN_BF16) *(uint4*)d = make_uint4(o[0], o[1], o[2], o[3]);
+                        else *(uint2*)d = make_uint2(o[0], o[1]);
                     }
                 }
             }

@@ -287,7 +287,8 @@ class Planner {
         if ((f32 || split) && prologue) {
             Step& g = h_->steps.back();
             if (g.kind == VD_STEP_GN_STATS && g.gn.rec && !g.gn.offset && g.gn.slots <= kRecMergeSlots) {
-                a.in_rec = g.gn.rec; a.in_slots = g.gn.slots; a.in_pixels = g.gn.P;
+                a.in_rec = g.gn.rec; a.in_slots = g.gn.slots; a.in_shift = rec_shift(g.gn.C, g.gn.G);
+                a.in_inv_n = 1.f / ((float)g.gn.P * (float)(g.gn.C / g.gn.G));
                 a.in_gamma = g.gn.gamma; a.in_beta = g.gn.beta; a.in_G = g.gn.G; a.in_eps = g.gn.eps;
                 a.scale = a.shift = nullptr;
                 g.skip = true;
@@ -307,6 +308,7 @@ class Planner {
             a.out_slots = slots;
             a.out_pending = tc_rec && pending(y_off) != kNone ? ptr<float>(pending(y_off)) : nullptr;
             a.out_G = cfg_.norm_groups;
+            a.out_shift = rec_shift(Cout, cfg_.norm_groups);
             rec_[y_off] = {rec_buf_[rec_toggle_], slots};
             max_slots_ = std::max(max_slots_, slots);
         }

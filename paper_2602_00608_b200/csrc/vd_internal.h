@@ -49,11 +49,11 @@ struct ConvArgs {
     const float4* in_rec;        // or null
     const float* in_gamma;       // [Cin]
     const float* in_beta;        // [Cin]
-    int in_slots, in_G, in_pixels;   // in_pixels: pixels the statistics are over
-    float in_eps;
+    int in_slots, in_G, in_shift;    // in_shift: log2 of the channels of a group
+    float in_eps, in_inv_n;          // in_inv_n: 1 / values of a group
     float4* out_rec;             // or null (conv_tc.cu too)
     const float* out_pending;    // conv_tc.cu: the records are those of y + out_pending[c] (null: of y)
-    int out_slots, out_G;
+    int out_slots, out_G, out_shift;
     // tensor-core kernel: ceil(2^32 / d) for the divisors of its tile numbering (tiles per image, channel
     // blocks, tiles per row), filled in by its launcher; 0 stands for d = 1
     unsigned int div_tiles, div_nblk, div_tx;
@@ -159,6 +159,10 @@ constexpr int kRecMergeSlots = 128;                             // up to here th
 inline bool rec_groups_ok(int channels, int groups) {          // records of such groups can be written and merged
     const int cpg = groups > 0 ? channels / groups : 0;
     return groups > 0 && channels % groups == 0 && (cpg == 4 || cpg == 8 || cpg == 16);
+}
+inline int rec_shift(int channels, int groups) {               // log2 of the channels of such a group
+    const int cpg = channels / groups;
+    return cpg == 4 ? 2 : cpg == 8 ? 3 : 4;
 }
 cudaError_t launch_gn_merge(const GnArgs& a, cudaStream_t s);  // a.rec -> a.scale, a.shift
 
