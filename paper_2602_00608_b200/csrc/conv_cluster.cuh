@@ -58,6 +58,14 @@ __device__ __forceinline__ bool wait_cluster(uint32_t bar, uint32_t parity, vola
     return true;
 }
 
+// The launch's parameters come through the constant cache, a line at a time: one thread reads a word of every line while the
+// kernel before is still running, so that nobody waits for the first use of one later.  (The sum goes to an unused word of
+// shared memory, or nothing would be read.)
+__device__ __forceinline__ void touch_params(const ConvArgs& a, volatile uint32_t* unused) {
+    *unused = (uint32_t)(size_t)a.bias + (uint32_t)(size_t)a.y + (uint32_t)a.out_dtype + (uint32_t)(size_t)a.bias2 + (uint32_t)(size_t)a.stat_gamma +
+              __float_as_uint(a.stat_eps) + (uint32_t)a.in_slots + __float_as_uint(a.in_inv_n) + (uint32_t)(size_t)a.out_rec + (uint32_t)a.out_shift + (uint32_t)a.silu + a.div_tx;
+}
+
 // half * scale and half * shift of the input channels [c0, c0 + nch) of `frame`, from the producing layer's records, by
 // eight warps (w = 0..7); c0 and nch are multiples of the group size.  A group has 8 lanes of a warp (32 where there are more
 // than 16 records); a lane's first two records are loaded by `load`, so that they are on their way before other loads, and

@@ -61,7 +61,7 @@ __device__ __forceinline__ unsigned long long pair(float x, float y) {
 struct FBars {
     uint64_t w_full[kMaxW];
     uint64_t rx_full;
-    uint32_t abort_flag;
+    uint32_t abort_flag, unused;
 };
 
 // Geometry of a build.  BN = 4: the frame head (at most four output channels; its weights are read with plain loads).
@@ -169,6 +169,7 @@ conv_f32_kernel(const ConvArgs a, const int S, const int n_w, const int ops_floa
     };
     InputStats st;
     if (a.in_rec) st.prepare(a, frame, c_first, nch, tid >> 5, lane, s_scale, s_shift);
+    if (tid == 0) touch_params(a, &bars->unused);
     griddep_wait();                                          // everything above is arithmetic, weights and parameters
     if (a.in_rec) st.load(a, lane);
     fetch(0);

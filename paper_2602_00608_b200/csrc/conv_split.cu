@@ -49,7 +49,7 @@ struct SBars {
     uint64_t a_full[kMaxA], a_empty[kMaxA];
     uint64_t b_full[kMaxB], b_empty[kMaxB];
     uint64_t acc_full, rx_full;
-    uint32_t tmem_base, abort_flag;
+    uint32_t tmem_base, abort_flag, unused;
 };
 
 // arrives, once the MMAs issued so far have completed, on the barrier at this offset in every CTA of `mask`
@@ -237,6 +237,7 @@ conv_split_kernel(const ConvArgs a, const ConvSplitShape sh, const __grid_consta
         InputStats stats;
         if (a.in_rec) stats.prepare(a, frame, k0 * 64, nch, pw, lane, s_scale, s_shift);
         const char* xb = (const char*)a.x + ((size_t)frame * H * W * a.Cin + k0 * 64 + (IN_BF16 ? j * 8 : j * 4)) * ESZ;
+        if (ptid == 0) touch_params(a, &bars->unused);
         griddep_wait();
         if (a.in_rec) stats.load(a, lane);
         uint32_t as = 0, aph = 0;
