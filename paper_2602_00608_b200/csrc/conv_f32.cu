@@ -29,9 +29,8 @@ namespace {
 using namespace cc;
 using namespace tc;
 
-constexpr int kThreads = 256, kTW = 8, kChunk = 16;          // threads, tile width, input channels per chunk
+constexpr int kThreads = 256, kChunk = 16;                   // threads, input channels per chunk
 constexpr int kMaxW = 8;                                     // weight stages
-constexpr int kRow = 12;                                     // floats per tile row in shared memory (10 used; 16-byte rows)
 
 enum { K3X3 = 0, K1X1 = 1, KPHASE = 2 };
 
@@ -64,17 +63,19 @@ struct FBars {
     uint32_t abort_flag, unused;
 };
 
-// Geometry of a build.  BN = 4: the frame head (at most four output channels; its weights are read with plain loads).
-template <int TH, int BN, int KIND> struct FCfg {
+// Geometry of a build: a tile of TH x TW pixels (a thread has eight pixels of a row).  BN = 4: the frame head (at most four
+// output channels; its weights are read with plain loads).
+template <int TH, int BN, int KIND, int TW = 8> struct FCfg {
     static constexpr int KH = KIND == K3X3 ? 3 : (KIND == K1X1 ? 1 : 2), TAPS = KH * KH;
-    static constexpr int RH = TH + KH - 1, RW = kTW + KH - 1;            // rows and columns of the input tile
-    static constexpr int CS = (RH * kRow + 7) / 8 * 8 + 4;               // floats per channel: four channels of a pixel on distinct banks
-    static constexpr int KT = kThreads / (TH * (BN / 4));                // thread groups along K
+    static constexpr int RH = TH + KH - 1, RW = TW + KH - 1;            // rows and columns of the input tile
+    static constexpr int ROW = TW + 4;                                   // floats per tile row (16-byte rows; KH - 1 of the four extra ones used)
+    static constexpr int CS = (RH * ROW + 7) / 8 * 8 + 4;                // floats per channel: four channels of a pixel on distinct banks
+    static constexpr int NG = TW / 8, KT = kThreads / (TH * NG * (BN / 4));             // thread groups along K
     static constexpr int IN_FLOATS = kChunk * CS;
     static constexpr int W_FLOATS = TAPS * kChunk * BN;
-    static constexpr int RX_FLOATS = TH * kTW * BN;                      // one partial of the tile
+    static constexpr int RX_FLOATS = TH * TW * BN;                       // one partial of the tile
     static constexpr int PART_FLOATS = KT / 2 * RX_FLOATS;               // partials of half the K groups at a time
-    static_assert(KT >= 2 && kThreads % (TH * (BN / 4)) == 0 && CS % 4 == 0, "thread layout");
+    static_assert(KT >= 2 && kThreads % (TH * NG * (BN / 4)) == 0 && CS % 4 == 0, "thread layout");
 };
 constexpr int kMaxSlice = 512;                               // input channels of one CTA
 constexpr int kFTail = 2 * kMaxSlice * 4 + 128;              // scale / shift of the slice, barriers
@@ -83,12 +84,13 @@ constexpr int kFTail = 2 * kMaxSlice * 4 + 128;              // scale / shift of
 // threads that write it (eight tile rows side by side) nor those that read it (eight pixels of a row) meet on a bank.
 template <int BN> __device__ __forceinline__ int piece(int R) { return BN < 32 ? 0 : (R ^ (R >> 3)) & 7; }
 
-template <int TH, int BN, int KIND>
+template <int TH, int BN, int KIND, int TW>
 __global__ void __launch_bounds__(kThreads, 2)
 conv_f32_kernel(const ConvArgs a, const int S, const int n_w, const int ops_floats, const __grid_constant__ CUtensorMap tm_w, unsigned int* status) {
-    using C = FCfg<TH, BN, KIND>;
+    using C = FCfg<TH, BN, KIND, TW>;
     constexpr bool HEAD = BN < 32;
-    constexpr int KH = C::KH, CS = C::CS, KT = C::KT;
+    constexpr int KH = C::KH, CS = C::CS, KT = C::KT, ROW = C::ROW;
+    static_assert(TW == 8 || HEAD, "wide tiles");
     extern __shared__ uint8_t smem_raw[];
     float* s_in = (float*)(((uintptr_t)smem_raw + 127) & ~(uintptr_t)127);           // two input chunks
     float* s_w = s_in + (2 * C::IN_FLOATS + 31) / 32 * 32;                           // n_w weight stages (head: the whole slice)
@@ -102,7 +104,7 @@ conv_f32_kernel(const ConvArgs a, const int S, const int n_w, const int ops_floa
     const int tid = threadIdx.x, lane = tid & 31;
     const int rank = S > 1 ? (int)ctarank() : 0;
     const int H = KIND == KPHASE ? a.Hs : a.H, W = KIND == KPHASE ? a.Ws : a.W;      // the tile grid is that of the source
-    const int tiles_x = (W + kTW - 1) / kTW, tiles = tiles_x * ((H + TH - 1) / TH);
+    const int tiles_x = (W + TW - 1) / TW, tiles = tiles_x * ((H + TH - 1) / TH);
     const int nblk = HEAD ? 1 : a.Cout / BN;
     int item = (int)blockIdx.x / S;
     const int n0 = (item % nblk) * BN;
@@ -110,7 +112,7 @@ conv_f32_kernel(const ConvArgs a, const int S, const int n_w, const int ops_floa
     const int par = KIND == KPHASE ? (item & 3) : 0;
     if (KIND == KPHASE) item >>= 2;
     const int tile = item % tiles, frame = item / tiles;
-    const int ty = (tile / tiles_x) * TH, tx = (tile % tiles_x) * kTW;
+    const int ty = (tile / tiles_x) * TH, tx = (tile % tiles_x) * TW;
     const int oy0 = KIND == K3X3 ? -1 : (KIND == KPHASE ? (par >> 1) - 1 : 0), ox0 = KIND == K3X3 ? -1 : (KIND == KPHASE ? (par & 1) - 1 : 0);
     const int chunks = (a.Cin + kChunk - 1) / kChunk;
     const int k0 = rank * chunks / S, units = (rank + 1) * chunks / S - k0;
@@ -149,7 +151,8 @@ conv_f32_kernel(const ConvArgs a, const int S, const int n_w, const int ops_floa
     const bool prologue = a.scale != nullptr || a.in_rec != nullptr, silu = a.silu != 0, round = a.bf16_operands != 0;
     float4 raw[NE];
     uint32_t vm = 0u;                                        // entries inside the image
-    const float* src[NE];
+    unsigned int src[NE];                                    // in pieces of four channels
+    const float4* const image = (const float4*)((const float*)a.x + (size_t)frame * H * W * a.Cin + c_first);
     const int quad = tid & 3;
 #pragma unroll
     for (int e = 0; e < NE; ++e) {
@@ -157,14 +160,14 @@ conv_f32_kernel(const ConvArgs a, const int S, const int n_w, const int ops_floa
         const int y = ty + oy0 + py, x = tx + ox0 + px;
         const bool v = py < C::RH && y >= 0 && y < H && x >= 0 && x < W;
         vm |= (v ? 1u : 0u) << e;
-        src[e] = (const float*)a.x + (((size_t)frame * H + (v ? y : 0)) * W + (v ? x : 0)) * a.Cin + c_first + quad * 4;
+        src[e] = v ? (unsigned int)(y * W + x) * (unsigned int)(a.Cin >> 2) + quad : 0u;
     }
     auto fetch = [&](int u) {
         const bool on = u * kChunk + quad * 4 < nch;         // (Cin is a multiple of 4)
 #pragma unroll
         for (int e = 0; e < NE; ++e) {
             raw[e] = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (on && (vm >> e & 1u)) raw[e] = __ldcg((const float4*)(src[e] + u * kChunk));
+            if (on && (vm >> e & 1u)) raw[e] = __ldcg(image + src[e] + u * (kChunk / 4));
         }
     };
     InputStats st;
@@ -184,9 +187,10 @@ conv_f32_kernel(const ConvArgs a, const int S, const int n_w, const int ops_floa
     }
 
     // thread = (K group, 4 channels, tile row); a warp holds 8 rows x 4 channel columns (head: 16 rows x 2 K groups)
+    const int ng = HEAD && TW > 8 ? tid / TH % C::NG : 0;    // eight-pixel group of the row
     const int row = HEAD ? tid % TH : (TH == 8 ? tid & 7 : (tid & 7) + ((tid >> 6) & 1) * 8);
     const int cg = HEAD ? 0 : (tid >> 3) & 7;
-    const int kt = HEAD ? tid / TH : tid / (TH * (BN / 4));
+    const int kt = HEAD ? tid / (TH * C::NG) : tid / (TH * (BN / 4));
     unsigned long long acc[8][2];
 #pragma unroll
     for (int p = 0; p < 8; ++p) acc[p][0] = acc[p][1] = 0ull;
@@ -212,7 +216,7 @@ conv_f32_kernel(const ConvArgs a, const int S, const int n_w, const int ops_floa
                         if (round) v[q] = __bfloat162float(__float2bfloat16_rn(v[q]));
                     }
                 }
-                float* d = buf + quad * 4 * CS + py * kRow + px;
+                float* d = buf + quad * 4 * CS + py * ROW + px;
 #pragma unroll
                 for (int q = 0; q < 4; ++q) d[q * CS] = v[q];
             }
@@ -223,7 +227,7 @@ conv_f32_kernel(const ConvArgs a, const int S, const int n_w, const int ops_floa
             if (tid == 0 && u > 0 && u - 1 + n_w < units) load_weights(u - 1 + n_w);
             (void)mbar_wait(smem_u32(&bars->w_full[u % n_w]), (u / n_w) & 1, abort_flag);
         }
-        const float* ip = buf + row * kRow;
+        const float* ip = buf + row * ROW + ng * 8;
         const float* wp = s_w + (HEAD ? u : u % n_w) * C::W_FLOATS + cg * 4;
         const int cmax = min(kChunk, nch - u * kChunk);
 #pragma unroll 1
@@ -231,7 +235,7 @@ conv_f32_kernel(const ConvArgs a, const int S, const int n_w, const int ops_floa
 #pragma unroll
             for (int ky = 0; ky < KH; ++ky) {
                 float p[8 + KH];
-                const float* q = ip + c * CS + ky * kRow;
+                const float* q = ip + c * CS + ky * ROW;
                 *(float4*)&p[0] = *(const float4*)q;
                 *(float4*)&p[4] = *(const float4*)(q + 4);
                 if (KH == 3) { const float2 t = *(const float2*)(q + 8); p[8] = t.x; p[9] = t.y; }
@@ -254,8 +258,8 @@ conv_f32_kernel(const ConvArgs a, const int S, const int n_w, const int ops_floa
 
     // ---- the K groups' partials are added in halves (a fixed order); the first group keeps the sum
     auto at = [&](int slab, int i) -> float4* {
-        const int R = row * kTW + i;
-        return (float4*)(part + (slab * TH * kTW + R) * BN + (cg ^ piece<BN>(R)) * 4);
+        const int R = row * TW + ng * 8 + i;
+        return (float4*)(part + (slab * TH * TW + R) * BN + (cg ^ piece<BN>(R)) * 4);
     };
     auto put = [&](int slab) {
 #pragma unroll
@@ -280,8 +284,8 @@ conv_f32_kernel(const ConvArgs a, const int S, const int n_w, const int ops_floa
         }
     }
     if (kt == 0) put(0);                                     // (where it has just read itself)
-    // ---- row R of the tile's TH x 8 belongs to CTA R / rpo of the cluster
-    const int rpo = TH * kTW / S;
+    // ---- row R of the tile's TH x TW belongs to CTA R / rpo of the cluster
+    const int rpo = TH * TW / S;
     if (S > 1) {
         if (kt == 0) fence_proxy_async_smem();
         __syncthreads();
@@ -298,8 +302,8 @@ conv_f32_kernel(const ConvArgs a, const int S, const int n_w, const int ops_floa
                         (KIND == KPHASE ? tile * 4 + par : tile) * S + rank,
                         [&](int local, int& oy, int& ox) -> bool {
                             const int R = rank * rpo + local;
-                            oy = ty + R / kTW;
-                            ox = tx + R % kTW;
+                            oy = ty + R / TW;
+                            ox = tx + R % TW;
                             const bool valid = oy < H && ox < W;
                             if (KIND == KPHASE) { oy = 2 * oy + (par >> 1); ox = 2 * ox + (par & 1); }
                             return valid;
@@ -345,20 +349,20 @@ __global__ void pack_weight_f32_phase_kernel(const T* w, float* packed, int Cout
 constexpr int kMaxDevices = 64;
 std::mutex g_mu;
 
-template <int TH, int BN, int KIND>
+template <int TH, int BN, int KIND, int TW = 8>
 int ops_floats(int n_w) {                                    // operand stages; the partials lie over them
-    using C = FCfg<TH, BN, KIND>;
+    using C = FCfg<TH, BN, KIND, TW>;
     return std::max((2 * C::IN_FLOATS + 31) / 32 * 32 + n_w * C::W_FLOATS, C::PART_FLOATS);
 }
-template <int TH, int BN, int KIND>
+template <int TH, int BN, int KIND, int TW = 8>
 int smem_bytes(int n_w, int splits) {
-    using C = FCfg<TH, BN, KIND>;
-    return (ops_floats<TH, BN, KIND>(n_w) + (splits > 1 ? C::RX_FLOATS : 0)) * 4 + kFTail + 128;
+    using C = FCfg<TH, BN, KIND, TW>;
+    return (ops_floats<TH, BN, KIND, TW>(n_w) + (splits > 1 ? C::RX_FLOATS : 0)) * 4 + kFTail + 128;
 }
 
-template <int TH, int BN, int KIND>
+template <int TH, int BN, int KIND, int TW = 8>
 cudaError_t launch_one(const ConvArgs& a, const ConvF32Plan& p, unsigned int* status, cudaStream_t s) {
-    auto kern = conv_f32_kernel<TH, BN, KIND>;
+    auto kern = conv_f32_kernel<TH, BN, KIND, TW>;
     static bool configured[kMaxDevices] = {};
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
@@ -373,12 +377,12 @@ cudaError_t launch_one(const ConvArgs& a, const ConvF32Plan& p, unsigned int* st
         }
     }
     const int H = KIND == KPHASE ? a.Hs : a.H, W = KIND == KPHASE ? a.Ws : a.W;
-    const long long grid = (long long)((W + kTW - 1) / kTW) * ((H + TH - 1) / TH) * (BN < 32 ? 1 : a.Cout / BN) * (KIND == KPHASE ? 4 : 1) * a.B * p.splits;
+    const long long grid = (long long)((W + TW - 1) / TW) * ((H + TH - 1) / TH) * (BN < 32 ? 1 : a.Cout / BN) * (KIND == KPHASE ? 4 : 1) * a.B * p.splits;
     if (grid > 0x7fffffffLL) return cudaErrorInvalidValue;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)grid);
     cfg.blockDim = dim3(kThreads);
-    cfg.dynamicSmemBytes = (size_t)smem_bytes<TH, BN, KIND>(p.n_w, p.splits);
+    cfg.dynamicSmemBytes = (size_t)smem_bytes<TH, BN, KIND, TW>(p.n_w, p.splits);
     cfg.stream = s;
     cudaLaunchAttribute attr[2];
     int na = 0;
@@ -392,7 +396,7 @@ cudaError_t launch_one(const ConvArgs& a, const ConvF32Plan& p, unsigned int* st
     }
     cfg.attrs = attr;
     cfg.numAttrs = na;
-    return cudaLaunchKernelEx(&cfg, kern, a, p.splits, p.n_w, ops_floats<TH, BN, KIND>(p.n_w), *(const CUtensorMap*)p.tmap, status);
+    return cudaLaunchKernelEx(&cfg, kern, a, p.splits, p.n_w, ops_floats<TH, BN, KIND, TW>(p.n_w), *(const CUtensorMap*)p.tmap, status);
 }
 
 int kind_of(const ConvArgs& a) { return a.upsample == 2 ? KPHASE : (a.ksize == 1 ? K1X1 : K3X3); }
@@ -419,7 +423,10 @@ bool conv_f32_choose(const ConvArgs& a, ConvF32Plan* p) {
     const int rows8 = (H + 7) / 8 * 8, rows16 = (H + 15) / 16 * 16;
     p->th = !head && rows16 * 7 > rows8 * 8 ? 8 : 16;
     p->bn = head ? 4 : 32;
-    const int tiles = ((W + kTW - 1) / kTW) * ((H + p->th - 1) / p->th), chunks = (a.Cin + kChunk - 1) / kChunk;
+    // the frame head of a large image: tiles 32 pixels wide (see FCfg), unless they are more than half padding
+    const long long wide = (long long)((W + 31) / 32) * ((H + 15) / 16);
+    p->tw = head && wide * std::max(a.B, 1) >= 148 && (W + 31) / 32 * 2 <= (W + 7) / 8 ? 32 : 8;
+    const int tiles = ((W + p->tw - 1) / p->tw) * ((H + p->th - 1) / p->th), chunks = (a.Cin + kChunk - 1) / kChunk;
     const long long ctas = (long long)tiles * (head ? 1 : a.Cout / 32) * (kind == KPHASE ? 4 : 1) * std::max(a.B, 1);
     int s = 1;
     while (s < 8 && 2 * s <= chunks && ctas * 2 * s <= 296) s *= 2;
@@ -443,7 +450,7 @@ bool conv_f32_choose(const ConvArgs& a, ConvF32Plan* p) {
 
 int conv_f32_slots(const ConvArgs& a, const ConvF32Plan& p, int groups) {
     const int H = a.upsample == 2 ? a.Hs : a.H, W = a.upsample == 2 ? a.Ws : a.W;
-    return ((W + kTW - 1) / kTW) * ((H + p.th - 1) / p.th) * (a.upsample == 2 ? 4 : 1) * p.splits * rec_parts(p.bn, a.Cout / groups);
+    return ((W + p.tw - 1) / p.tw) * ((H + p.th - 1) / p.th) * (a.upsample == 2 ? 4 : 1) * p.splits * rec_parts(p.bn, a.Cout / groups);
 }
 
 cudaError_t conv_f32_prepare(const ConvArgs& a, ConvF32Plan* p) {
@@ -468,7 +475,7 @@ cudaError_t launch_conv_f32(const ConvArgs& a, const ConvF32Plan& p, unsigned in
     if (a.in_rec && !rec_groups_ok(a.Cin, a.in_G)) return cudaErrorInvalidValue;
     if (a.out_rec && !rec_groups_ok(a.Cout, a.out_G)) return cudaErrorInvalidValue;
     const int kind = kind_of(a);
-    if (p.bn == 4) return launch_one<16, 4, K3X3>(a, p, status, s);
+    if (p.bn == 4) return p.tw == 32 ? launch_one<16, 4, K3X3, 32>(a, p, status, s) : launch_one<16, 4, K3X3>(a, p, status, s);
     if (p.th == 8) {
         if (kind == K3X3) return launch_one<8, 32, K3X3>(a, p, status, s);
         return kind == K1X1 ? launch_one<8, 32, K1X1>(a, p, status, s) : launch_one<8, 32, KPHASE>(a, p, status, s);

@@ -169,7 +169,7 @@ cudaError_t launch_gn_merge(const GnArgs& a, cudaStream_t s);  // a.rec -> a.sca
 // ---- single-precision convolution (conv_f32.cu)
 struct alignas(64) ConvF32Plan {
     unsigned char tmap[128];    // weights, fp32 [tap][Cin][Cout]
-    int th, bn;                 // tile height, output channels per CTA (4: frame head)
+    int th, tw, bn;             // tile, output channels per CTA (4: frame head)
     int splits;                 // CTAs that share K (the cluster)
     int n_w;                    // weight stages
     int valid;

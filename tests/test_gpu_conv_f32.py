@@ -20,6 +20,8 @@ CASES = [
     dict(B=2, H=8, W=11, Cin=128, Cout=64, k=3, upsample=2, prologue=False, silu=False, residual=False),
     dict(B=1, H=35, W=26, Cin=32, Cout=32, k=3, upsample=2, prologue=True, silu=True, residual=False),
     dict(B=2, H=19, W=23, Cin=128, Cout=3, k=3, upsample=False, prologue=True, silu=True, residual=False, out_nchw=True),
+    dict(B=2, H=135, W=290, Cin=36, Cout=3, k=3, upsample=False, prologue=True, silu=True, residual=False, out_nchw=True),   # 32-pixel tiles
+    dict(B=1, H=592, W=128, Cin=64, Cout=4, k=3, upsample=False, prologue=True, silu=True, residual=False, out_nchw=True),   # and a cluster
     dict(B=1, H=5, W=3, Cin=20, Cout=3, k=3, upsample=False, prologue=False, silu=False, residual=False, out_nchw=True),
 ]
 
