@@ -58,7 +58,7 @@ __device__ __forceinline__ bool wait_cluster(uint32_t bar, uint32_t parity, vola
     return true;
 }
 
-// The launch's parameters come through the constant cache, a line at a time: one thread reads a word of every line while the
+// The launch's parameters come through the constant cache, a line at a time: one warp reads a word of every line while the
 // kernel before is still running, so that nobody waits for the first use of one later.  (The sum goes to an unused word of
 // shared memory, or nothing would be read.)
 __device__ __forceinline__ void touch_params(const ConvArgs& a, volatile uint32_t* unused) {

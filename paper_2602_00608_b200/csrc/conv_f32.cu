@@ -172,7 +172,7 @@ conv_f32_kernel(const ConvArgs a, const int S, const int n_w, const int ops_floa
     };
     InputStats st;
     if (a.in_rec) st.prepare(a, frame, c_first, nch, tid >> 5, lane, s_scale, s_shift);
-    if (tid == 0) touch_params(a, &bars->unused);
+    if (tid < 32) touch_params(a, &bars->unused);
     griddep_wait();                                          // everything above is arithmetic, weights and parameters
     if (a.in_rec) st.load(a, lane);
     fetch(0);
@@ -180,8 +180,8 @@ conv_f32_kernel(const ConvArgs a, const int S, const int n_w, const int ops_floa
         if (a.in_rec) st.finish(a, nch, lane, 1.f, s_scale, s_shift);
         else
             for (int c = tid; c < nch; c += kThreads) {
-                s_scale[c] = __ldg(a.scale + (size_t)frame * a.Cin + c_first + c);
-                s_shift[c] = __ldg(a.shift + (size_t)frame * a.Cin + c_first + c);
+                s_scale[c] = __ldcg(a.scale + (size_t)frame * a.Cin + c_first + c);
+                s_shift[c] = __ldcg(a.shift + (size_t)frame * a.Cin + c_first + c);
             }
         __syncthreads();
     }

@@ -237,7 +237,7 @@ conv_split_kernel(const ConvArgs a, const ConvSplitShape sh, const __grid_consta
         InputStats stats;
         if (a.in_rec) stats.prepare(a, frame, k0 * 64, nch, pw, lane, s_scale, s_shift);
         const char* xb = (const char*)a.x + ((size_t)frame * H * W * a.Cin + k0 * 64 + (IN_BF16 ? j * 8 : j * 4)) * ESZ;
-        if (ptid == 0) touch_params(a, &bars->unused);
+        if (pw == 0) touch_params(a, &bars->unused);
         griddep_wait();
         if (a.in_rec) stats.load(a, lane);
         uint32_t as = 0, aph = 0;
@@ -261,8 +261,8 @@ conv_split_kernel(const ConvArgs a, const ConvSplitShape sh, const __grid_consta
                 if (a.in_rec) stats.finish(a, nch, lane, half, s_scale, s_shift);
                 else
                     for (int c = ptid; c < nch; c += kProd) {
-                        s_scale[c] = __ldg(a.scale + (size_t)frame * a.Cin + k0 * 64 + c) * half;
-                        s_shift[c] = __ldg(a.shift + (size_t)frame * a.Cin + k0 * 64 + c) * half;
+                        s_scale[c] = __ldcg(a.scale + (size_t)frame * a.Cin + k0 * 64 + c) * half;
+                        s_shift[c] = __ldcg(a.shift + (size_t)frame * a.Cin + k0 * 64 + c) * half;
                     }
                 named_barrier_sync(1, kProd);
             }

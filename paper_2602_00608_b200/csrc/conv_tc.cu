@@ -708,12 +708,12 @@ conv_tc_kernel(const ConvArgs a, const __grid_constant__ CUtensorMap tmap, const
             float sc[8], sh[8];
             auto load_affine = [&](const Pos& p) {               // GroupNorm scale/shift of the unit's channels
                 if (!prologue || (X2 && p.kc >= kchunks)) return;
-                // channels of v[0..3] and v[4..7] (see load_raw); the tiles of an item lie in one frame
+                // channels of v[0..3] and v[4..7] (see load_raw_at); the tiles of an item lie in one frame
                 const int ca = p.kc * 64 + (IN_BF16 ? j * 8 : j * 4), cb = IN_BF16 ? ca + 4 : ca + 32;
                 const float* ps = a.scale + (size_t)p.tile.b * a.Cin;
                 const float* pt = a.shift + (size_t)p.tile.b * a.Cin;
-                const float4 s0 = __ldg((const float4*)(ps + ca)), s1 = __ldg((const float4*)(ps + cb));
-                const float4 t0 = __ldg((const float4*)(pt + ca)), t1 = __ldg((const float4*)(pt + cb));
+                const float4 s0 = *(const float4*)(ps + ca), s1 = *(const float4*)(ps + cb);
+                const float4 t0 = *(const float4*)(pt + ca), t1 = *(const float4*)(pt + cb);
                 sc[0] = s0.x; sc[1] = s0.y; sc[2] = s0.z; sc[3] = s0.w; sc[4] = s1.x; sc[5] = s1.y; sc[6] = s1.z; sc[7] = s1.w;
                 sh[0] = t0.x; sh[1] = t0.y; sh[2] = t0.z; sh[3] = t0.w; sh[4] = t1.x; sh[5] = t1.y; sh[6] = t1.z; sh[7] = t1.w;
                 if (silu) {          // SiLU is evaluated as h + h*tanh(h) with h = v/2: the 1/2 folds into the affine map
@@ -805,12 +805,12 @@ conv_tc_kernel(const ConvArgs a, const __grid_constant__ CUtensorMap tmap, const
                 const bool pro = prologue && !second;
                 float sc[8], sh[8];
                 if (pro) {
-                    // channels of v[0..3] and v[4..7] (see load_raw); the tiles of an item lie in one frame
+                    // channels of v[0..3] and v[4..7] (see load_raw_at); the tiles of an item lie in one frame
                     const int ca = c0 + (IN_BF16 ? j * 8 : j * 4), cb = IN_BF16 ? ca + 4 : ca + 32;
                     const float* ps = a.scale + (size_t)tile0.b * a.Cin;
                     const float* pt = a.shift + (size_t)tile0.b * a.Cin;
-                    const float4 s0 = __ldg((const float4*)(ps + ca)), s1 = __ldg((const float4*)(ps + cb));
-                    const float4 t0 = __ldg((const float4*)(pt + ca)), t1 = __ldg((const float4*)(pt + cb));
+                    const float4 s0 = *(const float4*)(ps + ca), s1 = *(const float4*)(ps + cb);
+                    const float4 t0 = *(const float4*)(pt + ca), t1 = *(const float4*)(pt + cb);
                     sc[0] = s0.x; sc[1] = s0.y; sc[2] = s0.z; sc[3] = s0.w; sc[4] = s1.x; sc[5] = s1.y; sc[6] = s1.z; sc[7] = s1.w;
                     sh[0] = t0.x; sh[1] = t0.y; sh[2] = t0.z; sh[3] = t0.w; sh[4] = t1.x; sh[5] = t1.y; sh[6] = t1.z; sh[7] = t1.w;
                     if (silu) {          // SiLU is evaluated as h + h*tanh(h) with h = v/2: the 1/2 folds into the affine map

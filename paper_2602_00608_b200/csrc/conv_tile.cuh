@@ -35,27 +35,18 @@ constexpr int OUT_SLICE_BYTES = 128 * 128;                           // 128 pixe
 
 struct Raw8 { uint4 lo, hi; };   // eight channels of one pixel: bf16 -> lo only; fp32 -> lo + hi
 
+// The activations are streamed (no reuse within the SM): they bypass L1 allocation, which leaves the small L1 that remains
+// beside the shared-memory tiles to the data that is reused.  Not the non-coherent form (.nc): the kernel before is still
+// writing them while this one starts, and a .nc load may be moved up across the wait for it or hit what L1 kept from before
+// (seen: decodes that differed from call to call).
+__device__ __forceinline__ uint4 ldg_stream(const void* p) {
+    uint4 r;
+    asm volatile("ld.global.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w) : "l"(p) : "memory");
+    return r;
+}
 // bf16: the thread's 16 bytes are channels [8j, 8j+8) of the chunk.  fp32: two 16-byte loads,
 // channels [4j, 4j+4) and [32+4j, 32+4j+4), so that the eight threads of a pixel read two
 // contiguous 128-byte lines.
-__device__ __forceinline__ void load_raw(bool is_bf16, const void* x, size_t pix_off, int c0, int j, Raw8& r) {
-    if (is_bf16) {
-        r.lo = __ldg((const uint4*)((const __nv_bfloat16*)x + pix_off + c0 + j * 8));
-    } else {
-        const float* p = (const float*)x + pix_off + c0 + j * 4;
-        const float4 a = __ldg((const float4*)p), b = __ldg((const float4*)(p + 32));
-        r.lo = make_uint4(__float_as_uint(a.x), __float_as_uint(a.y), __float_as_uint(a.z), __float_as_uint(a.w));
-        r.hi = make_uint4(__float_as_uint(b.x), __float_as_uint(b.y), __float_as_uint(b.z), __float_as_uint(b.w));
-    }
-}
-// the same loads from the address of the thread's first channel.  The activations are streamed
-// (no reuse within the SM): they bypass L1 allocation, which leaves the small L1 that remains beside
-// the shared-memory tiles to the data that is reused.
-__device__ __forceinline__ uint4 ldg_stream(const void* p) {
-    uint4 r;
-    asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w) : "l"(p));
-    return r;
-}
 __device__ __forceinline__ void load_raw_at(bool is_bf16, const char* p, Raw8& r) {
     r.lo = ldg_stream(p);
     if (!is_bf16) r.hi = ldg_stream(p + 128);

@@ -66,11 +66,11 @@ __global__ void ingest_kernel(IngestArgs a) {
 // the result is bitwise reproducible and independent of the batch a sample is decoded in.
 template <typename T> __device__ __forceinline__ void load4(const T* p, float v[4]);
 template <> __device__ __forceinline__ void load4<float>(const float* p, float v[4]) {
-    const float4 t = __ldg((const float4*)p);
+    const float4 t = *(const float4*)p;
     v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
 }
 template <> __device__ __forceinline__ void load4<__nv_bfloat16>(const __nv_bfloat16* p, float v[4]) {
-    const uint2 t = __ldg((const uint2*)p);
+    const uint2 t = *(const uint2*)p;
     v[0] = __uint_as_float(t.x << 16); v[1] = __uint_as_float(t.x & 0xffff0000u);
     v[2] = __uint_as_float(t.y << 16); v[3] = __uint_as_float(t.y & 0xffff0000u);
 }
@@ -84,12 +84,12 @@ __device__ __forceinline__ uint64_t policy_evict_first() {
 }
 template <typename T> __device__ __forceinline__ void load4_stream(const T* p, float v[4], uint64_t pol);
 template <> __device__ __forceinline__ void load4_stream<float>(const float* p, float v[4], uint64_t pol) {
-    asm volatile("ld.global.nc.L1::no_allocate.L2::cache_hint.v4.f32 {%0, %1, %2, %3}, [%4], %5;"
-                 : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]) : "l"(p), "l"(pol));
+    asm volatile("ld.global.L1::no_allocate.L2::cache_hint.v4.f32 {%0, %1, %2, %3}, [%4], %5;"
+                 : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]) : "l"(p), "l"(pol) : "memory");
 }
 template <> __device__ __forceinline__ void load4_stream<__nv_bfloat16>(const __nv_bfloat16* p, float v[4], uint64_t pol) {
     uint2 t;
-    asm volatile("ld.global.nc.L1::no_allocate.L2::cache_hint.v2.u32 {%0, %1}, [%2], %3;" : "=r"(t.x), "=r"(t.y) : "l"(p), "l"(pol));
+    asm volatile("ld.global.L1::no_allocate.L2::cache_hint.v2.u32 {%0, %1}, [%2], %3;" : "=r"(t.x), "=r"(t.y) : "l"(p), "l"(pol) : "memory");
     v[0] = __uint_as_float(t.x << 16); v[1] = __uint_as_float(t.x & 0xffff0000u);
     v[2] = __uint_as_float(t.y << 16); v[3] = __uint_as_float(t.y & 0xffff0000u);
 }
@@ -444,19 +444,13 @@ cudaError_t conv_simt_dispatch(const ConvArgs& a, cudaStream_t s) {
 // in the single-precision path.  A CTA of eight warps takes QT queries and walks 64 keys at a time with a running maximum and
 // sum.  Scores: a warp has eight keys; a lane takes four channels of every 128 and keeps all 8 x QT partial sums, which one
 // halving exchange over the warp adds up (31 shuffles instead of 5 per sum).  Output: a thread has four channels and every
-// second half of the tile's keys.  K and V go straight from L2 to registers: no key is used twice by a thread, and staging
-// them cost more than the products (one warp per query, 8 queries per CTA: 8 CTAs at 64 tokens, 76 us; now @NOW@).
+// second key.  K and V go straight from L2 to registers: no key is used twice by a thread, and staging
+// them cost more than the products (one warp per query, 8 queries per CTA: 8 CTAs at 64 tokens, 76 us; now 12).
 // QT = 2 as long as the CTAs fit the chip at once, 4 beyond (K and V are read T / QT times).
 constexpr int kAttnTile = 64, kAttnMaxC = 512;
 
-template <typename T> __device__ __forceinline__ float4 attn_ld4(const T* p, bool vec) {
-    if (!vec) return make_float4(ld_f<T>(p, 0), ld_f<T>(p, 1), ld_f<T>(p, 2), ld_f<T>(p, 3));
-    if constexpr (sizeof(T) == 4) {
-        return __ldcg((const float4*)p);
-    } else {
-        const uint2 t = __ldcg((const uint2*)p);
-        return make_float4(__uint_as_float(t.x << 16), __uint_as_float(t.x & 0xffff0000u), __uint_as_float(t.y << 16), __uint_as_float(t.y & 0xffff0000u));
-    }
+__device__ __forceinline__ float4 attn_ld4(const float* p, bool vec) {
+    return vec ? __ldcg((const float4*)p) : make_float4(p[0], p[1], p[2], p[3]);
 }
 
 // Sums of v[0..N) over the warp: v[0] of lane i is the sum of value i / (32 / N).
@@ -478,8 +472,8 @@ template <int N> __device__ __forceinline__ void warp_sums(float (&v)[N], int la
     }
 }
 
-template <typename T, int QT>
-__global__ void __launch_bounds__(256, 2) attn_simt_kernel(AttnArgs a, bool vec) {
+template <int QT>
+__global__ void __launch_bounds__(256, 2) attn_f32_kernel(AttnArgs a, bool vec) {
     __shared__ __align__(16) float s_q[QT][kAttnMaxC];
     __shared__ __align__(16) float s_p[kAttnTile * QT];      // [key][query]
     __shared__ float s_corr[QT], s_l[QT];
@@ -488,12 +482,12 @@ __global__ void __launch_bounds__(256, 2) attn_simt_kernel(AttnArgs a, bool vec)
     griddep_wait();
     const int C = a.C, b = blockIdx.y, q0 = blockIdx.x * QT;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, half = tid >> 7, c4 = (tid & 127) * 4;
-    const T* q = (const T*)a.q + (size_t)b * a.T * a.ld_qkv;
-    const T* k = (const T*)a.k + (size_t)b * a.T * a.ld_qkv;
-    const T* v = (const T*)a.v + (size_t)b * a.T * a.ld_qkv;
+    const float* q = (const float*)a.q + (size_t)b * a.T * a.ld_qkv;
+    const float* k = (const float*)a.k + (size_t)b * a.T * a.ld_qkv;
+    const float* v = (const float*)a.v + (size_t)b * a.T * a.ld_qkv;
     for (int i = tid; i < QT * (kAttnMaxC / 4); i += 256) {
         const int t = i / (kAttnMaxC / 4), c = i % (kAttnMaxC / 4) * 4;
-        *(float4*)&s_q[t][c] = q0 + t < a.T && c < C ? attn_ld4<T>(q + (size_t)(q0 + t) * a.ld_qkv + c, vec) : make_float4(0.f, 0.f, 0.f, 0.f);
+        *(float4*)&s_q[t][c] = q0 + t < a.T && c < C ? attn_ld4(q + (size_t)(q0 + t) * a.ld_qkv + c, vec) : make_float4(0.f, 0.f, 0.f, 0.f);
     }
     float4 acc[QT];
 #pragma unroll
@@ -512,14 +506,14 @@ __global__ void __launch_bounds__(256, 2) attn_simt_kernel(AttnArgs a, bool vec)
 #pragma unroll
             for (int e = 0; e < 8; ++e) {
                 const int key = k0 + warp * 8 + e;
-                kv[e] = c < C && key < a.T ? attn_ld4<T>(k + (size_t)key * a.ld_qkv + c, vec) : make_float4(0.f, 0.f, 0.f, 0.f);
+                kv[e] = c < C && key < a.T ? attn_ld4(k + (size_t)key * a.ld_qkv + c, vec) : make_float4(0.f, 0.f, 0.f, 0.f);
             }
 #pragma unroll
             for (int t = 0; t < QT; ++t) {
                 const float4 qv = *(const float4*)&s_q[t][c];
 #pragma unroll
                 for (int e = 0; e < 8; ++e)
-                    sc[e * QT + t] = fmaf(qv.x, kv[e].x, fmaf(qv.y, kv[e].y, fmaf(qv.z, kv[e].z, fmaf(qv.w, kv[e].w, sc[e * QT + t]))));
+                    sc[e * QT + t] = fmaf(qv.w, kv[e].w, fmaf(qv.z, kv[e].z, fmaf(qv.y, kv[e].y, fmaf(qv.x, kv[e].x, sc[e * QT + t]))));
             }
         }
         warp_sums<8 * QT>(sc, lane);
@@ -553,16 +547,16 @@ __global__ void __launch_bounds__(256, 2) attn_simt_kernel(AttnArgs a, bool vec)
             }
             constexpr int U = 16;                            // keys on their way at a time
 #pragma unroll 1
-            for (int e0 = half * (kAttnTile / 2); e0 < (half + 1) * (kAttnTile / 2) && k0 + e0 < a.T; e0 += U) {
+            for (int e0 = half; e0 < kAttnTile && k0 + e0 < a.T; e0 += 2 * U) {
                 float4 vv[U];
 #pragma unroll
                 for (int e = 0; e < U; ++e)
-                    vv[e] = k0 + e0 + e < a.T ? attn_ld4<T>(v + (size_t)(k0 + e0 + e) * a.ld_qkv + c4, vec) : make_float4(0.f, 0.f, 0.f, 0.f);
+                    vv[e] = k0 + e0 + 2 * e < a.T ? attn_ld4(v + (size_t)(k0 + e0 + 2 * e) * a.ld_qkv + c4, vec) : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
                 for (int e = 0; e < U; ++e)
 #pragma unroll
                     for (int t = 0; t < QT; ++t) {
-                        const float p = s_p[(e0 + e) * QT + t];
+                        const float p = s_p[(e0 + 2 * e) * QT + t];
                         acc[t].x = fmaf(p, vv[e].x, acc[t].x); acc[t].y = fmaf(p, vv[e].y, acc[t].y);
                         acc[t].z = fmaf(p, vv[e].z, acc[t].z); acc[t].w = fmaf(p, vv[e].w, acc[t].w);
                     }
@@ -576,17 +570,89 @@ __global__ void __launch_bounds__(256, 2) attn_simt_kernel(AttnArgs a, bool vec)
     }
     __syncthreads();
     if (half == 0 && c4 < C) {
-        T* o = (T*)a.o + ((size_t)b * a.T + q0) * a.ld_o + c4;
+        float* o = (float*)a.o + ((size_t)b * a.T + q0) * a.ld_o + c4;
 #pragma unroll
         for (int t = 0; t < QT; ++t) {
             if (q0 + t >= a.T) break;
             const float inv = 1.f / s_l[t];
             const float4 r = s_o[t][c4 / 4];
-            st_f<T>(o, (size_t)t * a.ld_o, (acc[t].x + r.x) * inv);
-            st_f<T>(o, (size_t)t * a.ld_o + 1, (acc[t].y + r.y) * inv);
-            st_f<T>(o, (size_t)t * a.ld_o + 2, (acc[t].z + r.z) * inv);
-            st_f<T>(o, (size_t)t * a.ld_o + 3, (acc[t].w + r.w) * inv);
+            float* d = o + (size_t)t * a.ld_o;
+            d[0] = (acc[t].x + r.x) * inv; d[1] = (acc[t].y + r.y) * inv; d[2] = (acc[t].z + r.z) * inv; d[3] = (acc[t].w + r.w) * inv;
         }
+    }
+}
+
+// bf16 tensors, which take this path only where the FFMA kernels are asked for as a check: one warp per query, eight queries
+// per block sharing 32-key K/V tiles in shared memory; running maximum / running sum softmax, all in fp32.
+constexpr int kAttnQ = 8, kAttnKeys = 32;
+
+__global__ void __launch_bounds__(kAttnQ * 32) attn_bf16_kernel(AttnArgs a) {
+    using T = __nv_bfloat16;
+    griddep_launch();
+    griddep_wait();
+    extern __shared__ float smem[];
+    const int C = a.C;
+    float* s_q = smem;                               // [kAttnQ][C]
+    float* s_k = s_q + kAttnQ * C;                   // [kAttnKeys][C+1]
+    float* s_v = s_k + kAttnKeys * (C + 1);          // [kAttnKeys][C]
+    const int b = blockIdx.y;
+    const int q0 = blockIdx.x * kAttnQ;
+    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+    const T* q = (const T*)a.q + (size_t)b * a.T * a.ld_qkv;
+    const T* k = (const T*)a.k + (size_t)b * a.T * a.ld_qkv;
+    const T* v = (const T*)a.v + (size_t)b * a.T * a.ld_qkv;
+    T* o = (T*)a.o + (size_t)b * a.T * a.ld_o;
+
+    for (int idx = threadIdx.x; idx < kAttnQ * C; idx += blockDim.x) {
+        const int qi = idx / C, c = idx % C;
+        s_q[idx] = (q0 + qi < a.T) ? ld_f<T>(q, (size_t)(q0 + qi) * a.ld_qkv + c) : 0.f;
+    }
+    const int nacc = C / 32;                          // channels per lane (C multiple of 32, <= 512)
+    float acc[16];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) acc[i] = 0.f;
+    float m = -INFINITY, l = 0.f;
+
+    for (int k0 = 0; k0 < a.T; k0 += kAttnKeys) {
+        __syncthreads();
+        for (int idx = threadIdx.x; idx < kAttnKeys * C; idx += blockDim.x) {
+            const int ki = idx / C, c = idx % C;
+            const bool ok = k0 + ki < a.T;
+            s_k[ki * (C + 1) + c] = ok ? ld_f<T>(k, (size_t)(k0 + ki) * a.ld_qkv + c) : 0.f;
+            s_v[ki * C + c] = ok ? ld_f<T>(v, (size_t)(k0 + ki) * a.ld_qkv + c) : 0.f;
+        }
+        __syncthreads();
+        float sc = 0.f;
+        const float* qr = s_q + warp * C;
+        const float* kr = s_k + lane * (C + 1);
+        for (int c = 0; c < C; ++c) sc = fmaf(qr[c], kr[c], sc);
+        sc = (k0 + lane < a.T) ? sc * a.scale : -INFINITY;
+        float tmax = sc;
+#pragma unroll
+        for (int d = 16; d > 0; d >>= 1) tmax = fmaxf(tmax, __shfl_xor_sync(0xffffffffu, tmax, d));
+        const float m_new = fmaxf(m, tmax);
+        const float corr = expf(m - m_new);           // m = -inf at the first tile: exp(-inf) = 0
+        const float p = expf(sc - m_new);
+        float psum = p;
+#pragma unroll
+        for (int d = 16; d > 0; d >>= 1) psum += __shfl_xor_sync(0xffffffffu, psum, d);
+        l = l * corr + psum;
+        m = m_new;
+#pragma unroll
+        for (int i = 0; i < 16; ++i) acc[i] *= corr;
+        for (int ki = 0; ki < kAttnKeys; ++ki) {
+            const float pk = __shfl_sync(0xffffffffu, p, ki);
+            const float* vr = s_v + ki * C + lane;
+#pragma unroll
+            for (int i = 0; i < 16; ++i)
+                if (i < nacc) acc[i] = fmaf(pk, vr[i * 32], acc[i]);
+        }
+    }
+    if (q0 + warp < a.T) {
+        const float inv = 1.f / l;
+#pragma unroll
+        for (int i = 0; i < 16; ++i)
+            if (i < nacc) st_f<T>(o, (size_t)(q0 + warp) * a.ld_o + lane + i * 32, acc[i] * inv);
     }
 }
 
@@ -724,17 +790,18 @@ cudaError_t launch_conv_simt(const ConvArgs& a, cudaStream_t s) {
 
 cudaError_t launch_attn_simt(const AttnArgs& a, cudaStream_t s) {
     if (a.C % 32 != 0 || a.C > 512) return cudaErrorInvalidValue;
-    const uintptr_t align = (a.dtype == VD_BF16 ? 8 : 16) - 1;                      // of four channels at once
-    const bool vec = a.ld_qkv % 4 == 0 && (((uintptr_t)a.q | (uintptr_t)a.k | (uintptr_t)a.v) & align) == 0;
+    if (a.dtype == VD_BF16) {
+        const size_t smem = sizeof(float) * ((size_t)kAttnQ * a.C + (size_t)kAttnKeys * (a.C + 1) + (size_t)kAttnKeys * a.C);
+        const cudaError_t e = cudaFuncSetAttribute(attn_bf16_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        launch_pdl(attn_bf16_kernel, dim3((a.T + kAttnQ - 1) / kAttnQ, a.B), dim3(kAttnQ * 32), smem, s, a);
+        return cudaGetLastError();
+    }
+    const bool vec = a.ld_qkv % 4 == 0 && (((uintptr_t)a.q | (uintptr_t)a.k | (uintptr_t)a.v) & 15) == 0;
     const int qt = (long long)a.B * ((a.T + 1) / 2) <= 2 * 148 ? 2 : 4;
     const dim3 grid((a.T + qt - 1) / qt, a.B);
-    if (a.dtype == VD_BF16) {
-        if (qt == 2) launch_pdl(attn_simt_kernel<__nv_bfloat16, 2>, grid, dim3(256), 0, s, a, vec);
-        else launch_pdl(attn_simt_kernel<__nv_bfloat16, 4>, grid, dim3(256), 0, s, a, vec);
-    } else {
-        if (qt == 2) launch_pdl(attn_simt_kernel<float, 2>, grid, dim3(256), 0, s, a, vec);
-        else launch_pdl(attn_simt_kernel<float, 4>, grid, dim3(256), 0, s, a, vec);
-    }
+    if (qt == 2) launch_pdl(attn_f32_kernel<2>, grid, dim3(256), 0, s, a, vec);
+    else launch_pdl(attn_f32_kernel<4>, grid, dim3(256), 0, s, a, vec);
     return cudaGetLastError();
 }
 
