@@ -149,18 +149,19 @@ inline int rec_parts(int bn, int cpg) {
 }
 
 // Adds up the `nparts` partials of this CTA's `rpo` rows, adds bias and residual, writes the output and the statistics
-// records.  rx: [nparts][rpo][RXS] floats, 16-byte piece c of a row at c ^ swizzle(row).  ptid: 0..255.  locate(local row,
-// oy, ox) gives the row's output pixel and whether it exists; ready() returns when the partials have arrived.  The first
-// rows' addresses and residual and the record's address are made before that (the empty asm keeps them there).
+// records.  source(s): partial s, [rpo][RXS] floats, 16-byte piece c of a row at c ^ swizzle(row).  ptid: 0..255.
+// locate(local row, oy, ox) gives the row's output pixel and whether it exists; ready() returns when the partials have
+// arrived.  The first PRE rows' addresses and residual and the record's address are made before that (the empty asm keeps
+// them there).
 // A thread takes four channels (cg) of every RSTEP-th row, so a warp's share of a group comes from shuffles alone.  BN < 32:
 // the frame head (planes or packed pixels of a.Cout channels).
-template <int BN, int RXS, class Locate, class Swizzle, class Ready>
-__device__ __forceinline__ void finish_rows(const ConvArgs& a, const float* rx, int nparts, int rpo, int ptid, int frame, int n0, int OH, int OW,
+template <int BN, int RXS, int PRE, class Source, class Locate, class Swizzle, class Ready>
+__device__ __forceinline__ void finish_rows(const ConvArgs& a, Source source, int nparts, int rpo, int ptid, int frame, int n0, int OH, int OW,
                                             int slot0, Locate locate, Swizzle swizzle, Ready ready) {
     constexpr bool HEAD = BN < 32;
     constexpr int CPW = HEAD ? 1 : Split8<HEAD ? 64 : BN>::CPW, WC = HEAD ? 1 : Split8<HEAD ? 64 : BN>::WC, RL = 32 / CPW;
-    constexpr int RSTEP = HEAD ? kFinishThreads / (BN / 4) : RL * (8 / WC), CPW_LOG2 = CPW == 4 ? 2 : CPW - 1;
-    static_assert(CPW == 1 || CPW == 2 || CPW == 4, "columns of a warp");
+    constexpr int RSTEP = HEAD ? kFinishThreads / (BN / 4) : RL * (8 / WC), CPW_LOG2 = CPW == 8 ? 3 : CPW == 4 ? 2 : CPW - 1;
+    static_assert(CPW == 1 || CPW == 2 || CPW == 4 || CPW == 8, "columns of a warp");
     const int w = ptid >> 5, lane = ptid & 31;
     const int cg = HEAD ? ptid % (BN / 4) : (w % WC) * CPW + lane / RL, rg = HEAD ? ptid / (BN / 4) : (w / WC) * RL + lane % RL;
     const int co = n0 + cg * 4;
@@ -172,7 +173,6 @@ __device__ __forceinline__ void finish_rows(const ConvArgs& a, const float* rx, 
             bias.x += t.x; bias.y += t.y; bias.z += t.z; bias.w += t.w;
         }
     }
-    constexpr int PRE = 2;                                   // rows on their way at a time
     float4 res[PRE];
     size_t off[PRE];                                         // element of y (head: pixel of the frame)
     bool valid[PRE];
@@ -206,10 +206,10 @@ __device__ __forceinline__ void finish_rows(const ConvArgs& a, const float* rx, 
             const int local = first + i * RSTEP;
             float4 v = bias;
             if (valid[i]) {
-                const float* q = rx + local * RXS + (cg ^ swizzle(local)) * 4;
+                const int q = local * RXS + (cg ^ swizzle(local)) * 4;
 #pragma unroll 4
-                for (int s = 0; s < nparts; ++s, q += rpo * RXS) {
-                    const float4 p = *(const float4*)q;
+                for (int s = 0; s < nparts; ++s) {
+                    const float4 p = *(const float4*)(source(s) + q);
                     v.x += p.x; v.y += p.y; v.z += p.z; v.w += p.w;
                 }
                 if (HEAD) {

@@ -298,7 +298,7 @@ conv_f32_kernel(const ConvArgs a, const int S, const int n_w, const int ops_floa
         rx = part;
         __syncthreads();
     }
-    finish_rows<BN, BN>(a, rx, S, rpo, tid, frame, n0, KIND == KPHASE ? 2 * H : H, KIND == KPHASE ? 2 * W : W,
+    finish_rows<BN, BN, 2>(a, [&](int s) { return rx + s * rpo * BN; }, S, rpo, tid, frame, n0, KIND == KPHASE ? 2 * H : H, KIND == KPHASE ? 2 * W : W,
                         (KIND == KPHASE ? tile * 4 + par : tile) * S + rank,
                         [&](int local, int& oy, int& ox) -> bool {
                             const int R = rank * rpo + local;

@@ -21,6 +21,7 @@
 
 #include "conv_cluster.cuh"
 #include "conv_tile.cuh"
+#include "tc_pair.cuh"
 
 namespace vd {
 
@@ -37,8 +38,7 @@ using convtile::TILE_W;
 
 constexpr int kWarps = 10, kThreads = kWarps * 32;           // MMA, weights, eight producer / epilogue warps
 constexpr int kProd0 = 2, kProd = 8 * 32;
-constexpr int kBatch = (ITEMS + kProd - 1) / kProd;          // 6 (pixel, 8-channel) entries per producer thread and tile
-constexpr int kMaxA = 2, kMaxB = 9;
+constexpr int kMaxA = 2, kMaxB = 10;
 constexpr int kMaxSliceC = 512;                              // channels of one CTA's K slice
 constexpr int kTailBytes = 2 * kMaxSliceC * 4 + 256;         // after the operand stages: scale/shift of the slice, barriers
 
@@ -58,6 +58,86 @@ __device__ __forceinline__ void commit_to_cluster(uint32_t bar, uint16_t mask, u
                  "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;\n}\n"
                  ::"r"(bar), "h"(mask), "r"(on) : "memory");
 }
+
+// The operand of one tile, made by NPW warps: 18x10 halo pixels x 64 channels a chunk, an entry is (pixel, 8 channels).
+// fp32 input: four channels from the chunk's first half, four from its second.  `prepare` is what depends on the thread
+// alone; an entry's registers take the next chunk's values as soon as they have been read (515 -> 465 us for one 64x64
+// frame, most of whose layers give a CTA two chunks).
+template <int KIND, bool IN_BF16, int NPW> struct Operand {
+    static constexpr int NT = NPW * 32, N = (ITEMS + NT - 1) / NT, ESZ = IN_BF16 ? 2 : 4, HALVES = IN_BF16 ? 1 : 2, NV = 8 / HALVES;
+    static_assert(NT / 8 % 8 == 0, "an entry's swizzle is the first one's");
+    int goff[N];                                             // byte offset of the entry's source pixel
+    uint32_t soff, vm;                                       // where entry 0's operand goes (entry e: e * NT * 16 on); entries inside the image
+    const char* xb;
+    uint4 raw[HALVES][N];
+    __device__ __forceinline__ void prepare(const ConvArgs& a, int frame, int c_first, int ty, int tx, int H, int W, int ptid) {
+        const int j = ptid & 7, pix0 = ptid >> 3;
+        soff = (uint32_t)(pix0 * 128) + (IN_BF16 ? (uint32_t)((j ^ (pix0 & 7)) << 4) : (uint32_t)((((j >> 1) ^ (pix0 & 7)) << 4) + (j & 1) * 8));
+        vm = 0u;
+#pragma unroll
+        for (int e = 0; e < N; ++e) {
+            const int pix = (e * NT + ptid) >> 3, py = pix / PW, px = pix - py * PW;
+            const int oy = ty + py - 1, ox = tx + px - 1;
+            bool v = oy >= 0 && oy < H && ox >= 0 && ox < W && pix < NPIX;
+            if (KIND == K1X1) v = v && py >= 1 && py <= TILE_H && px >= 1 && px <= TILE_W;
+            vm |= (v ? 1u : 0u) << e;
+            goff[e] = v ? (oy * W + ox) * a.Cin * ESZ : 0;
+        }
+        xb = (const char*)a.x + ((size_t)frame * H * W * a.Cin + c_first + j * NV) * ESZ;
+    }
+    __device__ __forceinline__ void load(int u, int h, int e) {
+        if (vm >> e & 1u) raw[h][e] = convtile::ldg_stream(xb + (size_t)u * (64 * ESZ) + goff[e] + h * 128);
+    }
+    __device__ __forceinline__ void load_first() {
+#pragma unroll
+        for (int h = 0; h < HALVES; ++h)
+#pragma unroll
+            for (int e = 0; e < N; ++e) load(0, h, e);
+    }
+    __device__ __forceinline__ void transform(uint8_t* dst, int u, bool more, bool prologue, bool silu, const float* s_scale, const float* s_shift, int ptid) {
+        const int j = ptid & 7;
+#pragma unroll
+        for (int h = 0; h < HALVES; ++h) {
+            float sc[NV], sf[NV];
+            if (prologue) {
+                const int c = u * 64 + j * NV + h * 32;
+#pragma unroll
+                for (int i = 0; i < NV; i += 4) {
+                    *(float4*)&sc[i] = *(const float4*)(s_scale + c + i);
+                    *(float4*)&sf[i] = *(const float4*)(s_shift + c + i);
+                }
+            }
+#pragma unroll
+            for (int e = 0; e < N; ++e) {
+                if (e == N - 1 && ((e * NT + ptid) >> 3) >= NPIX) break;
+                uint32_t o[NV / 2];
+#pragma unroll
+                for (int i = 0; i < NV / 2; ++i) o[i] = 0u;
+                if (vm >> e & 1u) {
+                    float v[NV];
+                    const uint32_t r[4] = {raw[h][e].x, raw[h][e].y, raw[h][e].z, raw[h][e].w};
+#pragma unroll
+                    for (int i = 0; i < NV; ++i)
+                        v[i] = __uint_as_float(!IN_BF16 ? r[i & 3] : (i & 1) ? r[i >> 1] & 0xffff0000u : r[i >> 1] << 16);
+                    if (more) load(u + 1, h, e);
+                    if (prologue) {
+#pragma unroll
+                        for (int i = 0; i < NV; ++i) v[i] = fmaf(v[i], sc[i], sf[i]);
+                        if (silu) {
+#pragma unroll
+                            for (int i = 0; i < NV; ++i) v[i] = fmaf(v[i], tanh_fast(v[i]), v[i]);
+                        }
+                    }
+#pragma unroll
+                    for (int i = 0; i < NV / 2; ++i) o[i] = KIND == KPHASE ? pack_f16(v[2 * i], v[2 * i + 1]) : pack_bf16(v[2 * i], v[2 * i + 1]);
+                }
+                uint8_t* d = dst + (h ? soff ^ 64u : soff) + e * (NT * 16);
+                if constexpr (IN_BF16) *(uint4*)d = make_uint4(o[0], o[1], o[2], o[3]);
+                else *(uint2*)d = make_uint2(o[0], o[1]);
+            }
+        }
+    }
+};
 
 // BN: output channels per cluster (16: the frame head).  KIND: 3x3, 1x1, or one output parity of the phase-collapsed
 // upsampling convolution (2x2 taps of the source, fp16 operands; see conv_tc.cu).
@@ -214,45 +294,20 @@ conv_split_kernel(const ConvArgs a, const ConvSplitShape sh, const __grid_consta
         __syncwarp();
     } else {
         // ------------------------------------------------ operand prologue
-        const int ptid = tid - kProd0 * 32, j = ptid & 7, pw = warp - kProd0;
-        constexpr int ESZ = IN_BF16 ? 2 : 4;
+        const int ptid = tid - kProd0 * 32, pw = warp - kProd0;
         const bool prologue = a.scale != nullptr || a.in_rec != nullptr, silu = a.silu != 0;
         const int nch = nk * 64;
         const float half = silu ? 0.5f : 1.0f;               // SiLU is evaluated as h + h * tanh(h), h = v / 2
-        // what depends on the thread alone, before the kernel before has to be done
-        int goff[kBatch];                                    // byte offset of the entry's source pixel
-        // where its operand goes (entry e is kProd / 8 pixels, a multiple of the swizzle's eight rows, after entry 0)
-        const int pix0 = ptid >> 3;
-        const uint32_t soff = (uint32_t)(pix0 * 128) + (IN_BF16 ? (uint32_t)((j ^ (pix0 & 7)) << 4) : (uint32_t)((((j >> 1) ^ (pix0 & 7)) << 4) + (j & 1) * 8));
-        uint32_t vm = 0u;                                    // entries inside the image
-#pragma unroll
-        for (int e = 0; e < kBatch; ++e) {
-            const int pix = (e * kProd + ptid) >> 3, py = pix / PW, px = pix - py * PW;
-            const int oy = ty + py - 1, ox = tx + px - 1;
-            bool v = oy >= 0 && oy < H && ox >= 0 && ox < W && pix < NPIX;
-            if (KIND == K1X1) v = v && py >= 1 && py <= TILE_H && px >= 1 && px <= TILE_W;
-            vm |= (v ? 1u : 0u) << e;
-            goff[e] = v ? (oy * W + ox) * a.Cin * ESZ : 0;
-        }
+        Operand<KIND, IN_BF16, 8> op;
+        op.prepare(a, frame, k0 * 64, ty, tx, H, W, ptid);
         InputStats stats;
         if (a.in_rec) stats.prepare(a, frame, k0 * 64, nch, pw, lane, s_scale, s_shift);
-        const char* xb = (const char*)a.x + ((size_t)frame * H * W * a.Cin + k0 * 64 + (IN_BF16 ? j * 8 : j * 4)) * ESZ;
         if (pw == 0) touch_params(a, &bars->unused);
         griddep_wait();
         if (a.in_rec) stats.load(a, lane);
         uint32_t as = 0, aph = 0;
         bool ok = true;
-        // An entry's registers take the next chunk's values as soon as they have been read: 515 -> 465 us for one 64x64 frame,
-        // most of whose layers give a CTA two chunks.  fp32 input: 4 channels from the chunk's first half, 4 from its second.
-        constexpr int HALVES = IN_BF16 ? 1 : 2, NV = 8 / HALVES;
-        uint4 raw[HALVES][kBatch];
-        auto load = [&](int u, int h, int e) {
-            if (vm >> e & 1u) raw[h][e] = convtile::ldg_stream(xb + (size_t)u * (64 * ESZ) + goff[e] + h * 128);
-        };
-#pragma unroll
-        for (int h = 0; h < HALVES; ++h)
-#pragma unroll
-            for (int e = 0; e < kBatch; ++e) load(0, h, e);
+        op.load_first();
 #pragma unroll 1
         for (int u = 0; u < units; ++u) {
             const bool second = BN == 64 && KIND == K3X3 && u >= nk;
@@ -276,46 +331,7 @@ conv_split_kernel(const ConvArgs a, const ConvSplitShape sh, const __grid_consta
                     tma_load_4d(smem_u32(dst), &tm_x2, (q0 + u - nk) * 32, tx, ty, frame, smem_u32(&bars->a_full[as]));
                 }
             } else {
-#pragma unroll
-                for (int h = 0; h < HALVES; ++h) {
-                    float sc[NV], sf[NV];
-                    if (prologue) {
-                        const int c = u * 64 + j * NV + h * 32;
-#pragma unroll
-                        for (int i = 0; i < NV; i += 4) {
-                            *(float4*)&sc[i] = *(const float4*)(s_scale + c + i);
-                            *(float4*)&sf[i] = *(const float4*)(s_shift + c + i);
-                        }
-                    }
-#pragma unroll
-                    for (int e = 0; e < kBatch; ++e) {
-                        if (e == kBatch - 1 && ((e * kProd + ptid) >> 3) >= NPIX) break;
-                        uint32_t o[NV / 2];
-#pragma unroll
-                        for (int i = 0; i < NV / 2; ++i) o[i] = 0u;
-                        if (vm >> e & 1u) {
-                            float v[NV];
-                            const uint32_t r[4] = {raw[h][e].x, raw[h][e].y, raw[h][e].z, raw[h][e].w};
-#pragma unroll
-                            for (int i = 0; i < NV; ++i)
-                                v[i] = __uint_as_float(!IN_BF16 ? r[i & 3] : (i & 1) ? r[i >> 1] & 0xffff0000u : r[i >> 1] << 16);
-                            if (u + 1 < nk) load(u + 1, h, e);
-                            if (prologue) {
-#pragma unroll
-                                for (int i = 0; i < NV; ++i) v[i] = fmaf(v[i], sc[i], sf[i]);
-                                if (silu) {
-#pragma unroll
-                                    for (int i = 0; i < NV; ++i) v[i] = fmaf(v[i], tanh_fast(v[i]), v[i]);
-                                }
-                            }
-#pragma unroll
-                            for (int i = 0; i < NV / 2; ++i) o[i] = KIND == KPHASE ? pack_f16(v[2 * i], v[2 * i + 1]) : pack_bf16(v[2 * i], v[2 * i + 1]);
-                        }
-                        uint8_t* d = dst + (h ? soff ^ 64u : soff) + e * (kProd * 16);
-                        if constexpr (IN_BF16) *(uint4*)d = make_uint4(o[0], o[1], o[2], o[3]);
-                        else *(uint2*)d = make_uint2(o[0], o[1]);
-                    }
-                }
+                op.transform(dst, u, u + 1 < nk, prologue, silu, s_scale, s_shift, ptid);
             }
             fence_proxy_async_smem();
             __syncwarp();
@@ -363,7 +379,7 @@ conv_split_kernel(const ConvArgs a, const ConvSplitShape sh, const __grid_consta
             __syncwarp();
             cluster_arrive();                                // what is sent to this CTA has landed
         };
-        finish_rows<BN, RXS>(a, rx, S, rpo, ptid, frame, n0, KIND == KPHASE ? 2 * H : H, KIND == KPHASE ? 2 * W : W,
+        finish_rows<BN, RXS, 2>(a, [&](int s) { return rx + s * rpo * RXS; }, S, rpo, ptid, frame, n0, KIND == KPHASE ? 2 * H : H, KIND == KPHASE ? 2 * W : W,
                         (KIND == KPHASE ? tile * 4 + par : tile) * S + rank,
                         [&](int local, int& oy, int& ox) -> bool {
                             const int R = rank * rpo + local;
@@ -381,6 +397,228 @@ conv_split_kernel(const ConvArgs a, const ConvSplitShape sh, const __grid_consta
     if (warp == 0) {
         tc_fence_after();
         tmem_dealloc(tmem, (uint32_t)ACC_COLS);
+    }
+    if (tid == kProd0 * 32 && bars->abort_flag && status) {
+        if (atomicCAS(status, 0u, kStatusConvTimeout) == 0u) {
+            status[1] = blockIdx.x;
+            status[2] = (uint32_t)BN;
+        }
+    }
+}
+
+// ---- the same on pairs of CTAs
+// Where 64-channel blocks would stream the weights too often, a pair of CTAs takes two tiles x 256 output channels as one
+// tcgen05.mma.cta_group::2 (M = 256): a tap's weights come from L2 once for both tiles, and each CTA's shared memory holds
+// and feeds half of them.  S pairs share K; the exchange is between the CTAs of the same tile.  The pair's even CTA issues;
+// all "full" barriers are its own.
+constexpr int kPairBN = 256, kPairWarps = 16, kPairThreads = (kProd0 + kPairWarps) * 32, kPairSmemMax = 227 * 1024;
+
+// arrives, once the pair's MMAs issued so far have completed, on the barrier at this offset in every CTA of `mask`
+__device__ __forceinline__ void commit2_to_cluster(uint32_t bar, uint16_t mask, uint32_t on) {
+    asm volatile("{\n.reg .pred q;\nsetp.ne.b32 q, %2, 0;\n"
+                 "@q tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;\n}\n"
+                 ::"r"(bar), "h"(mask), "r"(on) : "memory");
+}
+
+template <bool IN_BF16>
+__global__ void __launch_bounds__(kPairThreads, 1)
+conv_pair_kernel(const ConvArgs a, const ConvSplitShape sh, const __grid_constant__ CUtensorMap tm_w, unsigned int* status) {
+    constexpr int TAPS = 9, BN = kPairBN, BST = BN / 2 * 128, RXS = BN + 4, ROWS = TILE_H * TILE_W, NT = kPairWarps * 32;
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+    const int n_a = sh.n_a, n_b = sh.n_b, S = sh.splits;
+    uint8_t* smem_a = smem;
+    uint8_t* smem_b = smem + n_a * A_TILE_BYTES;
+    // over the operand stages, once every MMA of the cluster is done: this CTA's partials, and the other CTA's of its rows
+    float* part = (float*)smem;
+    float* rx = part + ROWS * RXS;
+    float* s_scale = (float*)(smem + sh.tail_off);
+    float* s_shift = s_scale + kMaxSliceC;
+    SBars* bars = (SBars*)(s_shift + kMaxSliceC);
+    volatile uint32_t* abort_flag = &bars->abort_flag;
+
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int rank = (int)ctarank(), half = rank & 1, kp = rank >> 1, lead_cta = rank & ~1;
+    const int H = a.H, W = a.W;
+    const int tiles_x = (W + TILE_W - 1) / TILE_W, tiles = tiles_x * ((H + TILE_H - 1) / TILE_H), groups = (tiles + 1) / 2;
+    const int nblk = a.Cout / BN;
+    int item = (int)blockIdx.x / (2 * S);
+    const int n0 = (item % nblk) * BN;
+    item /= nblk;
+    const int tile = (item % groups) * 2 + half, frame = item / groups;
+    const int ty = tile / tiles_x * TILE_H, tx = tile % tiles_x * TILE_W;            // (beyond the last tile: below the image, nothing out)
+    const int kchunks = a.Cin >> 6, k0 = kp * kchunks / S, nk = (kp + 1) * kchunks / S - k0;
+
+    if (tid == 0) {
+        for (int i = 0; i < n_a; ++i) { mbar_init(smem_u32(&bars->a_full[i]), 2 * kPairWarps); mbar_init(smem_u32(&bars->a_empty[i]), 1); }
+        for (int i = 0; i < n_b; ++i) { mbar_init(smem_u32(&bars->b_full[i]), 2); mbar_init(smem_u32(&bars->b_empty[i]), 1); }
+        mbar_init(smem_u32(&bars->acc_full), S);             // one commit from every pair of the cluster
+        mbar_init(smem_u32(&bars->rx_full), 1);
+        bars->abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        fence_proxy_async_smem();
+        mbar_arrive_expect_tx(smem_u32(&bars->rx_full), ROWS / S * (S - 1) * RXS * 4);         // this CTA's rows from the other partials
+    }
+    if (warp == 0) tmem_alloc2(smem_u32(&bars->tmem_base), (uint32_t)BN);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    cluster_arrive();
+    cluster_wait();                                          // every CTA's barriers exist before anyone signals across
+    const uint32_t tmem = bars->tmem_base;
+    griddep_launch();
+
+    if (warp == 1) {
+        // ------------------------------------------------ this CTA's half of the weights (they do not depend on the kernel before)
+        if (lane == 0) {
+            uint32_t st = 0, ph = 0;
+            int issued = 0;
+            bool ok = true;
+            for (int u = 0; u < nk && ok; ++u) {
+#pragma unroll 1
+                for (int tap = 0; tap < TAPS; ++tap) {
+                    if (issued >= n_b) ok = mbar_wait(smem_u32(&bars->b_empty[st]), ph ^ 1, abort_flag);
+                    if (!ok) break;
+                    const uint32_t full = peer_addr(smem_u32(&bars->b_full[st]), lead_cta);
+                    mbar_arrive_expect_tx_cluster(full, BST);
+                    tma_load_2d_pair(smem_u32(smem_b + st * BST), &tm_w, (k0 + u) * 64, tap * a.Cout + n0 + half * (BN / 2), full);
+                    ++issued;
+                    if (++st == (uint32_t)n_b) { st = 0; ph ^= 1; }
+                }
+            }
+            if (!ok) {                                       // unwinding: let the copies in flight land first (the odd CTA cannot see that: it waits the limit)
+                for (int k = 0; k < min(issued, n_b); ++k) {
+                    if (st == 0) { st = n_b; ph ^= 1; }
+                    --st;
+                    const long long t0 = clock64();
+                    while (!mbar_try_wait(smem_u32(&bars->b_full[st]), ph) && clock64() - t0 < WAIT_LIMIT_CYCLES) {}
+                }
+            }
+        }
+    } else if (warp == 0) {
+        // ------------------------------------------------ MMA issue (warp-uniform, predicated on one elected lane)
+        if (half == 0) {
+            const uint32_t lead = elect_one();
+            constexpr uint32_t idesc = make_idesc_bf16(256, BN);
+            const uint32_t a_hi = desc_hi(PW * 128, 2), d_hi = desc_hi(1024, 2);
+            const uint32_t a_lo0 = desc_lo(smem_u32(smem_a)), b_lo0 = desc_lo(smem_u32(smem_b));
+            const uint16_t pair_mask = (uint16_t)(3u << rank), all = (uint16_t)((1u << (2 * S)) - 1u);
+            const int loads = nk * TAPS;
+            uint32_t as = 0, aph = 0, bs = 0, bph = 0, acc = 0;
+            int used = 0;                                    // a stage that no later load needs is not handed back
+            auto wait_on = [&](uint64_t* b, uint32_t ph) {
+                if (!mbar_try_wait(smem_u32(b), ph)) (void)mbar_wait(smem_u32(b), ph, abort_flag);
+                tc_fence_after();
+            };
+#pragma unroll 1
+            for (int u = 0; u < nk; ++u) {
+                if (*abort_flag) break;
+                wait_on(&bars->a_full[as], aph);
+                uint32_t a_lo = a_lo0 + as * (uint32_t)(A_TILE_BYTES >> 4);
+                int kx = 0;
+#pragma unroll 1
+                for (int tap = 0; tap < TAPS; ++tap) {
+                    wait_on(&bars->b_full[bs], bph);
+                    const uint32_t b_lo = b_lo0 + bs * (uint32_t)(BST >> 4);
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        umma2_bf16_split_on(tmem, a_lo + 2 * k, a_hi, b_lo + 2 * k, d_hi, idesc, acc, lead);
+                        acc = 1u;
+                    }
+                    if (++used + n_b <= loads) commit2_to_cluster(smem_u32(&bars->b_empty[bs]), pair_mask, lead);
+                    __syncwarp();
+                    if (++bs == (uint32_t)n_b) { bs = 0; bph ^= 1; }
+                    if (++kx == 3) { kx = 0; a_lo += (uint32_t)((PW - 2) * 8); } else a_lo += 8u;
+                }
+                if (u + n_a < nk) commit2_to_cluster(smem_u32(&bars->a_empty[as]), pair_mask, lead);
+                __syncwarp();
+                if (++as == (uint32_t)n_a) { as = 0; aph ^= 1; }
+            }
+            __syncwarp();
+            commit2_to_cluster(smem_u32(&bars->acc_full), all, lead);
+            __syncwarp();
+        }
+    } else {
+        // ------------------------------------------------ operand prologue
+        const int ptid = tid - kProd0 * 32, pw = warp - kProd0;
+        const bool prologue = a.scale != nullptr || a.in_rec != nullptr, silu = a.silu != 0;
+        const int nch = nk * 64;
+        const float scale = silu ? 0.5f : 1.0f;              // SiLU is evaluated as h + h * tanh(h), h = v / 2
+        Operand<K3X3, IN_BF16, kPairWarps> op;
+        op.prepare(a, frame, k0 * 64, ty, tx, H, W, ptid);
+        InputStats stats;
+        if (a.in_rec && pw < 8) stats.prepare(a, frame, k0 * 64, nch, pw, lane, s_scale, s_shift);
+        if (pw == 0) touch_params(a, &bars->unused);
+        griddep_wait();
+        if (a.in_rec && pw < 8) stats.load(a, lane);
+        op.load_first();
+        if (prologue) {
+            if (a.in_rec) {
+                if (pw < 8) stats.finish(a, nch, lane, scale, s_scale, s_shift);
+            } else {
+                for (int c = ptid; c < nch; c += NT) {
+                    s_scale[c] = __ldcg(a.scale + (size_t)frame * a.Cin + k0 * 64 + c) * scale;
+                    s_shift[c] = __ldcg(a.shift + (size_t)frame * a.Cin + k0 * 64 + c) * scale;
+                }
+            }
+            named_barrier_sync(1, NT);
+        }
+        uint32_t as = 0, aph = 0;
+#pragma unroll 1
+        for (int u = 0; u < nk; ++u) {
+            if (u >= n_a && !mbar_wait(smem_u32(&bars->a_empty[as]), aph ^ 1, abort_flag)) break;
+            op.transform(smem_a + as * A_TILE_BYTES, u, u + 1 < nk, prologue, silu, s_scale, s_shift, ptid);
+            fence_proxy_async_smem();
+            __syncwarp();
+            if (lane == 0) mbar_arrive_cluster(peer_addr(smem_u32(&bars->a_full[as]), lead_cta));
+            if (++as == (uint32_t)n_a) { as = 0; aph ^= 1; }
+        }
+        // ------------------------------------------------ exchange and epilogue: row R of the tile belongs to part R / rpo of K,
+        // and to eight of the sixteen warps
+        const int rpo = ROWS / S, rows = rpo / 2, first = (pw >> 3) * rows;
+        auto exchange = [&] {
+            (void)mbar_wait(smem_u32(&bars->acc_full), 0, abort_flag);       // every CTA of the cluster is done with its operands
+            tc_fence_after();
+            __syncwarp();
+            const int col = (pw >> 2) * (BN / 4);
+            float* row = part + ((warp & 3) * 32 + lane) * RXS + col;
+#pragma unroll 1
+            for (int p = 0; p < BN / 4; p += 32) {
+                uint32_t r[32];
+                tmem_ld32(tmem + (uint32_t)(col + p) + ((uint32_t)((warp & 3) * 32) << 16), r);
+                tmem_ld_wait();
+#pragma unroll
+                for (int c = 0; c < 8; ++c) *(uint4*)(row + p + 4 * c) = make_uint4(r[4 * c], r[4 * c + 1], r[4 * c + 2], r[4 * c + 3]);
+            }
+            tc_fence_before();
+            if (S > 1) fence_proxy_async_smem();
+            named_barrier_sync(1, NT);
+            if (S > 1) {
+                if (ptid < S && ptid != kp)
+                    copy_to_peer(peer_addr(smem_u32(rx + (kp < ptid ? kp : kp - 1) * rpo * RXS), (uint32_t)(ptid * 2 + half)), smem_u32(part + ptid * rpo * RXS),
+                                 (uint32_t)(rpo * RXS * 4), peer_addr(smem_u32(&bars->rx_full), (uint32_t)(ptid * 2 + half)));
+                __syncwarp();
+                (void)wait_cluster(smem_u32(&bars->rx_full), 0, abort_flag);
+            }
+            __syncwarp();
+            cluster_arrive();                                // what is sent to this CTA has landed
+        };
+        finish_rows<BN, RXS, 4>(a, [&](int s) { return (s == kp ? part + kp * rpo * RXS : rx + (s < kp ? s : s - 1) * rpo * RXS) + first * RXS; }, S, rows,
+                                ptid & 255, frame, n0, H, W, (tile * S + kp) * 2 + (pw >> 3),
+                                [&](int local, int& oy, int& ox) -> bool {
+                                    const int R = kp * rpo + first + local;
+                                    oy = ty + (R >> 3);
+                                    ox = tx + (R & 7);
+                                    return oy < H && ox < W;
+                                },
+                                [](int) { return 0; }, exchange);
+    }
+    __syncwarp();
+    if (warp < kProd0) cluster_arrive();
+    cluster_wait();                                          // the sources of this CTA's copies may go; the pair's accumulators have been read
+    if (warp == 0) {
+        tc_fence_after();
+        tmem_dealloc2(tmem, (uint32_t)BN);
     }
     if (tid == kProd0 * 32 && bars->abort_flag && status) {
         if (atomicCAS(status, 0u, kStatusConvTimeout) == 0u) {
@@ -433,6 +671,45 @@ cudaError_t launch_one(const ConvArgs& a, const ConvSplitPlan& p, unsigned int* 
     return cudaLaunchKernelEx(&cfg, kern, a, p.shape, *(const CUtensorMap*)p.tmap, *(const CUtensorMap*)p.tmap2, *(const CUtensorMap*)p.tmap_x2, status);
 }
 
+template <bool IB>
+cudaError_t launch_pair(const ConvArgs& a, const ConvSplitPlan& p, unsigned int* status, cudaStream_t s) {
+    auto kern = conv_pair_kernel<IB>;
+    static bool configured[kMaxDevices] = {};
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
+    {
+        std::lock_guard<std::mutex> lock(g_mu);
+        if (!configured[dev]) {
+            e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kPairSmemMax);
+            if (e != cudaSuccess) return e;
+            configured[dev] = true;
+        }
+    }
+    const long long tiles = (long long)((a.W + TILE_W - 1) / TILE_W) * ((a.H + TILE_H - 1) / TILE_H);
+    const long long grid = (tiles + 1) / 2 * (a.Cout / kPairBN) * a.B * 2 * p.shape.splits;
+    if (grid > 0x7fffffffLL) return cudaErrorInvalidValue;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3(kPairThreads);
+    cfg.dynamicSmemBytes = (size_t)p.smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[2];
+    int na = 0;
+    attr[na].id = cudaLaunchAttributeClusterDimension;
+    attr[na].val.clusterDim.x = (unsigned)(2 * p.shape.splits); attr[na].val.clusterDim.y = 1; attr[na].val.clusterDim.z = 1;
+    ++na;
+    if (pdl_enabled()) {
+        attr[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[na].val.programmaticStreamSerializationAllowed = 1;
+        ++na;
+    }
+    cfg.attrs = attr;
+    cfg.numAttrs = na;
+    return cudaLaunchKernelEx(&cfg, kern, a, p.shape, *(const CUtensorMap*)p.tmap, status);
+}
+
 int kind_of(const ConvArgs& a) { return a.upsample == 2 ? KPHASE : (a.ksize == 1 ? K1X1 : K3X3); }
 int tiles_of(const ConvArgs& a) {
     const int h = a.upsample == 2 ? a.Hs : a.H, w = a.upsample == 2 ? a.Ws : a.W;
@@ -446,6 +723,7 @@ bool conv_split_supported(const ConvArgs& a) {
 }
 
 int conv_split_slots(const ConvArgs& a, const ConvSplitPlan& p, int groups) {
+    if (p.bn == kPairBN) return (tiles_of(a) + 1) / 2 * 2 * p.shape.splits * 2 * rec_parts(p.bn, a.Cout / groups);
     return tiles_of(a) * (a.upsample == 2 ? 4 : 1) * p.shape.splits * rec_parts(p.bn, a.Cout / groups);
 }
 
@@ -462,7 +740,22 @@ bool conv_split_choose(const ConvArgs& a, ConvSplitPlan* p) {
     const long long ctas = (long long)tiles_of(a) * ((a.Cout + bn - 1) / bn) * (kind == KPHASE ? 4 : 1) * std::max(a.B, 1);
     int s = 1;
     while (s < 8 && 2 * s <= kchunks && ctas * 2 * s <= 296) s *= 2;
-    if (ctas * s > 296 || kchunks / s > 2) return false;
+    if (ctas * s > 296 || kchunks / s > 2) {
+        if (kind != K3X3 || a.x2 || a.Cout % kPairBN != 0) return false;
+        const long long pairs = (long long)(tiles_of(a) + 1) / 2 * (a.Cout / kPairBN) * std::max(a.B, 1);
+        if (kchunks < 2 || 4 * pairs > 132) return false;
+        s = 2;
+        const int nk = (kchunks + s - 1) / s, rows = TILE_H * TILE_W;
+        if (nk * 64 > kMaxSliceC) return false;
+        const int na = std::min(nk, kMaxA), a_bytes = na * A_TILE_BYTES, bst = kPairBN / 2 * 128;
+        const int nb = std::min(std::min(nk * taps, kMaxB), (kPairSmemMax - 1024 - kTailBytes - a_bytes) / bst);
+        const int ops = std::max(a_bytes + nb * bst, (rows + rows / s * (s - 1)) * (kPairBN + 4) * 4);
+        if (nb < 1 || ops + kTailBytes + 1024 > kPairSmemMax) return false;
+        p->bn = kPairBN;
+        p->shape = ConvSplitShape{s, na, nb, ops, a.Cout};
+        p->smem = ops + kTailBytes + 1024;
+        return true;
+    }
     // stages: as many as let two CTAs share an SM; a CTA with one unit needs one operand stage only
     const int nk = (kchunks + s - 1) / s, nq = a.x2 ? (a.Cin2 / 32 + s - 1) / s : 0;
     const int na = std::min(nk + nq, kMaxA), a_bytes = na * A_TILE_BYTES, bst = bn * 128;
@@ -481,7 +774,7 @@ cudaError_t conv_split_prepare(const ConvArgs& a, ConvSplitPlan* p) {
     const int rows = a.upsample == 2 ? 16 * a.Cout : a.ksize * a.ksize * p->shape.w_rows;
     const cuuint64_t wd[2] = {(cuuint64_t)a.Cin, (cuuint64_t)rows};
     const cuuint64_t ws[1] = {(cuuint64_t)a.Cin * 2};
-    const cuuint32_t wb[2] = {64, (cuuint32_t)p->bn};
+    const cuuint32_t wb[2] = {64, (cuuint32_t)(p->bn == kPairBN ? kPairBN / 2 : p->bn)};
     const cuuint32_t one[4] = {1, 1, 1, 1};
     if (enc((CUtensorMap*)p->tmap, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(a.w), wd, ws, wb, one, CU_TENSOR_MAP_INTERLEAVE_NONE,
             CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
@@ -513,6 +806,7 @@ cudaError_t launch_conv_split(const ConvArgs& a, const ConvSplitPlan& p, unsigne
     if (a.out_rec && !rec_groups_ok(a.Cout, a.out_G)) return cudaErrorInvalidValue;
     const bool ib = a.in_dtype == VD_BF16;
     const int kind = kind_of(a);
+    if (p.bn == kPairBN) return ib ? launch_pair<true>(a, p, status, s) : launch_pair<false>(a, p, status, s);
     if (p.bn == 16) return ib ? launch_one<16, K3X3, true>(a, p, status, s) : launch_one<16, K3X3, false>(a, p, status, s);
     if (kind == K3X3) return ib ? launch_one<64, K3X3, true>(a, p, status, s) : launch_one<64, K3X3, false>(a, p, status, s);
     if (kind == K1X1) return ib ? launch_one<64, K1X1, true>(a, p, status, s) : launch_one<64, K1X1, false>(a, p, status, s);

@@ -46,6 +46,7 @@
 #include <type_traits>
 
 #include "conv_tile.cuh"
+#include "tc_pair.cuh"
 #include "tc_common.cuh"
 #include "vd_internal.h"
 
@@ -185,75 +186,6 @@ struct PhaseSched {
     __device__ __forceinline__ int rot(int s) const { return lag ? ((s + 1 + 3 * K) & 3) : 0; }
     __device__ __forceinline__ int item_of(int q) const { return m_k ? (int)__umulhi((uint32_t)q, m_k) : q; }
 };
-
-// ---- cluster / cta_group::2 PTX
-__device__ __forceinline__ uint32_t cluster_ctarank() {
-    uint32_t r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-__device__ __forceinline__ uint32_t map_to_cta(uint32_t smem_addr, uint32_t cta) {     // shared::cta -> shared::cluster of `cta`
-    uint32_t r;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_addr), "r"(cta));
-    return r;
-}
-// Arrival on a barrier of the pair's leader CTA.  Release at CTA scope: the arriving warp's own shared-memory
-// stores (already made visible to the tensor core's proxy by its fence) are what the arrival publishes; nothing of
-// the peer CTA's memory is.  The cluster-scope form of the same instruction costs about 1600 cycles per arrival
-// here instead of about 100 (measured: stamps around the producers' hand-over).
-__device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr) {
-    asm volatile("mbarrier.arrive.release.cta.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive_cluster_relaxed(uint32_t cluster_addr) {
-    asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive_expect_tx_cluster(uint32_t cluster_addr, uint32_t bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.relaxed.cluster.shared::cluster.b64 _, [%0], %1;" ::"r"(cluster_addr), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void cluster_sync_all() {
-    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-// tile load into this CTA's shared memory whose completion is reported to a barrier of the leader CTA
-__device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const void* tmap, int x, int y, uint32_t leader_bar) {
-    asm volatile(
-        "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
-        ::"r"(dst), "l"(tmap), "r"(x), "r"(y), "r"(leader_bar) : "memory");
-}
-__device__ __forceinline__ void umma2_bf16_split(uint32_t d_tmem, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo, uint32_t b_hi,
-                                                 uint32_t idesc, uint32_t accumulate) {
-    asm volatile(
-        "{\n.reg .pred p;\n.reg .b64 da, db;\nsetp.ne.b32 p, %6, 0;\n"
-        "mov.b64 da, {%1, %2};\nmov.b64 db, {%3, %4};\n"
-        "tcgen05.mma.cta_group::2.kind::f16 [%0], da, db, %5, p;\n}\n"
-        ::"r"(d_tmem), "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(accumulate) : "memory");
-}
-__device__ __forceinline__ void umma2_bf16_split_on(uint32_t d_tmem, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo, uint32_t b_hi,
-                                                    uint32_t idesc, uint32_t accumulate, uint32_t on) {
-    asm volatile(
-        "{\n.reg .pred p, q;\n.reg .b64 da, db;\nsetp.ne.b32 p, %6, 0;\nsetp.ne.b32 q, %7, 0;\n"
-        "mov.b64 da, {%1, %2};\nmov.b64 db, {%3, %4};\n"
-        "@q tcgen05.mma.cta_group::2.kind::f16 [%0], da, db, %5, p;\n}\n"
-        ::"r"(d_tmem), "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(accumulate), "r"(on) : "memory");
-}
-__device__ __forceinline__ void umma2_commit_both_on(uint32_t bar, uint32_t on) {
-    const uint32_t peer = map_to_cta(bar, 1);
-    asm volatile("{\n.reg .pred q;\nsetp.ne.b32 q, %2, 0;\n"
-                 "@q tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];\n"
-                 "@q tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%1];\n}\n" ::"r"(bar), "r"(peer), "r"(on) : "memory");
-}
-// arrives (once the MMAs issued so far have completed) on the barrier at this offset in both CTAs of the pair:
-// one commit to the leader's own barrier, one to the peer's through its cluster address
-__device__ __forceinline__ void umma2_commit_both(uint32_t bar) {
-    asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
-    asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(map_to_cta(bar, 1)) : "memory");
-}
-__device__ __forceinline__ void tmem_alloc2(uint32_t smem_dst, uint32_t ncols) {
-    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_dst), "r"(ncols) : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
-}
-__device__ __forceinline__ void tmem_dealloc2(uint32_t taddr, uint32_t ncols) {
-    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
-}
 
 // ---- GroupNorm statistics of the output, taken in the epilogue (Section IV-B.1: the normalisation's reduction
 // rides on the tensor that is already on chip instead of reading it back from memory).

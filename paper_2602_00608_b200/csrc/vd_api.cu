@@ -278,8 +278,14 @@ class Planner {
                     h_->folds.push_back({v2, kNone, kNone, b2_off, w2_off, px2, Cin2, Cout});
                     a.bias2 = ptr<float>(v2);
                 }
-                if (pres != kNone) pending_[y_off] = pres;      // accumulated in place: what was pending stays pending
-                else pending_.erase(y_off);
+                if (pres != kNone && split && !a.bias2) {       // written anew: what was pending joins, and the records are those of all of y
+                    a.bias2 = ptr<float>(pres);
+                    pending_.erase(y_off);
+                } else if (pres != kNone) {
+                    pending_[y_off] = pres;                     // accumulated in place: what was pending stays pending
+                } else {
+                    pending_.erase(y_off);
+                }
             }
         }
         // ---- statistics as records (conv_cluster.cuh): where there are few, this layer merges them itself and the step
