@@ -67,15 +67,15 @@ __device__ __forceinline__ void touch_params(const ConvArgs& a, volatile uint32_
 }
 
 // half * scale and half * shift of the input channels [c0, c0 + nch) of `frame`, from the producing layer's records, by
-// eight warps (w = 0..7); c0 and nch are multiples of the group size.  A group has 8 lanes of a warp (32 where there are more
-// than 16 records); a lane's first two records are loaded by `load`, so that they are on their way before other loads, and
+// NW warps (w = 0..NW - 1); c0 and nch are multiples of the group size.  A group has 8 lanes of a warp (32 where there are more
+// than 16 records); a lane's first NR records are loaded by `load`, so that they are on their way before other loads, and
 // `finish` merges.  Deviations are from the first record's mean, so one round of loads and one of shuffles suffice.
 // Everything that does not need the kernel before is done ahead by `prepare`, gamma and beta into s_scale and s_shift
 // included (a lane reads back what it has put there itself); what stays in registers across the loads is kept small, since
 // a loaded value that is spilled has to be waited for.
-struct InputStats {
+template <int NW, int NR> struct InputStatsOf {
     const float4* rec;
-    float4 r0, r1;
+    float4 r[NR];
     int g;                                                   // this lane's group of the slice
     static __device__ __forceinline__ int lanes_log2(const ConvArgs& a) { return a.in_slots <= 16 ? 3 : 5; }
     __device__ __forceinline__ void prepare(const ConvArgs& a, int frame, int c0, int nch, int w, int lane, float* s_scale, float* s_shift) {
@@ -83,7 +83,7 @@ struct InputStats {
         g = (w << (5 - ll)) + (lane >> ll);
         rec = a.in_rec + ((size_t)frame * a.in_G + (c0 >> a.in_shift) + min(g, ng - 1)) * a.in_slots;
 #pragma unroll 1
-        for (int gg = g; gg < ng; gg += 8 << (5 - ll))
+        for (int gg = g; gg < ng; gg += NW << (5 - ll))
             for (int i = l; i < 1 << a.in_shift; i += L) {
                 const int c = (gg << a.in_shift) + i;
                 s_scale[c] = __ldg(a.in_gamma + c0 + c);
@@ -92,24 +92,27 @@ struct InputStats {
     }
     __device__ __forceinline__ void load(const ConvArgs& a, int lane) {
         const int ll = lanes_log2(a), L = 1 << ll, l = lane & (L - 1);
-        r0 = r1 = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (l < a.in_slots) r0 = __ldcg(rec + l);
-        if (l + L < a.in_slots) r1 = __ldcg(rec + l + L);
+#pragma unroll
+        for (int i = 0; i < NR; ++i) {
+            r[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (l + i * L < a.in_slots) r[i] = __ldcg(rec + l + i * L);
+        }
     }
     __device__ __forceinline__ void finish(const ConvArgs& a, int nch, int lane, float half, float* s_scale, float* s_shift) {
         const int ll = lanes_log2(a), L = 1 << ll, l = lane & (L - 1), ng = nch >> a.in_shift;
 #pragma unroll 1
         for (;;) {
-            const float ref = __shfl_sync(0xffffffffu, r0.y, lane & ~(L - 1));
-            const float d0 = r0.y - ref, d1 = r1.y - ref, n0 = r0.x * d0, n1 = r1.x * d1;
-            float s = n0 + n1, q = fmaf(n0, d0, r0.z) + fmaf(n1, d1, r1.z);
-#pragma unroll 1
-            for (int i = l + 2 * L; i < a.in_slots; i += L) {
-                const float4 r = __ldcg(rec + i);
-                const float d = r.y - ref, nd = r.x * d;
+            const float ref = __shfl_sync(0xffffffffu, r[0].y, lane & ~(L - 1));
+            float s = 0.f, q = 0.f;
+            auto add = [&](const float4& v) {
+                const float d = v.y - ref, nd = v.x * d;
                 s += nd;
-                q += fmaf(nd, d, r.z);
-            }
+                q += fmaf(nd, d, v.z);
+            };
+#pragma unroll
+            for (int i = 0; i < NR; ++i) add(r[i]);
+#pragma unroll 1
+            for (int i = l + NR * L; i < a.in_slots; i += L) add(__ldcg(rec + i));
             if (ll == 5) {
                 s += __shfl_xor_sync(0xffffffffu, s, 16); q += __shfl_xor_sync(0xffffffffu, q, 16);
                 s += __shfl_xor_sync(0xffffffffu, s, 8); q += __shfl_xor_sync(0xffffffffu, q, 8);
@@ -128,7 +131,7 @@ struct InputStats {
                     s_scale[c] = sc * half;
                     s_shift[c] = (s_shift[c] - mean * sc) * half;
                 }
-            const int step = 8 << (5 - ll);
+            const int step = NW << (5 - ll);
             if (g - (lane >> ll) + step >= ng) break;        // (the same for the whole warp)
             rec += (size_t)(min(g + step, ng - 1) - min(g, ng - 1)) * a.in_slots;
             g += step;
@@ -136,6 +139,7 @@ struct InputStats {
         }
     }
 };
+using InputStats = InputStatsOf<8, 2>;
 
 // The eight warps that write a CTA's rows: a warp has CPW four-channel columns of the BN channels (two at least: whole
 // 32-byte sectors), WC warps lie side by side and WR below one another.

@@ -411,7 +411,7 @@ conv_split_kernel(const ConvArgs a, const ConvSplitShape sh, const __grid_consta
 // tcgen05.mma.cta_group::2 (M = 256): a tap's weights come from L2 once for both tiles, and each CTA's shared memory holds
 // and feeds half of them.  S pairs share K; the exchange is between the CTAs of the same tile.  The pair's even CTA issues;
 // all "full" barriers are its own.
-constexpr int kPairBN = 256, kPairWarps = 16, kPairThreads = (kProd0 + kPairWarps) * 32, kPairSmemMax = 227 * 1024;
+constexpr int kPairBN = 256, kPairWarps = 16, kPairThreads = (kProd0 + kPairWarps) * 32, kPairSmemMax = 227 * 1024, kPairSplits = 2;
 
 // arrives, once the pair's MMAs issued so far have completed, on the barrier at this offset in every CTA of `mask`
 __device__ __forceinline__ void commit2_to_cluster(uint32_t bar, uint16_t mask, uint32_t on) {
@@ -423,15 +423,17 @@ __device__ __forceinline__ void commit2_to_cluster(uint32_t bar, uint16_t mask, 
 template <bool IN_BF16>
 __global__ void __launch_bounds__(kPairThreads, 1)
 conv_pair_kernel(const ConvArgs a, const ConvSplitShape sh, const __grid_constant__ CUtensorMap tm_w, unsigned int* status) {
-    constexpr int TAPS = 9, BN = kPairBN, BST = BN / 2 * 128, RXS = BN + 4, ROWS = TILE_H * TILE_W, NT = kPairWarps * 32;
+    constexpr int TAPS = 9, BN = kPairBN, BST = BN / 2 * 128, RXS = BN, ROWS = TILE_H * TILE_W, NT = kPairWarps * 32, S = kPairSplits;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    const int n_a = sh.n_a, n_b = sh.n_b, S = sh.splits;
+    const int n_a = sh.n_a, n_b = sh.n_b;
     uint8_t* smem_a = smem;
     uint8_t* smem_b = smem + n_a * A_TILE_BYTES;
-    // over the operand stages, once every MMA of the cluster is done: this CTA's partials, and the other CTA's of its rows
+    // over the operand stages, once every MMA of the cluster is done: this CTA's partials, and the other CTA's of its rows.
+    // 16-byte piece c of row R at c ^ swizzle(R): neither eight rows of a piece nor four rows of two pieces meet on a bank.
     float* part = (float*)smem;
     float* rx = part + ROWS * RXS;
+    auto swizzle = [](int R) { return (R & 3) * 2 + ((R >> 2) & 1); };
     float* s_scale = (float*)(smem + sh.tail_off);
     float* s_shift = s_scale + kMaxSliceC;
     SBars* bars = (SBars*)(s_shift + kMaxSliceC);
@@ -546,15 +548,15 @@ conv_pair_kernel(const ConvArgs a, const ConvSplitShape sh, const __grid_constan
         const float scale = silu ? 0.5f : 1.0f;              // SiLU is evaluated as h + h * tanh(h), h = v / 2
         Operand<K3X3, IN_BF16, kPairWarps> op;
         op.prepare(a, frame, k0 * 64, ty, tx, H, W, ptid);
-        InputStats stats;
-        if (a.in_rec && pw < 8) stats.prepare(a, frame, k0 * 64, nch, pw, lane, s_scale, s_shift);
+        InputStatsOf<kPairWarps, 4> stats;
+        if (a.in_rec) stats.prepare(a, frame, k0 * 64, nch, pw, lane, s_scale, s_shift);
         if (pw == 0) touch_params(a, &bars->unused);
         griddep_wait();
-        if (a.in_rec && pw < 8) stats.load(a, lane);
+        if (a.in_rec) stats.load(a, lane);
         op.load_first();
         if (prologue) {
             if (a.in_rec) {
-                if (pw < 8) stats.finish(a, nch, lane, scale, s_scale, s_shift);
+                stats.finish(a, nch, lane, scale, s_scale, s_shift);
             } else {
                 for (int c = ptid; c < nch; c += NT) {
                     s_scale[c] = __ldcg(a.scale + (size_t)frame * a.Cin + k0 * 64 + c) * scale;
@@ -580,15 +582,15 @@ conv_pair_kernel(const ConvArgs a, const ConvSplitShape sh, const __grid_constan
             (void)mbar_wait(smem_u32(&bars->acc_full), 0, abort_flag);       // every CTA of the cluster is done with its operands
             tc_fence_after();
             __syncwarp();
-            const int col = (pw >> 2) * (BN / 4);
-            float* row = part + ((warp & 3) * 32 + lane) * RXS + col;
+            const int col = (pw >> 2) * (BN / 4), R = (warp & 3) * 32 + lane;
+            float* row = part + R * RXS;
 #pragma unroll 1
             for (int p = 0; p < BN / 4; p += 32) {
                 uint32_t r[32];
                 tmem_ld32(tmem + (uint32_t)(col + p) + ((uint32_t)((warp & 3) * 32) << 16), r);
                 tmem_ld_wait();
 #pragma unroll
-                for (int c = 0; c < 8; ++c) *(uint4*)(row + p + 4 * c) = make_uint4(r[4 * c], r[4 * c + 1], r[4 * c + 2], r[4 * c + 3]);
+                for (int c = 0; c < 8; ++c) *(uint4*)(row + ((((col + p) >> 2) + c) ^ swizzle(R)) * 4) = make_uint4(r[4 * c], r[4 * c + 1], r[4 * c + 2], r[4 * c + 3]);
             }
             tc_fence_before();
             if (S > 1) fence_proxy_async_smem();
@@ -611,7 +613,7 @@ conv_pair_kernel(const ConvArgs a, const ConvSplitShape sh, const __grid_constan
                                     ox = tx + (R & 7);
                                     return oy < H && ox < W;
                                 },
-                                [](int) { return 0; }, exchange);
+                                swizzle, exchange);
     }
     __syncwarp();
     if (warp < kProd0) cluster_arrive();
@@ -743,13 +745,13 @@ bool conv_split_choose(const ConvArgs& a, ConvSplitPlan* p) {
     if (ctas * s > 296 || kchunks / s > 2) {
         if (kind != K3X3 || a.x2 || a.Cout % kPairBN != 0) return false;
         const long long pairs = (long long)(tiles_of(a) + 1) / 2 * (a.Cout / kPairBN) * std::max(a.B, 1);
-        if (kchunks < 2 || 4 * pairs > 132) return false;
-        s = 2;
+        if (kchunks < kPairSplits || 2 * kPairSplits * pairs > 132) return false;
+        s = kPairSplits;
         const int nk = (kchunks + s - 1) / s, rows = TILE_H * TILE_W;
         if (nk * 64 > kMaxSliceC) return false;
         const int na = std::min(nk, kMaxA), a_bytes = na * A_TILE_BYTES, bst = kPairBN / 2 * 128;
         const int nb = std::min(std::min(nk * taps, kMaxB), (kPairSmemMax - 1024 - kTailBytes - a_bytes) / bst);
-        const int ops = std::max(a_bytes + nb * bst, (rows + rows / s * (s - 1)) * (kPairBN + 4) * 4);
+        const int ops = std::max(a_bytes + nb * bst, (rows + rows / s * (s - 1)) * kPairBN * 4);
         if (nb < 1 || ops + kTailBytes + 1024 > kPairSmemMax) return false;
         p->bn = kPairBN;
         p->shape = ConvSplitShape{s, na, nb, ops, a.Cout};
