@@ -2,8 +2,8 @@
 // the exchange of partial sums through distributed shared memory, and GroupNorm statistics as records.
 //
 //   * A CTA adds up and writes 1/S of its cluster's output rows (row = pixel of the tile).  Every CTA lays its partials
-//     out in its own shared memory, and one bulk copy per owner carries an owner's rows there and counts the bytes on the
-//     owner's barrier: one wait, no cluster-wide barrier on the way.  (16-byte st.async stores straight from registers
+//     out in its own shared memory, and bulk copies carry an owner's rows there and count the bytes on the owner's barrier:
+//     one wait, no cluster-wide barrier on the way.  (16-byte st.async stores straight from registers
 //     took 2.3-3.7 us of a 12 us layer: 2048 packets per CTA.)  The owner adds the partials in a fixed order (bitwise
 //     reproducible).
 //   * While it writes its rows a CTA takes their statistics, and leaves one record (count, mean, sum of squared
@@ -153,15 +153,15 @@ inline int rec_parts(int bn, int cpg) {
 }
 
 // Adds up the `nparts` partials of this CTA's `rpo` rows, adds bias and residual, writes the output and the statistics
-// records.  source(s): partial s, [rpo][RXS] floats, 16-byte piece c of a row at c ^ swizzle(row).  ptid: 0..255.
+// records.  source(s, row, c): where channels [4c, 4c + 4) of row `row` of partial s lie.  ptid: 0..255.
 // locate(local row, oy, ox) gives the row's output pixel and whether it exists; ready() returns when the partials have
 // arrived.  The first PRE rows' addresses and residual and the record's address are made before that (the empty asm keeps
 // them there).
 // A thread takes four channels (cg) of every RSTEP-th row, so a warp's share of a group comes from shuffles alone.  BN < 32:
 // the frame head (planes or packed pixels of a.Cout channels).
-template <int BN, int RXS, int PRE, class Source, class Locate, class Swizzle, class Ready>
+template <int BN, int PRE, class Source, class Locate, class Ready>
 __device__ __forceinline__ void finish_rows(const ConvArgs& a, Source source, int nparts, int rpo, int ptid, int frame, int n0, int OH, int OW,
-                                            int slot0, Locate locate, Swizzle swizzle, Ready ready) {
+                                            int slot0, Locate locate, Ready ready) {
     constexpr bool HEAD = BN < 32;
     constexpr int CPW = HEAD ? 1 : Split8<HEAD ? 64 : BN>::CPW, WC = HEAD ? 1 : Split8<HEAD ? 64 : BN>::WC, RL = 32 / CPW;
     constexpr int RSTEP = HEAD ? kFinishThreads / (BN / 4) : RL * (8 / WC), CPW_LOG2 = CPW == 8 ? 3 : CPW == 4 ? 2 : CPW - 1;
@@ -210,10 +210,9 @@ __device__ __forceinline__ void finish_rows(const ConvArgs& a, Source source, in
             const int local = first + i * RSTEP;
             float4 v = bias;
             if (valid[i]) {
-                const int q = local * RXS + (cg ^ swizzle(local)) * 4;
 #pragma unroll 4
                 for (int s = 0; s < nparts; ++s) {
-                    const float4 p = *(const float4*)(source(s) + q);
+                    const float4 p = *(const float4*)source(s, local, cg);
                     v.x += p.x; v.y += p.y; v.z += p.z; v.w += p.w;
                 }
                 if (HEAD) {

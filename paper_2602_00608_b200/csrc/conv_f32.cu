@@ -82,7 +82,8 @@ constexpr int kFTail = 2 * kMaxSlice * 4 + 128;              // scale / shift of
 
 // A partial lies in memory as rows (pixels) of BN floats whose 16-byte pieces are permuted by the row, so that neither the
 // threads that write it (eight tile rows side by side) nor those that read it (eight pixels of a row) meet on a bank.
-template <int BN> __device__ __forceinline__ int piece(int R) { return BN < 32 ? 0 : (R ^ (R >> 3)) & 7; }
+// The frame head's rows are one piece long: there the pixels of a group of eight are permuted (displacement of row R).
+template <int BN, int TW> __device__ __forceinline__ int piece(int R) { return BN < 32 ? ((R ^ (R / TW)) & 7) - (R & 7) : (R ^ (R >> 3)) & 7; }
 
 template <int TH, int BN, int KIND, int TW>
 __global__ void __launch_bounds__(kThreads, 2)
@@ -259,7 +260,7 @@ conv_f32_kernel(const ConvArgs a, const int S, const int n_w, const int ops_floa
     // ---- the K groups' partials are added in halves (a fixed order); the first group keeps the sum
     auto at = [&](int slab, int i) -> float4* {
         const int R = row * TW + ng * 8 + i;
-        return (float4*)(part + (slab * TH * TW + R) * BN + (cg ^ piece<BN>(R)) * 4);
+        return (float4*)(part + (slab * TH * TW + R) * BN + (cg ^ piece<BN, TW>(R)) * 4);
     };
     auto put = [&](int slab) {
 #pragma unroll
@@ -298,7 +299,7 @@ conv_f32_kernel(const ConvArgs a, const int S, const int n_w, const int ops_floa
         rx = part;
         __syncthreads();
     }
-    finish_rows<BN, BN, 2>(a, [&](int s) { return rx + s * rpo * BN; }, S, rpo, tid, frame, n0, KIND == KPHASE ? 2 * H : H, KIND == KPHASE ? 2 * W : W,
+    finish_rows<BN, 2>(a, [&](int s, int local, int c) { return rx + (s * rpo + local) * BN + (c ^ piece<BN, TW>(rank * rpo + local)) * 4; }, S, rpo, tid, frame, n0, KIND == KPHASE ? 2 * H : H, KIND == KPHASE ? 2 * W : W,
                         (KIND == KPHASE ? tile * 4 + par : tile) * S + rank,
                         [&](int local, int& oy, int& ox) -> bool {
                             const int R = rank * rpo + local;
@@ -308,7 +309,6 @@ conv_f32_kernel(const ConvArgs a, const int S, const int n_w, const int ops_floa
                             if (KIND == KPHASE) { oy = 2 * oy + (par >> 1); ox = 2 * ox + (par & 1); }
                             return valid;
                         },
-                        [&](int local) { return piece<BN>(rank * rpo + local); },
                         [&] {
                             if (S > 1) {
                                 (void)wait_cluster(smem_u32(&bars->rx_full), 0, abort_flag);

@@ -52,6 +52,10 @@ struct SBars {
     uint32_t tmem_base, abort_flag, unused;
 };
 
+// 16-byte piece c of row R of a partial lies at this piece: eight rows of a piece, and four rows of two pieces side by side,
+// are on distinct banks.
+template <int BN> __device__ __forceinline__ int exchange_piece(int R, int c) { return BN < 64 ? c : c ^ ((R & 3) * 2 + ((R >> 2) & 1)); }
+
 // arrives, once the MMAs issued so far have completed, on the barrier at this offset in every CTA of `mask`
 __device__ __forceinline__ void commit_to_cluster(uint32_t bar, uint16_t mask, uint32_t on) {
     asm volatile("{\n.reg .pred q;\nsetp.ne.b32 q, %2, 0;\n"
@@ -147,16 +151,17 @@ conv_split_kernel(const ConvArgs a, const ConvSplitShape sh, const __grid_consta
                   const __grid_constant__ CUtensorMap tm_w2, const __grid_constant__ CUtensorMap tm_x2, unsigned int* status) {
     constexpr int TAPS = taps_of(KIND);
     constexpr int BST = BN * 128;                            // bytes of a weight stage
-    constexpr int RXS = BN < 32 ? BN : BN + 4;               // floats per row of the exchange buffer
+    constexpr int ROWS = TILE_H * TILE_W, CB = BN < 64 ? BN : 32, NB = BN / CB;       // a warp moves 32 rows x CB channels of the accumulator
     constexpr int ACC_COLS = BN < 32 ? 32 : BN;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     const int n_a = sh.n_a, n_b = sh.n_b, S = sh.splits;
     uint8_t* smem_a = smem;
     uint8_t* smem_b = smem + n_a * A_TILE_BYTES;
-    // over the operand stages, once every MMA of the cluster is done: this CTA's partials, and those of its rows
+    // over the operand stages, once every MMA of the cluster is done: this CTA's partials [NB][ROWS][CB], and those of its
+    // rows [S][NB][rows][CB]
     float* part = (float*)smem;
-    float* rx = S > 1 ? part + TILE_H * TILE_W * RXS : part;
+    float* rx = S > 1 ? part + ROWS * BN : part;
     float* s_scale = (float*)(smem + sh.tail_off);
     float* s_shift = s_scale + kMaxSliceC;
     SBars* bars = (SBars*)(s_shift + kMaxSliceC);
@@ -190,7 +195,7 @@ conv_split_kernel(const ConvArgs a, const ConvSplitShape sh, const __grid_consta
         bars->abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         fence_proxy_async_smem();
-        mbar_arrive_expect_tx(smem_u32(&bars->rx_full), TILE_H * TILE_W * RXS * 4);  // this CTA's rows from all S partials
+        mbar_arrive_expect_tx(smem_u32(&bars->rx_full), ROWS * BN * 4);  // this CTA's rows from all S partials
     }
     if (warp == 0) tmem_alloc(smem_u32(&bars->tmem_base), (uint32_t)ACC_COLS);
     tc_fence_before();
@@ -339,38 +344,33 @@ conv_split_kernel(const ConvArgs a, const ConvSplitShape sh, const __grid_consta
             if (++as == (uint32_t)n_a) { as = 0; aph ^= 1; }
         }
         // ------------------------------------------------ exchange and epilogue: row R of the tile belongs to CTA R / rpo
-        const int rpo = TILE_H * TILE_W / S;
+        const int rpo_log2 = 7 - (__ffs(S) - 1), rpo = 1 << rpo_log2;                 // (S is a power of two)
+        static_assert(ROWS == 128, "rows of a tile");
         auto exchange = [&] {
             (void)mbar_wait(smem_u32(&bars->acc_full), 0, abort_flag);       // every CTA of the cluster is done with its operands
             tc_fence_after();
             __syncwarp();
             cluster_wait();
-            const int col = BN < 64 ? 0 : (pw >> 2) * (BN / 2);
-            float* row = part + ((warp & 3) * 32 + lane) * RXS + col;
-            const uint32_t tacc = tmem + (uint32_t)col + ((uint32_t)((warp & 3) * 32) << 16);
-            if constexpr (BN < 64) {
-                uint32_t r[16];
-                tmem_ld16(tacc, r);
-                tmem_ld_wait();
-                if (pw < 4) {
+            const int cb = BN < 64 ? 0 : pw >> 2, R0 = (warp & 3) * 32;
+            float* row = part + (cb * ROWS + R0 + lane) * CB;
+            const uint32_t tacc = tmem + (uint32_t)(cb * CB) + ((uint32_t)R0 << 16);
+            const bool moves = BN >= 64 || pw < 4;
+            uint32_t r[CB];
+            if constexpr (BN < 64) tmem_ld16(tacc, r);
+            else tmem_ld32(tacc, r);
+            tmem_ld_wait();
+            if (moves) {
 #pragma unroll
-                    for (int c = 0; c < 4; ++c) *(uint4*)(row + 4 * c) = make_uint4(r[4 * c], r[4 * c + 1], r[4 * c + 2], r[4 * c + 3]);
-                }
-            } else {
-                static_assert(BN <= 64, "one pass of 32 columns per warp");
-                uint32_t r[32];
-                tmem_ld32(tacc, r);
-                tmem_ld_wait();
-#pragma unroll
-                for (int c = 0; c < 8; ++c) *(uint4*)(row + 4 * c) = make_uint4(r[4 * c], r[4 * c + 1], r[4 * c + 2], r[4 * c + 3]);
+                for (int c = 0; c < CB / 4; ++c) *(uint4*)(row + exchange_piece<BN>(lane, c) * 4) = make_uint4(r[4 * c], r[4 * c + 1], r[4 * c + 2], r[4 * c + 3]);
             }
             tc_fence_before();
-            if (S > 1) {
+            if (S > 1) {                                     // each warp sends what it has written: its owners' rows lie together
                 fence_proxy_async_smem();
-                named_barrier_sync(1, kProd);
-                if (ptid < S)
-                    copy_to_peer(peer_addr(smem_u32(rx + rank * rpo * RXS), (uint32_t)ptid), smem_u32(part + ptid * rpo * RXS), (uint32_t)(rpo * RXS * 4),
-                                 peer_addr(smem_u32(&bars->rx_full), (uint32_t)ptid));
+                __syncwarp();
+                const int n_log2 = min(rpo_log2, 5), n = 1 << n_log2, R = R0 + lane * n, owner = R >> rpo_log2;
+                if (moves && lane < 32 >> n_log2)
+                    copy_to_peer(peer_addr(smem_u32(rx + ((rank * NB + cb) * rpo + R - owner * rpo) * CB), (uint32_t)owner), smem_u32(part + (cb * ROWS + R) * CB),
+                                 (uint32_t)(n * CB * 4), peer_addr(smem_u32(&bars->rx_full), (uint32_t)owner));
                 __syncwarp();
                 (void)wait_cluster(smem_u32(&bars->rx_full), 0, abort_flag);
             } else {
@@ -379,7 +379,7 @@ conv_split_kernel(const ConvArgs a, const ConvSplitShape sh, const __grid_consta
             __syncwarp();
             cluster_arrive();                                // what is sent to this CTA has landed
         };
-        finish_rows<BN, RXS, 2>(a, [&](int s) { return rx + s * rpo * RXS; }, S, rpo, ptid, frame, n0, KIND == KPHASE ? 2 * H : H, KIND == KPHASE ? 2 * W : W,
+        finish_rows<BN, 2>(a, [&](int s, int local, int c) { return rx + ((s * NB + c / (CB / 4)) * rpo + local) * CB + exchange_piece<BN>(local, c % (CB / 4)) * 4; }, S, rpo, ptid, frame, n0, KIND == KPHASE ? 2 * H : H, KIND == KPHASE ? 2 * W : W,
                         (KIND == KPHASE ? tile * 4 + par : tile) * S + rank,
                         [&](int local, int& oy, int& ox) -> bool {
                             const int R = rank * rpo + local;
@@ -389,7 +389,7 @@ conv_split_kernel(const ConvArgs a, const ConvSplitShape sh, const __grid_consta
                             if (KIND == KPHASE) { oy = 2 * oy + (par >> 1); ox = 2 * ox + (par & 1); }
                             return valid;
                         },
-                        [](int) { return 0; }, exchange);
+                        exchange);
     }
     __syncwarp();
     if (warp < kProd0) cluster_arrive();
@@ -423,17 +423,16 @@ __device__ __forceinline__ void commit2_to_cluster(uint32_t bar, uint16_t mask, 
 template <bool IN_BF16>
 __global__ void __launch_bounds__(kPairThreads, 1)
 conv_pair_kernel(const ConvArgs a, const ConvSplitShape sh, const __grid_constant__ CUtensorMap tm_w, unsigned int* status) {
-    constexpr int TAPS = 9, BN = kPairBN, BST = BN / 2 * 128, RXS = BN, ROWS = TILE_H * TILE_W, NT = kPairWarps * 32, S = kPairSplits;
+    constexpr int TAPS = 9, BN = kPairBN, BST = BN / 2 * 128, ROWS = TILE_H * TILE_W, CB = 64, NT = kPairWarps * 32, S = kPairSplits, RPO = ROWS / S;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     const int n_a = sh.n_a, n_b = sh.n_b;
     uint8_t* smem_a = smem;
     uint8_t* smem_b = smem + n_a * A_TILE_BYTES;
-    // over the operand stages, once every MMA of the cluster is done: this CTA's partials, and the other CTA's of its rows.
-    // 16-byte piece c of row R at c ^ swizzle(R): neither eight rows of a piece nor four rows of two pieces meet on a bank.
+    // over the operand stages, once every MMA of the cluster is done: this CTA's partials [4][ROWS][CB], and the other CTA's
+    // of its rows [4][RPO][CB]
     float* part = (float*)smem;
-    float* rx = part + ROWS * RXS;
-    auto swizzle = [](int R) { return (R & 3) * 2 + ((R >> 2) & 1); };
+    float* rx = part + ROWS * BN;
     float* s_scale = (float*)(smem + sh.tail_off);
     float* s_shift = s_scale + kMaxSliceC;
     SBars* bars = (SBars*)(s_shift + kMaxSliceC);
@@ -459,7 +458,7 @@ conv_pair_kernel(const ConvArgs a, const ConvSplitShape sh, const __grid_constan
         bars->abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         fence_proxy_async_smem();
-        mbar_arrive_expect_tx(smem_u32(&bars->rx_full), ROWS / S * (S - 1) * RXS * 4);         // this CTA's rows from the other partials
+        mbar_arrive_expect_tx(smem_u32(&bars->rx_full), RPO * BN * 4);                  // this CTA's rows from the other partial
     }
     if (warp == 0) tmem_alloc2(smem_u32(&bars->tmem_base), (uint32_t)BN);
     tc_fence_before();
@@ -577,43 +576,47 @@ conv_pair_kernel(const ConvArgs a, const ConvSplitShape sh, const __grid_constan
         }
         // ------------------------------------------------ exchange and epilogue: row R of the tile belongs to part R / rpo of K,
         // and to eight of the sixteen warps
-        const int rpo = ROWS / S, rows = rpo / 2, first = (pw >> 3) * rows;
+        constexpr int rows = RPO / 2;
+        const int first = (pw >> 3) * rows;
         auto exchange = [&] {
             (void)mbar_wait(smem_u32(&bars->acc_full), 0, abort_flag);       // every CTA of the cluster is done with its operands
             tc_fence_after();
             __syncwarp();
-            const int col = (pw >> 2) * (BN / 4), R = (warp & 3) * 32 + lane;
-            float* row = part + R * RXS;
+            const int cb = pw >> 2, R0 = (warp & 3) * 32, owner = R0 / RPO;
+            float* row = part + (cb * ROWS + R0 + lane) * CB;
 #pragma unroll 1
-            for (int p = 0; p < BN / 4; p += 32) {
+            for (int p = 0; p < CB; p += 32) {
                 uint32_t r[32];
-                tmem_ld32(tmem + (uint32_t)(col + p) + ((uint32_t)((warp & 3) * 32) << 16), r);
+                tmem_ld32(tmem + (uint32_t)(cb * CB + p) + ((uint32_t)R0 << 16), r);
                 tmem_ld_wait();
 #pragma unroll
-                for (int c = 0; c < 8; ++c) *(uint4*)(row + ((((col + p) >> 2) + c) ^ swizzle(R)) * 4) = make_uint4(r[4 * c], r[4 * c + 1], r[4 * c + 2], r[4 * c + 3]);
+                for (int c = 0; c < 8; ++c) *(uint4*)(row + exchange_piece<BN>(lane, (p >> 2) + c) * 4) = make_uint4(r[4 * c], r[4 * c + 1], r[4 * c + 2], r[4 * c + 3]);
             }
             tc_fence_before();
-            if (S > 1) fence_proxy_async_smem();
-            named_barrier_sync(1, NT);
-            if (S > 1) {
-                if (ptid < S && ptid != kp)
-                    copy_to_peer(peer_addr(smem_u32(rx + (kp < ptid ? kp : kp - 1) * rpo * RXS), (uint32_t)(ptid * 2 + half)), smem_u32(part + ptid * rpo * RXS),
-                                 (uint32_t)(rpo * RXS * 4), peer_addr(smem_u32(&bars->rx_full), (uint32_t)(ptid * 2 + half)));
-                __syncwarp();
-                (void)wait_cluster(smem_u32(&bars->rx_full), 0, abort_flag);
+            fence_proxy_async_smem();
+            __syncwarp();
+            if (owner != kp && lane == 0) {
+                const uint32_t peer = (uint32_t)(owner * 2 + half);
+                copy_to_peer(peer_addr(smem_u32(rx + (cb * RPO + R0 - owner * RPO) * CB), peer), smem_u32(part + (cb * ROWS + R0) * CB), 32 * CB * 4,
+                             peer_addr(smem_u32(&bars->rx_full), peer));
             }
+            named_barrier_sync(1, NT);                       // this CTA's own share of its rows
+            (void)wait_cluster(smem_u32(&bars->rx_full), 0, abort_flag);
             __syncwarp();
             cluster_arrive();                                // what is sent to this CTA has landed
         };
-        finish_rows<BN, RXS, 4>(a, [&](int s) { return (s == kp ? part + kp * rpo * RXS : rx + (s < kp ? s : s - 1) * rpo * RXS) + first * RXS; }, S, rows,
+        finish_rows<BN, 4>(a, [&](int s, int local, int c) {
+                                    const int b = c / (CB / 4), R = first + local;
+                                    return (s == kp ? part + (b * ROWS + kp * RPO + R) * CB : rx + (b * RPO + R) * CB) + exchange_piece<BN>(R, c % (CB / 4)) * 4;
+                                }, S, rows,
                                 ptid & 255, frame, n0, H, W, (tile * S + kp) * 2 + (pw >> 3),
                                 [&](int local, int& oy, int& ox) -> bool {
-                                    const int R = kp * rpo + first + local;
+                                    const int R = kp * RPO + first + local;
                                     oy = ty + (R >> 3);
                                     ox = tx + (R & 7);
                                     return oy < H && ox < W;
                                 },
-                                swizzle, exchange);
+                                exchange);
     }
     __syncwarp();
     if (warp < kProd0) cluster_arrive();
@@ -762,7 +765,7 @@ bool conv_split_choose(const ConvArgs& a, ConvSplitPlan* p) {
     const int nk = (kchunks + s - 1) / s, nq = a.x2 ? (a.Cin2 / 32 + s - 1) / s : 0;
     const int na = std::min(nk + nq, kMaxA), a_bytes = na * A_TILE_BYTES, bst = bn * 128;
     const int nb = std::min(std::min(nk * taps + nq, kMaxB), (kSplitSmemMax - 1024 - kTailBytes - a_bytes) / bst);
-    const int ops = (std::max(a_bytes + nb * bst, (s > 1 ? 2 : 1) * TILE_H * TILE_W * (bn + 4) * 4) + 15) / 16 * 16;
+    const int ops = (std::max(a_bytes + nb * bst, (s > 1 ? 2 : 1) * TILE_H * TILE_W * bn * 4) + 15) / 16 * 16;
     if (ops + kTailBytes + 1024 > kSplitSmemMax) return false;
     p->bn = bn;
     p->shape = ConvSplitShape{s, na, nb, ops, head ? 16 : a.Cout};
