@@ -102,7 +102,7 @@ template <int BN, int CG = 1, bool PH = false, bool IN_BF16 = false> struct Tile
     // weight stages: as many as fit (the weight stream waits on the latency of L2, which the SM clock does not shorten)
     // (128-channel blocks: the staging of a bf16 input is half the size, which buys a fourth stage; measured, the MMA
     // warp of such a layer waits on weights for a quarter of its time with three)
-    static constexpr int B_STAGES = PH ? 4 : (CG == 2 ? (BN == 256 ? 7 : 8) : (BN == 256 ? 5 : (BN == 128 ? (IN_BF16 ? 4 : 3) : 8)));
+    static constexpr int B_STAGES = PH ? 4 : (CG == 2 ? (BN == 256 ? 7 : (IN_BF16 ? 8 : 5)) : (BN == 256 ? 5 : (BN == 128 ? (IN_BF16 ? 4 : 3) : 8)));
     static constexpr int B_GROUP = BN >= 128 ? 1 : 2;                // weight stages handed back per tcgen05.commit
     static constexpr int A_STAGES = PH ? 5 : 2;                    // phase form: a chunk stays until the parity that lags most has used it
     static constexpr int A_STAGE_BYTES = PAIR * A_TILE_BYTES;
@@ -1628,13 +1628,18 @@ bool conv_tc_stats_supported(const ConvArgs& a, int groups) {
 // 94 + 17 -> 97 + 8; 256->256 at 240x360 81 + 19.4 -> 87 + 10.2; with shortcut 512->256 at 240x360 163 + 24 -> 168 + 12, 256->128 at
 // 480x720 230 + 38 -> 236 + 21.  Where the epilogue paces the layer it loses: 128->128 at 480x720 109 + 27 -> 172 + 20, phase
 // form 256->256 to 480x720 186 + 64 -> 337 + 21.
-// 3x3 layers of 256-channel blocks with ten tiles or more per SM run as CTA pairs: the chip is at its power limit there, and a
-// pair reads each weight from L2 once instead of twice.  Eight 720x480 frames per decode 26.34 -> 25.80 ms, two 1280x720
-// frames 18.20 -> 17.85; smaller layers lose more to the signals between the two CTAs than they gain (one 720x480 frame,
-// whose layers have 96 to 675 tiles: 3.57 -> 3.64 ms).
+// Large 3x3 layers run as CTA pairs: the chip is at its power limit there, and a pair reads each weight from L2 once instead of
+// twice and feeds each tensor core half of it from shared memory.  256-channel blocks, from ten tiles per SM: eight 720x480
+// frames per decode 26.34 -> 25.80 ms, two 1280x720 frames 18.20 -> 17.85; below, the signals between the two CTAs cost more
+// than they save (one 720x480 frame, whose layers have 96 to 675 tiles: 3.57 -> 3.64 ms).  128-channel blocks, whose MMAs take
+// as many bytes of weights as of operand from shared memory (and would be limited by it), from seven tiles per SM:
+// 128->128 at 480x720 109 -> 98 us, 256->128 188 -> 173; eight 720x480 frames 25.87 -> 25.47 ms, two 1280x720 17.87 -> 17.60;
+// a 256x256 frame (512 tiles) 0.958 -> 0.961.
 static bool wide_layer(const ConvArgs& a) {
-    if (a.Cout % 256 != 0 || a.ksize != 3 || a.upsample || a.x2 || a.out_nchw || a.out_u8) return false;
-    return (long long)((a.H + TILE_H - 1) / TILE_H) * ((a.W + TILE_W - 1) / TILE_W) * a.B * (a.Cout / 256) >= 1500;
+    if (a.Cout % 128 != 0 || a.ksize != 3 || a.upsample || a.x2 || a.out_nchw || a.out_u8) return false;
+    const bool b256 = a.Cout % 256 == 0;
+    if (!b256 && a.stat_sum) return false;                    // statistics in the epilogue: 128-channel blocks have the one-CTA form only
+    return (long long)((a.H + TILE_H - 1) / TILE_H) * ((a.W + TILE_W - 1) / TILE_W) * a.B * (a.Cout / (b256 ? 256 : 128)) >= (b256 ? 1500 : 1000);
 }
 static bool rec_layer(const ConvArgs& a) {
     if (!conv_tc_supported(a) || a.Cout % 128 != 0 || a.residual || a.bias || a.bias2 || a.ksize != 3 || a.upsample) return false;
@@ -1685,7 +1690,7 @@ cudaError_t conv_tc_prepare(const ConvArgs& a, ConvTcPlan* plan) {
     const int bn = phase ? 128 : pick_bn(a.Cout);
     // 256-channel blocks of the folded upsampling form and the phase form run as two-CTA pairs (each CTA loads
     // half of the rows of a weight tile); the device must be able to co-schedule such pairs
-    // So do the other 3x3 layers of 256-channel blocks that are large enough (wide_layer).
+    // So do the other 3x3 layers that are large enough (wide_layer).
     int cg = (phase || (bn == 256 && a.upsample) || wide_layer(a)) ? 2 : 1;
     if (cg == 2 && !pairs_available()) {
         if (phase) return cudaErrorInvalidConfiguration;     // the phase form has no one-CTA variant
@@ -1812,6 +1817,7 @@ cudaError_t launch_conv_tc(const ConvArgs& a, const ConvTcPlan& plan, unsigned i
     if (plan.bn == 256 && plan.cg == 2) VD_CONV_CASE(256, 2, false, 3);          // (9-tap upsampling form: 3x3)
     if (plan.bn == 256) { if (k1) VD_CONV_CASE(256, 1, false, 1); VD_CONV_CASE(256, 1, false, 3); }
     if (k1) VD_CONV_CASE(128, 1, false, 1);
+    if (plan.cg == 2) VD_CONV_CASE(128, 2, false, 3);
     VD_CONV_CASE(128, 1, false, 3);
 #undef VD_CONV_CASE
 }

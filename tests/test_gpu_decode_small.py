@@ -1,5 +1,6 @@
 """Decodes whose layers are divided along K among clusters of CTAs, at the sizes where that can go wrong: a tile filled
-exactly and one pixel more, one row of tiles, several frames, frame sizes at which some levels are divided and others are not.
+exactly and one pixel more, one row of tiles, several frames, an odd number of tiles on pairs of CTAs (40x20: 25 tiles at 80x40),
+frame sizes at which some levels are divided and others are not.
 Against the FFMA kernels on every pixel, with canaries behind every workspace region, and bitwise the same for a frame decoded
 by itself and in a batch."""
 import pytest
@@ -9,7 +10,7 @@ from tests.util import BF16_MAX_ABS, BF16_REL_L2
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("h,w,b", [(16, 8, 1), (17, 9, 1), (3, 40, 2), (24, 16, 1)])
+@pytest.mark.parametrize("h,w,b", [(16, 8, 1), (17, 9, 1), (3, 40, 2), (24, 16, 1), (40, 20, 1)])
 def test_small_decodes_match_the_ffma_kernels(h, w, b):
     import torch
     from paper_2602_00608_b200 import binding as vd, synth
