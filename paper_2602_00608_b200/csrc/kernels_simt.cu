@@ -717,70 +717,112 @@ cudaError_t launch_gn_stats(const GnArgs& a, cudaStream_t s) {
     return cudaGetLastError();
 }
 
-// The first convolution (latent channels -> hundreds of channels): K = 9 * Cin <= 72 is too thin for the
-// tensor core and for the tiled FFMA kernel's staging.  A block computes 32 consecutive pixels x 128
-// output channels: the pixels' 3x3 neighbourhoods sit in shared memory, a thread holds 4 pixels x 4
-// channels and reads the weights ([tap][Cin][Cout] fp32) as coalesced float4 straight from L1/L2.
-constexpr int kThinPix = 32, kThinCout = 128, kThinMaxK = 72;
-template <int CIN>
-__global__ void __launch_bounds__(256) conv_thin_kernel(ConvArgs a) {
-    __shared__ float in_s[kThinPix][kThinMaxK + 1];
+// The first convolution (latent channels -> hundreds of channels): K = 9 * Cin <= 72 is too thin for the tensor core and for
+// the staging of the tiled FFMA kernels.  A block computes 64 (32, 16) consecutive pixels of a frame x 128 output channels; a
+// thread holds 8 (4, 2) pixels x 4 channels.  The weights go to shared memory while the kernel before is still running, the
+// pixels' 3x3 neighbourhoods as float4 of channels after it: per four k's and thread 4 + 8 shared loads of 16 bytes for 128
+// multiply-adds, and these loads are the bound (three blocks per SM, or blocks that walk the image with the weights in place,
+// are no faster).  The output's GroupNorm statistics leave as records (conv_cluster.cuh).  4->512, profiled, the tiled
+// kernel -> this one: 37x53 17 -> 12 us, 60x90 30 -> 21, two 90x160 frames 119 -> 57.
+constexpr int kThinCout = 128, kThinWarps = 8;
+// pixels of a thread: two where that gives small images more blocks (and few enough records for the next layer to merge
+// itself); else as many as shared memory has room for
+static int thin_px(const ConvArgs& a) { return a.H * a.W <= 256 ? 2 : a.Cin == 4 ? 8 : 4; }
+template <int CIN, int PX>
+__global__ void __launch_bounds__(256, 2) conv_thin_kernel(ConvArgs a) {
+    constexpr int K = 9 * CIN, K4 = K / 4, PIX = PX * kThinWarps;
+    __shared__ float4 s_x[K4][PIX];
+    __shared__ float4 s_w[K][kThinCout / 4];
     griddep_launch();
+    const int P = a.H * a.W, blocks = (P + PIX - 1) / PIX;
+    const int frame = blockIdx.x / blocks, block = blockIdx.x - frame * blocks, p0 = block * PIX;
+    const int co0 = blockIdx.y * kThinCout, tid = threadIdx.x, pg = tid >> 5, cg = tid & 31, co = co0 + cg * 4;
+    for (int i = tid; i < K * (kThinCout / 4); i += 256) {
+        const int k = i / (kThinCout / 4), c = i % (kThinCout / 4);
+        s_w[k][c] = __ldg((const float4*)((const float*)a.w + (size_t)k * a.Cout + co0) + c);
+    }
+    float4 bias = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (a.bias) bias = __ldg((const float4*)(a.bias + co));
+    const int px = p0 + (tid & (PIX - 1)), oy = px / a.W, ox = px - oy * a.W;        // this thread's pixel of the gather
+    const float4* x = (const float4*)a.x + (size_t)frame * P * (CIN / 4);
     griddep_wait();
-    constexpr int K = 9 * CIN;
-    const long long npix = (long long)a.B * a.H * a.W;
-    const long long p0 = (long long)blockIdx.x * kThinPix;
-    const int co0 = blockIdx.y * kThinCout;
-    const float* x = (const float*)a.x;
-    for (int i = threadIdx.x; i < kThinPix * K; i += 256) {
-        const int p = i / K, k = i - p * K;
-        const int tap = k / CIN, c = k - tap * CIN;
-        const long long g = p0 + p;
-        float v = 0.f;
-        if (g < npix) {
-            const int b = (int)(g / ((long long)a.H * a.W));
-            const int r = (int)(g - (long long)b * a.H * a.W);
-            const int oy = r / a.W + tap / 3 - 1, ox = r % a.W + tap % 3 - 1;
-            if (oy >= 0 && oy < a.H && ox >= 0 && ox < a.W) v = x[(((size_t)b * a.H + oy) * a.W + ox) * CIN + c];
-        }
-        in_s[p][k] = a.bf16_operands ? round_bf16(v) : v;
+#pragma unroll
+    for (int r = tid / PIX; r < K4; r += 256 / PIX) {
+        const int tap = r / (CIN / 4), yy = oy + tap / 3 - 1, xx = ox + tap % 3 - 1;
+        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (px < P && yy >= 0 && yy < a.H && xx >= 0 && xx < a.W) v = __ldcg(x + ((size_t)yy * a.W + xx) * (CIN / 4) + r % (CIN / 4));
+        if (a.bf16_operands) v = make_float4(round_bf16(v.x), round_bf16(v.y), round_bf16(v.z), round_bf16(v.w));
+        s_x[r][tid & (PIX - 1)] = v;
     }
     __syncthreads();
-    const int pg = threadIdx.x >> 5, cg = threadIdx.x & 31;          // 4 pixels, 4 channels per thread
-    const float* w = (const float*)a.w + co0 + cg * 4;
-    float acc[4][4];
+    float acc[PX][4];
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < PX; ++i)
 #pragma unroll
         for (int q = 0; q < 4; ++q) acc[i][q] = 0.f;
-#pragma unroll 12
-    for (int k = 0; k < K; ++k) {
-        const float4 wv = __ldg((const float4*)(w + (size_t)k * a.Cout));
+#pragma unroll 3
+    for (int k4 = 0; k4 < K4; ++k4) {
+        float4 xv[PX];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const float xv = in_s[pg * 4 + i][k];
-            acc[i][0] = fmaf(xv, wv.x, acc[i][0]); acc[i][1] = fmaf(xv, wv.y, acc[i][1]);
-            acc[i][2] = fmaf(xv, wv.z, acc[i][2]); acc[i][3] = fmaf(xv, wv.w, acc[i][3]);
+        for (int i = 0; i < PX; ++i) xv[i] = s_x[k4][pg * PX + i];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const float4 w = s_w[k4 * 4 + e][cg];
+#pragma unroll
+            for (int i = 0; i < PX; ++i) {
+                const float v = e == 0 ? xv[i].x : e == 1 ? xv[i].y : e == 2 ? xv[i].z : xv[i].w;
+                acc[i][0] = fmaf(v, w.x, acc[i][0]); acc[i][1] = fmaf(v, w.y, acc[i][1]);
+                acc[i][2] = fmaf(v, w.z, acc[i][2]); acc[i][3] = fmaf(v, w.w, acc[i][3]);
+            }
         }
     }
-    float4 bv = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (a.bias) bv = __ldg((const float4*)(a.bias + co0 + cg * 4));
+    const int n = min(max(P - p0 - pg * PX, 0), PX);         // pixels of this warp
+    float* y = (float*)a.y + ((size_t)frame * P + p0 + pg * PX) * a.Cout + co;
+    float sum = 0.f, sq = 0.f, pivot = 0.f;
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const long long g = p0 + pg * 4 + i;
-        if (g < npix)
-            *(float4*)((float*)a.y + (size_t)g * a.Cout + co0 + cg * 4) =
-                make_float4(acc[i][0] + bv.x, acc[i][1] + bv.y, acc[i][2] + bv.z, acc[i][3] + bv.w);
+    for (int i = 0; i < PX; ++i) {
+        const float4 v = make_float4(acc[i][0] + bias.x, acc[i][1] + bias.y, acc[i][2] + bias.z, acc[i][3] + bias.w);
+        if (i < n) *(float4*)(y + (size_t)i * a.Cout) = v;
+        if (a.out_rec) {                                     // a group is 1 << (out_shift - 2) lanes
+            if (i == 0) pivot = __shfl_sync(0xffffffffu, v.x, cg & ~((1 << (a.out_shift - 2)) - 1));
+            if (i < n) {
+                const float d0 = v.x - pivot, d1 = v.y - pivot, d2 = v.z - pivot, d3 = v.w - pivot;
+                sum += (d0 + d1) + (d2 + d3);
+                sq += fmaf(d0, d0, d1 * d1) + fmaf(d2, d2, d3 * d3);
+            }
+        }
+    }
+    if (a.out_rec) {
+#pragma unroll
+        for (int d = 1; d < 4; d <<= 1)
+            if (d < 1 << (a.out_shift - 2)) {
+                sum += __shfl_xor_sync(0xffffffffu, sum, d);
+                sq += __shfl_xor_sync(0xffffffffu, sq, d);
+            }
+        if ((cg & ((1 << (a.out_shift - 2)) - 1)) == 0) {
+            const float cnt = (float)(n << a.out_shift), dm = n ? sum / cnt : 0.f;
+            a.out_rec[((size_t)frame * a.out_G + (co >> a.out_shift)) * a.out_slots + block * kThinWarps + pg] =
+                make_float4(cnt, pivot + dm, fmaxf(fmaf(-dm, sum, sq), 0.f), 0.f);
+        }
     }
 }
 
+bool conv_thin_supported(const ConvArgs& a) {
+    return a.in_dtype == VD_F32 && a.out_dtype == VD_F32 && a.ksize == 3 && (a.Cin == 4 || a.Cin == 8) && a.Cout % kThinCout == 0 && !a.scale && !a.silu &&
+           !a.residual && !a.upsample && !a.out_nchw && !a.out_u8 && !a.x2;
+}
+int conv_thin_slots(const ConvArgs& a) { return (a.H * a.W + thin_px(a) * kThinWarps - 1) / (thin_px(a) * kThinWarps) * kThinWarps; }
+
 cudaError_t launch_conv_simt(const ConvArgs& a, cudaStream_t s) {
     const bool ib = a.in_dtype == VD_BF16, ob = a.out_dtype == VD_BF16;
-    if (!ib && !ob && a.ksize == 3 && (a.Cin == 4 || a.Cin == 8) && a.Cout % kThinCout == 0 && !a.scale && !a.residual &&
-        !a.upsample && !a.out_nchw && !a.x2) {
-        const long long npix = (long long)a.B * a.H * a.W;
-        dim3 grid((unsigned)((npix + kThinPix - 1) / kThinPix), a.Cout / kThinCout);
-        return a.Cin == 4 ? launch_pdl(conv_thin_kernel<4>, grid, dim3(256), 0, s, a) : launch_pdl(conv_thin_kernel<8>, grid, dim3(256), 0, s, a);
+    if (conv_thin_supported(a)) {
+        if (a.out_rec && !rec_groups_ok(a.Cout, a.out_G)) return cudaErrorInvalidValue;
+        const long long blocks = (long long)conv_thin_slots(a) / kThinWarps * a.B;
+        if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
+        const dim3 grid((unsigned)blocks, a.Cout / kThinCout);
+        auto launch = [&](auto kern) { return launch_pdl(kern, grid, dim3(256), 0, s, a); };
+        if (thin_px(a) == 2) return a.Cin == 4 ? launch(conv_thin_kernel<4, 2>) : launch(conv_thin_kernel<8, 2>);
+        return a.Cin == 4 ? launch(conv_thin_kernel<4, 8>) : launch(conv_thin_kernel<8, 4>);
     }
     if (ib && ob) return conv_simt_dispatch<__nv_bfloat16, __nv_bfloat16>(a, s);
     if (ib && !ob) return conv_simt_dispatch<__nv_bfloat16, float>(a, s);

@@ -230,7 +230,8 @@ class Planner {
         const bool split = tc && !(cfg_.flags & VD_FLAG_FUSED_STATS) && conv_split_choose(probe, &s.split);
         s.split.valid = split ? 1 : 0;
         bool f32 = false;
-        if (!tc && !(bf16() && (cfg_.flags & VD_FLAG_FORCE_SIMT))) {
+        const bool thin = !tc && conv_thin_supported(probe) && !(bf16() && (cfg_.flags & VD_FLAG_FORCE_SIMT));
+        if (!tc && !thin && !(bf16() && (cfg_.flags & VD_FLAG_FORCE_SIMT))) {
             probe.upsample = upsample ? ((cfg_.flags & VD_FLAG_UPSAMPLE_9TAP) ? 1 : 2) : 0;
             f32 = conv_f32_choose(probe, &s.f32);
             if (f32 && upsample) { phase = true; a.upsample = 2; }
@@ -307,8 +308,8 @@ class Planner {
         ConvArgs whole = a;
         whole.B = cfg_.max_batch;
         const bool tc_rec = tc && !split && !(cfg_.flags & VD_FLAG_FUSED_STATS) && !y_is_frames && conv_tc_records_supported(whole);
-        if ((f32 || split || tc_rec) && records && !y_is_frames && rec_groups_ok(Cout, cfg_.norm_groups)) {
-            const int slots = tc_rec ? conv_tc_slots(a) : split ? conv_split_slots(probe, s.split, cfg_.norm_groups) : conv_f32_slots(probe, s.f32, cfg_.norm_groups);
+        if ((f32 || split || thin || tc_rec) && records && !y_is_frames && rec_groups_ok(Cout, cfg_.norm_groups)) {
+            const int slots = thin ? conv_thin_slots(a) : tc_rec ? conv_tc_slots(a) : split ? conv_split_slots(probe, s.split, cfg_.norm_groups) : conv_f32_slots(probe, s.f32, cfg_.norm_groups);
             rec_toggle_ ^= 1;
             a.out_rec = ptr<float4>(rec_buf_[rec_toggle_]);
             a.out_slots = slots;
@@ -1064,7 +1065,7 @@ vd_status vd_op_conv2d(const vd_conv_desc* d, const void* x, const void* w_packe
         if (e == cudaSuccess) e = launch_conv_tc(a, plan, nullptr, (cudaStream_t)cuda_stream);
     } else {
         ConvF32Plan plan{};
-        if (conv_f32_choose(a, &plan)) {
+        if (!conv_thin_supported(a) && conv_f32_choose(a, &plan)) {
             e = conv_f32_prepare(a, &plan);
             if (e == cudaSuccess) e = launch_conv_f32(a, plan, nullptr, (cudaStream_t)cuda_stream);
         } else {

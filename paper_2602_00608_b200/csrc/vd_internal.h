@@ -113,6 +113,8 @@ void set_last_error(const char* msg);
 cudaError_t launch_ingest(const IngestArgs& a, cudaStream_t s);
 cudaError_t launch_gn_stats(const GnArgs& a, cudaStream_t s);          // one launch (the last block per sample finalises)
 cudaError_t launch_conv_simt(const ConvArgs& a, cudaStream_t s);
+bool conv_thin_supported(const ConvArgs& a);                   // the first convolution has a kernel of its own there
+int conv_thin_slots(const ConvArgs& a);                        // records per group and frame that it leaves
 cudaError_t launch_attn_simt(const AttnArgs& a, cudaStream_t s);
 // OIHW (or [out,in]) weight of dtype `w_dtype` -> fp32 [tap][Cin][Cout]
 // (Cout rows are written at column offset cout_offset of a packed matrix cout_total wide)

@@ -14,6 +14,9 @@ CASES = [
     dict(B=2, H=17, W=9, Cin=36, Cout=96, k=3, upsample=False, prologue=True, silu=True, residual=True),    # part-empty chunk
     dict(B=3, H=33, W=50, Cin=32, Cout=32, k=3, upsample=False, prologue=True, silu=True, residual=True),   # no cluster
     dict(B=1, H=9, W=7, Cin=4, Cout=512, k=3, upsample=False, prologue=False, silu=False, residual=False),
+    dict(B=3, H=33, W=21, Cin=4, Cout=256, k=3, upsample=False, prologue=False, silu=False, residual=False),      # thin: 64-pixel blocks
+    dict(B=2, H=19, W=23, Cin=8, Cout=128, k=3, upsample=False, prologue=False, silu=False, residual=False),      # thin: 32-pixel blocks
+    dict(B=2, H=5, W=13, Cin=8, Cout=128, k=3, upsample=False, prologue=False, silu=False, residual=False),       # thin: 16-pixel blocks
     dict(B=1, H=12, W=10, Cin=512, Cout=96, k=1, upsample=False, prologue=True, silu=False, residual=False),
     dict(B=2, H=21, W=30, Cin=64, Cout=32, k=1, upsample=False, prologue=False, silu=False, residual=True),
     dict(B=1, H=1, W=2, Cin=64, Cout=32, k=3, upsample=2, prologue=False, silu=False, residual=False),
