@@ -13,8 +13,9 @@
 //   * A nearest-2x upsampling 3x3 is four 2x2 convolutions of the source with weights summed in advance (fp32), one per
 //     output parity: 16 instead of 36 products per source pixel.
 // Measured on one B200 (profiled launches, direct kernel -> this one): 512->512 at 8x8 613 -> 31 us, at 16x16 604 -> 48;
-// 32->32 on four 256x256 frames 414 -> 164; frame head 32->3 on a 64x64 frame 29 -> 12.  Whole decodes: tiny layout 64x64
-// 652 -> 152 us, full-width layout 64x64 16.5 -> 1.39 ms.
+// 32->32 on four 256x256 frames 414 -> 142; frame head 32->3 on a 64x64 frame 29 -> 12, on four 256x256 frames (32-pixel tiles)
+// 83 -> 59.  Whole decodes, with the statistics as records: tiny layout 64x64 652 -> 127 us, full-width layout 64x64
+// 16.5 -> 1.25 ms.
 #include <string.h>
 
 #include <algorithm>

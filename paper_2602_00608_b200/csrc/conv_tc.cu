@@ -64,7 +64,7 @@ constexpr int WARP_SLICE_BYTES = 32 * 128;                           // one epil
 // item is two 16x8-pixel tiles whose MMAs consume every weight stage together, which halves the
 // weight traffic through shared memory and the bytes the TMA pipeline must keep in flight.
 //
-// CG = 2 (BN = 256 only): a cluster of two CTAs on neighbouring SMs issues every MMA as one
+// CG = 2 (folded and large layers, see wide_layer; here for BN = 256): a cluster of two CTAs on neighbouring SMs issues every MMA as one
 // tcgen05.mma.cta_group::2 of M = 256 (one tile per CTA) x N = 256.  Each CTA stages only its half of
 // every weight tile (128 rows) and the tensor cores of the pair read both halves, so the weight bytes
 // each SM pulls from L2 are halved; the one-CTA kernel is bound there by that traffic (32 KB per 513
