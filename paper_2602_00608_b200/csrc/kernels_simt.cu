@@ -6,6 +6,7 @@
 #include <mutex>
 #include <string>
 
+#include "conv_cluster.cuh"
 #include "vd_internal.h"
 
 namespace vd {
@@ -247,11 +248,14 @@ __global__ void __launch_bounds__(kGnThreads, 2) gn_stats_kernel(GnArgs a, int c
 // takes 16 channels (one, two or four groups) of one sample, an eighth of its pixels each; the eight sums meet in the first
 // CTA's shared memory, and that CTA writes scale and shift: no records in memory, no arrival counter, no second reading
 // phase.  Sums are of (x - K) with the reference value K of the pass above.
+// The first CTA's shared memory may be written once that CTA runs: every thread arrives on the cluster's barrier at the start
+// and waits for the others before the sums are sent, so the wait lies behind the reads.
 constexpr int kGnSplit = 8;
 template <typename T, int SPG>                       // SPG: four-channel slots per group (1, 2, 4)
 __global__ void __cluster_dims__(kGnSplit, 1, 1) __launch_bounds__(1024 / SPG) gn_cluster_kernel(GnArgs a) {
     constexpr int THREADS = 1024 / SPG, NG = 4 / SPG, ROWS = THREADS / 4, U = 8;
     __shared__ float2 s_warp[THREADS / 32][NG], s_all[NG][kGnSplit];
+    cc::cluster_arrive();
     griddep_launch();
     const int rank = blockIdx.x % kGnSplit, n = blockIdx.y, lane = threadIdx.x & 31;
     const int slot = threadIdx.x & 3, row = threadIdx.x >> 2, c0 = (int)blockIdx.x / kGnSplit * 16, cg = c0 + slot / SPG * (SPG * 4);
@@ -302,16 +306,17 @@ __global__ void __cluster_dims__(kGnSplit, 1, 1) __launch_bounds__(1024 / SPG) g
     }
     if (lane < 4 && lane % SPG == 0) s_warp[threadIdx.x / 32][lane / SPG] = make_float2(s, ss);
     __syncthreads();
+    cc::cluster_wait();                              // every CTA of the cluster runs
     if (threadIdx.x < NG) {
         float2 t = s_warp[0][threadIdx.x];
 #pragma unroll 8
         for (int w = 1; w < THREADS / 32; ++w) { t.x += s_warp[w][threadIdx.x].x; t.y += s_warp[w][threadIdx.x].y; }
-        uint32_t dst;
-        asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(dst) : "r"((uint32_t)__cvta_generic_to_shared(&s_all[threadIdx.x][rank])));
+        const uint32_t dst = cc::peer_addr(tc::smem_u32(&s_all[threadIdx.x][rank]), 0u);
         asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(dst), "f"(t.x), "f"(t.y) : "memory");
     }
     __syncwarp();
-    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    cc::cluster_arrive();
+    cc::cluster_wait();                              // the sums have arrived
     if (rank != 0 || threadIdx.x >= 16) return;
     const int g = threadIdx.x / (SPG * 4), c = c0 + threadIdx.x;
     float2 t = s_all[g][0];

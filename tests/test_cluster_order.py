@@ -1,0 +1,40 @@
+"""A CTA's shared memory may be addressed by another CTA of its cluster only once both are known to run, which a cluster barrier
+guarantees.  A missing wait shows on no run that happens to be slow enough, so the kernels' source is checked: in each kernel a
+cluster wait stands before the first access to another CTA's shared memory."""
+import glob
+import os
+import re
+
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2602_00608_b200", "csrc")
+WAIT = re.compile(r"cluster_wait\(\)|cluster_sync_all\(\)|barrier\.cluster\.wait")
+REMOTE = re.compile(r"st\.shared::cluster|copy_to_peer\(|mbar_arrive(?:_expect_tx)?_cluster\w*\(|commit2?_to_cluster\(|umma2_commit\w*\(")
+
+
+def kernels():
+    """(name, body) of every __global__ function."""
+    for path in sorted(glob.glob(os.path.join(CSRC, "*.cu"))):
+        text = re.sub(r"//[^\n]*", "", open(path).read())
+        for m in re.finditer(r"__global__", text):
+            open_at = text.index("{", m.end())
+            depth, i = 1, open_at + 1
+            while depth:
+                depth += {"{": 1, "}": -1}.get(text[i], 0)
+                i += 1
+            name = re.search(r"(\w+)\s*\((?!\()[^()]*\)\s*$|(\w+)\s*\(const", text[m.end():open_at])
+            yield os.path.basename(path), name.group(1) or name.group(2), text[open_at:i]
+
+
+WITH_REMOTE = [(f, n, b) for f, n, b in kernels() if REMOTE.search(b)]
+
+
+def test_the_cluster_kernels_are_found():
+    names = {n for _, n, _ in WITH_REMOTE}
+    assert {"gn_cluster_kernel", "conv_split_kernel", "conv_pair_kernel", "conv_f32_kernel", "conv_tc_kernel"} <= names, names
+
+
+@pytest.mark.parametrize("file,name,body", WITH_REMOTE, ids=[n for _, n, _ in WITH_REMOTE])
+def test_a_cluster_wait_precedes_remote_shared_memory(file, name, body):
+    wait, remote = WAIT.search(body), REMOTE.search(body)
+    assert wait and wait.start() < remote.start(), f"{file}: {name} reaches another CTA before it is known to run"

@@ -35,3 +35,12 @@ def test_gn_stats_of_a_small_sample_with_an_offset_and_in_a_batch(env):       # 
     assert torch.equal(sc[2:3], one[0]) and torch.equal(sh[2:3], one[1])
     got = x * sc.cpu().numpy()[:, :, None, None] + sh.cpu().numpy()[:, :, None, None]
     assert util.rel_l2(got, want) <= 2e-5       # scale x ~ 40: 2^-24 x 40 per element before the shift takes it off
+
+
+@pytest.mark.parametrize("P", [1, 3, 7])
+@pytest.mark.parametrize("C,G,bf16", [(128, 32, True), (256, 32, False), (512, 32, True)])
+def test_gn_stats_of_fewer_pixels_than_ctas(env, P, C, G, bf16):    # noqa: F811
+    """CTAs of the cluster without a pixel send their (zero) sums at once: nothing to read hides the wait for the first CTA."""
+    sc, sh, wsc, wsh = _gn_case(env, 41, 3, 1, P, C, G, bf16)
+    np.testing.assert_allclose(sc, wsc, rtol=2e-5)
+    np.testing.assert_allclose(sh, wsh, rtol=2e-5, atol=2e-5)
