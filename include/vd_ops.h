@@ -114,10 +114,22 @@ VD_API vd_status vd_conv_pack_weight(const vd_conv_desc* d, const void* w_oihw, 
  *   x        device NHWC [batch,in_h,in_w,c_in], in_dtype
  *   scale, shift   device fp32 [batch,c_in] or both NULL (no prologue); act = SiLU if d->silu
  *   bias     device fp32 [c_out] or NULL;  residual  device fp32 NHWC like y, or NULL
- *   y        device, out_dtype, NHWC (or NCHW if out_nchw) at the output resolution */
+ *   y        device, out_dtype, NHWC (or NCHW if out_nchw) at the output resolution
+ * The tensor-core kernel and the phase-collapsed form need x, w_packed, bias, residual and y at 16-byte boundaries; other
+ * fp32 layers take tensors at any boundary of their elements (on the direct kernel where one is not 16-byte aligned). */
 VD_API vd_status vd_op_conv2d(const vd_conv_desc* d, const void* x, const void* w_packed, const float* bias,
                               const float* scale, const float* shift, const float* residual, void* y,
                               void* cuda_stream);
+
+/* The kernel that vd_op_conv2d launches for these arguments (host-only; no pointer is followed). */
+typedef enum {
+    VD_ROUTE_DIRECT = 0,        /* tiled FFMA kernel, scalar accesses */
+    VD_ROUTE_THIN = 1,          /* first convolution (4 or 8 input channels), FFMA */
+    VD_ROUTE_F32 = 2,           /* register-tiled FFMA kernel, 16-byte accesses, K divided among a cluster */
+    VD_ROUTE_TC = 3             /* tcgen05 kernel */
+} vd_conv_route_kind;
+VD_API vd_status vd_conv_route(const vd_conv_desc* d, const void* x, const void* w_packed, const float* bias, const float* scale,
+                               const float* residual, const void* y, int32_t* route);
 
 /* vd_op_conv2d and, from the same launch, the statistics of GroupNorm(y) folded with the affine parameters
  * (Section IV-B.1: the normalisation's reduction is taken while the tile is on chip):

@@ -20,6 +20,7 @@ VD_FLAG_OUT_U8 = 0x4
 VD_FLAG_CANARY = 0x8
 VD_FLAG_FUSED_STATS = 0x10
 VD_IMPL_AUTO, VD_IMPL_SIMT, VD_IMPL_TC = 0, 1, 2
+VD_ROUTE_DIRECT, VD_ROUTE_THIN, VD_ROUTE_F32, VD_ROUTE_TC = 0, 1, 2, 3
 VD_STEP_INGEST, VD_STEP_GN_STATS, VD_STEP_CONV, VD_STEP_ATTENTION = 0, 1, 2, 3
 STATUS_NAMES = {0: "VD_OK", -1: "VD_ERR_INVALID_ARG", -2: "VD_ERR_UNSUPPORTED", -3: "VD_ERR_WORKSPACE",
                 -4: "VD_ERR_CUDA", -5: "VD_ERR_DEVICE_TIMEOUT"}
@@ -27,7 +28,7 @@ STATUS_NAMES = {0: "VD_OK", -1: "VD_ERR_INVALID_ARG", -2: "VD_ERR_UNSUPPORTED", 
 EXPORTED = [
     "vd_query_workspace", "vd_create", "vd_decode", "vd_decode_extrapolated", "vd_decode_host", "vd_get_status",
     "vd_last_error", "vd_destroy", "vd_num_steps", "vd_get_step", "vd_profile", "vd_debug_stop_after",
-    "vd_conv_packed_weight_bytes", "vd_conv_pack_weight", "vd_op_conv2d", "vd_conv_stats_scratch_bytes", "vd_op_conv2d_stats", "vd_gn_scratch_bytes", "vd_op_gn_stats",
+    "vd_conv_packed_weight_bytes", "vd_conv_pack_weight", "vd_op_conv2d", "vd_conv_route", "vd_conv_stats_scratch_bytes", "vd_op_conv2d_stats", "vd_gn_scratch_bytes", "vd_op_gn_stats",
     "vd_op_attention", "vd_attention_scratch_bytes", "vd_op_gn_stats_static", "vd_clear_status", "vd_decode_host_stream", "vd_debug_check_canaries", "vd_debug_status_offset", "vd_debug_wait_probe",
 ]
 
@@ -97,6 +98,7 @@ def lib():
         l.vd_conv_packed_weight_bytes.argtypes = [POINTER(VdConvDesc), POINTER(c_size_t)]
         l.vd_conv_pack_weight.argtypes = [POINTER(VdConvDesc), vp, c_int32, vp, vp]
         l.vd_op_conv2d.argtypes = [POINTER(VdConvDesc), vp, vp, vp, vp, vp, vp, vp, vp]
+        l.vd_conv_route.argtypes = [POINTER(VdConvDesc), vp, vp, vp, vp, vp, vp, POINTER(c_int32)]
         l.vd_conv_stats_scratch_bytes.argtypes = [c_int32, c_int32]
         l.vd_conv_stats_scratch_bytes.restype = c_size_t
         l.vd_op_conv2d_stats.argtypes = [POINTER(VdConvDesc), vp, vp, vp, vp, vp, vp, c_int32, c_float, vp, vp, vp, vp, vp, vp]
@@ -333,6 +335,13 @@ def op_conv2d(x_nhwc, w_oihw, bias=None, scale=None, shift=None, residual=None, 
         assert t is None or (t.dtype == torch.float32 and t.is_contiguous())
     _check(lib().vd_op_conv2d(byref(d), p(x_nhwc.contiguous()), p(packed), p(bias), p(scale), p(shift), p(residual), p(y), _stream_ptr()))
     return y
+
+
+def conv_route(desc: VdConvDesc, x=256, w=256, bias=0, scale=0, residual=0, y=256) -> int:
+    """The kernel vd_op_conv2d takes for a descriptor and tensors at these addresses (which are not followed)."""
+    r = c_int32(-1)
+    _check(lib().vd_conv_route(byref(desc), c_void_p(x), c_void_p(w), c_void_p(bias), c_void_p(scale), c_void_p(residual), c_void_p(y), byref(r)))
+    return int(r.value)
 
 
 def op_conv2d_stats(x_nhwc, w_oihw, gamma, beta, groups: int, eps: float, bias=None, scale=None, shift=None, *,

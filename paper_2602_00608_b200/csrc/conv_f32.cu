@@ -404,8 +404,12 @@ int kind_of(const ConvArgs& a) { return a.upsample == 2 ? KPHASE : (a.ksize == 1
 
 }  // namespace
 
+// The input is read as float4, and outside the frame head so are bias and residual, and the output is written so; the
+// weights come by bulk tensor loads.  Layers whose tensors are not aligned for that stay on the direct kernel.
 bool conv_f32_supported(const ConvArgs& a) {
     if (a.in_dtype != VD_F32 || (a.ksize != 1 && a.ksize != 3) || a.Cin % 4 != 0 || a.x2 || a.upsample == 1) return false;
+    if (!aligned16(a.x)) return false;
+    if (a.Cout % 32 == 0 && !(aligned16(a.w) && aligned16(a.bias) && aligned16(a.residual) && aligned16(a.y))) return false;
     if (a.upsample == 2) return a.ksize == 3 && a.Cout % 32 == 0 && !a.out_nchw && !a.out_u8 && a.out_dtype == VD_F32;
     if (a.Cout % 32 == 0) return !a.out_nchw && !a.out_u8 && a.out_dtype == VD_F32;
     // the frame head: its slice of the weights stays in shared memory

@@ -814,7 +814,8 @@ __global__ void __launch_bounds__(256, 2) conv_thin_kernel(ConvArgs a) {
 
 bool conv_thin_supported(const ConvArgs& a) {
     return a.in_dtype == VD_F32 && a.out_dtype == VD_F32 && a.ksize == 3 && (a.Cin == 4 || a.Cin == 8) && a.Cout % kThinCout == 0 && !a.scale && !a.silu &&
-           !a.residual && !a.upsample && !a.out_nchw && !a.out_u8 && !a.x2;
+           !a.residual && !a.upsample && !a.out_nchw && !a.out_u8 && !a.x2 &&
+           aligned16(a.x) && aligned16(a.w) && aligned16(a.bias) && aligned16(a.y);      // all read and written as float4
 }
 int conv_thin_slots(const ConvArgs& a) { return (a.H * a.W + thin_px(a) * kThinWarps - 1) / (thin_px(a) * kThinWarps) * kThinWarps; }
 

@@ -1007,8 +1007,14 @@ static vd_status resolve_impl(const vd_conv_desc* d, const ConvArgs& a, bool* tc
     const bool can = a.bf16_operands && conv_tc_supported(probe);
     if (d->impl == VD_IMPL_TC && !can) return fail(nullptr, VD_ERR_UNSUPPORTED, "the tensor-core convolution does not support this shape");
     *tc = d->impl == VD_IMPL_TC || (d->impl == VD_IMPL_AUTO && can);
-    if (!*tc && a.upsample == 2 && !conv_f32_supported(a)) return fail(nullptr, VD_ERR_UNSUPPORTED, "this layer has no phase-collapsed upsampling form");
+    if (!*tc && a.upsample == 2 && !conv_f32_supported(a)) return fail(nullptr, VD_ERR_UNSUPPORTED, "this layer has no phase-collapsed upsampling form, or its tensors are not 16-byte aligned");
     return VD_OK;
+}
+
+// the kernel of a layer that is not the tensor-core kernel's
+static vd_conv_route_kind ffma_route(const ConvArgs& a, ConvF32Plan* plan) {
+    if (conv_thin_supported(a)) return VD_ROUTE_THIN;
+    return conv_f32_choose(a, plan) ? VD_ROUTE_F32 : VD_ROUTE_DIRECT;
 }
 
 vd_status vd_conv_packed_weight_bytes(const vd_conv_desc* d, size_t* bytes) {
@@ -1065,7 +1071,7 @@ vd_status vd_op_conv2d(const vd_conv_desc* d, const void* x, const void* w_packe
         if (e == cudaSuccess) e = launch_conv_tc(a, plan, nullptr, (cudaStream_t)cuda_stream);
     } else {
         ConvF32Plan plan{};
-        if (!conv_thin_supported(a) && conv_f32_choose(a, &plan)) {
+        if (ffma_route(a, &plan) == VD_ROUTE_F32) {
             e = conv_f32_prepare(a, &plan);
             if (e == cudaSuccess) e = launch_conv_f32(a, plan, nullptr, (cudaStream_t)cuda_stream);
         } else {
@@ -1073,6 +1079,21 @@ vd_status vd_op_conv2d(const vd_conv_desc* d, const void* x, const void* w_packe
         }
     }
     return e == cudaSuccess ? VD_OK : cuda_fail(nullptr, e, "vd_op_conv2d");
+}
+
+vd_status vd_conv_route(const vd_conv_desc* d, const void* x, const void* w_packed, const float* bias, const float* scale,
+                        const float* residual, const void* y, int32_t* route) {
+    vd_status st = check_conv_desc(d);
+    if (st != VD_OK) return st;
+    if (!route) return fail(nullptr, VD_ERR_INVALID_ARG, "route is NULL");
+    ConvArgs a = conv_args_from_desc(d);
+    a.x = x; a.w = w_packed; a.bias = bias; a.scale = scale; a.shift = scale; a.residual = residual; a.y = const_cast<void*>(y);
+    bool tc;
+    st = resolve_impl(d, a, &tc);
+    if (st != VD_OK) return st;
+    ConvF32Plan plan{};
+    *route = tc ? VD_ROUTE_TC : ffma_route(a, &plan);
+    return VD_OK;
 }
 
 size_t vd_conv_stats_scratch_bytes(int32_t batch, int32_t groups) {

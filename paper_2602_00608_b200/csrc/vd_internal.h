@@ -109,6 +109,8 @@ cudaError_t launch_wait_probe(unsigned int* status_word, long long limit_cycles,
 // records `msg` as the text vd_last_error(NULL) returns (defined in vd_api.cu)
 void set_last_error(const char* msg);
 
+inline bool aligned16(const void* p) { return ((uintptr_t)p & 15) == 0; }
+
 // ---- FFMA kernels (kernels_simt.cu)
 cudaError_t launch_ingest(const IngestArgs& a, cudaStream_t s);
 cudaError_t launch_gn_stats(const GnArgs& a, cudaStream_t s);          // one launch (the last block per sample finalises)

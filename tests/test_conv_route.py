@@ -1,0 +1,72 @@
+"""Which kernel a single fp32 convolution takes, on the host: the kernels that read and write 16 bytes at a time must not be
+given tensors that lie elsewhere (a misaligned access ends the CUDA context); those stay on the direct kernel."""
+import pytest
+
+from paper_2602_00608_b200 import binding as vd
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    from paper_2602_00608_b200 import build
+    build.build()
+
+
+def desc(cin, cout, k=3, upsample=0, nchw=False, impl=vd.VD_IMPL_SIMT, h=12, w=10, b=1):
+    return vd.conv_desc(b, h, w, cin, cout, k, upsample, False, vd.VD_F32, vd.VD_F32, nchw, False, impl)
+
+
+LAYERS = {                     # descriptor, its kernel, the tensors that this kernel takes in 16-byte pieces
+    "f32": (desc(64, 32), vd.VD_ROUTE_F32, {"x", "w", "bias", "residual", "y"}),
+    "1x1": (desc(36, 96, 1), vd.VD_ROUTE_F32, {"x", "w", "bias", "residual", "y"}),
+    "head": (desc(64, 3, nchw=True), vd.VD_ROUTE_F32, {"x"}),
+    "thin": (desc(4, 256), vd.VD_ROUTE_THIN, {"x", "w", "bias", "y"}),
+    "thin8": (desc(8, 128), vd.VD_ROUTE_THIN, {"x", "w", "bias", "y"}),
+}
+
+
+@pytest.mark.parametrize("impl", [vd.VD_IMPL_SIMT, vd.VD_IMPL_AUTO])
+@pytest.mark.parametrize("name", LAYERS)
+def test_misaligned_tensors_take_the_direct_kernel(name, impl):
+    d, kernel, vector = LAYERS[name]
+    d.impl = impl
+    aligned = {"x": 1 << 20, "w": 2 << 20, "bias": 3 << 20, "y": 5 << 20}
+    if "residual" in vector:
+        aligned["residual"] = 4 << 20
+    assert vd.conv_route(d, **aligned) == kernel
+    for t in aligned:
+        for off in (4, 8, 12):
+            want = vd.VD_ROUTE_DIRECT if t in vector else kernel
+            assert vd.conv_route(d, **{**aligned, t: aligned[t] + off}) == want, (t, off)
+
+
+def test_phase_collapsed_layers_of_misaligned_tensors_are_refused():
+    d = desc(32, 32, upsample=2)
+    assert vd.conv_route(d) == vd.VD_ROUTE_F32
+    for t in ("x", "w", "y", "bias"):
+        with pytest.raises(vd.VdError) as e:
+            vd.conv_route(d, **{t: 1028})
+        assert e.value.status == vd.VD_ERR_UNSUPPORTED and "aligned" in str(e.value)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("cin,cout,k,nchw,moved", [
+    (36, 64, 3, False, "x"), (36, 64, 3, False, "bias"), (36, 64, 3, False, "residual"), (64, 96, 1, False, "x"),
+    (64, 96, 1, False, "bias"), (32, 3, 3, True, "x"), (32, 3, 3, True, "bias"), (4, 128, 3, False, "x"), (4, 128, 3, False, "bias")])
+def test_views_into_larger_buffers_give_the_same_result(cin, cout, k, nchw, moved):
+    import torch
+    g = torch.Generator(device="cuda").manual_seed(7)
+    B, H, W = 2, 9, 13
+
+    def tensor(name, *shape):
+        flat = torch.randn(int(torch.tensor(shape).prod()) + 1, device="cuda", generator=g)
+        return flat[1:].view(shape) if name == moved else flat[:-1].view(shape).clone()
+    x, bias, w = tensor("x", B, H, W, cin), tensor("bias", cout), torch.randn(cout, cin, k, k, device="cuda", generator=g)
+    res = tensor("residual", B, H, W, cout) if moved == "residual" else None
+    got = vd.op_conv2d(x, w, bias, residual=res, out_nchw=nchw, impl=vd.VD_IMPL_SIMT)
+    want = torch.nn.functional.conv2d(x.permute(0, 3, 1, 2).double(), w.double(), bias.double(), padding=k // 2)
+    if not nchw:
+        want = want.permute(0, 2, 3, 1)
+    if res is not None:
+        want = want + res.double()
+    # fp32 sums of at most 324 products in sequence: 2^-24 / sqrt(3) * sqrt(324 / 2)
+    assert float((got.double() - want).norm() / want.norm()) <= 1e-6
