@@ -78,7 +78,7 @@ template <int TH, int BN, int KIND, int TW = 8> struct FCfg {
     static constexpr int PART_FLOATS = KT / 2 * RX_FLOATS;               // partials of half the K groups at a time
     static_assert(KT >= 2 && kThreads % (TH * NG * (BN / 4)) == 0 && CS % 4 == 0, "thread layout");
 };
-constexpr int kMaxSlice = 512;                               // input channels of one CTA
+constexpr int kMaxSlice = 512, kMaxSplits = 8;               // input channels of one CTA; CTAs of a cluster
 constexpr int kFTail = 2 * kMaxSlice * 4 + 128;              // scale / shift of the slice, barriers
 
 // A partial lies in memory as rows (pixels) of BN floats whose 16-byte pieces are permuted by the row, so that neither the
@@ -405,10 +405,14 @@ int kind_of(const ConvArgs& a) { return a.upsample == 2 ? KPHASE : (a.ksize == 1
 }  // namespace
 
 // The input is read as float4, and outside the frame head so are bias and residual, and the output is written so; the
-// weights come by bulk tensor loads.  Layers whose tensors are not aligned for that stay on the direct kernel.
+// weights come by bulk tensor loads.  Layers whose tensors are not aligned for that stay on the direct kernel, and so do
+// inputs of more channels than a cluster's slices hold and frames whose pixels or four-channel pieces the kernel's 32-bit
+// indices do not reach.  What is supported here has a plan (conv_f32_choose).
 bool conv_f32_supported(const ConvArgs& a) {
     if (a.in_dtype != VD_F32 || (a.ksize != 1 && a.ksize != 3) || a.Cin % 4 != 0 || a.x2 || a.upsample == 1) return false;
-    if (!aligned16(a.x)) return false;
+    if (!aligned16(a.x) || a.Cin > kMaxSplits * kMaxSlice) return false;
+    const long long pixels = (long long)a.Hs * a.Ws;
+    if (pixels > 0x7fffffffLL || pixels * (a.Cin / 4) > 0xffffffffLL) return false;
     if (a.Cout % 32 == 0 && !(aligned16(a.w) && aligned16(a.bias) && aligned16(a.residual) && aligned16(a.y))) return false;
     if (a.upsample == 2) return a.ksize == 3 && a.Cout % 32 == 0 && !a.out_nchw && !a.out_u8 && a.out_dtype == VD_F32;
     if (a.Cout % 32 == 0) return !a.out_nchw && !a.out_u8 && a.out_dtype == VD_F32;
@@ -434,9 +438,8 @@ bool conv_f32_choose(const ConvArgs& a, ConvF32Plan* p) {
     const int tiles = ((W + p->tw - 1) / p->tw) * ((H + p->th - 1) / p->th), chunks = (a.Cin + kChunk - 1) / kChunk;
     const long long ctas = (long long)tiles * (head ? 1 : a.Cout / 32) * (kind == KPHASE ? 4 : 1) * std::max(a.B, 1);
     int s = 1;
-    while (s < 8 && 2 * s <= chunks && ctas * 2 * s <= 296) s *= 2;
+    while (s < kMaxSplits && 2 * s <= chunks && ctas * 2 * s <= 296) s *= 2;
     while ((chunks + s - 1) / s * kChunk > (head ? 128 : kMaxSlice)) s *= 2;
-    if (s > 8) return false;
     p->splits = s;
     const int units = (chunks + s - 1) / s;
     auto fit = [&](int base, int stage) { return std::min(std::min(units, kMaxW), (kSplitSmemMax - base) / stage); };

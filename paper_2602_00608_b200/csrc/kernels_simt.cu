@@ -821,6 +821,7 @@ int conv_thin_slots(const ConvArgs& a) { return (a.H * a.W + thin_px(a) * kThinW
 
 cudaError_t launch_conv_simt(const ConvArgs& a, cudaStream_t s) {
     const bool ib = a.in_dtype == VD_BF16, ob = a.out_dtype == VD_BF16;
+    if (a.upsample == 2) return cudaErrorInvalidValue;       // its weights are packed as sixteen 2x2 taps, which these kernels do not read
     if (conv_thin_supported(a)) {
         if (a.out_rec && !rec_groups_ok(a.Cout, a.out_G)) return cudaErrorInvalidValue;
         const long long blocks = (long long)conv_thin_slots(a) / kThinWarps * a.B;

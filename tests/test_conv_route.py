@@ -1,5 +1,7 @@
 """Which kernel a single fp32 convolution takes, on the host: the kernels that read and write 16 bytes at a time must not be
 given tensors that lie elsewhere (a misaligned access ends the CUDA context); those stay on the direct kernel."""
+import ctypes
+
 import pytest
 
 from paper_2602_00608_b200 import binding as vd
@@ -46,6 +48,26 @@ def test_phase_collapsed_layers_of_misaligned_tensors_are_refused():
         with pytest.raises(vd.VdError) as e:
             vd.conv_route(d, **{t: 1028})
         assert e.value.status == vd.VD_ERR_UNSUPPORTED and "aligned" in str(e.value)
+
+
+def test_phase_collapsed_layers_beyond_the_kernel_are_refused():
+    """No other FFMA kernel reads weights packed as sixteen 2x2 taps: what the kernel cannot plan must not be accepted."""
+    assert vd.conv_route(desc(4096, 32, upsample=2)) == vd.VD_ROUTE_F32
+    for d in (desc(4100, 32, upsample=2), desc(64, 32, upsample=2, h=32768, w=32768), desc(4, 32, upsample=2, h=65536, w=32768)):
+        with pytest.raises(vd.VdError) as e:
+            vd.conv_route(d)
+        assert e.value.status == vd.VD_ERR_UNSUPPORTED
+        n = ctypes.c_size_t()
+        assert vd.lib().vd_conv_packed_weight_bytes(ctypes.byref(d), ctypes.byref(n)) == vd.VD_ERR_UNSUPPORTED
+
+
+def test_layers_beyond_the_kernels_indices_take_the_direct_kernel():
+    assert vd.conv_route(desc(4096, 64)) == vd.VD_ROUTE_F32 and vd.conv_route(desc(4100, 64)) == vd.VD_ROUTE_DIRECT
+    # 2^32 - 1 pieces of four channels and 2^31 - 1 pixels of a frame are the last ones
+    assert vd.conv_route(desc(64, 32, h=16384, w=16383)) == vd.VD_ROUTE_F32
+    assert vd.conv_route(desc(64, 32, h=16384, w=16384)) == vd.VD_ROUTE_DIRECT
+    assert vd.conv_route(desc(4, 32, h=65536, w=32767)) == vd.VD_ROUTE_F32
+    assert vd.conv_route(desc(4, 32, h=65536, w=32768)) == vd.VD_ROUTE_DIRECT
 
 
 @pytest.mark.gpu
