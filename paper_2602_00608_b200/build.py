@@ -27,7 +27,7 @@ def _newer(target: str, deps) -> bool:
 def build(verbose: bool = False, force: bool = False) -> str:
     os.makedirs(OBJ, exist_ok=True)
     headers = [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith((".h", ".cuh"))]
-    headers.append(os.path.join(ROOT, "include", "vd.h"))
+    headers += [os.path.join(ROOT, "include", f) for f in ("vd.h", "vd_ops.h")]
     nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
 
     def compile_one(src: str) -> str:

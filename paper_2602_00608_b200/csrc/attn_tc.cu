@@ -11,7 +11,6 @@
 // core works on the next tile's scores while the softmax warps are busy.  The N x N score
 // matrix never exists in memory.  Every wait is bounded (see tc_common.cuh).
 #include <mutex>
-#include <cuda.h>
 
 #include "tc_common.cuh"
 #include "vd_internal.h"
@@ -321,23 +320,9 @@ __global__ void transpose_v_kernel(const __nv_bfloat16* v, __nv_bfloat16* vt, in
     }
 }
 
-typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
-                                  const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
-                                  CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-EncodeTiledFn get_encode_fn() {
-    static EncodeTiledFn fn = nullptr;
-    if (!fn) {
-        void* p = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &q) == cudaSuccess && q == cudaDriverEntryPointSuccess)
-            fn = (EncodeTiledFn)p;
-    }
-    return fn;
-}
-
 bool encode_2d(CUtensorMap* tm, const void* base, uint64_t cols, uint64_t rows, uint64_t row_stride_bytes, uint32_t box_cols,
                uint32_t box_rows) {
-    EncodeTiledFn enc = get_encode_fn();
+    EncodeTiledFn enc = encode_fn();
     if (!enc) return false;
     const cuuint64_t dims[2] = {cols, rows};
     const cuuint64_t strides[1] = {row_stride_bytes};

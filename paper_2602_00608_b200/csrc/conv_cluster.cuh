@@ -11,11 +11,13 @@
 //     channels (Chan's formula, a fixed order), or a small launch does where there are many.  The normalisation then
 //     costs neither a read of the tensor nor, mostly, a launch.
 #pragma once
-#include <cuda.h>
 #include <cuda_bf16.h>
 #include <stdint.h>
 
+#include <mutex>
+
 #include "tc_common.cuh"
+#include "tc_pair.cuh"
 #include "vd_internal.h"
 
 namespace vd {
@@ -23,16 +25,6 @@ namespace cc {
 
 constexpr int kFinishThreads = 256;                          // eight warps add up and write the rows
 
-__device__ __forceinline__ uint32_t ctarank() {
-    uint32_t r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-__device__ __forceinline__ uint32_t peer_addr(uint32_t smem_addr, uint32_t cta) {
-    uint32_t r;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_addr), "r"(cta));
-    return r;
-}
 // `bytes` (a multiple of 16) from this CTA's shared memory into another CTA's (cluster addresses); their arrival is
 // counted on that CTA's barrier `bar`
 __device__ __forceinline__ void copy_to_peer(uint32_t dst, uint32_t src, uint32_t bytes, uint32_t bar) {
@@ -264,17 +256,42 @@ __device__ __forceinline__ void finish_rows(const ConvArgs& a, Source source, in
     }
 }
 
-typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
-                                  const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
-                                  CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-inline EncodeTiledFn encode_fn() {
-    static EncodeTiledFn fn = [] {
-        void* p = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        return cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &q) == cudaSuccess && q == cudaDriverEntryPointSuccess
-                   ? (EncodeTiledFn)p : (EncodeTiledFn) nullptr;
-    }();
-    return fn;
+// ---- launches of kernels that run as clusters
+// `smem_max`: the kernel's shared-memory limit, set once per device.
+constexpr int kMaxDevices = 64;
+template <auto KERNEL> cudaError_t set_smem_limit(int smem_max) {
+    static std::mutex mu;
+    static bool done[kMaxDevices] = {};
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
+    std::lock_guard<std::mutex> lock(mu);
+    if (!done[dev]) {
+        e = cudaFuncSetAttribute(KERNEL, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max);
+        if (e != cudaSuccess) return e;
+        done[dev] = true;
+    }
+    return cudaSuccess;
+}
+struct ClusterShape { long long ctas; int threads, smem, smem_max, cluster; };
+template <auto KERNEL, class... Args> cudaError_t launch_clusters(const ClusterShape& c, cudaStream_t s, Args&&... args) {
+    cudaError_t e = set_smem_limit<KERNEL>(c.smem_max);
+    if (e != cudaSuccess) return e;
+    if (c.ctas > 0x7fffffffLL) return cudaErrorInvalidValue;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)c.ctas);
+    cfg.blockDim = dim3((unsigned)c.threads);
+    cfg.dynamicSmemBytes = (size_t)c.smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)c.cluster; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = pdl_enabled() ? 2 : 1;
+    return cudaLaunchKernelEx(&cfg, KERNEL, std::forward<Args>(args)...);
 }
 
 }  // namespace cc

@@ -19,7 +19,6 @@
 #include <string.h>
 
 #include <algorithm>
-#include <mutex>
 
 #include "conv_cluster.cuh"
 
@@ -104,7 +103,7 @@ conv_f32_kernel(const ConvArgs a, const int S, const int n_w, const int ops_floa
     volatile uint32_t* abort_flag = &bars->abort_flag;
 
     const int tid = threadIdx.x, lane = tid & 31;
-    const int rank = S > 1 ? (int)ctarank() : 0;
+    const int rank = S > 1 ? (int)cluster_ctarank() : 0;
     const int H = KIND == KPHASE ? a.Hs : a.H, W = KIND == KPHASE ? a.Ws : a.W;      // the tile grid is that of the source
     const int tiles_x = (W + TW - 1) / TW, tiles = tiles_x * ((H + TH - 1) / TH);
     const int nblk = HEAD ? 1 : a.Cout / BN;
@@ -293,8 +292,8 @@ conv_f32_kernel(const ConvArgs a, const int S, const int n_w, const int ops_floa
         __syncthreads();
         cluster_wait();
         if (tid < S)
-            copy_to_peer(peer_addr(smem_u32(rx + rank * rpo * BN), (uint32_t)tid), smem_u32(part + tid * rpo * BN), (uint32_t)(rpo * BN * 4),
-                         peer_addr(smem_u32(&bars->rx_full), (uint32_t)tid));
+            copy_to_peer(map_to_cta(smem_u32(rx + rank * rpo * BN), (uint32_t)tid), smem_u32(part + tid * rpo * BN), (uint32_t)(rpo * BN * 4),
+                         map_to_cta(smem_u32(&bars->rx_full), (uint32_t)tid));
         __syncwarp();
     } else {
         rx = part;
@@ -347,9 +346,6 @@ __global__ void pack_weight_f32_phase_kernel(const T* w, float* packed, int Cout
     }
 }
 
-constexpr int kMaxDevices = 64;
-std::mutex g_mu;
-
 template <int TH, int BN, int KIND, int TW = 8>
 int ops_floats(int n_w) {                                    // operand stages; the partials lie over them
     using C = FCfg<TH, BN, KIND, TW>;
@@ -363,41 +359,10 @@ int smem_bytes(int n_w, int splits) {
 
 template <int TH, int BN, int KIND, int TW = 8>
 cudaError_t launch_one(const ConvArgs& a, const ConvF32Plan& p, unsigned int* status, cudaStream_t s) {
-    auto kern = conv_f32_kernel<TH, BN, KIND, TW>;
-    static bool configured[kMaxDevices] = {};
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
-    {
-        std::lock_guard<std::mutex> lock(g_mu);
-        if (!configured[dev]) {
-            e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSplitSmemMax);
-            if (e != cudaSuccess) return e;
-            configured[dev] = true;
-        }
-    }
     const int H = KIND == KPHASE ? a.Hs : a.H, W = KIND == KPHASE ? a.Ws : a.W;
-    const long long grid = (long long)((W + TW - 1) / TW) * ((H + TH - 1) / TH) * (BN < 32 ? 1 : a.Cout / BN) * (KIND == KPHASE ? 4 : 1) * a.B * p.splits;
-    if (grid > 0x7fffffffLL) return cudaErrorInvalidValue;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)grid);
-    cfg.blockDim = dim3(kThreads);
-    cfg.dynamicSmemBytes = (size_t)smem_bytes<TH, BN, KIND, TW>(p.n_w, p.splits);
-    cfg.stream = s;
-    cudaLaunchAttribute attr[2];
-    int na = 0;
-    attr[na].id = cudaLaunchAttributeClusterDimension;
-    attr[na].val.clusterDim.x = (unsigned)p.splits; attr[na].val.clusterDim.y = 1; attr[na].val.clusterDim.z = 1;
-    ++na;
-    if (pdl_enabled()) {
-        attr[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[na].val.programmaticStreamSerializationAllowed = 1;
-        ++na;
-    }
-    cfg.attrs = attr;
-    cfg.numAttrs = na;
-    return cudaLaunchKernelEx(&cfg, kern, a, p.splits, p.n_w, ops_floats<TH, BN, KIND, TW>(p.n_w), *(const CUtensorMap*)p.tmap, status);
+    const long long ctas = (long long)((W + TW - 1) / TW) * ((H + TH - 1) / TH) * (BN < 32 ? 1 : a.Cout / BN) * (KIND == KPHASE ? 4 : 1) * a.B * p.splits;
+    return launch_clusters<conv_f32_kernel<TH, BN, KIND, TW>>({ctas, kThreads, smem_bytes<TH, BN, KIND, TW>(p.n_w, p.splits), kSplitSmemMax, p.splits}, s,
+                                                              a, p.splits, p.n_w, ops_floats<TH, BN, KIND, TW>(p.n_w), *(const CUtensorMap*)p.tmap, status);
 }
 
 int kind_of(const ConvArgs& a) { return a.upsample == 2 ? KPHASE : (a.ksize == 1 ? K1X1 : K3X3); }

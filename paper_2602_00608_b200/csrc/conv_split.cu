@@ -17,7 +17,6 @@
 #include <string.h>
 
 #include <algorithm>
-#include <mutex>
 
 #include "conv_cluster.cuh"
 #include "conv_tile.cuh"
@@ -169,7 +168,7 @@ conv_split_kernel(const ConvArgs a, const ConvSplitShape sh, const __grid_consta
     volatile uint32_t* abort_flag = &bars->abort_flag;
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int rank = (int)ctarank();
+    const int rank = (int)cluster_ctarank();
 
     // ---- this cluster's item: (frame, tile, output parity, channel block); for KPHASE the tile grid is that of the source
     const int H = KIND == KPHASE ? a.Hs : a.H, W = KIND == KPHASE ? a.Ws : a.W;
@@ -369,8 +368,8 @@ conv_split_kernel(const ConvArgs a, const ConvSplitShape sh, const __grid_consta
                 __syncwarp();
                 const int n_log2 = min(rpo_log2, 5), n = 1 << n_log2, R = R0 + lane * n, owner = R >> rpo_log2;
                 if (moves && lane < 32 >> n_log2)
-                    copy_to_peer(peer_addr(smem_u32(rx + ((rank * NB + cb) * rpo + R - owner * rpo) * CB), (uint32_t)owner), smem_u32(part + (cb * ROWS + R) * CB),
-                                 (uint32_t)(n * CB * 4), peer_addr(smem_u32(&bars->rx_full), (uint32_t)owner));
+                    copy_to_peer(map_to_cta(smem_u32(rx + ((rank * NB + cb) * rpo + R - owner * rpo) * CB), (uint32_t)owner), smem_u32(part + (cb * ROWS + R) * CB),
+                                 (uint32_t)(n * CB * 4), map_to_cta(smem_u32(&bars->rx_full), (uint32_t)owner));
                 __syncwarp();
                 (void)wait_cluster(smem_u32(&bars->rx_full), 0, abort_flag);
             } else {
@@ -439,7 +438,7 @@ conv_pair_kernel(const ConvArgs a, const ConvSplitShape sh, const __grid_constan
     volatile uint32_t* abort_flag = &bars->abort_flag;
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int rank = (int)ctarank(), half = rank & 1, kp = rank >> 1, lead_cta = rank & ~1;
+    const int rank = (int)cluster_ctarank(), half = rank & 1, kp = rank >> 1, lead_cta = rank & ~1;
     const int H = a.H, W = a.W;
     const int tiles_x = (W + TILE_W - 1) / TILE_W, tiles = tiles_x * ((H + TILE_H - 1) / TILE_H), groups = (tiles + 1) / 2;
     const int nblk = a.Cout / BN;
@@ -480,7 +479,7 @@ conv_pair_kernel(const ConvArgs a, const ConvSplitShape sh, const __grid_constan
                 for (int tap = 0; tap < TAPS; ++tap) {
                     if (issued >= n_b) ok = mbar_wait(smem_u32(&bars->b_empty[st]), ph ^ 1, abort_flag);
                     if (!ok) break;
-                    const uint32_t full = peer_addr(smem_u32(&bars->b_full[st]), lead_cta);
+                    const uint32_t full = map_to_cta(smem_u32(&bars->b_full[st]), lead_cta);
                     mbar_arrive_expect_tx_cluster(full, BST);
                     tma_load_2d_pair(smem_u32(smem_b + st * BST), &tm_w, (k0 + u) * 64, tap * a.Cout + n0 + half * (BN / 2), full);
                     ++issued;
@@ -571,7 +570,7 @@ conv_pair_kernel(const ConvArgs a, const ConvSplitShape sh, const __grid_constan
             op.transform(smem_a + as * A_TILE_BYTES, u, u + 1 < nk, prologue, silu, s_scale, s_shift, ptid);
             fence_proxy_async_smem();
             __syncwarp();
-            if (lane == 0) mbar_arrive_cluster(peer_addr(smem_u32(&bars->a_full[as]), lead_cta));
+            if (lane == 0) mbar_arrive_cluster(map_to_cta(smem_u32(&bars->a_full[as]), lead_cta));
             if (++as == (uint32_t)n_a) { as = 0; aph ^= 1; }
         }
         // ------------------------------------------------ exchange and epilogue: row R of the tile belongs to part R / rpo of K,
@@ -597,8 +596,8 @@ conv_pair_kernel(const ConvArgs a, const ConvSplitShape sh, const __grid_constan
             __syncwarp();
             if (owner != kp && lane == 0) {
                 const uint32_t peer = (uint32_t)(owner * 2 + half);
-                copy_to_peer(peer_addr(smem_u32(rx + (cb * RPO + R0 - owner * RPO) * CB), peer), smem_u32(part + (cb * ROWS + R0) * CB), 32 * CB * 4,
-                             peer_addr(smem_u32(&bars->rx_full), peer));
+                copy_to_peer(map_to_cta(smem_u32(rx + (cb * RPO + R0 - owner * RPO) * CB), peer), smem_u32(part + (cb * ROWS + R0) * CB), 32 * CB * 4,
+                             map_to_cta(smem_u32(&bars->rx_full), peer));
             }
             named_barrier_sync(1, NT);                       // this CTA's own share of its rows
             (void)wait_cluster(smem_u32(&bars->rx_full), 0, abort_flag);
@@ -633,98 +632,31 @@ conv_pair_kernel(const ConvArgs a, const ConvSplitShape sh, const __grid_constan
     }
 }
 
-constexpr int kMaxDevices = 64;
-std::mutex g_mu;
-
-template <int BN, int KIND, bool IB>
-cudaError_t launch_one(const ConvArgs& a, const ConvSplitPlan& p, unsigned int* status, cudaStream_t s) {
-    auto kern = conv_split_kernel<BN, KIND, IB>;
-    static bool configured[kMaxDevices] = {};
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
-    {
-        std::lock_guard<std::mutex> lock(g_mu);
-        if (!configured[dev]) {
-            e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSplitSmemMax);
-            if (e != cudaSuccess) return e;
-            configured[dev] = true;
-        }
-    }
-    const int H = KIND == KPHASE ? a.Hs : a.H, W = KIND == KPHASE ? a.Ws : a.W;
-    const long long grid = (long long)((W + TILE_W - 1) / TILE_W) * ((H + TILE_H - 1) / TILE_H) * ((a.Cout + BN - 1) / BN) *
-                           (KIND == KPHASE ? 4 : 1) * a.B * p.shape.splits;
-    if (grid > 0x7fffffffLL) return cudaErrorInvalidValue;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)grid);
-    cfg.blockDim = dim3(kThreads);
-    cfg.dynamicSmemBytes = (size_t)p.smem;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[2];
-    int na = 0;
-    attr[na].id = cudaLaunchAttributeClusterDimension;
-    attr[na].val.clusterDim.x = (unsigned)p.shape.splits; attr[na].val.clusterDim.y = 1; attr[na].val.clusterDim.z = 1;
-    ++na;
-    if (pdl_enabled()) {
-        attr[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[na].val.programmaticStreamSerializationAllowed = 1;
-        ++na;
-    }
-    cfg.attrs = attr;
-    cfg.numAttrs = na;
-    return cudaLaunchKernelEx(&cfg, kern, a, p.shape, *(const CUtensorMap*)p.tmap, *(const CUtensorMap*)p.tmap2, *(const CUtensorMap*)p.tmap_x2, status);
-}
-
-template <bool IB>
-cudaError_t launch_pair(const ConvArgs& a, const ConvSplitPlan& p, unsigned int* status, cudaStream_t s) {
-    auto kern = conv_pair_kernel<IB>;
-    static bool configured[kMaxDevices] = {};
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
-    {
-        std::lock_guard<std::mutex> lock(g_mu);
-        if (!configured[dev]) {
-            e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kPairSmemMax);
-            if (e != cudaSuccess) return e;
-            configured[dev] = true;
-        }
-    }
-    const long long tiles = (long long)((a.W + TILE_W - 1) / TILE_W) * ((a.H + TILE_H - 1) / TILE_H);
-    const long long grid = (tiles + 1) / 2 * (a.Cout / kPairBN) * a.B * 2 * p.shape.splits;
-    if (grid > 0x7fffffffLL) return cudaErrorInvalidValue;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)grid);
-    cfg.blockDim = dim3(kPairThreads);
-    cfg.dynamicSmemBytes = (size_t)p.smem;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[2];
-    int na = 0;
-    attr[na].id = cudaLaunchAttributeClusterDimension;
-    attr[na].val.clusterDim.x = (unsigned)(2 * p.shape.splits); attr[na].val.clusterDim.y = 1; attr[na].val.clusterDim.z = 1;
-    ++na;
-    if (pdl_enabled()) {
-        attr[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[na].val.programmaticStreamSerializationAllowed = 1;
-        ++na;
-    }
-    cfg.attrs = attr;
-    cfg.numAttrs = na;
-    return cudaLaunchKernelEx(&cfg, kern, a, p.shape, *(const CUtensorMap*)p.tmap, status);
-}
-
 int kind_of(const ConvArgs& a) { return a.upsample == 2 ? KPHASE : (a.ksize == 1 ? K1X1 : K3X3); }
 int tiles_of(const ConvArgs& a) {
     const int h = a.upsample == 2 ? a.Hs : a.H, w = a.upsample == 2 ? a.Ws : a.W;
     return ((w + TILE_W - 1) / TILE_W) * ((h + TILE_H - 1) / TILE_H);
 }
 
+template <int BN, int KIND, bool IB>
+cudaError_t launch_one(const ConvArgs& a, const ConvSplitPlan& p, unsigned int* status, cudaStream_t s) {
+    const long long ctas = (long long)tiles_of(a) * ((a.Cout + BN - 1) / BN) * (KIND == KPHASE ? 4 : 1) * a.B * p.shape.splits;
+    return launch_clusters<conv_split_kernel<BN, KIND, IB>>({ctas, kThreads, p.smem, kSplitSmemMax, p.shape.splits}, s, a, p.shape, *(const CUtensorMap*)p.tmap,
+                                                            *(const CUtensorMap*)p.tmap2, *(const CUtensorMap*)p.tmap_x2, status);
+}
+
+template <bool IB>
+cudaError_t launch_pair(const ConvArgs& a, const ConvSplitPlan& p, unsigned int* status, cudaStream_t s) {
+    const long long ctas = (long long)(tiles_of(a) + 1) / 2 * (a.Cout / kPairBN) * a.B * 2 * p.shape.splits;
+    return launch_clusters<conv_pair_kernel<IB>>({ctas, kPairThreads, p.smem, kPairSmemMax, 2 * p.shape.splits}, s, a, p.shape, *(const CUtensorMap*)p.tmap, status);
+}
+
 }  // namespace
 
+// (The upsampling form and the frame head read the residual stream: fp32 input only.)
 bool conv_split_supported(const ConvArgs& a) {
-    return conv_tc_supported(a) && a.upsample != 1 && !(a.residual && a.out_dtype != VD_F32);
+    return conv_tc_supported(a) && a.upsample != 1 && !(a.residual && a.out_dtype != VD_F32) &&
+           !(a.in_dtype == VD_BF16 && (a.upsample == 2 || a.Cout % 128 != 0));
 }
 
 int conv_split_slots(const ConvArgs& a, const ConvSplitPlan& p, int groups) {
@@ -815,10 +747,10 @@ cudaError_t launch_conv_split(const ConvArgs& a, const ConvSplitPlan& p, unsigne
     const bool ib = a.in_dtype == VD_BF16;
     const int kind = kind_of(a);
     if (p.bn == kPairBN) return ib ? launch_pair<true>(a, p, status, s) : launch_pair<false>(a, p, status, s);
-    if (p.bn == 16) return ib ? launch_one<16, K3X3, true>(a, p, status, s) : launch_one<16, K3X3, false>(a, p, status, s);
+    if (p.bn == 16) return launch_one<16, K3X3, false>(a, p, status, s);
     if (kind == K3X3) return ib ? launch_one<64, K3X3, true>(a, p, status, s) : launch_one<64, K3X3, false>(a, p, status, s);
     if (kind == K1X1) return ib ? launch_one<64, K1X1, true>(a, p, status, s) : launch_one<64, K1X1, false>(a, p, status, s);
-    return ib ? launch_one<64, KPHASE, true>(a, p, status, s) : launch_one<64, KPHASE, false>(a, p, status, s);
+    return launch_one<64, KPHASE, false>(a, p, status, s);
 }
 
 }  // namespace vd

@@ -36,7 +36,6 @@
 //     form: one halo tile of 16x8 SOURCE pixels, four parity accumulators, 16 instead of 36 tap
 //     products (see TileCfg and PhaseSched).
 // Every wait is bounded: on expiry the CTA records a code in the status word and unwinds.
-#include <cuda.h>
 #include <cuda_fp16.h>
 #include <stdlib.h>
 #include <string.h>
@@ -1465,27 +1464,13 @@ __global__ void pack_weight_phase_kernel(const T* w, __half* packed, int Cout, i
     }
 }
 
-typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
-                                  const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
-                                  CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-EncodeTiledFn get_encode_fn() {
-    static EncodeTiledFn fn = nullptr;
-    if (!fn) {
-        void* p = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &q) == cudaSuccess && q == cudaDriverEntryPointSuccess)
-            fn = (EncodeTiledFn)p;
-    }
-    return fn;
-}
-
 int padded_cout(int Cout) { return (Cout % 128 == 0) ? Cout : 16; }
 int pick_bn(int Cout) {
     return (Cout % 128 != 0) ? 16 : ((Cout % 256 == 0) ? 256 : 128);
 }
 
 bool encode_weights(CUtensorMap* tm, const void* w, int Cin, int rows, int bn) {
-    EncodeTiledFn enc = get_encode_fn();
+    EncodeTiledFn enc = encode_fn();
     if (!enc) return false;
     const cuuint64_t dims[2] = {(cuuint64_t)Cin, (cuuint64_t)rows};
     const cuuint64_t strides[1] = {(cuuint64_t)Cin * 2};
@@ -1698,7 +1683,7 @@ cudaError_t conv_tc_prepare(const ConvArgs& a, ConvTcPlan* plan) {
     }
     plan->cg = cg;
     plan->phase = phase ? 1 : 0;
-    EncodeTiledFn enc = get_encode_fn();
+    EncodeTiledFn enc = encode_fn();
     if (!enc) return cudaErrorNotSupported;
     const bool ob = a.out_dtype == VD_BF16;
     const cuuint64_t es = ob ? 2 : 4;

@@ -311,7 +311,7 @@ __global__ void __cluster_dims__(kGnSplit, 1, 1) __launch_bounds__(1024 / SPG) g
         float2 t = s_warp[0][threadIdx.x];
 #pragma unroll 8
         for (int w = 1; w < THREADS / 32; ++w) { t.x += s_warp[w][threadIdx.x].x; t.y += s_warp[w][threadIdx.x].y; }
-        const uint32_t dst = cc::peer_addr(tc::smem_u32(&s_all[threadIdx.x][rank]), 0u);
+        const uint32_t dst = tc::map_to_cta(tc::smem_u32(&s_all[threadIdx.x][rank]), 0u);
         asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(dst), "f"(t.x), "f"(t.y) : "memory");
     }
     __syncwarp();
