@@ -74,6 +74,9 @@ typedef enum { VD_ARCH_TINY = 0, VD_ARCH_SDVAE = 1 } vd_arch;
                                      the sums double their instruction count; measured 3.77 against 3.70 ms per
                                      720x480 frame). */
 
+#define VD_FLAG_NO_CLUSTERS 0x20u  /* debugging: plan no layer whose CTAs divide its sums among a thread-block cluster, as
+                                     vd_create does by itself on a device that cannot hold such a cluster */
+
 typedef struct {
     uint32_t struct_size;       /* sizeof(vd_config), for versioning */
     int32_t arch;               /* vd_arch */

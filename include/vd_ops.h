@@ -47,7 +47,7 @@ typedef struct {
     int32_t out_u8;             /* 1: the output is the display-packed uint8 NHWC frame (VD_FLAG_OUT_U8) */
     int32_t stats_fused;        /* 1: a convolution whose epilogue also produces the statistics (scale, shift) of the
                                    GroupNorm that follows; that GroupNorm has no step of its own then */
-    int32_t reserved;
+    int32_t cluster;            /* CTAs of a thread-block cluster that divide the step's sums among them (1: undivided) */
     int64_t out_pending_offset; /* >= 0: byte offset in the workspace of an fp32 vector [out_channels]; the step's stored
                                    output lacks this per-channel constant (a bias left out of the epilogue and accounted
                                    for by the steps that read the tensor): layer output = stored + pending[c].  -1: none */

@@ -19,6 +19,7 @@ VD_FLAG_UPSAMPLE_9TAP = 0x2
 VD_FLAG_OUT_U8 = 0x4
 VD_FLAG_CANARY = 0x8
 VD_FLAG_FUSED_STATS = 0x10
+VD_FLAG_NO_CLUSTERS = 0x20
 VD_IMPL_AUTO, VD_IMPL_SIMT, VD_IMPL_TC = 0, 1, 2
 VD_ROUTE_DIRECT, VD_ROUTE_THIN, VD_ROUTE_F32, VD_ROUTE_TC = 0, 1, 2, 3
 VD_STEP_INGEST, VD_STEP_GN_STATS, VD_STEP_CONV, VD_STEP_ATTENTION = 0, 1, 2, 3
@@ -50,7 +51,7 @@ class VdStepInfo(Structure):
                 ("out_nchw", c_int32), ("out_offset", c_int64), ("flops_per_frame", c_double),
                 ("bytes_per_frame", c_double), ("weight_bytes", c_double), ("c_in2", c_int32),
                 ("has_residual", c_int32), ("phase_collapsed", c_int32), ("out_u8", c_int32),
-                ("stats_fused", c_int32), ("reserved", c_int32), ("out_pending_offset", c_int64)]
+                ("stats_fused", c_int32), ("cluster", c_int32), ("out_pending_offset", c_int64)]
 
 
 class VdConvDesc(Structure):

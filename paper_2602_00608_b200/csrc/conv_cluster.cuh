@@ -274,6 +274,36 @@ template <auto KERNEL> cudaError_t set_smem_limit(int smem_max) {
     }
     return cudaSuccess;
 }
+// Can the current device hold a cluster of `cluster` such CTAs at all?  (A part of a GPU may have too few SMs side by side.)
+// Asked once per device and size, for the largest shared memory that the kernel is launched with.
+template <auto KERNEL> bool clusters_fit(int threads, int smem_max, int cluster) {
+    static std::mutex mu;
+    static signed char known[kMaxDevices][4] = {};           // by log2 of the size: 0 not asked, 1 yes, -1 no
+    int dev = 0, l = 0;
+    while (1 << l < cluster) ++l;
+    if (l == 0) return true;
+    if (l > 3 || cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices || set_smem_limit<KERNEL>(smem_max) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    std::lock_guard<std::mutex> lock(mu);
+    if (!known[dev][l]) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)cluster);
+        cfg.blockDim = dim3((unsigned)threads);
+        cfg.dynamicSmemBytes = (size_t)smem_max;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = (unsigned)cluster; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        int n = 0;
+        const cudaError_t e = cudaOccupancyMaxActiveClusters(&n, (const void*)KERNEL, &cfg);
+        if (e != cudaSuccess) cudaGetLastError();
+        known[dev][l] = e == cudaSuccess && n > 0 ? 1 : -1;
+    }
+    return known[dev][l] > 0;
+}
 struct ClusterShape { long long ctas; int threads, smem, smem_max, cluster; };
 template <auto KERNEL, class... Args> cudaError_t launch_clusters(const ClusterShape& c, cudaStream_t s, Args&&... args) {
     cudaError_t e = set_smem_limit<KERNEL>(c.smem_max);

@@ -77,7 +77,7 @@ template <int TH, int BN, int KIND, int TW = 8> struct FCfg {
     static constexpr int PART_FLOATS = KT / 2 * RX_FLOATS;               // partials of half the K groups at a time
     static_assert(KT >= 2 && kThreads % (TH * NG * (BN / 4)) == 0 && CS % 4 == 0, "thread layout");
 };
-constexpr int kMaxSlice = 512, kMaxSplits = 8;               // input channels of one CTA; CTAs of a cluster
+constexpr int kMaxSlice = 512, kMaxSplits = kF32MaxSplits;   // input channels of one CTA; CTAs of a cluster
 constexpr int kFTail = 2 * kMaxSlice * 4 + 128;              // scale / shift of the slice, barriers
 
 // A partial lies in memory as rows (pixels) of BN floats whose 16-byte pieces are permuted by the row, so that neither the
@@ -388,7 +388,7 @@ bool conv_f32_supported(const ConvArgs& a) {
 // Tile height 8 where 16 would be more than an eighth padding; K divided among a cluster as long as two CTAs per SM are
 // not exceeded (a CTA's time is proportional to its share of K, and below that the other SMs idle: 512->512 at 8x8 is 16
 // CTAs undivided).
-bool conv_f32_choose(const ConvArgs& a, ConvF32Plan* p) {
+bool conv_f32_choose(const ConvArgs& a, ConvF32Plan* p, int max_splits) {
     p->valid = 0;
     if (!conv_f32_supported(a)) return false;
     const int kind = kind_of(a);
@@ -403,8 +403,9 @@ bool conv_f32_choose(const ConvArgs& a, ConvF32Plan* p) {
     const int tiles = ((W + p->tw - 1) / p->tw) * ((H + p->th - 1) / p->th), chunks = (a.Cin + kChunk - 1) / kChunk;
     const long long ctas = (long long)tiles * (head ? 1 : a.Cout / 32) * (kind == KPHASE ? 4 : 1) * std::max(a.B, 1);
     int s = 1;
-    while (s < kMaxSplits && 2 * s <= chunks && ctas * 2 * s <= 296) s *= 2;
+    while (s < max_splits && 2 * s <= chunks && ctas * 2 * s <= 296) s *= 2;
     while ((chunks + s - 1) / s * kChunk > (head ? 128 : kMaxSlice)) s *= 2;
+    if (s > max_splits) return false;
     p->splits = s;
     const int units = (chunks + s - 1) / s;
     auto fit = [&](int base, int stage) { return std::min(std::min(units, kMaxW), (kSplitSmemMax - base) / stage); };
@@ -443,18 +444,33 @@ cudaError_t conv_f32_prepare(const ConvArgs& a, ConvF32Plan* p) {
     return cudaSuccess;
 }
 
+// f(Build<...>) for the build that the plan takes
+namespace {
+template <int TH, int BN, int KIND, int TW = 8> struct Build {
+    static cudaError_t launch(const ConvArgs& a, const ConvF32Plan& p, unsigned int* status, cudaStream_t s) { return launch_one<TH, BN, KIND, TW>(a, p, status, s); }
+    static bool fits(const ConvF32Plan& p) { return clusters_fit<conv_f32_kernel<TH, BN, KIND, TW>>(kThreads, kSplitSmemMax, p.splits); }
+};
+template <class F> auto with_build(const ConvArgs& a, const ConvF32Plan& p, F f) {
+    const int kind = kind_of(a);
+    if (p.bn == 4) return p.tw == 32 ? f(Build<16, 4, K3X3, 32>()) : f(Build<16, 4, K3X3>());
+    if (p.th == 8) {
+        if (kind == K3X3) return f(Build<8, 32, K3X3>());
+        return kind == K1X1 ? f(Build<8, 32, K1X1>()) : f(Build<8, 32, KPHASE>());
+    }
+    if (kind == K3X3) return f(Build<16, 32, K3X3>());
+    return kind == K1X1 ? f(Build<16, 32, K1X1>()) : f(Build<16, 32, KPHASE>());
+}
+}  // namespace
+
+bool conv_f32_fits(const ConvArgs& a, const ConvF32Plan& p) {
+    return with_build(a, p, [&](auto build) { return build.fits(p); });
+}
+
 cudaError_t launch_conv_f32(const ConvArgs& a, const ConvF32Plan& p, unsigned int* status, cudaStream_t s) {
     if (!p.valid) return cudaErrorInvalidValue;
     if (a.in_rec && !rec_groups_ok(a.Cin, a.in_G)) return cudaErrorInvalidValue;
     if (a.out_rec && !rec_groups_ok(a.Cout, a.out_G)) return cudaErrorInvalidValue;
-    const int kind = kind_of(a);
-    if (p.bn == 4) return p.tw == 32 ? launch_one<16, 4, K3X3, 32>(a, p, status, s) : launch_one<16, 4, K3X3>(a, p, status, s);
-    if (p.th == 8) {
-        if (kind == K3X3) return launch_one<8, 32, K3X3>(a, p, status, s);
-        return kind == K1X1 ? launch_one<8, 32, K1X1>(a, p, status, s) : launch_one<8, 32, KPHASE>(a, p, status, s);
-    }
-    if (kind == K3X3) return launch_one<16, 32, K3X3>(a, p, status, s);
-    return kind == K1X1 ? launch_one<16, 32, K1X1>(a, p, status, s) : launch_one<16, 32, KPHASE>(a, p, status, s);
+    return with_build(a, p, [&](auto build) { return build.launch(a, p, status, s); });
 }
 
 cudaError_t launch_pack_weight_f32_phase(const void* w, int w_dtype, float* packed, int Cout, int Cin, cudaStream_t s) {

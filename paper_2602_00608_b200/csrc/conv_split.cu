@@ -740,17 +740,38 @@ cudaError_t conv_split_prepare(const ConvArgs& a, ConvSplitPlan* p) {
     return cudaSuccess;
 }
 
+// f(Build<...>) for the build that the plan takes
+namespace {
+template <int BN, int KIND, bool IB> struct Build {
+    static cudaError_t launch(const ConvArgs& a, const ConvSplitPlan& p, unsigned int* status, cudaStream_t s) { return launch_one<BN, KIND, IB>(a, p, status, s); }
+    static bool fits(const ConvSplitPlan& p) { return clusters_fit<conv_split_kernel<BN, KIND, IB>>(kThreads, kSplitSmemMax, p.shape.splits); }
+};
+template <bool IB> struct PairBuild {
+    static cudaError_t launch(const ConvArgs& a, const ConvSplitPlan& p, unsigned int* status, cudaStream_t s) { return launch_pair<IB>(a, p, status, s); }
+    static bool fits(const ConvSplitPlan& p) { return clusters_fit<conv_pair_kernel<IB>>(kPairThreads, kPairSmemMax, 2 * p.shape.splits); }
+};
+template <class F> auto with_build(const ConvArgs& a, const ConvSplitPlan& p, F f) {
+    const bool ib = a.in_dtype == VD_BF16;
+    const int kind = kind_of(a);
+    if (p.bn == kPairBN) return ib ? f(PairBuild<true>()) : f(PairBuild<false>());
+    if (p.bn == 16) return f(Build<16, K3X3, false>());
+    if (kind == K3X3) return ib ? f(Build<64, K3X3, true>()) : f(Build<64, K3X3, false>());
+    if (kind == K1X1) return ib ? f(Build<64, K1X1, true>()) : f(Build<64, K1X1, false>());
+    return f(Build<64, KPHASE, false>());
+}
+}  // namespace
+
+bool conv_split_fits(const ConvArgs& a, const ConvSplitPlan& p) {
+    return with_build(a, p, [&](auto build) { return build.fits(p); });
+}
+
+int conv_split_cluster(const ConvSplitPlan& p) { return p.shape.splits * (p.bn == kPairBN ? 2 : 1); }
+
 cudaError_t launch_conv_split(const ConvArgs& a, const ConvSplitPlan& p, unsigned int* status, cudaStream_t s) {
     if (!p.valid || a.B > p.batch) return cudaErrorInvalidValue;
     if (a.in_rec && !rec_groups_ok(a.Cin, a.in_G)) return cudaErrorInvalidValue;
     if (a.out_rec && !rec_groups_ok(a.Cout, a.out_G)) return cudaErrorInvalidValue;
-    const bool ib = a.in_dtype == VD_BF16;
-    const int kind = kind_of(a);
-    if (p.bn == kPairBN) return ib ? launch_pair<true>(a, p, status, s) : launch_pair<false>(a, p, status, s);
-    if (p.bn == 16) return launch_one<16, K3X3, false>(a, p, status, s);
-    if (kind == K3X3) return ib ? launch_one<64, K3X3, true>(a, p, status, s) : launch_one<64, K3X3, false>(a, p, status, s);
-    if (kind == K1X1) return ib ? launch_one<64, K1X1, true>(a, p, status, s) : launch_one<64, K1X1, false>(a, p, status, s);
-    return launch_one<64, KPHASE, false>(a, p, status, s);
+    return with_build(a, p, [&](auto build) { return build.launch(a, p, status, s); });
 }
 
 }  // namespace vd

@@ -696,15 +696,24 @@ cudaError_t launch_ingest(const IngestArgs& a, cudaStream_t s) {
     return cudaGetLastError();
 }
 
-cudaError_t launch_gn_stats(const GnArgs& a, cudaStream_t s) {
-    if (a.C % 4 != 0 || a.C / 4 > kGnThreads || a.G > kGnThreads || (a.C / a.G) % 4 != 0) return cudaErrorInvalidValue;
+bool gn_takes_clusters(const GnArgs& a) {
     const int spg = a.C / a.G / 4;
     // Up to here the clusters' few CTAs read a sample faster than the other kernel's phases run (the line depends on the
     // sample size only, like everything below).  Measured by itself, one sample, us, other kernel -> this one, a 2 us memset
     // included in both: 512 channels 32x32 10.3 -> 6.3, 60x90 10.4 -> 8.2; 256 channels 128x128 12.2 -> 8.6, bf16 240x360
     // 14.5 -> 20.7; 128 channels 296x424 14.5 -> 16.5.  Whole decodes: 424x296 1565 -> 1536 us with the line at 3 million
     // elements, 1567 at 12 million and 1666 at 20 million (the next layer's lines leave L2 later).
-    if (a.C % 16 == 0 && (spg == 1 || spg == 2 || spg == 4) && (long long)a.P * a.C <= 3000000) {
+    return !a.no_clusters && a.C % 16 == 0 && (spg == 1 || spg == 2 || spg == 4) && (long long)a.P * a.C <= 3000000;
+}
+
+bool gn_clusters_fit() {
+    return cc::clusters_fit<gn_cluster_kernel<float, 1>>(1024, 0, kGnSplit) && cc::clusters_fit<gn_cluster_kernel<__nv_bfloat16, 1>>(1024, 0, kGnSplit);
+}
+
+cudaError_t launch_gn_stats(const GnArgs& a, cudaStream_t s) {
+    if (a.C % 4 != 0 || a.C / 4 > kGnThreads || a.G > kGnThreads || (a.C / a.G) % 4 != 0) return cudaErrorInvalidValue;
+    if (gn_takes_clusters(a) && gn_clusters_fit()) {
+        const int spg = a.C / a.G / 4;
         const dim3 grid(a.C / 16 * kGnSplit, a.B), block(1024 / spg);
         if (a.dtype == VD_BF16)
             return spg == 4 ? launch_pdl(gn_cluster_kernel<__nv_bfloat16, 4>, grid, block, 0, s, a)

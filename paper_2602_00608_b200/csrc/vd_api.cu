@@ -107,7 +107,9 @@ namespace {
 // sizes/offsets are computed (all pointers are offsets from 0).
 class Planner {
   public:
-    Planner(vd_handle_s* h, char* base) : h_(h), base_(base), cfg_(h->cfg) {}
+    // clusters: layers and statistics whose CTAs divide their sums among a cluster may be planned; pad: bytes left free
+    // ahead of the last layer's regions
+    Planner(vd_handle_s* h, char* base, bool clusters, size_t pad = 0) : h_(h), base_(base), cfg_(h->cfg), clusters_(clusters), pad_(pad) {}
 
     // With VD_FLAG_CANARY every region is followed by a 256-byte guard that vd_create fills with a pattern
     // and vd_debug_check_canaries verifies: a kernel that writes past the end of its buffer (or before the start of
@@ -186,8 +188,10 @@ class Planner {
             s.gn.rec = ptr<float4>(rec_[x_off].off);
             s.gn.slots = rec_[x_off].slots;
         }
+        s.gn.no_clusters = clusters_ ? 0 : 1;
         fill_info(s, name, 0, C, C, 0, 0, H, W, C, VD_F32, 0, -1);
         s.info.launches = 1;
+        if (!s.gn.rec && gn_takes_clusters(s.gn)) s.info.cluster = 8;
         s.info.bytes_per_frame = (double)H * W * C * elt(dtype);
         h_->steps.push_back(s);
     }
@@ -227,13 +231,13 @@ class Planner {
         // fp32 layers: the direct kernel remains for the bf16 layout's cross-check path (and the 9-tap upsampling form)
         probe.B = cfg_.max_batch;
         probe.upsample = a.upsample;
-        const bool split = tc && !(cfg_.flags & VD_FLAG_FUSED_STATS) && conv_split_choose(probe, &s.split);
+        const bool split = tc && clusters_ && !(cfg_.flags & VD_FLAG_FUSED_STATS) && conv_split_choose(probe, &s.split);
         s.split.valid = split ? 1 : 0;
         bool f32 = false;
         const bool thin = !tc && conv_thin_supported(probe) && !(bf16() && (cfg_.flags & VD_FLAG_FORCE_SIMT));
         if (!tc && !thin && !(bf16() && (cfg_.flags & VD_FLAG_FORCE_SIMT))) {
             probe.upsample = upsample ? ((cfg_.flags & VD_FLAG_UPSAMPLE_9TAP) ? 1 : 2) : 0;
-            f32 = conv_f32_choose(probe, &s.f32);
+            f32 = conv_f32_choose(probe, &s.f32, clusters_ ? kF32MaxSplits : 1);
             if (f32 && upsample) { phase = true; a.upsample = 2; }
         }
         s.f32.valid = f32 ? 1 : 0;
@@ -331,6 +335,7 @@ class Planner {
         s.info.weight_bytes = (double)ksize * ksize * Cin * Cout * elt(cfg_.dtype);
         s.info.has_residual = residual_off >= 0;
         s.info.phase_collapsed = phase ? 1 : 0;
+        s.info.cluster = split ? conv_split_cluster(s.split) : f32 ? s.f32.splits : 1;
         if (!y_is_frames && pending(y_off) != kNone) s.info.out_pending_offset = (int64_t)pending(y_off);
         if (!shortcut_name.empty()) {
             s.info.c_in2 = Cin2;
@@ -350,6 +355,7 @@ class Planner {
         s.info.out_h = H; s.info.out_w = W; s.info.out_channels = oc; s.info.out_dtype = odt;
         s.info.out_nchw = nchw; s.info.out_offset = off;
         s.info.out_pending_offset = -1;
+        s.info.cluster = 1;
     }
 
     // x -> shortcut(x) + conv2(silu(gn2(conv1(silu(gn1(x))))))
@@ -416,7 +422,7 @@ class Planner {
     vd_status plan() {
         vd_handle_s scratch;
         scratch.cfg = cfg_;
-        Planner first(&scratch, nullptr);
+        Planner first(&scratch, nullptr, clusters_);
         first.layout(0);
         return layout(first.max_slots_);
     }
@@ -532,6 +538,7 @@ class Planner {
     }
 
     void head(int C, int H, int W) {
+        cur_ += pad_;
         add_gn("norm_out", xs_[cur_x_], VD_F32, H, W, C, "norm_out");
         const bool u8 = (cfg_.flags & VD_FLAG_OUT_U8) != 0;
         add_conv("conv_out", {"conv_out"}, cfg_.out_channels, xs_[cur_x_], VD_F32, H, W, C, 3, false, true, true, -1, 0,
@@ -542,6 +549,8 @@ class Planner {
     vd_handle_s* h_;
     char* base_;
     const vd_config& cfg_;
+    const bool clusters_;
+    const size_t pad_;
     size_t cur_ = 0;
     size_t stat_off_ = 0;
     std::map<size_t, size_t> pending_;   // tensor offset -> offset of its pending-bias vector
@@ -575,7 +584,7 @@ vd_status validate_cfg(const vd_config* cfg, std::string& err) {
         return VD_ERR_INVALID_ARG;
     }
     if (!(cfg->norm_eps > 0.f) || !(cfg->norm_eps < 1.f)) { err = "norm_eps must be in (0,1)"; return VD_ERR_INVALID_ARG; }
-    if (cfg->flags & ~(VD_FLAG_FORCE_SIMT | VD_FLAG_UPSAMPLE_9TAP | VD_FLAG_OUT_U8 | VD_FLAG_CANARY | VD_FLAG_FUSED_STATS)) { err = "unknown flag bits"; return VD_ERR_INVALID_ARG; }
+    if (cfg->flags & ~(VD_FLAG_FORCE_SIMT | VD_FLAG_UPSAMPLE_9TAP | VD_FLAG_OUT_U8 | VD_FLAG_CANARY | VD_FLAG_FUSED_STATS | VD_FLAG_NO_CLUSTERS)) { err = "unknown flag bits"; return VD_ERR_INVALID_ARG; }
     return VD_OK;
 }
 
@@ -592,6 +601,27 @@ const vd_tensor* find_tensor(const vd_tensor* t, int n, const std::string& name)
     for (int i = 0; i < n; ++i)
         if (t[i].name && name == t[i].name) return &t[i];
     return nullptr;
+}
+
+size_t plan_bytes(const vd_config& cfg, bool clusters) {
+    vd_handle_s h;
+    h.cfg = cfg;
+    Planner(&h, nullptr, clusters).plan();
+    return h.total;
+}
+// Workspace of either plan: which one a device takes is known in vd_create only.
+size_t workspace_of(const vd_config& cfg) {
+    const size_t without = plan_bytes(cfg, false);
+    return (cfg.flags & VD_FLAG_NO_CLUSTERS) ? without : std::max(without, plan_bytes(cfg, true));
+}
+
+// Can the current device hold the clusters of the plan's steps?
+bool plan_fits(const vd_handle_s& h) {
+    for (const Step& st : h.steps) {
+        if (st.kind == VD_STEP_CONV && st.split.valid && !conv_split_fits(st.conv, st.split)) return false;
+        if (st.kind == VD_STEP_CONV && st.f32.valid && !conv_f32_fits(st.conv, st.f32)) return false;
+    }
+    return true;
 }
 
 cudaError_t launch_step(const vd_handle_s* h, const Step& st, int B, const void* latents, const void* v_prev,
@@ -690,11 +720,7 @@ vd_status vd_query_workspace(const vd_config* cfg, size_t* bytes) {
     vd_status st = validate_cfg(cfg, err);
     if (st != VD_OK) return fail(nullptr, st, err);
     if (!bytes) return fail(nullptr, VD_ERR_INVALID_ARG, "bytes is NULL");
-    vd_handle_s tmp;
-    tmp.cfg = *cfg;
-    Planner p(&tmp, nullptr);
-    p.plan();
-    *bytes = tmp.total;
+    *bytes = workspace_of(*cfg);
     return VD_OK;
 }
 
@@ -714,17 +740,21 @@ vd_status vd_create(const vd_config* cfg, const vd_tensor* weights, int32_t n_we
     if (e != cudaSuccess) return cuda_fail(nullptr, e, "device query");
     if (major != 10) return fail(nullptr, VD_ERR_UNSUPPORTED, "this library runs on sm_100 devices only");
 
-    vd_handle_s* h = new vd_handle_s();
-    h->cfg = *cfg;
-    h->ws = (char*)workspace;
-    h->ws_bytes = workspace_bytes;
-    Planner p(h, h->ws);
-    p.plan();
-    if (workspace_bytes < h->total) {
+    const size_t need = workspace_of(*cfg);
+    if (workspace_bytes < need) {
         char msg[128];
-        snprintf(msg, sizeof(msg), "workspace too small: %zu bytes given, %zu needed", workspace_bytes, h->total);
-        delete h;
+        snprintf(msg, sizeof(msg), "workspace too small: %zu bytes given, %zu needed", workspace_bytes, need);
         return fail(nullptr, VD_ERR_WORKSPACE, msg);
+    }
+    vd_handle_s* h = nullptr;
+    for (bool clusters = !(cfg->flags & VD_FLAG_NO_CLUSTERS);; clusters = false) {
+        h = new vd_handle_s();
+        h->cfg = *cfg;
+        h->ws = (char*)workspace;
+        h->ws_bytes = workspace_bytes;
+        Planner(h, h->ws, clusters, need - plan_bytes(*cfg, clusters)).plan();      // (either plan ends where the workspace does)
+        if (!clusters || plan_fits(*h)) break;
+        delete h;
     }
     cudaStream_t s = (cudaStream_t)cuda_stream;
     e = cudaMemsetAsync(h->ws + h->status_off, 0, 256, s);
@@ -1071,7 +1101,8 @@ vd_status vd_op_conv2d(const vd_conv_desc* d, const void* x, const void* w_packe
         if (e == cudaSuccess) e = launch_conv_tc(a, plan, nullptr, (cudaStream_t)cuda_stream);
     } else {
         ConvF32Plan plan{};
-        if (ffma_route(a, &plan) == VD_ROUTE_F32) {
+        const bool f32 = ffma_route(a, &plan) == VD_ROUTE_F32 && (conv_f32_fits(a, plan) || conv_f32_choose(a, &plan, 1));
+        if (f32) {
             e = conv_f32_prepare(a, &plan);
             if (e == cudaSuccess) e = launch_conv_f32(a, plan, nullptr, (cudaStream_t)cuda_stream);
         } else {

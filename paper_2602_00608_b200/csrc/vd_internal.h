@@ -78,6 +78,7 @@ struct GnArgs {
                             // left out), and shift takes scale * offset in, so scale * x + shift normalises x + offset
     const float4* rec;      // or the producing layer's statistics records [B][G][slots] (launch_gn_merge)
     int slots;
+    int no_clusters;        // 1: the kernel without clusters
 };
 constexpr int kGnMaxChunks = 296;      // two blocks per SM on a 148-SM device
 // bytes of the partial records / of the whole scratch (records, then the arrival counters)
@@ -114,6 +115,8 @@ inline bool aligned16(const void* p) { return ((uintptr_t)p & 15) == 0; }
 // ---- FFMA kernels (kernels_simt.cu)
 cudaError_t launch_ingest(const IngestArgs& a, cudaStream_t s);
 cudaError_t launch_gn_stats(const GnArgs& a, cudaStream_t s);          // one launch (the last block per sample finalises)
+bool gn_takes_clusters(const GnArgs& a);                       // by the sample's size; the device is not asked
+bool gn_clusters_fit();                                        // on the current device
 cudaError_t launch_conv_simt(const ConvArgs& a, cudaStream_t s);
 bool conv_thin_supported(const ConvArgs& a);                   // the first convolution has a kernel of its own there
 int conv_thin_slots(const ConvArgs& a);                        // records per group and frame that it leaves
@@ -179,7 +182,9 @@ struct alignas(64) ConvF32Plan {
     int valid;
 };
 bool conv_f32_supported(const ConvArgs& a);
-bool conv_f32_choose(const ConvArgs& a, ConvF32Plan* plan);    // a.B = the handle's batch
+constexpr int kF32MaxSplits = 8;
+bool conv_f32_choose(const ConvArgs& a, ConvF32Plan* plan, int max_splits = kF32MaxSplits);    // a.B = the handle's batch
+bool conv_f32_fits(const ConvArgs& a, const ConvF32Plan& plan);    // can the current device hold the plan's clusters?
 int conv_f32_slots(const ConvArgs& a, const ConvF32Plan& plan, int groups);
 cudaError_t conv_f32_prepare(const ConvArgs& a, ConvF32Plan* plan);
 cudaError_t launch_conv_f32(const ConvArgs& a, const ConvF32Plan& plan, unsigned int* status_word, cudaStream_t s);
@@ -202,6 +207,8 @@ struct alignas(64) ConvSplitPlan {
 };
 bool conv_split_supported(const ConvArgs& a);
 bool conv_split_choose(const ConvArgs& a, ConvSplitPlan* plan);   // a.B = the handle's batch; false: conv_tc.cu is the faster one
+bool conv_split_fits(const ConvArgs& a, const ConvSplitPlan& plan);
+int conv_split_cluster(const ConvSplitPlan& plan);             // CTAs of a cluster
 int conv_split_slots(const ConvArgs& a, const ConvSplitPlan& plan, int groups);
 cudaError_t conv_split_prepare(const ConvArgs& a, ConvSplitPlan* plan);
 cudaError_t launch_conv_split(const ConvArgs& a, const ConvSplitPlan& plan, unsigned int* status_word, cudaStream_t s);
