@@ -38,7 +38,9 @@ typedef struct {
     int32_t out_nchw;           /* 1 if the output is NCHW (the frames), else NHWC */
     int64_t out_offset;         /* byte offset of the output in the workspace, -1 if it is `frames` */
     double flops_per_frame;     /* 2*taps*Cin*Cout*P for a conv, 4*T*T*C for attention, 0 otherwise */
-    double bytes_per_frame;     /* algorithmic HBM bytes as stored (inputs once, output once, residual once) */
+    double bytes_per_frame;     /* algorithmic HBM bytes as stored (inputs once, output once, residual once); statistics: the
+                                   tensor, or the records that its producer left of it, or 0 where the next layer merges
+                                   those itself (launches is 0 then) */
     double weight_bytes;        /* parameter bytes read once per launch (shared by the batch) */
     int32_t c_in2;              /* > 0: a 1x1 shortcut on a second input of c_in2 channels is fused in */
     int32_t has_residual;       /* 1: an fp32 residual tensor is added in the epilogue */

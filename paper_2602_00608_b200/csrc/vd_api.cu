@@ -192,7 +192,7 @@ class Planner {
         fill_info(s, name, 0, C, C, 0, 0, H, W, C, VD_F32, 0, -1);
         s.info.launches = 1;
         if (!s.gn.rec && gn_takes_clusters(s.gn)) s.info.cluster = 8;
-        s.info.bytes_per_frame = (double)H * W * C * elt(dtype);
+        s.info.bytes_per_frame = s.gn.rec ? 16.0 * cfg_.norm_groups * s.gn.slots : (double)H * W * C * elt(dtype);
         h_->steps.push_back(s);
     }
 
@@ -304,6 +304,7 @@ class Planner {
                 a.scale = a.shift = nullptr;
                 g.skip = true;
                 g.info.launches = 0;
+                g.info.bytes_per_frame = 0.0;
             }
         }
         if (!y_is_frames) rec_.erase(y_off);

@@ -30,3 +30,26 @@ def test_small_decodes_match_the_ffma_kernels(h, w, b):
     # two paths that each meet the bound against the exact result differ by at most twice the bound
     d = got.float() - want.float()
     assert float(d.norm() / want.float().norm()) <= 2 * BF16_REL_L2 and float(d.abs().max()) <= 2 * BF16_MAX_ABS
+
+
+@pytest.mark.parametrize("h,w", [(8, 8), (60, 90)])
+def test_statistics_steps_count_what_they_read(h, w):
+    """A pass reads the tensor; where the layer before has left records the step reads those, or is no launch and reads nothing."""
+    from paper_2602_00608_b200 import binding as vd, synth
+    wl = synth.WORKLOADS[2]
+    dec = vd.Decoder(wl.arch, wl.dtype, h, w, 1, wl.groups, wl.eps, synth.workload_weights(wl))
+    seen = set()
+    for s in dec.steps():
+        if s["kind"] != vd.VD_STEP_GN_STATS:
+            continue
+        values = s["out_h"] * s["out_w"] * s["c_in"]
+        if s["launches"] == 0:
+            assert s["bytes_per_frame"] == 0
+            seen.add("merged by the next layer")
+        elif s["bytes_per_frame"] in (2 * values, 4 * values):
+            seen.add("pass")
+        else:
+            assert s["bytes_per_frame"] % (16 * wl.groups) == 0 and 0 < s["bytes_per_frame"] < values
+            seen.add("merged")
+    # 8x8: every layer leaves few records and merges them; 60x90: no level is divided along K, some leave records
+    assert seen == ({"merged by the next layer"} if h == 8 else {"merged", "pass"})
