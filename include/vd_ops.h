@@ -88,7 +88,10 @@ VD_API vd_status vd_debug_stop_after(vd_handle h, int32_t index);
  * Operator-level entry points: the fused building blocks of the chain of Section IV-B.1,
  * callable on caller-provided device tensors (internal NHWC layout).  Used by per-kernel tests.
  * ---------------------------------------------------------------------------------------- */
-typedef enum { VD_IMPL_AUTO = 0, VD_IMPL_SIMT = 1, VD_IMPL_TC = 2 } vd_impl;
+typedef enum {
+    VD_IMPL_AUTO = 0, VD_IMPL_SIMT = 1, VD_IMPL_TC = 2,
+    VD_IMPL_TC_SPLIT = 3        /* tcgen05 kernels that divide K among a cluster (convolutions of small images) */
+} vd_impl;
 
 typedef struct {
     uint32_t struct_size;
@@ -128,10 +131,39 @@ typedef enum {
     VD_ROUTE_DIRECT = 0,        /* tiled FFMA kernel, scalar accesses */
     VD_ROUTE_THIN = 1,          /* first convolution (4 or 8 input channels), FFMA */
     VD_ROUTE_F32 = 2,           /* register-tiled FFMA kernel, 16-byte accesses, K divided among a cluster */
-    VD_ROUTE_TC = 3             /* tcgen05 kernel */
+    VD_ROUTE_TC = 3,            /* tcgen05 kernel */
+    VD_ROUTE_SPLIT = 4,         /* tcgen05 kernel, K divided among the CTAs of a cluster */
+    VD_ROUTE_SPLIT_PAIRS = 5    /* the same on CTA pairs */
 } vd_conv_route_kind;
 VD_API vd_status vd_conv_route(const vd_conv_desc* d, const void* x, const void* w_packed, const float* bias, const float* scale,
                                const float* residual, const void* y, int32_t* route);
+
+/* vd_op_conv2d with what a decode hands from layer to layer besides tensors; every field may be zero. */
+typedef struct {
+    uint32_t struct_size;
+    int32_t c_in2;              /* fused 1x1 shortcut (tensor-core kernels): y += w2 * x2 + bias2 */
+    const void* x2;             /* device fp32 NHWC [batch,h,w,c_in2] */
+    const float* w2;            /* device fp32 [c_out,c_in2] */
+    const float* bias2;         /* device fp32 [c_out], or NULL */
+    const void* in_records;     /* statistics records of x [batch][in_groups][in_slots] of 16 bytes instead of scale and shift
+                                   (VD_ROUTE_F32, VD_ROUTE_SPLIT, VD_ROUTE_SPLIT_PAIRS) */
+    const float* in_gamma;      /* device fp32 [c_in] */
+    const float* in_beta;
+    int32_t in_slots, in_groups;
+    float in_eps;
+    int32_t out_groups;         /* > 0: the statistics records of y are written to out_records */
+    void* out_records;          /* [batch][out_groups][vd_conv_record_slots] of 16 bytes (count, mean, sum of squared deviations, 0) */
+    const float* out_pending;   /* VD_ROUTE_TC: the records are those of y + out_pending[c]; or NULL */
+} vd_conv_extra;
+/* Records per group and frame that this layer leaves (host-only); VD_ERR_UNSUPPORTED if its kernel leaves none. */
+VD_API vd_status vd_conv_record_slots(const vd_conv_desc* d, const vd_conv_extra* ex, int32_t* slots);
+VD_API vd_status vd_op_conv2d_ex(const vd_conv_desc* d, const vd_conv_extra* ex, const void* x, const void* w_packed,
+                                 const float* bias, const float* scale, const float* shift, const float* residual, void* y,
+                                 void* cuda_stream);
+/* Folds the records of a [batch,pixels,c] tensor into scale and shift as vd_op_gn_stats does from the tensor. */
+VD_API vd_status vd_op_merge_records(const void* records, int32_t slots, int32_t batch, int32_t pixels, int32_t c, int32_t groups,
+                                     float eps, const float* gamma, const float* beta, const float* offset, float* scale,
+                                     float* shift, void* cuda_stream);
 
 /* vd_op_conv2d and, from the same launch, the statistics of GroupNorm(y) folded with the affine parameters
  * (Section IV-B.1: the normalisation's reduction is taken while the tile is on chip):

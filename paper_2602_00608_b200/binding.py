@@ -20,8 +20,8 @@ VD_FLAG_OUT_U8 = 0x4
 VD_FLAG_CANARY = 0x8
 VD_FLAG_FUSED_STATS = 0x10
 VD_FLAG_NO_CLUSTERS = 0x20
-VD_IMPL_AUTO, VD_IMPL_SIMT, VD_IMPL_TC = 0, 1, 2
-VD_ROUTE_DIRECT, VD_ROUTE_THIN, VD_ROUTE_F32, VD_ROUTE_TC = 0, 1, 2, 3
+VD_IMPL_AUTO, VD_IMPL_SIMT, VD_IMPL_TC, VD_IMPL_TC_SPLIT = 0, 1, 2, 3
+VD_ROUTE_DIRECT, VD_ROUTE_THIN, VD_ROUTE_F32, VD_ROUTE_TC, VD_ROUTE_SPLIT, VD_ROUTE_SPLIT_PAIRS = 0, 1, 2, 3, 4, 5
 VD_STEP_INGEST, VD_STEP_GN_STATS, VD_STEP_CONV, VD_STEP_ATTENTION = 0, 1, 2, 3
 STATUS_NAMES = {0: "VD_OK", -1: "VD_ERR_INVALID_ARG", -2: "VD_ERR_UNSUPPORTED", -3: "VD_ERR_WORKSPACE",
                 -4: "VD_ERR_CUDA", -5: "VD_ERR_DEVICE_TIMEOUT"}
@@ -29,7 +29,7 @@ STATUS_NAMES = {0: "VD_OK", -1: "VD_ERR_INVALID_ARG", -2: "VD_ERR_UNSUPPORTED", 
 EXPORTED = [
     "vd_query_workspace", "vd_create", "vd_decode", "vd_decode_extrapolated", "vd_decode_host", "vd_get_status",
     "vd_last_error", "vd_destroy", "vd_num_steps", "vd_get_step", "vd_profile", "vd_debug_stop_after",
-    "vd_conv_packed_weight_bytes", "vd_conv_pack_weight", "vd_op_conv2d", "vd_conv_route", "vd_conv_stats_scratch_bytes", "vd_op_conv2d_stats", "vd_gn_scratch_bytes", "vd_op_gn_stats",
+    "vd_conv_packed_weight_bytes", "vd_conv_pack_weight", "vd_op_conv2d", "vd_conv_route", "vd_op_conv2d_ex", "vd_conv_record_slots", "vd_op_merge_records", "vd_conv_stats_scratch_bytes", "vd_op_conv2d_stats", "vd_gn_scratch_bytes", "vd_op_gn_stats",
     "vd_op_attention", "vd_attention_scratch_bytes", "vd_op_gn_stats_static", "vd_clear_status", "vd_decode_host_stream", "vd_debug_check_canaries", "vd_debug_status_offset", "vd_debug_wait_probe",
 ]
 
@@ -59,6 +59,13 @@ class VdConvDesc(Structure):
                 ("c_in", c_int32), ("c_out", c_int32), ("ksize", c_int32), ("upsample", c_int32), ("silu", c_int32),
                 ("in_dtype", c_int32), ("out_dtype", c_int32), ("out_nchw", c_int32), ("bf16_operands", c_int32),
                 ("impl", c_int32)]
+
+
+class VdConvExtra(Structure):
+    _fields_ = [("struct_size", c_uint32), ("c_in2", c_int32), ("x2", c_void_p), ("w2", c_void_p), ("bias2", c_void_p),
+                ("in_records", c_void_p), ("in_gamma", c_void_p), ("in_beta", c_void_p), ("in_slots", c_int32),
+                ("in_groups", c_int32), ("in_eps", c_float), ("out_groups", c_int32), ("out_records", c_void_p),
+                ("out_pending", c_void_p)]
 
 
 class VdError(RuntimeError):
@@ -100,6 +107,9 @@ def lib():
         l.vd_conv_pack_weight.argtypes = [POINTER(VdConvDesc), vp, c_int32, vp, vp]
         l.vd_op_conv2d.argtypes = [POINTER(VdConvDesc), vp, vp, vp, vp, vp, vp, vp, vp]
         l.vd_conv_route.argtypes = [POINTER(VdConvDesc), vp, vp, vp, vp, vp, vp, POINTER(c_int32)]
+        l.vd_op_conv2d_ex.argtypes = [POINTER(VdConvDesc), POINTER(VdConvExtra), vp, vp, vp, vp, vp, vp, vp, vp]
+        l.vd_conv_record_slots.argtypes = [POINTER(VdConvDesc), POINTER(VdConvExtra), POINTER(c_int32)]
+        l.vd_op_merge_records.argtypes = [vp, c_int32, c_int32, c_int32, c_int32, c_int32, c_float, vp, vp, vp, vp, vp, vp]
         l.vd_conv_stats_scratch_bytes.argtypes = [c_int32, c_int32]
         l.vd_conv_stats_scratch_bytes.restype = c_size_t
         l.vd_op_conv2d_stats.argtypes = [POINTER(VdConvDesc), vp, vp, vp, vp, vp, vp, c_int32, c_float, vp, vp, vp, vp, vp, vp]
@@ -316,8 +326,13 @@ def conv_desc(batch, in_h, in_w, c_in, c_out, ksize, upsample, silu, in_dtype, o
 
 
 def op_conv2d(x_nhwc, w_oihw, bias=None, scale=None, shift=None, residual=None, *, upsample=False, silu=False,
-              out_dtype=None, out_nchw=False, bf16_operands=False, impl=VD_IMPL_AUTO):
-    """Fused convolution on device tensors; x is NHWC, w is [Cout,Cin,k,k]; returns y (NHWC or NCHW)."""
+              out_dtype=None, out_nchw=False, bf16_operands=False, impl=VD_IMPL_AUTO, shortcut=None, in_records=None,
+              groups=0, pending=None):
+    """Fused convolution on device tensors; x is NHWC, w is [Cout,Cin,k,k]; returns y (NHWC or NCHW).
+
+    shortcut: (x2 NHWC fp32, w2 [Cout,Cin2] fp32, bias2 or None), a fused 1x1 convolution.  in_records: (records, gamma, beta,
+    eps), the statistics of x as records [B,G,slots,4] instead of scale and shift.  groups > 0: returns (y, records of y),
+    those of y + pending[c] if given."""
     import torch
     b, h, w, cin = x_nhwc.shape
     cout, _, k, _ = w_oihw.shape
@@ -332,10 +347,39 @@ def op_conv2d(x_nhwc, w_oihw, bias=None, scale=None, shift=None, residual=None, 
     shape = (b, cout, oh, ow) if out_nchw else (b, oh, ow, cout)
     y = torch.empty(shape, dtype=_torch_dtype(od), device=x_nhwc.device)
     p = lambda t: None if t is None else c_void_p(t.data_ptr())
-    for t in (bias, scale, shift, residual):
+    for t in (bias, scale, shift, residual, pending) + (shortcut or ()) + tuple(in_records or ())[:3]:
         assert t is None or (t.dtype == torch.float32 and t.is_contiguous())
-    _check(lib().vd_op_conv2d(byref(d), p(x_nhwc.contiguous()), p(packed), p(bias), p(scale), p(shift), p(residual), p(y), _stream_ptr()))
-    return y
+    x_nhwc = x_nhwc.contiguous()
+    if shortcut is None and in_records is None and not groups:
+        _check(lib().vd_op_conv2d(byref(d), p(x_nhwc), p(packed), p(bias), p(scale), p(shift), p(residual), p(y), _stream_ptr()))
+        return y
+    ex = VdConvExtra(struct_size=ctypes.sizeof(VdConvExtra), out_groups=groups, out_pending=p(pending))
+    if shortcut is not None:
+        ex.x2, ex.w2, ex.bias2, ex.c_in2 = p(shortcut[0]), p(shortcut[1]), p(shortcut[2]), shortcut[0].shape[3]
+    if in_records is not None:
+        rec, ex.in_gamma, ex.in_beta, ex.in_eps = in_records[0], p(in_records[1]), p(in_records[2]), in_records[3]
+        assert rec.shape[0] == b and rec.shape[3] == 4
+        ex.in_records, ex.in_groups, ex.in_slots = p(rec), rec.shape[1], rec.shape[2]
+    records = None
+    if groups:
+        slots = c_int32(0)
+        _check(lib().vd_conv_record_slots(byref(d), byref(ex), byref(slots)))
+        records = torch.empty((b, groups, slots.value, 4), dtype=torch.float32, device=x_nhwc.device)
+        ex.out_records = p(records)
+    _check(lib().vd_op_conv2d_ex(byref(d), byref(ex), p(x_nhwc), p(packed), p(bias), p(scale), p(shift), p(residual), p(y), _stream_ptr()))
+    return (y, records) if groups else y
+
+
+def op_merge_records(records, pixels: int, gamma, beta, eps: float, offset=None):
+    """Scale and shift of a GroupNorm from the records [B,G,slots,4] of a tensor (of x + offset[c] if given)."""
+    import torch
+    b, groups, slots, _ = records.shape
+    c = gamma.numel()
+    scale = torch.empty((b, c), dtype=torch.float32, device=records.device)
+    shift = torch.empty((b, c), dtype=torch.float32, device=records.device)
+    p = lambda t: None if t is None else c_void_p(t.data_ptr())
+    _check(lib().vd_op_merge_records(p(records), slots, b, pixels, c, groups, eps, p(gamma), p(beta), p(offset), p(scale), p(shift), _stream_ptr()))
+    return scale, shift
 
 
 def conv_route(desc: VdConvDesc, x=256, w=256, bias=0, scale=0, residual=0, y=256) -> int:

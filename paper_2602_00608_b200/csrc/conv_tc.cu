@@ -1635,7 +1635,8 @@ static bool rec_layer(const ConvArgs& a) {
 // pass, which overlaps its neighbours there: 256x256 frame 1049 us without, 1073 with, 424x296 1539 / 1571; four 256x256
 // frames 2772 / 2673.
 // On CTA pairs the hand-over costs more than it saves (two 1280x720 frames 17.85 ms without, 18.00 with).
-bool conv_tc_records_supported(const ConvArgs& a) { return rec_layer(a) && !wide_layer(a) && (double)a.H * a.W * a.Cout * a.B >= 6e6; }
+bool conv_tc_can_record(const ConvArgs& a) { return rec_layer(a) && !wide_layer(a); }
+bool conv_tc_records_supported(const ConvArgs& a) { return conv_tc_can_record(a) && (double)a.H * a.W * a.Cout * a.B >= 6e6; }
 int conv_tc_slots(const ConvArgs& a) { return ((a.W + TILE_W - 1) / TILE_W) * ((a.H + TILE_H - 1) / TILE_H) * REC_WARPS; }
 
 bool conv_tc_pairs_available() { return pairs_available(); }

@@ -1016,7 +1016,7 @@ static vd_status check_conv_desc(const vd_conv_desc* d) {
     if (d->ksize != 1 && d->ksize != 3) return fail(nullptr, VD_ERR_INVALID_ARG, "ksize must be 1 or 3");
     if ((d->in_dtype != VD_F32 && d->in_dtype != VD_BF16) || (d->out_dtype != VD_F32 && d->out_dtype != VD_BF16))
         return fail(nullptr, VD_ERR_INVALID_ARG, "bad dtype");
-    if (d->impl < VD_IMPL_AUTO || d->impl > VD_IMPL_TC) return fail(nullptr, VD_ERR_INVALID_ARG, "bad impl");
+    if (d->impl < VD_IMPL_AUTO || d->impl > VD_IMPL_TC_SPLIT) return fail(nullptr, VD_ERR_INVALID_ARG, "bad impl");
     if (d->upsample < 0 || d->upsample > 2) return fail(nullptr, VD_ERR_INVALID_ARG, "upsample must be 0, 1 or 2");
     return VD_OK;
 }
@@ -1036,16 +1036,25 @@ static vd_status resolve_impl(const vd_conv_desc* d, const ConvArgs& a, bool* tc
     ConvArgs probe = a;
     probe.B = 1;
     const bool can = a.bf16_operands && conv_tc_supported(probe);
-    if (d->impl == VD_IMPL_TC && !can) return fail(nullptr, VD_ERR_UNSUPPORTED, "the tensor-core convolution does not support this shape");
-    *tc = d->impl == VD_IMPL_TC || (d->impl == VD_IMPL_AUTO && can);
+    if ((d->impl == VD_IMPL_TC || d->impl == VD_IMPL_TC_SPLIT) && !can) return fail(nullptr, VD_ERR_UNSUPPORTED, "the tensor-core convolution does not support this shape");
+    *tc = d->impl == VD_IMPL_TC || d->impl == VD_IMPL_TC_SPLIT || (d->impl == VD_IMPL_AUTO && can);
     if (!*tc && a.upsample == 2 && !conv_f32_supported(a)) return fail(nullptr, VD_ERR_UNSUPPORTED, "this layer has no phase-collapsed upsampling form, or its tensors are not 16-byte aligned");
     return VD_OK;
 }
 
-// the kernel of a layer that is not the tensor-core kernel's
-static vd_conv_route_kind ffma_route(const ConvArgs& a, ConvF32Plan* plan) {
-    if (conv_thin_supported(a)) return VD_ROUTE_THIN;
-    return conv_f32_choose(a, plan) ? VD_ROUTE_F32 : VD_ROUTE_DIRECT;
+// the kernel of a layer, and its plan where that kernel has one
+struct ConvPlans { ConvSplitPlan split; ConvF32Plan f32; };
+static vd_status resolve_route(const vd_conv_desc* d, const ConvArgs& a, vd_conv_route_kind* route, ConvPlans* plans) {
+    bool tc;
+    vd_status st = resolve_impl(d, a, &tc);
+    if (st != VD_OK) return st;
+    if (d->impl == VD_IMPL_TC_SPLIT) {
+        if (!conv_split_choose(a, &plans->split)) return fail(nullptr, VD_ERR_UNSUPPORTED, "this layer's K is not divided among a cluster");
+        *route = conv_split_cluster(plans->split) == plans->split.shape.splits ? VD_ROUTE_SPLIT : VD_ROUTE_SPLIT_PAIRS;
+    } else {
+        *route = tc ? VD_ROUTE_TC : conv_thin_supported(a) ? VD_ROUTE_THIN : conv_f32_choose(a, &plans->f32) ? VD_ROUTE_F32 : VD_ROUTE_DIRECT;
+    }
+    return VD_OK;
 }
 
 vd_status vd_conv_packed_weight_bytes(const vd_conv_desc* d, size_t* bytes) {
@@ -1075,42 +1084,110 @@ vd_status vd_conv_pack_weight(const vd_conv_desc* d, const void* w_oihw, int32_t
     return e == cudaSuccess ? VD_OK : cuda_fail(nullptr, e, "vd_conv_pack_weight");
 }
 
-vd_status vd_op_conv2d(const vd_conv_desc* d, const void* x, const void* w_packed, const float* bias, const float* scale,
-                       const float* shift, const float* residual, void* y, void* cuda_stream) {
+// the descriptor's layer with what `ex` (or null) adds to it; pointers of the tensors are the caller's to fill in
+static vd_status conv_args_with_extra(const vd_conv_desc* d, const vd_conv_extra* ex, ConvArgs* a) {
+    *a = conv_args_from_desc(d);
+    if (!ex) return VD_OK;
+    if (ex->struct_size != sizeof(vd_conv_extra)) return fail(nullptr, VD_ERR_INVALID_ARG, "bad conv extra");
+    if ((ex->x2 != nullptr) != (ex->w2 != nullptr) || (ex->x2 && ex->c_in2 < 1)) return fail(nullptr, VD_ERR_INVALID_ARG, "x2, w2 and c_in2 go together");
+    if (ex->in_records && (!ex->in_gamma || !ex->in_beta || ex->in_slots < 1 || !rec_groups_ok(d->c_in, ex->in_groups)))
+        return fail(nullptr, VD_ERR_INVALID_ARG, "records of the input need gamma, beta, slots and groups of 4, 8 or 16 channels");
+    if (ex->out_groups && !rec_groups_ok(d->c_out, ex->out_groups)) return fail(nullptr, VD_ERR_INVALID_ARG, "records need groups of 4, 8 or 16 channels");
+    if (ex->x2) { a->x2 = ex->x2; a->w2 = ex->w2; a->bias2 = ex->bias2; a->Cin2 = ex->c_in2; }
+    if (ex->in_records) {
+        a->in_rec = (const float4*)ex->in_records; a->in_gamma = ex->in_gamma; a->in_beta = ex->in_beta;
+        a->in_slots = ex->in_slots; a->in_G = ex->in_groups; a->in_shift = rec_shift(d->c_in, ex->in_groups); a->in_eps = ex->in_eps;
+        a->in_inv_n = 1.f / ((float)d->in_h * (float)d->in_w * (float)(d->c_in / ex->in_groups));
+    }
+    return VD_OK;
+}
+
+// records per group and frame of the layer's output; 0: its kernel leaves none
+static int record_slots(const ConvArgs& a, vd_conv_route_kind route, const ConvPlans& plans, int groups) {
+    switch (route) {
+        case VD_ROUTE_THIN: return conv_thin_slots(a);
+        case VD_ROUTE_F32: return a.Cout % 32 == 0 ? conv_f32_slots(a, plans.f32, groups) : 0;
+        case VD_ROUTE_TC: return conv_tc_can_record(a) ? conv_tc_slots(a) : 0;
+        case VD_ROUTE_SPLIT: case VD_ROUTE_SPLIT_PAIRS: return a.out_nchw ? 0 : conv_split_slots(a, plans.split, groups);
+        default: return 0;
+    }
+}
+
+vd_status vd_conv_record_slots(const vd_conv_desc* d, const vd_conv_extra* ex, int32_t* slots) {
+    vd_status st = check_conv_desc(d);
+    if (st != VD_OK) return st;
+    if (!ex || !slots || ex->out_groups < 1) return fail(nullptr, VD_ERR_INVALID_ARG, "extra with out_groups and slots must be given");
+    ConvArgs a;
+    vd_conv_route_kind route;
+    ConvPlans plans{};
+    st = conv_args_with_extra(d, ex, &a);
+    if (st == VD_OK) st = resolve_route(d, a, &route, &plans);
+    if (st != VD_OK) return st;
+    *slots = record_slots(a, route, plans, ex->out_groups);
+    return *slots > 0 ? VD_OK : fail(nullptr, VD_ERR_UNSUPPORTED, "this layer's kernel leaves no statistics records");
+}
+
+vd_status vd_op_conv2d_ex(const vd_conv_desc* d, const vd_conv_extra* ex, const void* x, const void* w_packed, const float* bias,
+                          const float* scale, const float* shift, const float* residual, void* y, void* cuda_stream) {
     vd_status st = check_conv_desc(d);
     if (st != VD_OK) return st;
     if (!x || !w_packed || !y) return fail(nullptr, VD_ERR_INVALID_ARG, "NULL pointer");
     if ((scale == nullptr) != (shift == nullptr)) return fail(nullptr, VD_ERR_INVALID_ARG, "scale and shift go together");
     if (d->batch == 0) return VD_OK;
-    ConvArgs a = conv_args_from_desc(d);
-    a.x = x; a.w = w_packed; a.bias = bias; a.scale = scale; a.shift = shift; a.residual = residual; a.y = y;
-    bool tc;
-    st = resolve_impl(d, a, &tc);
+    ConvArgs a;
+    st = conv_args_with_extra(d, ex, &a);
     if (st != VD_OK) return st;
+    a.x = x; a.w = w_packed; a.bias = bias; a.scale = scale; a.shift = shift; a.residual = residual; a.y = y;
+    vd_conv_route_kind route;
+    ConvPlans plans{};
+    st = resolve_route(d, a, &route, &plans);
+    if (st != VD_OK) return st;
+    cudaStream_t s = (cudaStream_t)cuda_stream;
+    if (route == VD_ROUTE_F32 && !conv_f32_fits(a, plans.f32) && !conv_f32_choose(a, &plans.f32, 1)) route = VD_ROUTE_DIRECT;
+    if (a.in_rec && (scale || (route != VD_ROUTE_F32 && route != VD_ROUTE_SPLIT && route != VD_ROUTE_SPLIT_PAIRS)))
+        return fail(nullptr, VD_ERR_UNSUPPORTED, "this layer's kernel takes no records of its input");
+    if (a.x2 && route < VD_ROUTE_TC) return fail(nullptr, VD_ERR_UNSUPPORTED, "the fused shortcut exists in the tensor-core kernels only");
+    if (ex && ex->out_groups) {
+        if (!ex->out_records) return fail(nullptr, VD_ERR_INVALID_ARG, "out_records is NULL");
+        a.out_slots = record_slots(a, route, plans, ex->out_groups);
+        if (a.out_slots < 1) return fail(nullptr, VD_ERR_UNSUPPORTED, "this layer's kernel leaves no statistics records");
+        a.out_rec = (float4*)ex->out_records; a.out_G = ex->out_groups; a.out_shift = rec_shift(a.Cout, ex->out_groups);
+        a.out_pending = ex->out_pending;
+    }
     cudaError_t e;
-    if (tc) {
-        ConvTcPlan plan{};
-        if (a.residual && a.residual != (const float*)a.y) {
-            // the tensor-core kernel accumulates into its output: seed it with the residual
-            const size_t n = (size_t)a.B * a.H * a.W * a.Cout * sizeof(float);
-            e = a.out_dtype == VD_F32 ? cudaMemcpyAsync(a.y, a.residual, n, cudaMemcpyDeviceToDevice, (cudaStream_t)cuda_stream)
-                                      : cudaErrorInvalidValue;
-            if (e != cudaSuccess) return cuda_fail(nullptr, e, "vd_op_conv2d (a residual needs an fp32 output)");
-            a.residual = (const float*)a.y;
+    switch (route) {
+        case VD_ROUTE_TC: {
+            ConvTcPlan plan{};
+            if (a.residual && a.residual != (const float*)a.y) {
+                // the tensor-core kernel accumulates into its output: seed it with the residual
+                const size_t n = (size_t)a.B * a.H * a.W * a.Cout * sizeof(float);
+                e = a.out_dtype == VD_F32 ? cudaMemcpyAsync(a.y, a.residual, n, cudaMemcpyDeviceToDevice, s) : cudaErrorInvalidValue;
+                if (e != cudaSuccess) return cuda_fail(nullptr, e, "vd_op_conv2d (a residual needs an fp32 output)");
+                a.residual = (const float*)a.y;
+            }
+            e = conv_tc_prepare(a, &plan);
+            if (e == cudaSuccess) e = launch_conv_tc(a, plan, nullptr, s);
+            break;
         }
-        e = conv_tc_prepare(a, &plan);
-        if (e == cudaSuccess) e = launch_conv_tc(a, plan, nullptr, (cudaStream_t)cuda_stream);
-    } else {
-        ConvF32Plan plan{};
-        const bool f32 = ffma_route(a, &plan) == VD_ROUTE_F32 && (conv_f32_fits(a, plan) || conv_f32_choose(a, &plan, 1));
-        if (f32) {
-            e = conv_f32_prepare(a, &plan);
-            if (e == cudaSuccess) e = launch_conv_f32(a, plan, nullptr, (cudaStream_t)cuda_stream);
-        } else {
-            e = launch_conv_simt(a, (cudaStream_t)cuda_stream);
-        }
+        case VD_ROUTE_SPLIT:
+        case VD_ROUTE_SPLIT_PAIRS:
+            if (!conv_split_fits(a, plans.split)) return fail(nullptr, VD_ERR_UNSUPPORTED, "this device cannot hold the layer's clusters");
+            e = conv_split_prepare(a, &plans.split);
+            if (e == cudaSuccess) e = launch_conv_split(a, plans.split, nullptr, s);
+            break;
+        case VD_ROUTE_F32:
+            e = conv_f32_prepare(a, &plans.f32);
+            if (e == cudaSuccess) e = launch_conv_f32(a, plans.f32, nullptr, s);
+            break;
+        default:
+            e = launch_conv_simt(a, s);
     }
     return e == cudaSuccess ? VD_OK : cuda_fail(nullptr, e, "vd_op_conv2d");
+}
+
+vd_status vd_op_conv2d(const vd_conv_desc* d, const void* x, const void* w_packed, const float* bias, const float* scale,
+                       const float* shift, const float* residual, void* y, void* cuda_stream) {
+    return vd_op_conv2d_ex(d, nullptr, x, w_packed, bias, scale, shift, residual, y, cuda_stream);
 }
 
 vd_status vd_conv_route(const vd_conv_desc* d, const void* x, const void* w_packed, const float* bias, const float* scale,
@@ -1120,12 +1197,23 @@ vd_status vd_conv_route(const vd_conv_desc* d, const void* x, const void* w_pack
     if (!route) return fail(nullptr, VD_ERR_INVALID_ARG, "route is NULL");
     ConvArgs a = conv_args_from_desc(d);
     a.x = x; a.w = w_packed; a.bias = bias; a.scale = scale; a.shift = scale; a.residual = residual; a.y = const_cast<void*>(y);
-    bool tc;
-    st = resolve_impl(d, a, &tc);
-    if (st != VD_OK) return st;
-    ConvF32Plan plan{};
-    *route = tc ? VD_ROUTE_TC : ffma_route(a, &plan);
-    return VD_OK;
+    vd_conv_route_kind r;
+    ConvPlans plans{};
+    st = resolve_route(d, a, &r, &plans);
+    if (st == VD_OK) *route = r;
+    return st;
+}
+
+vd_status vd_op_merge_records(const void* records, int32_t slots, int32_t batch, int32_t pixels, int32_t c, int32_t groups, float eps,
+                              const float* gamma, const float* beta, const float* offset, float* scale, float* shift, void* cuda_stream) {
+    if (!records || !gamma || !beta || !scale || !shift) return fail(nullptr, VD_ERR_INVALID_ARG, "NULL pointer");
+    if (slots < 1 || batch < 0 || pixels < 1 || c < 1 || !rec_groups_ok(c, groups)) return fail(nullptr, VD_ERR_INVALID_ARG, "bad sizes of statistics records");
+    if (batch == 0) return VD_OK;
+    GnArgs a{};
+    a.B = batch; a.P = pixels; a.C = c; a.G = groups; a.eps = eps; a.gamma = gamma; a.beta = beta; a.scale = scale; a.shift = shift;
+    a.offset = offset; a.rec = (const float4*)records; a.slots = slots;
+    const cudaError_t e = launch_gn_merge(a, (cudaStream_t)cuda_stream);
+    return e == cudaSuccess ? VD_OK : cuda_fail(nullptr, e, "vd_op_merge_records");
 }
 
 size_t vd_conv_stats_scratch_bytes(int32_t batch, int32_t groups) {
@@ -1147,7 +1235,7 @@ vd_status vd_op_conv2d_stats(const vd_conv_desc* d, const void* x, const void* w
     bool tc;
     st = resolve_impl(d, a, &tc);
     if (st != VD_OK) return st;
-    if (!tc || !conv_tc_stats_supported(a, groups))
+    if (!tc || d->impl == VD_IMPL_TC_SPLIT || !conv_tc_stats_supported(a, groups))
         return fail(nullptr, VD_ERR_UNSUPPORTED, "this layer's epilogue cannot take GroupNorm statistics");
     a.stat_sum = (unsigned long long*)scratch;
     a.stat_counter = (unsigned int*)((char*)scratch + conv_stat_sum_bytes(a.B, groups));

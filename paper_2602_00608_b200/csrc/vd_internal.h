@@ -136,7 +136,8 @@ cudaError_t launch_fill_rows(float* dst, const float* src, int C, int B, cudaStr
 // ---- tcgen05 kernels (conv_tc.cu, attn_tc.cu)
 bool conv_tc_supported(const ConvArgs& a);
 bool conv_tc_stats_supported(const ConvArgs& a, int groups);   // the epilogue can take the next GroupNorm's statistics
-bool conv_tc_records_supported(const ConvArgs& a);             // the kernel can leave statistics records of this layer's output
+bool conv_tc_can_record(const ConvArgs& a);                    // the kernel can leave statistics records of this layer's output
+bool conv_tc_records_supported(const ConvArgs& a);             // and it pays
 int conv_tc_slots(const ConvArgs& a);
 bool conv_tc_pairs_available();          // can the current device co-schedule the kernels' CTA pairs?
 size_t conv_tc_packed_bytes(int Cout, int Cin, int taps, bool phase);
