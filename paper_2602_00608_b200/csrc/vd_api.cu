@@ -420,13 +420,15 @@ class Planner {
     }
 
     // Laid out twice: how much room the statistics records need is known once every layer has its kernel.
-    vd_status plan() {
+    struct Size { int rec_slots; size_t bytes; };            // of the records; of the whole plan
+    static Size measure(const vd_config& cfg, bool clusters) {
         vd_handle_s scratch;
-        scratch.cfg = cfg_;
-        Planner first(&scratch, nullptr, clusters_);
-        first.layout(0);
-        return layout(first.max_slots_);
+        scratch.cfg = cfg;
+        Planner p(&scratch, nullptr, clusters);
+        p.layout(0);
+        return {p.max_slots_, scratch.total + 2 * align_up(p.rec_bytes(p.max_slots_), 256)};
     }
+    size_t rec_bytes(int slots) const { return (size_t)cfg_.max_batch * cfg_.norm_groups * slots * sizeof(float4); }
 
     vd_status layout(int rec_slots) {
         const int h = cfg_.latent_h, w = cfg_.latent_w, B = cfg_.max_batch;
@@ -474,7 +476,7 @@ class Planner {
         stat_off_ = alloc(conv_stat_scratch_bytes(B, cfg_.norm_groups));
         h_->stat_off = stat_off_;
         h_->stat_bytes = conv_stat_scratch_bytes(B, cfg_.norm_groups);
-        for (int i = 0; i < 2; ++i) rec_buf_[i] = alloc((size_t)B * cfg_.norm_groups * rec_slots * sizeof(float4));
+        for (int i = 0; i < 2; ++i) rec_buf_[i] = alloc(rec_bytes(rec_slots));
         zbuf_ = alloc((size_t)B * P0 * lc * 4);
         xs_[0] = alloc((size_t)B * max_x * 4);
         xs_[1] = alloc((size_t)B * max_x * 4);
@@ -604,17 +606,17 @@ const vd_tensor* find_tensor(const vd_tensor* t, int n, const std::string& name)
     return nullptr;
 }
 
-size_t plan_bytes(const vd_config& cfg, bool clusters) {
-    vd_handle_s h;
-    h.cfg = cfg;
-    Planner(&h, nullptr, clusters).plan();
-    return h.total;
-}
-// Workspace of either plan: which one a device takes is known in vd_create only.
-size_t workspace_of(const vd_config& cfg) {
-    const size_t without = plan_bytes(cfg, false);
-    return (cfg.flags & VD_FLAG_NO_CLUSTERS) ? without : std::max(without, plan_bytes(cfg, true));
-}
+// Both plans of a configuration, without ([0]) and with clusters: which one a device takes is known in vd_create only, so the
+// workspace holds either.
+struct PlanSizes {
+    Planner::Size of[2];
+    size_t workspace;
+    explicit PlanSizes(const vd_config& cfg) {
+        of[0] = Planner::measure(cfg, false);
+        of[1] = (cfg.flags & VD_FLAG_NO_CLUSTERS) ? of[0] : Planner::measure(cfg, true);
+        workspace = std::max(of[0].bytes, of[1].bytes);
+    }
+};
 
 // Can the current device hold the clusters of the plan's steps?
 bool plan_fits(const vd_handle_s& h) {
@@ -721,7 +723,7 @@ vd_status vd_query_workspace(const vd_config* cfg, size_t* bytes) {
     vd_status st = validate_cfg(cfg, err);
     if (st != VD_OK) return fail(nullptr, st, err);
     if (!bytes) return fail(nullptr, VD_ERR_INVALID_ARG, "bytes is NULL");
-    *bytes = workspace_of(*cfg);
+    *bytes = PlanSizes(*cfg).workspace;
     return VD_OK;
 }
 
@@ -741,10 +743,10 @@ vd_status vd_create(const vd_config* cfg, const vd_tensor* weights, int32_t n_we
     if (e != cudaSuccess) return cuda_fail(nullptr, e, "device query");
     if (major != 10) return fail(nullptr, VD_ERR_UNSUPPORTED, "this library runs on sm_100 devices only");
 
-    const size_t need = workspace_of(*cfg);
-    if (workspace_bytes < need) {
+    const PlanSizes sizes(*cfg);
+    if (workspace_bytes < sizes.workspace) {
         char msg[128];
-        snprintf(msg, sizeof(msg), "workspace too small: %zu bytes given, %zu needed", workspace_bytes, need);
+        snprintf(msg, sizeof(msg), "workspace too small: %zu bytes given, %zu needed", workspace_bytes, sizes.workspace);
         return fail(nullptr, VD_ERR_WORKSPACE, msg);
     }
     vd_handle_s* h = nullptr;
@@ -753,7 +755,8 @@ vd_status vd_create(const vd_config* cfg, const vd_tensor* weights, int32_t n_we
         h->cfg = *cfg;
         h->ws = (char*)workspace;
         h->ws_bytes = workspace_bytes;
-        Planner(h, h->ws, clusters, need - plan_bytes(*cfg, clusters)).plan();      // (either plan ends where the workspace does)
+        const Planner::Size& size = sizes.of[clusters];
+        Planner(h, h->ws, clusters, sizes.workspace - size.bytes).layout(size.rec_slots);       // (either plan ends where the workspace does)
         if (!clusters || plan_fits(*h)) break;
         delete h;
     }
