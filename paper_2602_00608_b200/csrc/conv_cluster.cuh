@@ -39,14 +39,13 @@ __device__ __forceinline__ bool try_wait_cluster(uint32_t bar, uint32_t parity) 
                  : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
     return ok != 0u;
 }
-// bounded like mbar_wait, for data that other CTAs of the cluster have stored
+// Bounded like mbar_wait, for data that other CTAs of the cluster send.  It does not return early when a wait of this CTA has
+// already given up: the others send theirs all the same, and it must not land in shared memory that is gone.
 __device__ __forceinline__ bool wait_cluster(uint32_t bar, uint32_t parity, volatile uint32_t* abort_flag) {
     if (try_wait_cluster(bar, parity)) return true;
     const long long t0 = clock64();
-    while (!try_wait_cluster(bar, parity)) {
-        if (*abort_flag) return false;
+    while (!try_wait_cluster(bar, parity))
         if (clock64() - t0 > tc::WAIT_LIMIT_CYCLES) { *abort_flag = 1; return false; }
-    }
     return true;
 }
 

@@ -12,18 +12,27 @@ WAIT = re.compile(r"cluster_wait\(\)|cluster_sync_all\(\)|barrier\.cluster\.wait
 REMOTE = re.compile(r"st\.shared::cluster|copy_to_peer\(|mbar_arrive(?:_expect_tx)?_cluster\w*\(|commit2?_to_cluster\(|umma2_commit\w*\(")
 
 
+def source():
+    return {os.path.basename(p): re.sub(r"//[^\n]*", "", open(p).read()) for p in sorted(glob.glob(os.path.join(CSRC, "*.cu*")))}
+
+
+def body_at(text, start):
+    """The braces' content from the first one after `start`."""
+    open_at = text.index("{", start)
+    depth, i = 1, open_at + 1
+    while depth:
+        depth += {"{": 1, "}": -1}.get(text[i], 0)
+        i += 1
+    return open_at, text[open_at:i]
+
+
 def kernels():
     """(name, body) of every __global__ function."""
-    for path in sorted(glob.glob(os.path.join(CSRC, "*.cu"))):
-        text = re.sub(r"//[^\n]*", "", open(path).read())
+    for file, text in source().items():
         for m in re.finditer(r"__global__", text):
-            open_at = text.index("{", m.end())
-            depth, i = 1, open_at + 1
-            while depth:
-                depth += {"{": 1, "}": -1}.get(text[i], 0)
-                i += 1
+            open_at, body = body_at(text, m.end())
             name = re.search(r"(\w+)\s*\((?!\()[^()]*\)\s*$|(\w+)\s*\(const", text[m.end():open_at])
-            yield os.path.basename(path), name.group(1) or name.group(2), text[open_at:i]
+            yield file, name.group(1) or name.group(2), body
 
 
 WITH_REMOTE = [(f, n, b) for f, n, b in kernels() if REMOTE.search(b)]
@@ -38,3 +47,11 @@ def test_the_cluster_kernels_are_found():
 def test_a_cluster_wait_precedes_remote_shared_memory(file, name, body):
     wait, remote = WAIT.search(body), REMOTE.search(body)
     assert wait and wait.start() < remote.start(), f"{file}: {name} reaches another CTA before it is known to run"
+
+
+def test_what_other_ctas_send_is_waited_for_after_a_wait_gave_up():
+    """The other CTAs of the cluster send their partial sums in any case: only the limit may end the wait for them."""
+    text = source()["conv_cluster.cuh"]
+    body = body_at(text, text.index("bool wait_cluster("))[1]
+    assert "WAIT_LIMIT_CYCLES" in body
+    assert not re.search(r"if\s*\(\s*\*abort_flag", body)
