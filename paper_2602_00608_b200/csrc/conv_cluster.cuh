@@ -49,6 +49,15 @@ __device__ __forceinline__ bool wait_cluster(uint32_t bar, uint32_t parity, vola
     return true;
 }
 
+// Where a wait gave up, loads into shared memory may still be on their way when everybody else is done: load k of `issued`
+// (into stage k % stages, counted on that stage's barrier) has landed when this returns, or the limit has passed.
+__device__ __forceinline__ void land_loads(const uint64_t* full, int stages, int issued) {
+    for (int k = max(issued - stages, 0); k < issued; ++k) {
+        const long long t0 = clock64();
+        while (!tc::mbar_try_wait(tc::smem_u32(full + k % stages), (k / stages) & 1) && clock64() - t0 < tc::WAIT_LIMIT_CYCLES) {}
+    }
+}
+
 // The launch's parameters come through the constant cache, a line at a time: one warp reads a word of every line while the
 // kernel before is still running, so that nobody waits for the first use of one later.  (The sum goes to an unused word of
 // shared memory, or nothing would be read.)

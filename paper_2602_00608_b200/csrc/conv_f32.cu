@@ -61,6 +61,7 @@ struct FBars {
     uint64_t w_full[kMaxW];
     uint64_t rx_full;
     uint32_t abort_flag, unused;
+    int issued;                                              // weight loads
 };
 
 // Geometry of a build: a tile of TH x TW pixels (a thread has eight pixels of a row).  BN = 4: the frame head (at most four
@@ -79,6 +80,7 @@ template <int TH, int BN, int KIND, int TW = 8> struct FCfg {
 };
 constexpr int kMaxSlice = 512, kMaxSplits = kF32MaxSplits;   // input channels of one CTA; CTAs of a cluster
 constexpr int kFTail = 2 * kMaxSlice * 4 + 128;              // scale / shift of the slice, barriers
+static_assert(sizeof(FBars) <= 128, "barrier block");
 
 // A partial lies in memory as rows (pixels) of BN floats whose 16-byte pieces are permuted by the row, so that neither the
 // threads that write it (eight tile rows side by side) nor those that read it (eight pixels of a row) meet on a bank.
@@ -128,6 +130,7 @@ conv_f32_kernel(const ConvArgs a, const int S, const int n_w, const int ops_floa
         for (int i = 0; i < kMaxW; ++i) mbar_init(smem_u32(&bars->w_full[i]), 1);
         mbar_init(smem_u32(&bars->rx_full), 1);
         bars->abort_flag = 0;
+        bars->issued = HEAD ? 0 : min(units, n_w);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         fence_proxy_async_smem();
         mbar_arrive_expect_tx(smem_u32(&bars->rx_full), C::RX_FLOATS * 4);           // this CTA's rows from all S * KT partials
@@ -225,7 +228,10 @@ conv_f32_kernel(const ConvArgs a, const int S, const int n_w, const int ops_floa
         if (u + 1 < units) fetch(u + 1);
         __syncthreads();                                     // chunk u is complete; every thread is done with chunk u - 1
         if (!HEAD) {
-            if (tid == 0 && u > 0 && u - 1 + n_w < units) load_weights(u - 1 + n_w);
+            if (tid == 0 && u > 0 && u - 1 + n_w < units && !*abort_flag) {
+                bars->issued = u + n_w;
+                load_weights(u - 1 + n_w);
+            }
             (void)mbar_wait(smem_u32(&bars->w_full[u % n_w]), (u / n_w) & 1, abort_flag);
         }
         const float* ip = buf + row * ROW + ng * 8;
@@ -316,8 +322,9 @@ conv_f32_kernel(const ConvArgs a, const int S, const int n_w, const int ops_floa
                                 cluster_arrive();            // what is sent to this CTA has landed
                             }
                         });
-    if (tid == 0 && bars->abort_flag && status) {
-        if (atomicCAS(status, 0u, kStatusConvTimeout) == 0u) {
+    if (tid == 0 && bars->abort_flag) {
+        land_loads(bars->w_full, n_w, bars->issued);
+        if (status && atomicCAS(status, 0u, kStatusConvTimeout) == 0u) {
             status[1] = blockIdx.x;
             status[2] = (uint32_t)BN;
         }

@@ -228,14 +228,9 @@ conv_split_kernel(const ConvArgs a, const ConvSplitShape sh, const __grid_consta
                     if (++st == (uint32_t)n_b) { st = 0; ph ^= 1; }
                 }
             }
-            if (!ok) {                                       // unwinding: let the copies in flight land first
-                for (int k = 0; k < min(issued, n_b); ++k) {
-                    if (st == 0) { st = n_b; ph ^= 1; }
-                    --st;
-                    const long long t0 = clock64();
-                    while (!mbar_try_wait(smem_u32(&bars->b_full[st]), ph) && clock64() - t0 < WAIT_LIMIT_CYCLES) {}
-                }
-            }
+            // what a CTA that gave up has on its way lands before the others may leave (the last arrival below)
+            (void)mbar_wait(smem_u32(&bars->acc_full), 0, abort_flag);
+            if (*abort_flag) land_loads(bars->b_full, n_b, issued);
         }
         __syncwarp();
         cluster_wait();
@@ -486,14 +481,10 @@ conv_pair_kernel(const ConvArgs a, const ConvSplitShape sh, const __grid_constan
                     if (++st == (uint32_t)n_b) { st = 0; ph ^= 1; }
                 }
             }
-            if (!ok) {                                       // unwinding: let the copies in flight land first (the odd CTA cannot see that: it waits the limit)
-                for (int k = 0; k < min(issued, n_b); ++k) {
-                    if (st == 0) { st = n_b; ph ^= 1; }
-                    --st;
-                    const long long t0 = clock64();
-                    while (!mbar_try_wait(smem_u32(&bars->b_full[st]), ph) && clock64() - t0 < WAIT_LIMIT_CYCLES) {}
-                }
-            }
+            // what a pair that gave up has on its way lands before anybody may leave (the last arrival below); both halves are
+            // counted on the even CTA's barriers
+            (void)mbar_wait(smem_u32(&bars->acc_full), 0, abort_flag);
+            if (half == 0 && *abort_flag) land_loads(bars->b_full, n_b, issued);
         }
     } else if (warp == 0) {
         // ------------------------------------------------ MMA issue (warp-uniform, predicated on one elected lane)

@@ -55,3 +55,16 @@ def test_what_other_ctas_send_is_waited_for_after_a_wait_gave_up():
     body = body_at(text, text.index("bool wait_cluster("))[1]
     assert "WAIT_LIMIT_CYCLES" in body
     assert not re.search(r"if\s*\(\s*\*abort_flag", body)
+
+
+def test_loads_on_their_way_land_after_a_wait_gave_up():
+    """A CTA whose wait ran into its limit must not end, or reuse the stages, while bulk loads are on their way into them."""
+    for name in ("conv_split_kernel", "conv_pair_kernel", "conv_f32_kernel"):
+        body = next(b for _, n, b in kernels() if n == name)
+        landed = re.search(r"abort_flag\)\s*\{?\s*land_loads\(", body)
+        assert landed, name
+        if name == "conv_f32_kernel":                        # and nothing new is loaded
+            assert re.search(r"!\*abort_flag\) \{\s*bars->issued = u \+ n_w;\s*load_weights\(", body)
+        else:                                                # whatever wait it was: once the accumulators are complete, before the last arrival
+            wait = body.rindex("mbar_wait(smem_u32(&bars->acc_full)", 0, landed.start())
+            assert landed.start() - wait < 200 and landed.start() < body.rindex("cluster_arrive()")
