@@ -86,7 +86,9 @@ typedef struct {
     int32_t latent_channels;    /* 4 */
     int32_t out_channels;       /* 3 */
     int32_t latent_h, latent_w; /* frames are 8*latent_h x 8*latent_w */
-    int32_t max_batch;          /* largest `batch` vd_decode will be given */
+    int32_t max_batch;          /* largest `batch` vd_decode will be given.  A handle's kernels, and the order of their
+                                   sums, are chosen for it: a frame's bits do not depend on the batch of the call, but they
+                                   differ (by rounding) between handles of different max_batch */
     int32_t norm_groups;        /* 32 (SDVAE) / 8 (TINY) in the benchmark configurations */
     float norm_eps;             /* 1e-6 */
     uint32_t flags;

@@ -659,9 +659,11 @@ int conv_split_slots(const ConvArgs& a, const ConvSplitPlan& p, int groups) {
 // Measured with both (one B200): up to there a layer with its normalisation takes 8-12 us against 25-45 on conv_tc.cu;
 // with 512 channels per CTA (256x256 frame, 64x64 level) this kernel's narrow channel blocks stream the weights four
 // times as often as conv_tc.cu's, and a 424x296 frame took 1.73 instead of 1.57 ms.
-// Beyond, 3x3 layers run on pairs with K in two as long as the clusters of four fit the chip at once (33 of them): a layer with
-// its normalisation 22 us against 40 on conv_tc.cu (64x64 and 37x53 pixels, 512 channels); 256x256 frame 1016 -> 957 us,
-// 424x296 1534 -> 1455.  Pairs without the division (60x90, 74x106) gain nothing over conv_tc.cu.
+// Beyond, 3x3 layers run on pairs with K in two as long as the clusters of four fit the chip at once (33 of them; from 10, where
+// 64-channel blocks no longer do): a layer with its normalisation 22 us against 40 on conv_tc.cu (64x64 and 37x53 pixels, 512
+// channels, 32 and 22 pairs); 256x256 frame 1016 -> 957 us, 424x296 1534 -> 1455; with 10, 12 and 14 pairs at the second level
+// (160x128, 192x128, 224x128 frames) 790 -> 736, 810 -> 755, 802 -> 744.  Pairs without the division (60x90, 74x106) gain
+// nothing over conv_tc.cu.  (296 and 132: two CTAs and 0.9 CTAs per SM of 148; on fewer SMs the layers take more waves.)
 bool conv_split_choose(const ConvArgs& a, ConvSplitPlan* p) {
     p->valid = 0;
     if (!conv_split_supported(a)) return false;

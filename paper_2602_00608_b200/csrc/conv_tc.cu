@@ -1614,12 +1614,13 @@ bool conv_tc_stats_supported(const ConvArgs& a, int groups) {
 // 480x720 230 + 38 -> 236 + 21.  Where the epilogue paces the layer it loses: 128->128 at 480x720 109 + 27 -> 172 + 20, phase
 // form 256->256 to 480x720 186 + 64 -> 337 + 21.
 // Large 3x3 layers run as CTA pairs: the chip is at its power limit there, and a pair reads each weight from L2 once instead of
-// twice and feeds each tensor core half of it from shared memory.  256-channel blocks, from ten tiles per SM: eight 720x480
-// frames per decode 26.34 -> 25.80 ms, two 1280x720 frames 18.20 -> 17.85; below, the signals between the two CTAs cost more
-// than they save (one 720x480 frame, whose layers have 96 to 675 tiles: 3.57 -> 3.64 ms).  128-channel blocks, whose MMAs take
-// as many bytes of weights as of operand from shared memory (and would be limited by it), from seven tiles per SM:
-// 128->128 at 480x720 109 -> 98 us, 256->128 188 -> 173; eight 720x480 frames 25.87 -> 25.47 ms, two 1280x720 17.87 -> 17.60;
-// a 256x256 frame (512 tiles) 0.958 -> 0.961.
+// twice and feeds each tensor core half of it from shared memory.  256-channel blocks, from 1500 items (tile x block): eight
+// 720x480 frames per decode 26.34 -> 25.80 ms, two 1280x720 frames 18.20 -> 17.85; below, the signals between the two CTAs cost
+// more than they save (one 720x480 frame, whose layers have 96 to 675 tiles: 3.57 -> 3.64 ms).  128-channel blocks, whose MMAs
+// take as many bytes of weights as of operand from shared memory (and would be limited by it), from 1000 items:
+// 128->128 at 480x720 109 -> 98 us, 256->128 188 -> 173; eight 720x480 frames 25.87 -> 25.47 ms, two 1280x720 17.87 -> 17.60.
+// Whole decodes by the tiles of their last level, one CTA -> pairs: 512 (256x256) 956 -> 959 us; 640 1256 -> 1252, 768 1320 -> 1321,
+// 880 1350 -> 1349, 1007 (424x296) 1487-1515 -> 1476-1511: no difference from 640 to 1007, so the line may lie anywhere there.
 static bool wide_layer(const ConvArgs& a) {
     if (a.Cout % 128 != 0 || a.ksize != 3 || a.upsample || a.x2 || a.out_nchw || a.out_u8) return false;
     const bool b256 = a.Cout % 256 == 0;

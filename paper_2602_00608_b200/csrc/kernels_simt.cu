@@ -701,8 +701,10 @@ bool gn_takes_clusters(const GnArgs& a) {
     // Up to here the clusters' few CTAs read a sample faster than the other kernel's phases run (the line depends on the
     // sample size only, like everything below).  Measured by itself, one sample, us, other kernel -> this one, a 2 us memset
     // included in both: 512 channels 32x32 10.3 -> 6.3, 60x90 10.4 -> 8.2; 256 channels 128x128 12.2 -> 8.6, bf16 240x360
-    // 14.5 -> 20.7; 128 channels 296x424 14.5 -> 16.5.  Whole decodes: 424x296 1565 -> 1536 us with the line at 3 million
-    // elements, 1567 at 12 million and 1666 at 20 million (the next layer's lines leave L2 later).
+    // 14.5 -> 20.7; 128 channels 296x424 14.5 -> 16.5.  The line is that of whole decodes, where the other kernel's pass leaves
+    // the next layer's lines in L2: 424x296 1565 -> 1536 us with it at 3 million elements, 1567 at 12 million, 1666 at 20 million;
+    // from 3 to 4.5 million (256 channels at 128x128 then come here) 256x256 957 -> 962, 288x224 1062 -> 1067, 320x192
+    // 1007 -> 1013, 424x296 1470 -> 1472, four 256x256 frames 2648 -> 2634.
     return !a.no_clusters && a.C % 16 == 0 && (spg == 1 || spg == 2 || spg == 4) && (long long)a.P * a.C <= 3000000;
 }
 

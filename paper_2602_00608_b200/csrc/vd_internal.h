@@ -23,11 +23,11 @@ struct ConvArgs {
     int H, W;               // output resolution (= source, or 2x source with upsample)
     int Cin, Cout, ksize;
     int upsample;           // 0 none; 1 nearest-2x folded into the addressing (9 taps on the 2x grid); 2 phase-collapsed
-                            // (four 2x2 convolutions of the source with pre-summed weights; tensor-core kernel only)
+                            // (four 2x2 convolutions of the source with pre-summed weights; not in the direct kernel)
     int silu;
     int in_dtype, out_dtype, out_nchw, bf16_operands;
     int out_u8;             // 1: y is the display-packed frame, NHWC uint8 [B,H,W,Cout] (out_dtype and out_nchw are ignored)
-    // optional fused 1x1 shortcut (tensor-core kernel only): y += W2 * x2 + bias2
+    // optional fused 1x1 shortcut (tensor-core kernels only): y += W2 * x2 + bias2
     const void* x2;         // fp32 NHWC [B,H,W,Cin2] at the output resolution, or null
     const void* w2;         // fp32 [Cout][Cin2] (tensor-core kernel: the shortcut's products are tf32)
     const float* bias2;     // [Cout] or null
@@ -114,7 +114,7 @@ inline bool aligned16(const void* p) { return ((uintptr_t)p & 15) == 0; }
 
 // ---- FFMA kernels (kernels_simt.cu)
 cudaError_t launch_ingest(const IngestArgs& a, cudaStream_t s);
-cudaError_t launch_gn_stats(const GnArgs& a, cudaStream_t s);          // one launch (the last block per sample finalises)
+cudaError_t launch_gn_stats(const GnArgs& a, cudaStream_t s);          // one launch
 bool gn_takes_clusters(const GnArgs& a);                       // by the sample's size; the device is not asked
 bool gn_clusters_fit();                                        // on the current device
 cudaError_t launch_conv_simt(const ConvArgs& a, cudaStream_t s);
