@@ -55,11 +55,14 @@ __device__ __forceinline__ void umma2_bf16_split_on(uint32_t d_tmem, uint32_t a_
         "@q tcgen05.mma.cta_group::2.kind::f16 [%0], da, db, %5, p;\n}\n"
         ::"r"(d_tmem), "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(accumulate), "r"(on) : "memory");
 }
-__device__ __forceinline__ void umma2_commit_both_on(uint32_t bar, uint32_t on) {
-    const uint32_t peer = map_to_cta(bar, 1);
+// arrives, once the MMAs issued so far have completed, on a barrier of this CTA and one of its peer (a cluster address)
+__device__ __forceinline__ void umma2_commit_pair_on(uint32_t bar, uint32_t peer_bar, uint32_t on) {
     asm volatile("{\n.reg .pred q;\nsetp.ne.b32 q, %2, 0;\n"
                  "@q tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];\n"
-                 "@q tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%1];\n}\n" ::"r"(bar), "r"(peer), "r"(on) : "memory");
+                 "@q tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%1];\n}\n" ::"r"(bar), "r"(peer_bar), "r"(on) : "memory");
+}
+__device__ __forceinline__ void umma2_commit_both_on(uint32_t bar, uint32_t on) {
+    umma2_commit_pair_on(bar, map_to_cta(bar, 1), on);
 }
 // arrives (once the MMAs issued so far have completed) on the barrier at this offset in both CTAs of the pair:
 // one commit to the leader's own barrier, one to the peer's through its cluster address

@@ -399,7 +399,7 @@ class Planner {
         s.kind = VD_STEP_ATTENTION;
         const int es = elt(act_dtype());
         s.attn = AttnArgs{ptr<void>(qkv_), ptr<void>(qkv_ + (size_t)C * es), ptr<void>(qkv_ + (size_t)2 * C * es),
-                          ptr<void>(attno_), act_dtype(), 0, H * W, C, 3 * C, C, 1.0f / sqrtf((float)C), ptr<void>(vt_)};
+                          ptr<void>(attno_), act_dtype(), 0, H * W, C, 3 * C, C, 1.0f / sqrtf((float)C), ptr<void>(vt_), clusters_ ? 0 : 1};
         s.use_tc = bf16() && !(cfg_.flags & VD_FLAG_FORCE_SIMT) && attn_tc_supported(s.attn);
         fill_info(s, p + ".core", s.use_tc, C, C, 0, 0, H, W, C, act_dtype(), 0, (long)attno_);
         if (s.use_tc) s.info.launches = 2;               // V transpose + attention core
@@ -822,6 +822,13 @@ vd_status vd_create(const vd_config* cfg, const vd_tensor* weights, int32_t n_we
             AttnArgs pa = st.attn;
             pa.B = cfg->max_batch;
             e = attn_tc_prepare(pa, &st.attn_tc);
+            if (e == cudaErrorInvalidConfiguration) {       // the device holds no CTA pair
+                st.use_tc = false;
+                st.info.impl = VD_IMPL_SIMT;
+                st.info.launches = 1;
+                continue;
+            }
+            if (e == cudaSuccess && st.attn_tc.splits > 1) st.info.cluster = 2 * st.attn_tc.splits;
             if (e != cudaSuccess) { delete h; return cuda_fail(nullptr, e, "attention tensor maps"); }
         }
     }
@@ -1288,7 +1295,7 @@ vd_status vd_op_attention(const void* q, const void* k, const void* v, void* o, 
     if (impl < VD_IMPL_AUTO || impl > VD_IMPL_TC) return fail(nullptr, VD_ERR_INVALID_ARG, "bad impl");
     if (batch == 0) return VD_OK;
     AttnArgs a{q, k, v, o, dtype, batch, tokens, channels, ld_qkv, ld_o, scale, scratch};
-    const bool can = attn_tc_supported(a) && scratch != nullptr;
+    const bool can = attn_tc_supported(a) && scratch != nullptr && attn_tc_available();
     if (impl == VD_IMPL_TC && !can) return fail(nullptr, VD_ERR_UNSUPPORTED, "the tensor-core attention does not support this shape");
     const bool tc = impl == VD_IMPL_TC || (impl == VD_IMPL_AUTO && can);
     cudaError_t e = tc ? launch_attn_tc(a, nullptr, nullptr, (cudaStream_t)cuda_stream) : launch_attn_simt(a, (cudaStream_t)cuda_stream);

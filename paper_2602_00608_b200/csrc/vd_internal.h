@@ -91,6 +91,7 @@ struct AttnArgs {
     int B, T, C, ld_qkv, ld_o;
     float scale;
     void* vt;               // scratch for the tensor-core kernel: V transposed, [B][C][round_up(T,64)] bf16
+    int no_clusters;        // 1: the keys are not divided among a cluster
 };
 
 struct IngestArgs {
@@ -215,12 +216,14 @@ cudaError_t conv_split_prepare(const ConvArgs& a, ConvSplitPlan* plan);
 cudaError_t launch_conv_split(const ConvArgs& a, const ConvSplitPlan& plan, unsigned int* status_word, cudaStream_t s);
 
 bool attn_tc_supported(const AttnArgs& a);
+bool attn_tc_available();               // can the current device hold the kernel's CTA pairs?
 size_t attn_tc_scratch_bytes(int B, int T, int C);
 // Launch-invariant state of the tensor-core attention: the TMA descriptors of q, k and the transposed v.
 struct alignas(64) AttnTcPlan {
     unsigned char tq[128], tk[128], tv[128];
     const void* q; const void* k; const void* vt;
     int batch, tokens, valid;
+    int splits;                 // CTA pairs that share the keys of a query tile; 0: the kernel of up to 128 tokens
 };
 cudaError_t attn_tc_prepare(const AttnArgs& a, AttnTcPlan* plan);      // a.B = the largest batch the plan must serve
 cudaError_t launch_attn_tc(const AttnArgs& a, const AttnTcPlan* plan, unsigned int* status_word, cudaStream_t s);
