@@ -283,12 +283,17 @@ attn_tc_kernel(const AttnTcParams a, const __grid_constant__ CUtensorMap tm_q, c
                 if (j + 1 < j1) load_k(j + 1);
                 if (ok) load_v(j);
             }
+            // Everything has landed once it has been multiplied.  If a wait gave up anywhere, what is on its way lands before the
+            // CTA's memory goes (counted in the pair's first CTA; the other one lets the limit pass).
+            for (int k = 0; k < STAGES && ok; ++k) {
+                ok = mbar_wait(smem_u32(&bars->empty[st]), ph ^ 1, abort_flag);
+                if (ok && ++st == STAGES) { st = 0; ph ^= 1; }
+            }
             if (!ok) {
-                // unwinding: let the copies already in flight land before the CTA's memory is released
+                const long long t0 = clock64();
                 for (int k = 0; k < min(issued, STAGES); ++k) {
                     if (st == 0) { st = STAGES; ph ^= 1; }
                     --st;
-                    const long long t0 = clock64();
                     while (!mbar_try_wait(smem_u32(&bars->full[st]), ph) && clock64() - t0 < WAIT_LIMIT_CYCLES) {}
                 }
             }
