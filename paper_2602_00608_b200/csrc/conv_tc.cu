@@ -280,26 +280,6 @@ template <class Cfg> __host__ __device__ constexpr int tail_bufs(bool rec) {
     const int n = Cfg::SMEM_B / (4 * WARP_SLICE_BYTES) >= 2 ? Cfg::SMEM_B / (4 * WARP_SLICE_BYTES) : 2;
     return rec && n > 4 ? 4 : n;
 }
-__device__ __forceinline__ unsigned long long add2(unsigned long long a, unsigned long long b) {
-    unsigned long long r;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ unsigned long long sqacc2(unsigned long long d, unsigned long long q) {
-    unsigned long long r;
-    asm("fma.rn.f32x2 %0, %1, %1, %2;" : "=l"(r) : "l"(d), "l"(q));
-    return r;
-}
-__device__ __forceinline__ unsigned long long pack2(float x, float y) {
-    unsigned long long r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
-    return r;
-}
-__device__ __forceinline__ float sum2(unsigned long long v) {
-    float x, y;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(v));
-    return x + y;
-}
 template <class Cfg, int BN, bool OUT_BF16>
 __device__ __forceinline__ void rec_warp(const ConvArgs& a, const Sched& sched, Bars* bars, RecBars* rbars, const uint8_t* smem_out, const uint8_t* smem_b,
                                          float* s_pend, int j, int lane) {
@@ -378,7 +358,7 @@ __device__ __forceinline__ void rec_warp(const ConvArgs& a, const Sched& sched, 
                                                                    : pack2(__uint_as_float(v[it].z), __uint_as_float(v[it].w));
                             const unsigned long long d0 = add2(x0, ko[h][0]), d1 = add2(x1, ko[h][1]);
                             s[h][0] = add2(s[h][0], d0); s[h][1] = add2(s[h][1], d1);
-                            q[h][0] = sqacc2(d0, q[h][0]); q[h][1] = sqacc2(d1, q[h][1]);
+                            q[h][0] = fmaf2(d0, d0, q[h][0]); q[h][1] = fmaf2(d1, d1, q[h][1]);
                         }
                     }
                 }

@@ -13,6 +13,8 @@ namespace vd {
 
 namespace {
 
+using namespace tc;
+
 template <typename T> __device__ __forceinline__ float ld_f(const T* p, size_t i);
 template <> __device__ __forceinline__ float ld_f<float>(const float* p, size_t i) { return p[i]; }
 template <> __device__ __forceinline__ float ld_f<__nv_bfloat16>(const __nv_bfloat16* p, size_t i) {
@@ -244,7 +246,321 @@ __global__ void __launch_bounds__(kGnThreads, 2) gn_stats_kernel(GnArgs a, int c
     if (threadIdx.x == 0) a.counters[n] = 0u;        // ready for the next launch
 }
 
-// The same statistics for tensors small enough that the pass above is mostly its own latency: a cluster of eight CTAs
+__device__ __forceinline__ void bulk_load_stream(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar, uint64_t pol) {
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1], %2, [%3], %4;"
+                 ::"r"(dst), "l"(src), "r"(bytes), "r"(bar), "l"(pol) : "memory");
+}
+
+// ---- the pass for handles whose decodes may be of several frames
+constexpr int kGnBlocks = 296;                            // two per SM of a 148-SM device (a block waits for no other)
+constexpr int kGnStages = 4, kGnStageBytes = 16384;
+constexpr unsigned int kGnMine = 0x40000000u;
+
+// What a thread knows and adds up: a 16-byte piece of a pixel (one or two quads of channels) of every `rows`-th pixel.
+template <typename T> struct GnSums {
+    static constexpr int E = 16 / (int)sizeof(T), Q = E / 4;
+    int cpg, quads, ppp, rows, piece, row;               // channels of a group; quads and pieces of a pixel; pixels side by side
+    bool on;
+    float off_k[Q], off_c[E];                            // what a per-channel offset adds: to the quads' references, to the channels
+    float kv[Q][4];                                      // raw reference pixels
+    unsigned long long nk[E / 2], s[Q], ss[Q];           // minus the references (the offset taken in); sums by channel parity
+    __device__ __forceinline__ void init(const GnArgs& a, int tid) {
+        cpg = a.C / a.G; quads = a.C / 4; ppp = a.C / E; rows = kGnThreads / ppp;
+        piece = tid % ppp; row = tid / ppp; on = row < rows;
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+            const int c = piece * E + q * 4;
+            off_k[q] = 0.f;
+            off_c[4 * q] = off_c[4 * q + 1] = off_c[4 * q + 2] = off_c[4 * q + 3] = 0.f;
+            if (a.offset) {
+                const float4 og = __ldg((const float4*)(a.offset + c / cpg * cpg)), oc = __ldg((const float4*)(a.offset + c));
+                off_k[q] = 0.25f * ((og.x + og.y) + (og.z + og.w));
+                off_c[4 * q] = oc.x; off_c[4 * q + 1] = oc.y; off_c[4 * q + 2] = oc.z; off_c[4 * q + 3] = oc.w;
+            }
+        }
+    }
+    __device__ __forceinline__ void load_refs(const GnArgs& a, int n) {
+#pragma unroll
+        for (int q = 0; q < Q; ++q) load4<T>((const T*)a.x + ((size_t)n * a.P + a.P / 2) * a.C + (piece * E + q * 4) / cpg * cpg, kv[q]);
+    }
+    __device__ __forceinline__ void start() {
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+            // d = (x + off) - k = x - (k - off)
+            const float k = 0.25f * ((kv[q][0] + kv[q][1]) + (kv[q][2] + kv[q][3])) + off_k[q];
+            nk[2 * q] = pack2(off_c[4 * q] - k, off_c[4 * q + 1] - k);
+            nk[2 * q + 1] = pack2(off_c[4 * q + 2] - k, off_c[4 * q + 3] - k);
+            s[q] = ss[q] = 0ull;
+        }
+    }
+    __device__ __forceinline__ void add(const uint4& r) {
+        const uint32_t w[4] = {r.x, r.y, r.z, r.w};
+#pragma unroll
+        for (int e = 0; e < E / 2; ++e) {
+            const unsigned long long v = sizeof(T) == 4 ? pack2(__uint_as_float(w[(2 * e) & 3]), __uint_as_float(w[(2 * e + 1) & 3]))
+                                                        : pack2(__uint_as_float(w[e] << 16), __uint_as_float(w[e] & 0xffff0000u));
+            const unsigned long long d = add2(v, nk[e]);
+            s[e / 2] = add2(s[e / 2], d);
+            ss[e / 2] = fmaf2(d, d, ss[e / 2]);
+        }
+    }
+    __device__ __forceinline__ void put(float2* sm) const {
+        if (!on) return;
+#pragma unroll
+        for (int q = 0; q < Q; ++q) sm[row * quads + piece * Q + q] = make_float2(sum2(s[q]), sum2(ss[q]));
+    }
+    // A group's members in the block, rows x (quads of the group), added by 2 to 32 neighbouring threads: valid in the first
+    // of them, which are the threads with (tid & (lanes - 1)) == 0, group tid / lanes.
+    __device__ __forceinline__ float2 group(const float2* sm, int G, int tid, int lanes) const {
+        const int g = tid / lanes, qpg = cpg / 4;
+        float2 acc = make_float2(0.f, 0.f);
+        if (g < G)
+            for (int e = tid & (lanes - 1); e < rows * qpg; e += lanes) {
+                const int r = (qpg & (qpg - 1)) == 0 ? e >> (__ffs(qpg) - 1) : e / qpg;
+                const float2 v = sm[r * quads + g * qpg + (e - r * qpg)];
+                acc.x += v.x;
+                acc.y += v.y;
+            }
+        for (int d = lanes >> 1; d > 0; d >>= 1) {
+            acc.x += __shfl_xor_sync(0xffffffffu, acc.x, d);
+            acc.y += __shfl_xor_sync(0xffffffffu, acc.y, d);
+        }
+        return acc;
+    }
+};
+
+// Folds sample n's records into scale and shift, by the 512 summing threads: thread t adds the records k = t / G,
+// t / G + slices, ... of group t % G (a warp reads whole records: coalesced), the slices are added in a fixed order through
+// shared memory, and every thread then writes scale and shift of the channels c = t, t + 512, ...
+template <typename T>
+__device__ __forceinline__ void gn_fold(const GnArgs& a, int n, int chunks, int tid, float2* sm, float* s_mean, float* s_rstd) {
+    constexpr int kLoads = 8;
+    const int cpg = a.C / a.G;
+    float ref = 0.f;
+    if (tid < a.G) {
+        float kf[4];
+        load4<T>((const T*)a.x + ((size_t)n * a.P + a.P / 2) * a.C + tid * cpg, kf);
+        ref = 0.25f * ((kf[0] + kf[1]) + (kf[2] + kf[3]));
+        if (a.offset) {
+            const float4 of = __ldg((const float4*)(a.offset + tid * cpg));
+            ref += 0.25f * ((of.x + of.y) + (of.z + of.w));
+        }
+    }
+    __threadfence();
+    const int slices = kGnThreads / a.G;                 // >= 1 (checked by the launcher)
+    const int g = tid % a.G, sl = tid / a.G;
+    float2 acc = make_float2(0.f, 0.f);
+    if (sl < slices) {
+        const float2* rec = (const float2*)a.partial + (size_t)n * kGnMaxChunks * a.G + g;
+        for (int k0 = sl; k0 < chunks; k0 += kLoads * slices) {
+            float2 r[kLoads];
+#pragma unroll
+            for (int i = 0; i < kLoads; ++i) {               // (a record that does not exist re-reads the first and counts as zero)
+                const int k = k0 + i * slices;
+                const float2* q = rec + (size_t)(k < chunks ? k : sl) * a.G;
+                asm volatile("ld.global.cg.v2.f32 {%0, %1}, [%2];" : "=f"(r[i].x), "=f"(r[i].y) : "l"(q));
+            }
+#pragma unroll
+            for (int i = 0; i < kLoads; ++i) {
+                const bool in = k0 + i * slices < chunks;
+                acc.x += in ? r[i].x : 0.f;
+                acc.y += in ? r[i].y : 0.f;
+            }
+        }
+    }
+    sm[tid] = acc;
+    named_barrier_sync(1, kGnThreads);
+    if (tid < a.G) {
+        float2 t = make_float2(0.f, 0.f);
+#pragma unroll 4
+        for (int q = 0; q < slices; ++q) {
+            const float2 v = sm[q * a.G + tid];
+            t.x += v.x;
+            t.y += v.y;
+        }
+        const float inv_n = 1.f / ((float)a.P * (float)cpg);
+        const float md = t.x * inv_n;
+        const float var = fmaxf(fmaf(-md, md, t.y * inv_n), 0.f);
+        s_mean[tid] = ref + md;
+        s_rstd[tid] = 1.f / sqrtf(var + a.eps);
+    }
+    named_barrier_sync(1, kGnThreads);
+    for (int c = tid; c < a.C; c += kGnThreads) {
+        const int gc = c / cpg;
+        const float sc = __ldg(a.gamma + c) * s_rstd[gc];
+        a.scale[(size_t)n * a.C + c] = sc;
+        a.shift[(size_t)n * a.C + c] = __ldg(a.beta + c) - (s_mean[gc] - (a.offset ? __ldg(a.offset + c) : 0.f)) * sc;
+    }
+    if (tid == 0) a.counters[n] = 0u;                    // ready for the next launch
+    named_barrier_sync(1, kGnThreads);                   // (the next fold writes the same shared memory)
+}
+
+// Records and references are those of the kernel above.  Its one block per chunk leaves every wave of 296 blocks to fill and drain
+// by itself; here the two resident blocks of an SM walk the chunks of all samples, and nothing on the way may empty the pipe:
+// bulk copies (a chunk is one run of bytes) keep 128 KB per SM under way while chunks are summed; a warp of its own writes the
+// records and arrives (a fence and an atomic take microseconds behind the loads); samples are folded after the last chunk (a
+// block that stops to fold falls behind, is last again, and delays every sample after).  Bound by memory.
+// Measured, a decode's launches, the kernel above -> this one, us: eight 720x480 frames, fp32 512 channels at 120x180 (354 MB)
+// 102 -> 66, 256 at 240x360 146 -> 122, 256 at 480x720 (2.8 GB) 442 -> 430; bf16 512 at 120x180 (177 MB) 81 -> 60, 256 at 240x360
+// 105 -> 85, 128 at 480x720 160 -> 138; four 256x256 frames 128 channels 40 -> 33; all statistics of eight frames 2.91 -> 2.54 ms.  A
+// single frame's blocks all run at once, and there this kernel's hand-overs cost 1 us more than they save (14 -> 15, 16 -> 17
+// in 256x256): handles for one frame keep the other one.
+template <typename T>
+__global__ void __launch_bounds__(kGnThreads + 64, 2) gn_batch_kernel(GnArgs a, int chunks, int pix_per_chunk, int items) {
+    constexpr int S = kGnStages, PPS = kGnStageBytes / (kGnThreads * 16);
+    using Sums = GnSums<T>;
+    extern __shared__ __align__(128) uint8_t ring[];
+    __shared__ float2 sm[kGnThreads * Sums::Q], s_rec[kGnThreads];
+    __shared__ float s_mean[kGnThreads], s_rstd[kGnThreads];
+    __shared__ uint32_t s_last;                          // bit k: this block's chunk k (below 32) was its sample's last to arrive
+    __shared__ int s_more;                               // a later one was (its counter then holds kGnMine + the block)
+    __shared__ uint64_t full[S], empty[S];
+    __shared__ uint32_t s_abort;
+    volatile uint32_t* abort_flag = &s_abort;
+    // named barriers: 1 the summing warps; 2 a chunk's sums are there; 3 they have been read; 4 all is recorded
+    constexpr int kSums = 2, kRead = 3, kDone = 4, kBoth = kGnThreads + 32;
+    griddep_launch();
+    const int tid = threadIdx.x;
+    if (tid == 0) {
+        for (int i = 0; i < S; ++i) { mbar_init(smem_u32(&full[i]), 1); mbar_init(smem_u32(&empty[i]), kGnThreads / 32); }
+        s_abort = 0u;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    __syncthreads();
+    const int rows = kGnThreads / (a.C / Sums::E);
+    const size_t pixbytes = (size_t)a.C * sizeof(T);
+    const int stage_pix = kGnStageBytes / (rows * (int)pixbytes) * rows;     // whole rounds of the block's rows
+    int n = (int)blockIdx.x / chunks, chunk = (int)blockIdx.x - n * chunks, k = 0;
+    auto next = [&]() {
+        chunk += (int)gridDim.x;
+        while (chunk >= chunks) { chunk -= chunks; ++n; }
+        ++k;
+    };
+
+    if (tid >= kGnThreads + 32) {
+        // ------------------------------------------------ loads
+        if (tid == kGnThreads + 32) {
+            const uint64_t pol = policy_evict_first();
+            uint32_t st = 0, ph = 0;
+            int issued = 0;
+            bool ok = true;
+            griddep_wait();
+            for (int item = (int)blockIdx.x; item < items && ok; item += (int)gridDim.x, next()) {
+                const int p0 = chunk * pix_per_chunk, len = min(a.P, p0 + pix_per_chunk) - p0;
+                const char* src = (const char*)a.x + ((size_t)n * a.P + p0) * pixbytes;
+                for (int p = 0; p < len; p += stage_pix) {
+                    ok = mbar_wait(smem_u32(&empty[st]), ph ^ 1u, abort_flag);
+                    if (!ok) break;
+                    const uint32_t bytes = (uint32_t)(min(stage_pix, len - p) * (int)pixbytes), bar = smem_u32(&full[st]);
+                    mbar_arrive_expect_tx(bar, bytes);
+                    bulk_load_stream(smem_u32(ring) + st * kGnStageBytes, src + (size_t)p * pixbytes, bytes, bar, pol);
+                    ++issued;
+                    if (++st == (uint32_t)S) { st = 0; ph ^= 1u; }
+                }
+            }
+            // everything has landed once it has been summed; if a wait gave up, what is on its way lands first
+            for (int i = 0; i < S && ok; ++i) {
+                ok = mbar_wait(smem_u32(&empty[st]), ph ^ 1u, abort_flag);
+                if (ok && ++st == (uint32_t)S) { st = 0; ph ^= 1u; }
+            }
+            if (!ok) {
+                const long long t0 = clock64();
+                for (int i = 0; i < min(issued, S); ++i) {
+                    if (st == 0) { st = S; ph ^= 1u; }
+                    --st;
+                    while (!mbar_try_wait(smem_u32(&full[st]), ph) && clock64() - t0 < WAIT_LIMIT_CYCLES) {}
+                }
+            }
+        }
+        return;
+    }
+    if (tid >= kGnThreads) {
+        // ------------------------------------------------ records and arrivals
+        const int lane = tid - kGnThreads;
+        griddep_wait();
+        int n_before = 0;
+        unsigned int arrived = 0, last = 0, more = 0;
+        auto look = [&](int j) {                         // the answer to the arrival of chunk j
+            if (arrived != (unsigned int)chunks - 1u) return;
+            if (j < 32) last |= 1u << j;
+            else { a.counters[n_before] = kGnMine + blockIdx.x; more = 1u; }
+        };
+        for (int item = (int)blockIdx.x; item < items; item += (int)gridDim.x, next()) {
+            named_barrier_sync(kSums, kBoth);
+            float2* rec = (float2*)a.partial + ((size_t)n * kGnMaxChunks + chunk) * a.G;
+            for (int g = lane; g < a.G; g += 32) rec[g] = s_rec[g];
+            named_barrier_arrive(kRead, kBoth);
+            __threadfence();
+            __syncwarp();
+            if (lane == 0) {
+                if (k > 0) look(k - 1);
+                arrived = atomicAdd(a.counters + n, 1u);
+            }
+            n_before = n;
+        }
+        if (lane == 0) { look(k - 1); s_last = last; s_more = (int)more; }
+        named_barrier_arrive(kDone, kBoth);
+        return;
+    }
+
+    // ---------------------------------------------------- sums
+    Sums sums;
+    sums.init(a, tid);                                   // (the offset does not depend on the kernel before this one)
+    int lanes = 32;                                      // threads that add up a group
+    while (lanes * a.G > kGnThreads) lanes >>= 1;
+    const bool even = rows * sums.ppp == kGnThreads && stage_pix * (int)pixbytes == kGnStageBytes;
+    const uint32_t slot0 = smem_u32(ring) + (uint32_t)tid * 16u;     // (the row's and the piece's place in a stage)
+    griddep_wait();
+    sums.load_refs(a, n);
+    uint32_t st = 0, ph = 0;
+    for (int item = (int)blockIdx.x; item < items; item += (int)gridDim.x, next()) {
+        const int len = min(a.P, (chunk + 1) * pix_per_chunk) - chunk * pix_per_chunk;
+        const int n_next = (item + (int)gridDim.x) / chunks;         // (another sample: a block has one chunk of each)
+        sums.start();
+        // the next sample's references, asked for a chunk ahead; from memory two ahead (a load waits behind the stream's)
+        if (n_next < a.B) sums.load_refs(a, n_next);
+        if (n_next + 1 < a.B && tid * 128 < (int)pixbytes)
+            asm volatile("prefetch.global.L2 [%0];" ::"l"((const char*)a.x + ((size_t)(n_next + 1) * a.P + a.P / 2) * pixbytes + tid * 128));
+        for (int p = 0; p < len; p += stage_pix) {
+            (void)mbar_wait(smem_u32(&full[st]), ph, abort_flag);
+            const uint32_t src = slot0 + st * kGnStageBytes;
+            if (even && len - p >= stage_pix) {          // a full stage of a width that divides it: no counting
+                uint4 w[PPS];
+#pragma unroll
+                for (int u = 0; u < PPS; ++u) w[u] = lds_u4(src + (uint32_t)(u * kGnThreads * 16));
+#pragma unroll
+                for (int u = 0; u < PPS; ++u) sums.add(w[u]);
+            } else {
+                const int cnt = sums.on ? min(stage_pix, len - p) - sums.row : 0;
+                for (int r = 0; r < cnt; r += rows) sums.add(lds_u4(src + (uint32_t)(r * sums.ppp) * 16u));
+            }
+            __syncwarp();
+            if ((tid & 31) == 0) mbar_arrive(smem_u32(&empty[st]));
+            if (++st == (uint32_t)S) { st = 0; ph ^= 1u; }
+        }
+        if (k > 0) named_barrier_sync(kRead, kBoth);     // the sums of the chunk before have been read
+        sums.put(sm);
+        named_barrier_sync(1, kGnThreads);
+        const float2 total = sums.group(sm, a.G, tid, lanes);
+        if (tid / lanes < a.G && (tid & (lanes - 1)) == 0) s_rec[tid / lanes] = total;
+        named_barrier_arrive(kSums, kBoth);
+    }
+    named_barrier_sync(kRead, kBoth);
+    named_barrier_sync(kDone, kBoth);
+    for (uint32_t m = s_last; m != 0u; m &= m - 1u)
+        gn_fold<T>(a, ((int)blockIdx.x + (__ffs((int)m) - 1) * (int)gridDim.x) / chunks, chunks, tid, sm, s_mean, s_rstd);
+    if (s_more)
+        for (int j = 32; j < k; ++j) {
+            const int nj = ((int)blockIdx.x + j * (int)gridDim.x) / chunks;
+            if (__ldcg(a.counters + nj) == kGnMine + blockIdx.x) gn_fold<T>(a, nj, chunks, tid, sm, s_mean, s_rstd);
+        }
+    if (tid == 0 && s_abort && a.status && atomicCAS(a.status, 0u, kStatusGnTimeout) == 0u) {
+        a.status[1] = blockIdx.x;
+        a.status[2] = 0u;
+    }
+}
+
+// The same statistics for tensors small enough that the passes above are mostly their own latency: a cluster of eight CTAs
 // takes 16 channels (one, two or four groups) of one sample, an eighth of its pixels each; the eight sums meet in the first
 // CTA's shared memory, and that CTA writes scale and shift: no records in memory, no arrival counter, no second reading
 // phase.  Sums are of (x - K) with the reference value K of the pass above.
@@ -712,6 +1028,17 @@ bool gn_clusters_fit() {
     return cc::clusters_fit<gn_cluster_kernel<float, 1>>(1024, 0, kGnSplit) && cc::clusters_fit<gn_cluster_kernel<__nv_bfloat16, 1>>(1024, 0, kGnSplit);
 }
 
+namespace {
+template <typename T>
+cudaError_t launch_gn_batch(const GnArgs& a, int chunks, int ppc, cudaStream_t s) {
+    constexpr int SMEM = kGnStages * kGnStageBytes;
+    const cudaError_t e = cc::set_smem_limit<gn_batch_kernel<T>>(SMEM);
+    if (e != cudaSuccess) return e;
+    const int items = chunks * a.B;
+    return launch_pdl(gn_batch_kernel<T>, dim3(min(items, kGnBlocks)), dim3(kGnThreads + 64), SMEM, s, a, chunks, ppc, items);
+}
+}  // namespace
+
 cudaError_t launch_gn_stats(const GnArgs& a, cudaStream_t s) {
     if (a.C % 4 != 0 || a.C / 4 > kGnThreads || a.G > kGnThreads || (a.C / a.G) % 4 != 0) return cudaErrorInvalidValue;
     if (gn_takes_clusters(a) && gn_clusters_fit()) {
@@ -724,7 +1051,12 @@ cudaError_t launch_gn_stats(const GnArgs& a, cudaStream_t s) {
              : spg == 2 ? launch_pdl(gn_cluster_kernel<float, 2>, grid, block, 0, s, a) : launch_pdl(gn_cluster_kernel<float, 1>, grid, block, 0, s, a);
     }
     // chunks per sample depend on the sample size only (so a frame's statistics, and with them
-    // the frame, do not depend on the batch it is decoded in): at least 32 pixels per chunk
+    // the frame, do not depend on the batch it is decoded in): at least 32 (16) pixels per chunk
+    if (!a.single && aligned16(a.x) && (a.dtype != VD_BF16 || a.C % 8 == 0)) {       // (every pixel is whole 16-byte pieces)
+        if (a.B < 1 || a.B > 65535) return cudaErrorInvalidConfiguration;
+        const int ppc = max(16, (a.P + kGnMaxChunks - 1) / kGnMaxChunks), chunks = (a.P + ppc - 1) / ppc;
+        return a.dtype == VD_BF16 ? launch_gn_batch<__nv_bfloat16>(a, chunks, ppc, s) : launch_gn_batch<float>(a, chunks, ppc, s);
+    }
     int ppc = max(32, (a.P + kGnMaxChunks - 1) / kGnMaxChunks);
     int chunks = (a.P + ppc - 1) / ppc;
     dim3 grid(chunks, a.B);

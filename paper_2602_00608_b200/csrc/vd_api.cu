@@ -189,6 +189,7 @@ class Planner {
             s.gn.slots = rec_[x_off].slots;
         }
         s.gn.no_clusters = clusters_ ? 0 : 1;
+        s.gn.single = cfg_.max_batch == 1 ? 1 : 0;
         fill_info(s, name, 0, C, C, 0, 0, H, W, C, VD_F32, 0, -1);
         s.info.launches = 1;
         if (!s.gn.rec && gn_takes_clusters(s.gn)) s.info.cluster = 8;
@@ -640,6 +641,7 @@ cudaError_t launch_step(const vd_handle_s* h, const Step& st, int B, const void*
         case VD_STEP_GN_STATS: {
             GnArgs a = st.gn;
             a.B = B;
+            a.status = status;
             return a.rec ? launch_gn_merge(a, s) : launch_gn_stats(a, s);
         }
         case VD_STEP_CONV: {
@@ -937,7 +939,7 @@ vd_status vd_get_status(vd_handle h) {
     if (word[0] != 0) {
         char msg[160];
         const char* who = word[0] == kStatusConvTimeout ? "convolution" : word[0] == kStatusAttnTimeout ? "attention"
-                          : word[0] == kStatusWaitProbe ? "wait probe" : "unknown";
+                          : word[0] == kStatusGnTimeout ? "statistics" : word[0] == kStatusWaitProbe ? "wait probe" : "unknown";
         snprintf(msg, sizeof(msg), "a %s kernel gave up on a bounded wait (code 0x%x, block %u, detail 0x%x)", who, word[0], word[1], word[2]);
         return fail(h, VD_ERR_DEVICE_TIMEOUT, msg);
     }

@@ -79,6 +79,8 @@ struct GnArgs {
     const float4* rec;      // or the producing layer's statistics records [B][G][slots] (launch_gn_merge)
     int slots;
     int no_clusters;        // 1: the kernel without clusters
+    unsigned int* status;   // status word, or null
+    int single;             // 1: B is 1 in every call that this one's results may be compared with
 };
 constexpr int kGnMaxChunks = 296;      // two blocks per SM on a 148-SM device
 // bytes of the partial records / of the whole scratch (records, then the arrival counters)
@@ -105,7 +107,7 @@ struct IngestArgs {
 };
 
 // codes the kernels latch in the status word when a bounded wait runs out
-constexpr unsigned int kStatusConvTimeout = 0xC0DE0001u, kStatusAttnTimeout = 0xC0DE0002u, kStatusWaitProbe = 0xC0DE0003u;
+constexpr unsigned int kStatusConvTimeout = 0xC0DE0001u, kStatusAttnTimeout = 0xC0DE0002u, kStatusWaitProbe = 0xC0DE0003u, kStatusGnTimeout = 0xC0DE0004u;
 cudaError_t launch_wait_probe(unsigned int* status_word, long long limit_cycles, cudaStream_t s);   // wait_probe.cu
 
 // records `msg` as the text vd_last_error(NULL) returns (defined in vd_api.cu)
