@@ -90,7 +90,8 @@ VD_API vd_status vd_debug_stop_after(vd_handle h, int32_t index);
  * ---------------------------------------------------------------------------------------- */
 typedef enum {
     VD_IMPL_AUTO = 0, VD_IMPL_SIMT = 1, VD_IMPL_TC = 2,
-    VD_IMPL_TC_SPLIT = 3        /* tcgen05 kernels that divide K among a cluster (convolutions of small images) */
+    VD_IMPL_TC_SPLIT = 3,       /* tcgen05 kernels that divide K among a cluster (convolutions of small images) */
+    VD_IMPL_TC_F32 = 4          /* single-precision 3x3 convolution on the tensor cores (operands as pairs of tf32 numbers) */
 } vd_impl;
 
 typedef struct {
@@ -133,7 +134,8 @@ typedef enum {
     VD_ROUTE_F32 = 2,           /* register-tiled FFMA kernel, 16-byte accesses, K divided among a cluster */
     VD_ROUTE_TC = 3,            /* tcgen05 kernel */
     VD_ROUTE_SPLIT = 4,         /* tcgen05 kernel, K divided among the CTAs of a cluster */
-    VD_ROUTE_SPLIT_PAIRS = 5    /* the same on CTA pairs */
+    VD_ROUTE_SPLIT_PAIRS = 5,   /* the same on CTA pairs */
+    VD_ROUTE_F32_TC = 6         /* single-precision tcgen05 kernel, K divided among a cluster */
 } vd_conv_route_kind;
 VD_API vd_status vd_conv_route(const vd_conv_desc* d, const void* x, const void* w_packed, const float* bias, const float* scale,
                                const float* residual, const void* y, int32_t* route);
@@ -146,7 +148,7 @@ typedef struct {
     const float* w2;            /* device fp32 [c_out,c_in2] */
     const float* bias2;         /* device fp32 [c_out], or NULL */
     const void* in_records;     /* statistics records of x [batch][in_groups][in_slots] of 16 bytes instead of scale and shift
-                                   (VD_ROUTE_F32, VD_ROUTE_SPLIT, VD_ROUTE_SPLIT_PAIRS) */
+                                   (VD_ROUTE_F32, VD_ROUTE_F32_TC, VD_ROUTE_SPLIT, VD_ROUTE_SPLIT_PAIRS) */
     const float* in_gamma;      /* device fp32 [c_in] */
     const float* in_beta;
     int32_t in_slots, in_groups;

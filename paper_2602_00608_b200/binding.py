@@ -20,7 +20,7 @@ VD_FLAG_OUT_U8 = 0x4
 VD_FLAG_CANARY = 0x8
 VD_FLAG_FUSED_STATS = 0x10
 VD_FLAG_NO_CLUSTERS = 0x20
-VD_IMPL_AUTO, VD_IMPL_SIMT, VD_IMPL_TC, VD_IMPL_TC_SPLIT = 0, 1, 2, 3
+VD_IMPL_AUTO, VD_IMPL_SIMT, VD_IMPL_TC, VD_IMPL_TC_SPLIT, VD_IMPL_TC_F32 = 0, 1, 2, 3, 4
 VD_ROUTE_DIRECT, VD_ROUTE_THIN, VD_ROUTE_F32, VD_ROUTE_TC, VD_ROUTE_SPLIT, VD_ROUTE_SPLIT_PAIRS = 0, 1, 2, 3, 4, 5
 VD_STEP_INGEST, VD_STEP_GN_STATS, VD_STEP_CONV, VD_STEP_ATTENTION = 0, 1, 2, 3
 STATUS_NAMES = {0: "VD_OK", -1: "VD_ERR_INVALID_ARG", -2: "VD_ERR_UNSUPPORTED", -3: "VD_ERR_WORKSPACE",

@@ -26,6 +26,7 @@ struct Step {
     ConvTcPlan tc;
     ConvSplitPlan split;         // valid: the layer runs on conv_split.cu
     ConvF32Plan f32;             // valid: the layer runs on conv_f32.cu
+    ConvF32TcPlan f32_tc;        // valid: on conv_f32_tc.cu
     AttnTcPlan attn_tc;
     bool skip;                   // statistics that the consuming layer merges from its producer's records: no launch
     // batch-dependent pointers are rebased per call: strides per frame
@@ -56,6 +57,7 @@ struct WeightJob {           // repack work done once in vd_create
     int Cout, Cin, taps;
     int cout_total, cout_offset;
     size_t dst_off;
+    bool f32_tc = false;     // fp32 weights as pairs of tf32 numbers
 };
 
 size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
@@ -132,15 +134,15 @@ class Planner {
     struct ConvW { size_t w_off, b_off; bool tc; };
 
     // registers the repack of a conv weight (possibly a stack of several source tensors along Cout)
-    ConvW conv_weight(const std::vector<std::string>& names, int Cout_each, int Cin, int taps, bool tc, bool phase) {
+    ConvW conv_weight(const std::vector<std::string>& names, int Cout_each, int Cin, int taps, bool tc, bool phase, bool f32_tc) {
         const int Cout = Cout_each * (int)names.size();
         ConvW r;
         r.tc = tc;
-        const size_t wbytes = tc ? conv_tc_packed_bytes(Cout, Cin, taps, phase) : (size_t)(phase ? 16 : taps) * Cin * Cout * 4;
+        const size_t wbytes = tc ? conv_tc_packed_bytes(Cout, Cin, taps, phase) : f32_tc ? conv_f32_tc_packed_bytes(Cout, Cin, phase) : (size_t)(phase ? 16 : taps) * Cin * Cout * 4;
         r.w_off = alloc(wbytes);
         r.b_off = alloc((size_t)Cout * 4);
         for (size_t i = 0; i < names.size(); ++i) {
-            h_->jobs.push_back({names[i] + ".weight", 0, tc, phase, Cout_each, Cin, taps, Cout, (int)i * Cout_each, r.w_off});
+            h_->jobs.push_back({names[i] + ".weight", 0, tc, phase, Cout_each, Cin, taps, Cout, (int)i * Cout_each, r.w_off, f32_tc});
             h_->jobs.push_back({names[i] + ".bias", 1, false, false, Cout_each, 0, 0, 0, 0, r.b_off + (size_t)i * Cout_each * 4});
         }
         return r;
@@ -241,8 +243,10 @@ class Planner {
             f32 = conv_f32_choose(probe, &s.f32, clusters_ ? kF32MaxSplits : 1);
             if (f32 && upsample) { phase = true; a.upsample = 2; }
         }
-        s.f32.valid = f32 ? 1 : 0;
-        ConvW cw = conv_weight(wnames, Cout_each, Cin, ksize * ksize, tc, phase);
+        const bool f32_tc = f32 && wnames.size() == 1 && conv_f32_tc_choose(probe, &s.f32_tc, clusters_ ? kF32MaxSplits : 1) && conv_f32_tc_pays(probe);
+        s.f32_tc.valid = f32_tc ? 1 : 0;
+        s.f32.valid = f32 && !f32_tc ? 1 : 0;
+        ConvW cw = conv_weight(wnames, Cout_each, Cin, ksize * ksize, tc, phase, f32_tc);
         a.w = ptr<void>(cw.w_off);
         a.bias = ptr<float>(cw.b_off);
         if (!shortcut_name.empty()) {          // only requested when the tensor-core kernel takes this layer
@@ -315,7 +319,8 @@ class Planner {
         whole.B = cfg_.max_batch;
         const bool tc_rec = tc && !split && !(cfg_.flags & VD_FLAG_FUSED_STATS) && !y_is_frames && conv_tc_records_supported(whole);
         if ((f32 || split || thin || tc_rec) && records && !y_is_frames && rec_groups_ok(Cout, cfg_.norm_groups)) {
-            const int slots = thin ? conv_thin_slots(a) : tc_rec ? conv_tc_slots(a) : split ? conv_split_slots(probe, s.split, cfg_.norm_groups) : conv_f32_slots(probe, s.f32, cfg_.norm_groups);
+            const int slots = thin ? conv_thin_slots(a) : tc_rec ? conv_tc_slots(a) : split ? conv_split_slots(probe, s.split, cfg_.norm_groups)
+                              : f32_tc ? conv_f32_tc_slots(probe, s.f32_tc, cfg_.norm_groups) : conv_f32_slots(probe, s.f32, cfg_.norm_groups);
             rec_toggle_ ^= 1;
             a.out_rec = ptr<float4>(rec_buf_[rec_toggle_]);
             a.out_slots = slots;
@@ -337,7 +342,7 @@ class Planner {
         s.info.weight_bytes = (double)ksize * ksize * Cin * Cout * elt(cfg_.dtype);
         s.info.has_residual = residual_off >= 0;
         s.info.phase_collapsed = phase ? 1 : 0;
-        s.info.cluster = split ? conv_split_cluster(s.split) : f32 ? s.f32.splits : 1;
+        s.info.cluster = split ? conv_split_cluster(s.split) : f32_tc ? s.f32_tc.splits : f32 ? s.f32.splits : 1;
         if (!y_is_frames && pending(y_off) != kNone) s.info.out_pending_offset = (int64_t)pending(y_off);
         if (!shortcut_name.empty()) {
             s.info.c_in2 = Cin2;
@@ -624,6 +629,7 @@ bool plan_fits(const vd_handle_s& h) {
     for (const Step& st : h.steps) {
         if (st.kind == VD_STEP_CONV && st.split.valid && !conv_split_fits(st.conv, st.split)) return false;
         if (st.kind == VD_STEP_CONV && st.f32.valid && !conv_f32_fits(st.conv, st.f32)) return false;
+        if (st.kind == VD_STEP_CONV && st.f32_tc.valid && !conv_f32_tc_fits(st.conv, st.f32_tc)) return false;
     }
     return true;
 }
@@ -649,6 +655,7 @@ cudaError_t launch_step(const vd_handle_s* h, const Step& st, int B, const void*
             a.B = B;
             if (!a.y) a.y = frames;
             if (st.split.valid) return launch_conv_split(a, st.split, status, s);
+            if (st.f32_tc.valid) return launch_conv_f32_tc(a, st.f32_tc, status, s);
             if (st.f32.valid) return launch_conv_f32(a, st.f32, status, s);
             return st.use_tc ? launch_conv_tc(a, st.tc, status, s) : launch_conv_simt(a, s);
         }
@@ -786,6 +793,8 @@ vd_status vd_create(const vd_config* cfg, const vd_tensor* weights, int32_t n_we
             e = launch_to_f32(t->dptr, t->dtype, (float*)(h->ws + j.dst_off), j.kind == 1 ? j.Cout : (int64_t)j.Cout * j.Cin, s);
         } else if (j.tc) {
             e = launch_pack_weight_tc(t->dptr, t->dtype, h->ws + j.dst_off, j.Cout, j.Cin, j.taps, j.cout_total, j.cout_offset, j.phase, s);
+        } else if (j.f32_tc) {
+            e = launch_pack_weight_f32_tc(t->dptr, t->dtype, (float*)(h->ws + j.dst_off), j.Cout, j.Cin, j.phase, s);
         } else if (j.phase) {
             e = launch_pack_weight_f32_phase(t->dptr, t->dtype, (float*)(h->ws + j.dst_off), j.Cout, j.Cin, s);
         } else {
@@ -803,8 +812,8 @@ vd_status vd_create(const vd_config* cfg, const vd_tensor* weights, int32_t n_we
         if (e != cudaSuccess) { delete h; return cuda_fail(nullptr, e, "bias rows"); }
     }
     for (Step& st : h->steps) {
-        if (st.kind == VD_STEP_CONV && st.f32.valid) {
-            e = conv_f32_prepare(st.conv, &st.f32);
+        if (st.kind == VD_STEP_CONV && (st.f32.valid || st.f32_tc.valid)) {
+            e = st.f32.valid ? conv_f32_prepare(st.conv, &st.f32) : conv_f32_tc_prepare(st.conv, &st.f32_tc);
             if (e != cudaSuccess) { delete h; return cuda_fail(nullptr, e, "weight tensor map"); }
         }
         if (st.kind == VD_STEP_CONV && st.use_tc) {
@@ -1028,7 +1037,7 @@ static vd_status check_conv_desc(const vd_conv_desc* d) {
     if (d->ksize != 1 && d->ksize != 3) return fail(nullptr, VD_ERR_INVALID_ARG, "ksize must be 1 or 3");
     if ((d->in_dtype != VD_F32 && d->in_dtype != VD_BF16) || (d->out_dtype != VD_F32 && d->out_dtype != VD_BF16))
         return fail(nullptr, VD_ERR_INVALID_ARG, "bad dtype");
-    if (d->impl < VD_IMPL_AUTO || d->impl > VD_IMPL_TC_SPLIT) return fail(nullptr, VD_ERR_INVALID_ARG, "bad impl");
+    if (d->impl < VD_IMPL_AUTO || d->impl > VD_IMPL_TC_F32) return fail(nullptr, VD_ERR_INVALID_ARG, "bad impl");
     if (d->upsample < 0 || d->upsample > 2) return fail(nullptr, VD_ERR_INVALID_ARG, "upsample must be 0, 1 or 2");
     return VD_OK;
 }
@@ -1049,18 +1058,22 @@ static vd_status resolve_impl(const vd_conv_desc* d, const ConvArgs& a, bool* tc
     probe.B = 1;
     const bool can = a.bf16_operands && conv_tc_supported(probe);
     if ((d->impl == VD_IMPL_TC || d->impl == VD_IMPL_TC_SPLIT) && !can) return fail(nullptr, VD_ERR_UNSUPPORTED, "the tensor-core convolution does not support this shape");
+    if (d->impl == VD_IMPL_TC_F32 && !conv_f32_tc_supported(a)) return fail(nullptr, VD_ERR_UNSUPPORTED, "the single-precision tensor-core convolution does not support this layer");
     *tc = d->impl == VD_IMPL_TC || d->impl == VD_IMPL_TC_SPLIT || (d->impl == VD_IMPL_AUTO && can);
     if (!*tc && a.upsample == 2 && !conv_f32_supported(a)) return fail(nullptr, VD_ERR_UNSUPPORTED, "this layer has no phase-collapsed upsampling form, or its tensors are not 16-byte aligned");
     return VD_OK;
 }
 
 // the kernel of a layer, and its plan where that kernel has one
-struct ConvPlans { ConvSplitPlan split; ConvF32Plan f32; };
+struct ConvPlans { ConvSplitPlan split; ConvF32Plan f32; ConvF32TcPlan f32_tc; };
 static vd_status resolve_route(const vd_conv_desc* d, const ConvArgs& a, vd_conv_route_kind* route, ConvPlans* plans) {
     bool tc;
     vd_status st = resolve_impl(d, a, &tc);
     if (st != VD_OK) return st;
-    if (d->impl == VD_IMPL_TC_SPLIT) {
+    if (d->impl == VD_IMPL_TC_F32) {
+        if (!conv_f32_tc_choose(a, &plans->f32_tc)) return fail(nullptr, VD_ERR_UNSUPPORTED, "the single-precision tensor-core convolution has no plan for this layer");
+        *route = VD_ROUTE_F32_TC;
+    } else if (d->impl == VD_IMPL_TC_SPLIT) {
         if (!conv_split_choose(a, &plans->split)) return fail(nullptr, VD_ERR_UNSUPPORTED, "this layer's K is not divided among a cluster");
         *route = conv_split_cluster(plans->split) == plans->split.shape.splits ? VD_ROUTE_SPLIT : VD_ROUTE_SPLIT_PAIRS;
     } else {
@@ -1077,7 +1090,8 @@ vd_status vd_conv_packed_weight_bytes(const vd_conv_desc* d, size_t* bytes) {
     st = resolve_impl(d, conv_args_from_desc(d), &tc);
     if (st != VD_OK) return st;
     const int taps = d->ksize * d->ksize;
-    *bytes = tc ? conv_tc_packed_bytes(d->c_out, d->c_in, taps, d->upsample == 2) : (size_t)(d->upsample == 2 ? 16 : taps) * d->c_in * d->c_out * 4;
+    *bytes = tc ? conv_tc_packed_bytes(d->c_out, d->c_in, taps, d->upsample == 2)
+             : d->impl == VD_IMPL_TC_F32 ? conv_f32_tc_packed_bytes(d->c_out, d->c_in, d->upsample == 2) : (size_t)(d->upsample == 2 ? 16 : taps) * d->c_in * d->c_out * 4;
     return VD_OK;
 }
 
@@ -1091,6 +1105,7 @@ vd_status vd_conv_pack_weight(const vd_conv_desc* d, const void* w_oihw, int32_t
     if (st != VD_OK) return st;
     const int taps = d->ksize * d->ksize;
     cudaError_t e = tc ? launch_pack_weight_tc(w_oihw, w_dtype, packed, d->c_out, d->c_in, taps, d->c_out, 0, d->upsample == 2, (cudaStream_t)cuda_stream)
+                       : d->impl == VD_IMPL_TC_F32 ? launch_pack_weight_f32_tc(w_oihw, w_dtype, (float*)packed, d->c_out, d->c_in, d->upsample == 2, (cudaStream_t)cuda_stream)
                        : d->upsample == 2 ? launch_pack_weight_f32_phase(w_oihw, w_dtype, (float*)packed, d->c_out, d->c_in, (cudaStream_t)cuda_stream)
                        : launch_pack_weight_simt(w_oihw, w_dtype, (float*)packed, d->c_out, d->c_in, taps, d->c_out, 0, (cudaStream_t)cuda_stream);
     return e == cudaSuccess ? VD_OK : cuda_fail(nullptr, e, "vd_conv_pack_weight");
@@ -1119,6 +1134,7 @@ static int record_slots(const ConvArgs& a, vd_conv_route_kind route, const ConvP
     switch (route) {
         case VD_ROUTE_THIN: return conv_thin_slots(a);
         case VD_ROUTE_F32: return a.Cout % 32 == 0 ? conv_f32_slots(a, plans.f32, groups) : 0;
+        case VD_ROUTE_F32_TC: return conv_f32_tc_slots(a, plans.f32_tc, groups);
         case VD_ROUTE_TC: return conv_tc_can_record(a) ? conv_tc_slots(a) : 0;
         case VD_ROUTE_SPLIT: case VD_ROUTE_SPLIT_PAIRS: return a.out_nchw ? 0 : conv_split_slots(a, plans.split, groups);
         default: return 0;
@@ -1156,7 +1172,7 @@ vd_status vd_op_conv2d_ex(const vd_conv_desc* d, const vd_conv_extra* ex, const 
     if (st != VD_OK) return st;
     cudaStream_t s = (cudaStream_t)cuda_stream;
     if (route == VD_ROUTE_F32 && !conv_f32_fits(a, plans.f32) && !conv_f32_choose(a, &plans.f32, 1)) route = VD_ROUTE_DIRECT;
-    if (a.in_rec && (scale || (route != VD_ROUTE_F32 && route != VD_ROUTE_SPLIT && route != VD_ROUTE_SPLIT_PAIRS)))
+    if (a.in_rec && (scale || (route != VD_ROUTE_F32 && route != VD_ROUTE_F32_TC && route != VD_ROUTE_SPLIT && route != VD_ROUTE_SPLIT_PAIRS)))
         return fail(nullptr, VD_ERR_UNSUPPORTED, "this layer's kernel takes no records of its input");
     if (a.x2 && route < VD_ROUTE_TC) return fail(nullptr, VD_ERR_UNSUPPORTED, "the fused shortcut exists in the tensor-core kernels only");
     if (ex && ex->out_groups) {
@@ -1186,6 +1202,11 @@ vd_status vd_op_conv2d_ex(const vd_conv_desc* d, const vd_conv_extra* ex, const 
             if (!conv_split_fits(a, plans.split)) return fail(nullptr, VD_ERR_UNSUPPORTED, "this device cannot hold the layer's clusters");
             e = conv_split_prepare(a, &plans.split);
             if (e == cudaSuccess) e = launch_conv_split(a, plans.split, nullptr, s);
+            break;
+        case VD_ROUTE_F32_TC:
+            if (!conv_f32_tc_fits(a, plans.f32_tc)) return fail(nullptr, VD_ERR_UNSUPPORTED, "this device cannot hold the layer's clusters");
+            e = conv_f32_tc_prepare(a, &plans.f32_tc);
+            if (e == cudaSuccess) e = launch_conv_f32_tc(a, plans.f32_tc, nullptr, s);
             break;
         case VD_ROUTE_F32:
             e = conv_f32_prepare(a, &plans.f32);

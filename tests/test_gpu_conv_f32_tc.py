@@ -1,0 +1,65 @@
+"""The single-precision convolution on the tensor cores, at the sizes where it can go wrong: tiles cut by the image edge, one to
+eight CTAs that share K, more taps than accumulators, the four parities of the upsampling form.
+
+Small whole numbers are exact in tf32 and their sums in fp32, so the result is that of a 64-bit convolution bit for bit; numbers
+with 24 significant bits show that the operands keep all of them."""
+import pytest
+
+from tests.test_gpu_conv_split import exact_conv, ints, vd            # noqa: F401  (vd is a fixture)
+
+pytestmark = pytest.mark.gpu
+
+# B, H, W, Cin, Cout, up
+SHAPES = [
+    (1, 1, 1, 32, 32, 0), (2, 17, 9, 64, 96, 0), (1, 16, 8, 256, 32, 0), (1, 8, 8, 512, 512, 0), (3, 33, 50, 32, 32, 0), (1, 30, 21, 96, 64, 0),
+    (1, 24, 24, 512, 512, 0), (1, 61, 57, 128, 128, 0), (2, 33, 30, 96, 192, 0),
+    (1, 3, 2, 64, 32, 2), (2, 17, 9, 128, 64, 2), (1, 8, 8, 512, 512, 2), (2, 33, 19, 32, 32, 2),
+]
+
+
+@pytest.mark.parametrize("shape", SHAPES)
+def test_whole_numbers_are_exact(vd, shape):                          # noqa: F811
+    import torch
+    B, H, W, Cin, Cout, up = shape
+    g = torch.Generator(device="cuda").manual_seed(H * 1000 + W * 10 + Cin)
+    x, w, bias = ints(g, -4, 4, B, H, W, Cin), ints(g, -2, 2, Cout, Cin, 3, 3), ints(g, -8, 8, Cout)
+    scale, shift = 2.0 ** ints(g, -1, 1, B, Cin), ints(g, -1, 1, B, Cin)
+    want = exact_conv(x.double() * scale[:, None, None, :].double() + shift[:, None, None, :].double(), w, 3, up) + bias.double()
+    res = None if up else ints(g, -64, 64, *want.shape)
+    got = vd.op_conv2d(x, w, bias, scale, shift, res, upsample=up, impl=vd.VD_IMPL_TC_F32)
+    assert torch.equal(got, (want if res is None else want + res.double()).float())
+
+
+@pytest.mark.parametrize("shape", [(2, 17, 9, 64, 96, 0), (1, 8, 8, 512, 512, 0), (3, 33, 50, 32, 32, 0), (1, 64, 64, 128, 128, 0), (1, 8, 8, 512, 512, 2)])
+def test_operands_keep_24_bits(vd, shape):                            # noqa: F811
+    """A tap's sum has four truncating steps (2^-23 at most of a sum that grows to its size), each operand's remainder is below
+    2^-24, and at most 144 sums are added with rounding (2^-24 / sqrt(3) each, on a sum that grows: sqrt(144 / 2))."""
+    import torch
+    B, H, W, Cin, Cout, up = shape
+    g = torch.Generator(device="cuda").manual_seed(7)
+    rnd = lambda *s: torch.randn(*s, device="cuda", generator=g)
+    x, w = rnd(B, H, W, Cin), rnd(Cout, Cin, 3, 3) / (9 * Cin) ** 0.5
+    want = exact_conv(x, w, 3, up)
+    got = vd.op_conv2d(x, w, upsample=up, impl=vd.VD_IMPL_TC_F32).double()
+    bound = 4 * 2.0 ** -23 / 2 + 2.0 ** -24 + 2.0 ** -24 / 3 ** 0.5 * (144 / 2) ** 0.5
+    if up:
+        bound += 2.0 ** -24                                           # the sums of up to four weights are rounded once
+    assert float((got - want).norm() / want.norm()) <= bound
+
+
+@pytest.mark.parametrize("B,H,W,Cin,Cout,cpg", [(2, 17, 9, 64, 128, 4), (1, 16, 16, 512, 512, 16), (1, 33, 50, 32, 64, 8)])
+def test_records_of_the_output_and_of_the_input(vd, B, H, W, Cin, Cout, cpg):      # noqa: F811
+    import torch
+    g = torch.Generator(device="cuda").manual_seed(9)
+    rnd = lambda *s: torch.randn(*s, device="cuda", generator=g)
+    x, w, gamma, beta = rnd(B, H, W, Cin), rnd(Cout, Cin, 3, 3) / (9 * Cin) ** 0.5, 1 + 0.1 * rnd(Cout), 0.1 * rnd(Cout)
+    y, rec = vd.op_conv2d(x, w, impl=vd.VD_IMPL_TC_F32, groups=Cout // cpg)
+    want = vd.op_gn_stats(y, gamma, beta, Cout // cpg, 1e-6)
+    got = vd.op_merge_records(rec, H * W, gamma, beta, 1e-6)
+    for a, b in zip(got, want):
+        assert torch.allclose(a, b, rtol=2e-5, atol=2e-5)             # fp32 sums of some 1e3 to 1e5 values, in two orders
+    if rec.shape[2] <= 128:                                           # and merged by the next layer
+        w2 = rnd(32, Cout, 3, 3) / (9 * Cout) ** 0.5
+        a = vd.op_conv2d(y, w2, scale=want[0], shift=want[1], silu=True, impl=vd.VD_IMPL_TC_F32)
+        b = vd.op_conv2d(y, w2, silu=True, impl=vd.VD_IMPL_TC_F32, in_records=(rec, gamma, beta, 1e-6))
+        assert float((a - b).norm() / a.norm()) <= 1e-5
