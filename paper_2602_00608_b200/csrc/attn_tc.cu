@@ -128,10 +128,11 @@ attn_tc_kernel(const AttnTcParams a, const __grid_constant__ CUtensorMap tm_q, c
         // same (quarter & 1), which share a named barrier.
         float* red = s_red + row;
         const uint32_t lane_base = (uint32_t)(quarter * 32) << 16, half_cols = (uint32_t)(warp >> 2) * 64u;
-        for (int j = j0; j < j1 && ok; ++j) {
+        // After a wait gave up a warp walks on over whatever is there: the four warps of a row meet at their barriers however each
+        // of them learns of it, and nothing of it is written in the end.
+        for (int j = j0; j < j1; ++j) {
             const int i = j - j0, buf = i & 1;
-            ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bars->s_full[buf]), (i >> 1) & 1, abort_flag));
-            if (!ok) break;
+            ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bars->s_full[buf]), (i >> 1) & 1, abort_flag)) && ok;
             tc_fence_after();
             uint32_t r0[32], r1[32];
             tmem_ld32(tmem_s + lane_base + (uint32_t)buf * 128u + half_cols, r0);
@@ -191,8 +192,7 @@ attn_tc_kernel(const AttnTcParams a, const __grid_constant__ CUtensorMap tm_q, c
             const bool any_grow = __any_sync(0xffffffffu, grow) && i > 0;
             if (i > 0) {
                 // P and O are free once the previous tile's P.V product has completed
-                ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bars->pv_done), (i - 1) & 1, abort_flag));
-                if (!ok) break;
+                ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bars->pv_done), (i - 1) & 1, abort_flag)) && ok;
                 tc_fence_after();
             }
             if (any_grow) {                                        // this warp's half of the row's accumulator columns
@@ -218,13 +218,13 @@ attn_tc_kernel(const AttnTcParams a, const __grid_constant__ CUtensorMap tm_q, c
             __syncwarp();
             if (lane == 0) mbar_arrive_cluster(leader_bar(&bars->p_full));
         }
-        if (ok) ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bars->pv_done), (j1 - j0 - 1) & 1, abort_flag));
+        ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bars->pv_done), (j1 - j0 - 1) & 1, abort_flag)) && ok;
+        tc_fence_after();
+        // the row's sum over its four threads
+        red[kb * ROWS] = l;
+        named_barrier_sync(1 + (quarter & 1), SOFTMAX_WARPS * 16);
+        l = (red[0] + red[ROWS]) + (red[2 * ROWS] + red[3 * ROWS]);
         if (ok) {
-            tc_fence_after();
-            // the row's sum over its four threads
-            red[kb * ROWS] = l;
-            named_barrier_sync(1 + (quarter & 1), SOFTMAX_WARPS * 16);
-            l = (red[0] + red[ROWS]) + (red[2 * ROWS] + red[3 * ROWS]);
             const float inv = 1.f / l;
             const bool inside = q0 + row < a.T;
             const int ch0 = (warp >> 2) * 256 + (quarter >> 1) * 128;      // this thread's 128 channels

@@ -68,3 +68,35 @@ def test_loads_on_their_way_land_after_a_wait_gave_up():
         else:                                                # whatever wait it was: once the accumulators are complete, before the last arrival
             wait = body.rindex("mbar_wait(smem_u32(&bars->acc_full)", 0, landed.start())
             assert landed.start() - wait < 200 and landed.start() < body.rindex("cluster_arrive()")
+
+
+BARRIER = re.compile(r"named_barrier_sync\(")
+
+
+def enclosing(body, at):
+    """What stands before each brace that is open at `at`: conditions, loops, lambdas, from the outermost in."""
+    open_braces = []
+    for i in range(at):
+        if body[i] == "{":
+            open_braces.append(i)
+        elif body[i] == "}":
+            open_braces.pop()
+    return [re.split(r"[{}]|;(?![^()]*\))", body[:i])[-1].strip() for i in open_braces], open_braces
+
+
+WITH_BARRIERS = [(f, n, b) for f, n, b in kernels() if BARRIER.search(b)]
+
+
+@pytest.mark.parametrize("file,name,body", WITH_BARRIERS, ids=[n for _, n, _ in WITH_BARRIERS])
+def test_every_warp_reaches_its_named_barriers_after_a_wait_gave_up(file, name, body):
+    """Warps learn of a wait that gave up one by one.  If one of them left for the end of the kernel, the others would stand in their
+    named barrier for good: whether a warp comes to a barrier must not depend on its waits, once it has waited at all."""
+    for m in BARRIER.finditer(body):
+        headers, braces = enclosing(body, m.start())
+        if any(re.search(r"\bu == 0\b", h) for h in headers):        # the first pass of a loop: before any wait
+            continue
+        for h, at in zip(headers, braces):
+            assert not re.search(r"\bok\b|abort_flag", h), f"{file}: {name}: a barrier under `{h}`"
+            if re.match(r"(for|while)\b", h):
+                loop = body_at(body, at)[1]
+                assert not re.search(r"\b(break|return)\b", loop), f"{file}: {name}: a barrier in a loop that a warp may leave"
