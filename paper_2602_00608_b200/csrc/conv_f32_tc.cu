@@ -284,7 +284,7 @@ conv_f32_tc_kernel(const ConvArgs a, const TShape sh, const __grid_constant__ CU
                     }
                 named_barrier_sync(1, kProd);
             }
-            if (u > 0 && !mbar_wait(smem_u32(&bars->a_empty), (uint32_t)(u - 1) & 1u, abort_flag)) break;
+            if (u > 0 && !__all_sync(0xffffffffu, mbar_wait(smem_u32(&bars->a_empty), (uint32_t)(u - 1) & 1u, abort_flag))) break;
             op.transform(smem_a, u, prologue, silu, s_scale, s_shift, ptid);
             if (u + 1 < nk) op.load(u + 1);
             fence_proxy_async_smem();

@@ -321,7 +321,7 @@ conv_split_kernel(const ConvArgs a, const ConvSplitShape sh, const __grid_consta
                 named_barrier_sync(1, kProd);
             }
             if (u >= n_a) {
-                ok = mbar_wait(smem_u32(&bars->a_empty[as]), aph ^ 1, abort_flag);
+                ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bars->a_empty[as]), aph ^ 1, abort_flag));
                 if (!ok) break;
             }
             if (second) {                                    // 16 x 8 pixels x 32 fp32 channels, as they lie in memory
@@ -557,7 +557,7 @@ conv_pair_kernel(const ConvArgs a, const ConvSplitShape sh, const __grid_constan
         uint32_t as = 0, aph = 0;
 #pragma unroll 1
         for (int u = 0; u < nk; ++u) {
-            if (u >= n_a && !mbar_wait(smem_u32(&bars->a_empty[as]), aph ^ 1, abort_flag)) break;
+            if (u >= n_a && !__all_sync(0xffffffffu, mbar_wait(smem_u32(&bars->a_empty[as]), aph ^ 1, abort_flag))) break;
             op.transform(smem_a + as * A_TILE_BYTES, u, u + 1 < nk, prologue, silu, s_scale, s_shift, ptid);
             fence_proxy_async_smem();
             __syncwarp();

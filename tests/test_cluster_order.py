@@ -100,3 +100,18 @@ def test_every_warp_reaches_its_named_barriers_after_a_wait_gave_up(file, name, 
             if re.match(r"(for|while)\b", h):
                 loop = body_at(body, at)[1]
                 assert not re.search(r"\b(break|return)\b", loop), f"{file}: {name}: a barrier in a loop that a warp may leave"
+
+
+ONE_LANE = re.compile(r"\b(lane|tid|ptid) == |\bif \(lead\)|elected")
+WITH_ALIGNED = [(f, n, b) for f, n, b in kernels() if re.search(r"tmem_ld\d*\(|__syncwarp\(", b) and "mbar_wait" in b]
+
+
+@pytest.mark.parametrize("file,name,body", WITH_ALIGNED, ids=[n for _, n, _ in WITH_ALIGNED])
+def test_a_warp_decides_as_one_whether_a_wait_gave_up(file, name, body):
+    """Where whole warps wait, the answer that they act on is voted on: lanes that part would meet the warp's barriers and tensor
+    memory instructions at different places."""
+    for m in re.finditer(r"\bmbar_wait(?:<[^>]*>)?\(", body):
+        before = re.split(r"[;{}]", body[:m.start()])[-1]
+        if "(void)" in before or "__all_sync(" in before or any(ONE_LANE.search(h) for h in enclosing(body, m.start())[0]):
+            continue
+        raise AssertionError(f"{file}: {name}: {before.strip()} mbar_wait(...) is not voted on")
