@@ -284,18 +284,17 @@ attn_tc_kernel(const AttnTcParams a, const __grid_constant__ CUtensorMap tm_q, c
                 if (ok) load_v(j);
             }
             // Everything has landed once it has been multiplied.  If a wait gave up anywhere, what is on its way lands before the
-            // CTA's memory goes (counted in the pair's first CTA; the other one lets the limit pass).
+            // CTA's memory goes (both CTAs' loads are counted in the pair's first one; the other one lets the limit pass).
             for (int k = 0; k < STAGES && ok; ++k) {
                 ok = mbar_wait(smem_u32(&bars->empty[st]), ph ^ 1, abort_flag);
                 if (ok && ++st == STAGES) { st = 0; ph ^= 1; }
             }
-            if (!ok) {
+            if (!ok && rank == 0) {
+                cc::land_loads(&bars->q_full, 1, 1);
+                cc::land_loads(bars->full, STAGES, issued);
+            } else if (!ok) {
                 const long long t0 = clock64();
-                for (int k = 0; k < min(issued, STAGES); ++k) {
-                    if (st == 0) { st = STAGES; ph ^= 1; }
-                    --st;
-                    while (!mbar_try_wait(smem_u32(&bars->full[st]), ph) && clock64() - t0 < WAIT_LIMIT_CYCLES) {}
-                }
+                while (clock64() - t0 < WAIT_LIMIT_CYCLES) {}
             }
         }
     } else if (rank == 0) {

@@ -463,14 +463,7 @@ __global__ void __launch_bounds__(kGnThreads + 64, 2) gn_batch_kernel(GnArgs a, 
                 ok = mbar_wait(smem_u32(&empty[st]), ph ^ 1u, abort_flag);
                 if (ok && ++st == (uint32_t)S) { st = 0; ph ^= 1u; }
             }
-            if (!ok) {
-                const long long t0 = clock64();
-                for (int i = 0; i < min(issued, S); ++i) {
-                    if (st == 0) { st = S; ph ^= 1u; }
-                    --st;
-                    while (!mbar_try_wait(smem_u32(&full[st]), ph) && clock64() - t0 < WAIT_LIMIT_CYCLES) {}
-                }
-            }
+            if (!ok) cc::land_loads(full, S, issued);
         }
         return;
     }

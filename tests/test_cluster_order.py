@@ -115,3 +115,11 @@ def test_a_warp_decides_as_one_whether_a_wait_gave_up(file, name, body):
         if "(void)" in before or "__all_sync(" in before or any(ONE_LANE.search(h) for h in enclosing(body, m.start())[0]):
             continue
         raise AssertionError(f"{file}: {name}: {before.strip()} mbar_wait(...) is not voted on")
+
+
+@pytest.mark.parametrize("kernel", ["attn_tc_kernel", "gn_batch_kernel"])
+def test_the_landing_starts_from_the_last_load(kernel):
+    """The wait for everything to be consumed may itself give up half-way, and has moved on then: where the copies on their way are,
+    the number of the loads says."""
+    body = next(b for _, n, b in kernels() if n == kernel)
+    assert re.search(r"land_loads\((?:bars->)?full, \w+, issued\)", body) and "--st" not in body
