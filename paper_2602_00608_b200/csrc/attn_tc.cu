@@ -46,7 +46,7 @@ constexpr int kMaxSplits = 4;                                // pairs of a clust
 struct Bars {
     uint64_t q_full, full[STAGES], empty[STAGES];
     uint64_t s_full[2], s_free[2];
-    uint64_t p_full, pv_done;
+    uint64_t p_full, pv_done, drained;
     uint32_t tmem_base, abort_flag;
 };
 constexpr int RED_BYTES = 4 * ROWS * 4;                      // what the four threads of a row tell one another
@@ -105,6 +105,7 @@ attn_tc_kernel(const AttnTcParams a, const __grid_constant__ CUtensorMap tm_q, c
         for (int i = 0; i < 2; ++i) { mbar_init(smem_u32(&bars->s_full[i]), 1); mbar_init(smem_u32(&bars->s_free[i]), 2 * SOFTMAX_WARPS); }
         mbar_init(smem_u32(&bars->p_full), 2 * SOFTMAX_WARPS);
         mbar_init(smem_u32(&bars->pv_done), 1);
+        mbar_init(smem_u32(&bars->drained), 1);
         bars->abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         fence_proxy_async_smem();
@@ -354,6 +355,12 @@ attn_tc_kernel(const AttnTcParams a, const __grid_constant__ CUtensorMap tm_q, c
             if (j + 1 < j1) issue_qk(j + 1 - j0);
             issue_pv(j - j0, (min(BKV, a.T - j * BKV) + 63) >> 6);
         }
+        if (*abort_flag) {                                   // nobody else waits for the products under way
+            commit(&bars->drained);
+            __syncwarp();
+            (void)cc::wait_cluster(smem_u32(&bars->drained), 0, abort_flag);
+            __syncwarp();
+        }
     }
 
     tc_fence_before();
@@ -572,6 +579,8 @@ attn_small_kernel(const AttnTcParams a, const __grid_constant__ CUtensorMap tm_q
             for (int i = 0; i < 4; ++i) umma_bf16_split_on(tmem_o, pa + i * 2, hi, va + i * 2, hi, idesc, (k | i) != 0 ? 1u : 0u, on);
         }
         umma_commit_on(smem_u32(&bars->o_full), on);
+        __syncwarp();
+        if (*abort_flag) (void)cc::wait_cluster(smem_u32(&bars->o_full), 0, abort_flag);     // (the others no longer wait for the products under way)
         __syncwarp();
     }
     tc_fence_before();

@@ -253,6 +253,8 @@ conv_f32_tc_kernel(const ConvArgs a, const TShape sh, const __grid_constant__ CU
         cluster_wait();
         commit_to_cluster(smem_u32(&bars->acc_full), (uint16_t)((1u << S) - 1u), lead);
         __syncwarp();
+        if (*abort_flag) (void)wait_cluster(smem_u32(&bars->acc_full), 0, abort_flag);       // (the others no longer wait for the products under way)
+        __syncwarp();
     } else {
         // ------------------------------------------------ operand prologue, and the taps' sums
         const int ptid = tid - kProd0 * 32, pw = warp - kProd0;

@@ -123,3 +123,13 @@ def test_the_landing_starts_from_the_last_load(kernel):
     the number of the loads says."""
     body = next(b for _, n, b in kernels() if n == kernel)
     assert re.search(r"land_loads\((?:bars->)?full, \w+, issued\)", body) and "--st" not in body
+
+
+@pytest.mark.parametrize("kernel,bar,last", [("attn_tc_kernel", "drained", "tmem_dealloc2("), ("attn_small_kernel", "o_full", "tmem_dealloc("),
+                                             ("conv_f32_tc_kernel", "acc_full", "tmem_dealloc(")])
+def test_products_under_way_complete_before_tensor_memory_goes(kernel, bar, last):
+    """After a wait gave up the issuing warp goes on or leaves, and nobody else waits for the products that it has in flight: it
+    does so itself, and a flag that is already up does not end that wait."""
+    body = next(b for _, n, b in kernels() if n == kernel)
+    wait = re.search(r"if \(\*abort_flag\)[^;]*(?:;[^;]*){0,2}wait_cluster\(smem_u32\(&bars->" + bar, body)
+    assert wait and wait.start() < body.rindex(last)
