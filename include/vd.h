@@ -82,7 +82,10 @@ typedef struct {
     int32_t arch;               /* vd_arch */
     int32_t dtype;              /* vd_dtype of latents, frames and weights.  VD_BF16: bf16 operands and
                                    intra-block tensors, fp32 accumulation, fp32 residual stream.
-                                   VD_F32: fp32 throughout (FFMA kernels). */
+                                   VD_F32: fp32 throughout, no operand or sum in fewer bits; wide 3x3 layers
+                                   multiply on the tensor cores, each operand as three bf16 numbers that add up to
+                                   it, products exact but for what is below 2^-24 of them, the others on the
+                                   FFMA kernels. */
     int32_t latent_channels;    /* 4 */
     int32_t out_channels;       /* 3 */
     int32_t latent_h, latent_w; /* frames are 8*latent_h x 8*latent_w */

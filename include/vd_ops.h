@@ -91,7 +91,7 @@ VD_API vd_status vd_debug_stop_after(vd_handle h, int32_t index);
 typedef enum {
     VD_IMPL_AUTO = 0, VD_IMPL_SIMT = 1, VD_IMPL_TC = 2,
     VD_IMPL_TC_SPLIT = 3,       /* tcgen05 kernels that divide K among a cluster (convolutions of small images) */
-    VD_IMPL_TC_F32 = 4          /* single-precision 3x3 convolution on the tensor cores (operands as pairs of tf32 numbers) */
+    VD_IMPL_TC_F32 = 4          /* single-precision 3x3 convolution on the tensor cores (operands as three bf16 numbers each) */
 } vd_impl;
 
 typedef struct {

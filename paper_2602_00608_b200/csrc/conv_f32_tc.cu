@@ -1,25 +1,27 @@
-// Single-precision 3x3 convolutions (upsampling ones too) on the tensor cores: every fp32 operand is two tf32 numbers.
+// Single-precision 3x3 convolutions (upsampling ones too) on the tensor cores: every fp32 operand is three bf16 numbers.
 //
-// x = hi + lo, hi = x rounded to tf32 (11 significant bits), lo = x - hi rounded to tf32: what is lost of x is below 2^-24 |x|.
-// A product takes three tf32 products, hi hi + hi lo + lo hi (lo lo is below 2^-24 of it), so the operands are as good as
-// fp32's.  The tensor core truncates its running sum at every step of K = 8, which would make long sums worse than the FMA
-// kernel's (conv_f32.cu), whose additions round: so a sum has four steps only, a tap of 32 channels; the warps that have made
-// the operand read it and add it to their registers with rounding while the next taps run, in a ring of four accumulators.
-// Relative 2-norm error against 64 bits, FMA kernel / this one / this one with nine to eighteen steps per sum: 512->512 at 16x16 3.1e-7 /
-// 1.7e-7 / 3.8e-7, at 24x24 4.3e-7 / 2.1e-7 / 1.4e-6, 256->256 at 48x48 4.3e-7 / 1.8e-7 / 7.1e-7, 128->128 at 64x64 3.1e-7 / 1.7e-7 / 3.9e-7,
-// 32->32 at 128x128 2.2e-7 / 1.5e-7 / 2.3e-7.  Of 1x1 layers and of fewer than 576 products the FMA kernel's sums are the better
-// ones (512 products 1.3e-7 / 1.5e-7): they stay there.
+// x = x0 + x1 + x2, each the rest rounded to bf16: 8 + 8 + 8 significant bits are all 24 of x, and bf16 has fp32's exponents, so
+// nothing of an operand is lost (of one below 2^-110 in size up to 2^-134, half of bf16's smallest step).  A product takes six
+// bf16 products, which are exact; x1 w2 + x2 w1 + x2 w2 are left out: 2^-24 of it at most, as much as rounding it would cost
+// (|x1| is up to 2^-8, |x2| up to 2^-17 of x's power of two).  The tensor core truncates its running sum at every step of K = 16,
+// so a sum has two steps only, a tap of 32 channels, and the products of either size have their own: the largest, of 16 bits
+// each, mostly add up exactly, and what is cut from the others is below 2^-31.  The warps that have made the operand read the sums
+// and add them to their registers, smallest first, with rounding, while the next tap runs: two accumulators in turn.
+// Relative 2-norm error against 64 bits, FMA kernel (conv_f32.cu) / this one, normally distributed operands: 512->512 at 16x16 3.1e-7 /
+// 1.2e-7, at 24x24 4.2e-7 / 1.7e-7, 256->256 at 48x48 4.3e-7 / 1.3e-7, 128->128 at 64x64 3.1e-7 / 1.1e-7, 32->32 at 128x128 2.3e-7 / 0.9e-7;
+// sizes that spread over 2^24: 512->512 at 24x24 4.1e-7 / 1.7e-7; positive ones, whose truncations add up: 1.3e-7 / 1.0e-7 there, 0.57e-7 /
+// 0.62e-7 at 8x8 (with a row of taps per sum, which is 7 % faster in the full-width 64x64 decode, 1.14e-7); one product per output 2.5e-8 / 2.6e-8.
 //
 // The shape is that of conv_split.cu: a cluster of S CTAs shares one tile of 16 x 8 pixels x 32 output channels, each takes 1/S of
 // the 32-channel chunks, the partial sums meet in distributed shared memory, statistics are records.  A chunk's operand is
-// two tiles of 180 halo pixels x 32 channels (hi, lo; 128-byte rows, swizzled), written once and read by nine taps through
-// views; a tap's weights are one box of 64 rows, hi above lo, so that one MMA of N = 64 multiplies A hi with both and one of
-// N = 32 multiplies A lo with hi.  Two CTAs share an SM.  Bound by the taps' hand-over (issue, sum, barrier: about 500 cycles for
-// 350 of MMAs) and by the chain of latencies around it.
-// us, launches of a decode, FMA kernel -> this one: 512->512 at 8x8 28.7 -> 26.7, at 16x16 43.3 -> 29.0, upsampling to 16x16 30.7 -> 27.5, to
-// 32x32 75.7 -> 45.0; 512->256 at 32x32 74.4 -> 45.4, 256->256 43.1 -> 29.0, 128->128 at 64x64 45.4 -> 31.1; 32->32 on four 256x256
-// frames 141 -> 109, at 128x128 45 -> 37.  Decodes: 64x64 of the full-width layout 1250 -> 838 us, sixteen 256x256 frames of the small
-// one 2758 -> 2389 (2291 with the 64-channel layers too).
+// three tiles of 180 halo pixels x 32 channels (64-byte rows, swizzled), written once and read by nine taps through views; a
+// tap's weights are one box of 96 rows, the parts one above the other, so that x0 takes one MMA of N = 96 with all three, x1 one
+// of 64 and x2 one of 32, each added where products of that size are.  Two CTAs share an SM.  Bound by the taps' hand-over (issue,
+// sum, barrier) and by the chain of latencies around it.
+// us, launches of a decode, FMA kernel -> this one: 512->512 at 8x8 28.9 -> 26.7, at 16x16 43.4 -> 29.0, upsampling to 16x16 30.6 -> 27.5, to
+// 32x32 76.0 -> 43.8; 512->256 at 32x32 76.1 -> 45.3, 256->256 43.2 -> 28.9, 128->128 at 64x64 45.4 -> 31.0; 32->32 on four 256x256
+// frames 142 -> 109, at 128x128 45 -> 37.  Decodes: 64x64 of the full-width layout 1254 -> 831 us, sixteen 256x256 frames of the small
+// one 2770 -> 2184.
 #include <string.h>
 
 #include <algorithm>
@@ -34,7 +36,6 @@ namespace {
 
 using namespace cc;
 using namespace tc;
-using convtile::A_TILE_BYTES;
 using convtile::NPIX;
 using convtile::PW;
 using convtile::TILE_H;
@@ -44,8 +45,10 @@ constexpr int kWarps = 10, kThreads = kWarps * 32;           // MMA, weights, ei
 constexpr int kProd0 = 2, kProd = 8 * 32;
 constexpr int BN = 32, kChunk = 32, ROWS = TILE_H * TILE_W;  // output channels of a cluster, input channels of a chunk, rows of a tile
 constexpr int kMaxB = 9, kMaxSlice = 512;                    // weight stages; input channels of a CTA
-constexpr int A_BYTES = 2 * A_TILE_BYTES, B_BYTES = 2 * BN * 128;
-constexpr int ACCS = 4, ACC_COLS = 2 * BN;                   // accumulators of a tap each, in turn: columns [hi hi | hi lo + lo hi]
+constexpr int PARTS = 3;                                     // bf16 numbers of an operand
+constexpr int ROW_BYTES = kChunk * 2;                        // a pixel's, or an output channel's, part: 64 bytes (64-byte swizzle)
+constexpr int A_PART_BYTES = (NPIX * ROW_BYTES + 1023) / 1024 * 1024, A_BYTES = PARTS * A_PART_BYTES, B_BYTES = PARTS * BN * ROW_BYTES;
+constexpr int ACCS = 2, ACC_COLS = 128;                      // accumulators of a tap each, in turn: columns [x0 w0 | x0 w1 + x1 w0 | x0 w2 + x1 w1 + x2 w0]
 constexpr int kTailBytes = 2 * kMaxSlice * 4 + 320;
 
 enum { K3X3 = 0, KPHASE = 1 };
@@ -61,10 +64,12 @@ struct TBars {
 static_assert(sizeof(TBars) <= 320, "barrier block");
 struct TShape { int splits, n_b, tail_off; };
 
-__device__ __forceinline__ float to_tf32(float x) {
-    uint32_t r;
-    asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
-    return __uint_as_float(r);
+// the next parts of two numbers (the first in the low half), the largest first; the rests stay
+__device__ __forceinline__ uint32_t take_bf16(float& v0, float& v1) {
+    const uint32_t p = pack_bf16(v0, v1);
+    v0 -= __uint_as_float(p << 16);
+    v1 -= __uint_as_float(p & 0xffff0000u);
+    return p;
 }
 // 16-byte piece c of row R of a partial: eight rows of a piece, and four rows of two pieces side by side, are on distinct banks
 __device__ __forceinline__ int exchange_piece(int R, int c) { return c ^ ((R & 3) * 2 + ((R >> 2) & 1)); }
@@ -78,12 +83,12 @@ __device__ __forceinline__ void commit_to_cluster(uint32_t bar, uint16_t mask, u
 struct Operand {
     static constexpr int N = (NPIX * 8 + kProd - 1) / kProd;
     int goff[N];                                             // element offset of the entry's source pixel
-    uint32_t soff, vm;                                       // where entry 0 goes (entry e: e * kProd * 16 on); entries inside the image
+    uint32_t soff, vm;                                       // where entry 0 goes (entry e: e * kProd * 8 on); entries inside the image
     const float* xb;
     float4 raw[N];
     __device__ __forceinline__ void prepare(const ConvArgs& a, int frame, int c_first, int ty, int tx, int H, int W, int ptid) {
         const int j = ptid & 7, pix0 = ptid >> 3;
-        soff = (uint32_t)(pix0 * 128 + ((j ^ (pix0 & 7)) << 4));
+        soff = (uint32_t)(pix0 * ROW_BYTES + (((j >> 1) ^ (pix0 >> 1 & 3)) << 4) + (j & 1) * 8);
         vm = 0u;
 #pragma unroll
         for (int e = 0; e < N; ++e) {
@@ -110,21 +115,22 @@ struct Operand {
 #pragma unroll
         for (int e = 0; e < N; ++e) {
             if (e == N - 1 && ((e * kProd + ptid) >> 3) >= NPIX) break;
-            float hi[4] = {0.f, 0.f, 0.f, 0.f}, lo[4] = {0.f, 0.f, 0.f, 0.f};
+            float v[4] = {0.f, 0.f, 0.f, 0.f};
             if (vm >> e & 1u) {                              // outside the image the transformed tensor is zero
                 const float x[4] = {raw[e].x, raw[e].y, raw[e].z, raw[e].w}, s4[4] = {sc.x, sc.y, sc.z, sc.w}, f4[4] = {sf.x, sf.y, sf.z, sf.w};
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
-                    float v = x[q];
-                    if (prologue) v = fmaf(v, s4[q], f4[q]);
-                    if (silu) v = v / (1.0f + expf(-v));
-                    hi[q] = to_tf32(v);
-                    lo[q] = to_tf32(v - hi[q]);
+                    v[q] = x[q];
+                    if (prologue) v[q] = fmaf(v[q], s4[q], f4[q]);
+                    if (silu) v[q] = v[q] / (1.0f + expf(-v[q]));
                 }
             }
-            uint8_t* d = dst + soff + e * (kProd * 16);
-            *(float4*)d = make_float4(hi[0], hi[1], hi[2], hi[3]);
-            *(float4*)(d + A_TILE_BYTES) = make_float4(lo[0], lo[1], lo[2], lo[3]);
+            uint8_t* d = dst + soff + e * (kProd * 8);
+#pragma unroll
+            for (int p = 0; p < PARTS; ++p) {
+                const uint32_t lo = take_bf16(v[0], v[1]), hi = take_bf16(v[2], v[3]);
+                *(uint2*)(d + p * A_PART_BYTES) = make_uint2(lo, hi);
+            }
         }
     }
 };
@@ -198,7 +204,7 @@ conv_f32_tc_kernel(const ConvArgs a, const TShape sh, const __grid_constant__ CU
                     if (!ok) break;
                     const uint32_t full = smem_u32(&bars->b_full[st]);
                     mbar_arrive_expect_tx(full, B_BYTES);
-                    tma_load_2d(smem_u32(smem_b + st * B_BYTES), &tm_w, (k0 + u) * kChunk, ((par * TAPS + tap) * nblk + blk) * (2 * BN), full);
+                    tma_load_2d(smem_u32(smem_b + st * B_BYTES), &tm_w, (k0 + u) * kChunk, ((par * TAPS + tap) * nblk + blk) * (PARTS * BN), full);
                     ++issued;
                     if (++st == (uint32_t)n_b) { st = 0; ph ^= 1; }
                 }
@@ -212,8 +218,9 @@ conv_f32_tc_kernel(const ConvArgs a, const TShape sh, const __grid_constant__ CU
     } else if (warp == 0) {
         // ------------------------------------------------ MMA issue (warp-uniform, predicated on one elected lane)
         const uint32_t lead = elect_one();
-        constexpr uint32_t idesc_both = make_idesc_tf32(128, 2 * BN), idesc_hi = make_idesc_tf32(128, BN);
-        const uint32_t a_desc = desc_hi(PW * 128, 2), b_desc = desc_hi(1024, 2);
+        constexpr uint32_t idesc3 = make_idesc_bf16(128, 3 * BN), idesc2 = make_idesc_bf16(128, 2 * BN), idesc1 = make_idesc_bf16(128, BN);
+        constexpr uint32_t SWIZZLE_64B = 4;
+        const uint32_t a_desc = desc_hi(PW * ROW_BYTES, SWIZZLE_64B), b_desc = desc_hi(8 * ROW_BYTES, SWIZZLE_64B);
         const uint32_t a_lo0 = desc_lo(smem_u32(smem_a)), b_lo0 = desc_lo(smem_u32(smem_b));
         uint32_t bs = 0, bph = 0;
         int used = 0;                                        // (a stage that no later load needs is not handed back)
@@ -225,26 +232,28 @@ conv_f32_tc_kernel(const ConvArgs a, const TShape sh, const __grid_constant__ CU
         for (int u = 0; u < nk; ++u) {
             if (*abort_flag) break;
             wait_on(&bars->a_full, (uint32_t)u & 1u);
-            uint32_t a_hi = a_lo0 + (KIND == KPHASE ? (uint32_t)(((par >> 1) * PW + (par & 1)) * 8) : 0u);
+            constexpr uint32_t PIX = ROW_BYTES >> 4, PART = A_PART_BYTES >> 4;
+            uint32_t a0 = a_lo0 + (KIND == KPHASE ? (uint32_t)((par >> 1) * PW + (par & 1)) * PIX : 0u);
             constexpr int COLS = KIND == K3X3 ? 3 : 2;
             int kx = 0;
 #pragma unroll 1
             for (int tap = 0; tap < TAPS; ++tap, ++used) {
                 wait_on(&bars->b_full[bs], bph);
-                const uint32_t b_lo = b_lo0 + bs * (uint32_t)(B_BYTES >> 4), a_lo = a_hi + (uint32_t)(A_TILE_BYTES >> 4);
+                const uint32_t b = b_lo0 + bs * (uint32_t)(B_BYTES >> 4);
                 const int acc = used & (ACCS - 1);
                 const uint32_t td = tmem + (uint32_t)(acc * ACC_COLS);
                 wait_on(&bars->t_empty[acc], (uint32_t)((used / ACCS) & 1) ^ 1u);
 #pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    umma_tf32_split_on(td, a_hi + 2 * k, a_desc, b_lo + 2 * k, b_desc, idesc_both, k == 0 ? 0u : 1u, lead);
-                    umma_tf32_split_on(td + BN, a_lo + 2 * k, a_desc, b_lo + 2 * k, b_desc, idesc_hi, 1u, lead);
+                for (int k = 0; k < 2; ++k) {
+                    umma_bf16_split_on(td, a0 + 2 * k, a_desc, b + 2 * k, b_desc, idesc3, k == 0 ? 0u : 1u, lead);
+                    umma_bf16_split_on(td + BN, a0 + PART + 2 * k, a_desc, b + 2 * k, b_desc, idesc2, 1u, lead);
+                    umma_bf16_split_on(td + 2 * BN, a0 + 2 * PART + 2 * k, a_desc, b + 2 * k, b_desc, idesc1, 1u, lead);
                 }
                 umma_commit_on(smem_u32(&bars->t_full[acc]), lead);
                 if (used + 1 + n_b <= loads) umma_commit_on(smem_u32(&bars->b_empty[bs]), lead);
                 __syncwarp();
                 if (++bs == (uint32_t)n_b) { bs = 0; bph ^= 1; }
-                if (++kx == COLS) { kx = 0; a_hi += (uint32_t)((PW - COLS + 1) * 8); } else a_hi += 8u;
+                if (++kx == COLS) { kx = 0; a0 += (uint32_t)(PW - COLS + 1) * PIX; } else a0 += PIX;
             }
             if (u + 1 < nk) umma_commit_on(smem_u32(&bars->a_empty), lead);
             __syncwarp();
@@ -298,15 +307,20 @@ conv_f32_tc_kernel(const ConvArgs a, const TShape sh, const __grid_constant__ CU
                 ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bars->t_full[acc]), (uint32_t)(used / ACCS) & 1u, abort_flag));
                 if (!ok) break;
                 tc_fence_after();
-                uint32_t big[16], small[16];
-                tmem_ld16(tacc + (uint32_t)(acc * ACC_COLS), big);
-                tmem_ld16(tacc + (uint32_t)(acc * ACC_COLS + BN), small);
+                const uint32_t at = tacc + (uint32_t)(acc * ACC_COLS);
+                uint32_t r[16], t[16];                       // smallest terms first
+                tmem_ld16(at + 2 * BN, r);
+                tmem_ld16(at + BN, t);
+                tmem_ld_wait();
+#pragma unroll
+                for (int c = 0; c < 16; ++c) r[c] = __float_as_uint(__uint_as_float(r[c]) + __uint_as_float(t[c]));
+                tmem_ld16(at, t);
                 tmem_ld_wait();
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(smem_u32(&bars->t_empty[acc]));           // (in registers: the accumulator may go)
 #pragma unroll
-                for (int c = 0; c < 16; ++c) v[c] += __uint_as_float(big[c]) + __uint_as_float(small[c]);
+                for (int c = 0; c < 16; ++c) v[c] += __uint_as_float(t[c]) + __uint_as_float(r[c]);
             }
         }
         // ------------------------------------------------ exchange and epilogue: row R of the tile belongs to CTA R / rpo
@@ -359,10 +373,10 @@ conv_f32_tc_kernel(const ConvArgs a, const TShape sh, const __grid_constant__ CU
     }
 }
 
-// OIHW -> [tap][block of 32 output channels][hi, lo][32][Cin]; phase: the sixteen taps of the phase-collapsed upsampling form
+// OIHW -> bf16 [tap][block of 32 output channels][part][32][Cin]; phase: the sixteen taps of the phase-collapsed upsampling form
 // (parity * 4 + dy * 2 + dx, each the sum of the 3x3 taps that read the same source pixel, in conv_f32.cu's order).
 template <typename T>
-__global__ void pack_weight_f32_tc_kernel(const T* w, float* packed, int Cout, int Cin, int taps, bool phase) {
+__global__ void pack_weight_f32_tc_kernel(const T* w, __nv_bfloat16* packed, int Cout, int Cin, int taps, bool phase) {
     const int64_t total = (int64_t)taps * Cout * Cin;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
         const int c = (int)(i % Cin), o = (int)((i / Cin) % Cout), tap = (int)(i / ((int64_t)Cin * Cout));
@@ -377,10 +391,12 @@ __global__ void pack_weight_f32_tc_kernel(const T* w, float* packed, int Cout, i
                 const size_t j = ((size_t)o * Cin + c) * 9 + ky * 3 + kx;
                 v += sizeof(T) == 2 ? __bfloat162float(((const __nv_bfloat16*)w)[j]) : ((const float*)w)[j];
             }
-        const float hi = to_tf32(v);
-        const size_t row = ((size_t)tap * (Cout / BN) + o / BN) * (2 * BN) + o % BN;
-        packed[row * Cin + c] = hi;
-        packed[(row + BN) * Cin + c] = to_tf32(v - hi);
+        const size_t row = ((size_t)tap * (Cout / BN) + o / BN) * (PARTS * BN) + o % BN;
+        for (int p = 0; p < PARTS; ++p) {
+            const __nv_bfloat16 part = __float2bfloat16_rn(v);
+            packed[(row + p * BN) * Cin + c] = part;
+            v -= __bfloat162float(part);
+        }
     }
 }
 
@@ -425,8 +441,10 @@ bool conv_f32_tc_choose(const ConvArgs& a, ConvF32TcPlan* p, int max_splits) {
 }
 
 // Narrow layers of few tiles stay on the FMA kernel: there a layer is the chain of latencies, which the taps' hand-over lengthens.
-// us, FMA kernel / this one: 64 channels at 8x8 12.4 / 16.3, at 16x16 14.5 / 16.9; 32 at 64x64 16.7 / 18.8; 64 channels, four frames,
-// 32x32 (32 tiles) 19.1 / 20.5; 64x64 (128 tiles) 43 / 31, its upsampling from 32x32 (128 tiles and parities) 26 / 22.
+// us, FMA kernel / this one, the same layer again and again: 64 channels, 1 tile 10.3 / 12.4, 2 tiles 11.9 / 13.8, 24 16.5 / 14.4,
+// 48 24.6 / 18.1, 72 24.6 / 18.5, 128 39.0 / 25.1; upsampling, tiles times parities, 32 12.4 / 12.4, 64 18.5 / 14.8, 96 26.7 / 20.5, 128 26.7 /
+// 20.6; 32 channels, 24 tiles 12.4 / 14.2, 48 and 72 12.4 / 14.4, 96 16.4 / 14.4, 128 16.5 / 14.4.  From 128 on this one gains in all of them.
+// 128 channels: 1 tile 10.3 / 12.4, 2 tiles 12.4 / 13.3, 32 39.0 / 25.6; 512 from the smallest on (24.7 / 22.6).
 bool conv_f32_tc_pays(const ConvArgs& a) {
     return a.Cin >= 128 || (long long)tiles_of(a) * (a.upsample == 2 ? 4 : 1) * std::max(a.B, 1) >= 128;
 }
@@ -439,17 +457,17 @@ int conv_f32_tc_slots(const ConvArgs& a, const ConvF32TcPlan& p, int groups) {
     return tiles_of(a) * (a.upsample == 2 ? 4 : 1) * p.splits * rec_parts(BN, a.Cout / groups);
 }
 
-size_t conv_f32_tc_packed_bytes(int Cout, int Cin, bool phase) { return (size_t)(phase ? 16 : 9) * Cout * Cin * 8; }
+size_t conv_f32_tc_packed_bytes(int Cout, int Cin, bool phase) { return (size_t)(phase ? 16 : 9) * Cout * Cin * PARTS * 2; }
 
 cudaError_t conv_f32_tc_prepare(const ConvArgs& a, ConvF32TcPlan* p) {
     EncodeTiledFn enc = encode_fn();
     if (!enc) return cudaErrorNotSupported;
-    const cuuint64_t d[2] = {(cuuint64_t)a.Cin, (cuuint64_t)(a.upsample == 2 ? 16 : 9) * a.Cout * 2};
-    const cuuint64_t st[1] = {(cuuint64_t)a.Cin * 4};
-    const cuuint32_t box[2] = {kChunk, 2 * BN};
+    const cuuint64_t d[2] = {(cuuint64_t)a.Cin, (cuuint64_t)(a.upsample == 2 ? 16 : 9) * a.Cout * PARTS};
+    const cuuint64_t st[1] = {(cuuint64_t)a.Cin * 2};
+    const cuuint32_t box[2] = {kChunk, PARTS * BN};
     const cuuint32_t one[2] = {1, 1};
-    if (enc((CUtensorMap*)p->tmap, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<void*>(a.w), d, st, box, one, CU_TENSOR_MAP_INTERLEAVE_NONE,
-            CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+    if (enc((CUtensorMap*)p->tmap, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(a.w), d, st, box, one, CU_TENSOR_MAP_INTERLEAVE_NONE,
+            CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
         return cudaErrorInvalidValue;
     p->valid = 1;
     return cudaSuccess;
@@ -462,11 +480,11 @@ cudaError_t launch_conv_f32_tc(const ConvArgs& a, const ConvF32TcPlan& p, unsign
     return with_build(a, [&](auto build) { return build.launch(a, p, status, s); });
 }
 
-cudaError_t launch_pack_weight_f32_tc(const void* w, int w_dtype, float* packed, int Cout, int Cin, bool phase, cudaStream_t s) {
+cudaError_t launch_pack_weight_f32_tc(const void* w, int w_dtype, void* packed, int Cout, int Cin, bool phase, cudaStream_t s) {
     const int t = phase ? 16 : 9;
     const int grid = (int)std::min<int64_t>(((int64_t)t * Cout * Cin + 255) / 256, 148 * 16);
-    if (w_dtype == VD_BF16) pack_weight_f32_tc_kernel<__nv_bfloat16><<<grid, 256, 0, s>>>((const __nv_bfloat16*)w, packed, Cout, Cin, t, phase);
-    else pack_weight_f32_tc_kernel<float><<<grid, 256, 0, s>>>((const float*)w, packed, Cout, Cin, t, phase);
+    if (w_dtype == VD_BF16) pack_weight_f32_tc_kernel<__nv_bfloat16><<<grid, 256, 0, s>>>((const __nv_bfloat16*)w, (__nv_bfloat16*)packed, Cout, Cin, t, phase);
+    else pack_weight_f32_tc_kernel<float><<<grid, 256, 0, s>>>((const float*)w, (__nv_bfloat16*)packed, Cout, Cin, t, phase);
     return cudaGetLastError();
 }
 

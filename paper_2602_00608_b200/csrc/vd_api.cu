@@ -57,7 +57,7 @@ struct WeightJob {           // repack work done once in vd_create
     int Cout, Cin, taps;
     int cout_total, cout_offset;
     size_t dst_off;
-    bool f32_tc = false;     // fp32 weights as pairs of tf32 numbers
+    bool f32_tc = false;     // fp32 weights as three bf16 numbers each
 };
 
 size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
@@ -794,7 +794,7 @@ vd_status vd_create(const vd_config* cfg, const vd_tensor* weights, int32_t n_we
         } else if (j.tc) {
             e = launch_pack_weight_tc(t->dptr, t->dtype, h->ws + j.dst_off, j.Cout, j.Cin, j.taps, j.cout_total, j.cout_offset, j.phase, s);
         } else if (j.f32_tc) {
-            e = launch_pack_weight_f32_tc(t->dptr, t->dtype, (float*)(h->ws + j.dst_off), j.Cout, j.Cin, j.phase, s);
+            e = launch_pack_weight_f32_tc(t->dptr, t->dtype, h->ws + j.dst_off, j.Cout, j.Cin, j.phase, s);
         } else if (j.phase) {
             e = launch_pack_weight_f32_phase(t->dptr, t->dtype, (float*)(h->ws + j.dst_off), j.Cout, j.Cin, s);
         } else {
@@ -1105,7 +1105,7 @@ vd_status vd_conv_pack_weight(const vd_conv_desc* d, const void* w_oihw, int32_t
     if (st != VD_OK) return st;
     const int taps = d->ksize * d->ksize;
     cudaError_t e = tc ? launch_pack_weight_tc(w_oihw, w_dtype, packed, d->c_out, d->c_in, taps, d->c_out, 0, d->upsample == 2, (cudaStream_t)cuda_stream)
-                       : d->impl == VD_IMPL_TC_F32 ? launch_pack_weight_f32_tc(w_oihw, w_dtype, (float*)packed, d->c_out, d->c_in, d->upsample == 2, (cudaStream_t)cuda_stream)
+                       : d->impl == VD_IMPL_TC_F32 ? launch_pack_weight_f32_tc(w_oihw, w_dtype, packed, d->c_out, d->c_in, d->upsample == 2, (cudaStream_t)cuda_stream)
                        : d->upsample == 2 ? launch_pack_weight_f32_phase(w_oihw, w_dtype, (float*)packed, d->c_out, d->c_in, (cudaStream_t)cuda_stream)
                        : launch_pack_weight_simt(w_oihw, w_dtype, (float*)packed, d->c_out, d->c_in, taps, d->c_out, 0, (cudaStream_t)cuda_stream);
     return e == cudaSuccess ? VD_OK : cuda_fail(nullptr, e, "vd_conv_pack_weight");

@@ -195,9 +195,9 @@ cudaError_t launch_conv_f32(const ConvArgs& a, const ConvF32Plan& plan, unsigned
 // OIHW 3x3 -> the sixteen pre-summed 2x2 taps of the phase-collapsed upsampling form, fp32 [16][Cin][Cout]
 cudaError_t launch_pack_weight_f32_phase(const void* w, int w_dtype, float* packed, int Cout, int Cin, cudaStream_t s);
 
-// ---- single-precision 3x3 convolution on the tensor cores, operands as pairs of tf32 numbers (conv_f32_tc.cu)
+// ---- single-precision 3x3 convolution on the tensor cores, operands as three bf16 numbers each (conv_f32_tc.cu)
 struct alignas(64) ConvF32TcPlan {
-    unsigned char tmap[128];    // weights, [tap][block of 32 output channels][hi, lo][32][Cin]
+    unsigned char tmap[128];    // weights, bf16 [tap][block of 32 output channels][part][32][Cin]
     int splits;                 // CTAs that share K (the cluster)
     int n_b;                    // weight stages
     int tail_off, smem, valid;
@@ -210,7 +210,7 @@ int conv_f32_tc_slots(const ConvArgs& a, const ConvF32TcPlan& plan, int groups);
 size_t conv_f32_tc_packed_bytes(int Cout, int Cin, bool phase);
 cudaError_t conv_f32_tc_prepare(const ConvArgs& a, ConvF32TcPlan* plan);
 cudaError_t launch_conv_f32_tc(const ConvArgs& a, const ConvF32TcPlan& plan, unsigned int* status_word, cudaStream_t s);
-cudaError_t launch_pack_weight_f32_tc(const void* w, int w_dtype, float* packed, int Cout, int Cin, bool phase, cudaStream_t s);
+cudaError_t launch_pack_weight_f32_tc(const void* w, int w_dtype, void* packed, int Cout, int Cin, bool phase, cudaStream_t s);
 
 // ---- tcgen05 convolution divided along K for small images (conv_split.cu)
 struct ConvSplitShape {

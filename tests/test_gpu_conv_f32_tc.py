@@ -1,8 +1,8 @@
 """The single-precision convolution on the tensor cores, at the sizes where it can go wrong: tiles cut by the image edge, one to
 eight CTAs that share K, more taps than accumulators, the four parities of the upsampling form.
 
-Small whole numbers are exact in tf32 and their sums in fp32, so the result is that of a 64-bit convolution bit for bit; numbers
-with 24 significant bits show that the operands keep all of them."""
+Small whole numbers are exact in one bf16 number and their sums in fp32, so the result is that of a 64-bit convolution bit for bit;
+numbers with 24 significant bits, alone in their sums, show that the operands keep all of them."""
 import pytest
 
 from tests.test_gpu_conv_split import exact_conv, ints, vd            # noqa: F401  (vd is a fixture)
@@ -32,8 +32,9 @@ def test_whole_numbers_are_exact(vd, shape):                          # noqa: F8
 
 @pytest.mark.parametrize("shape", [(2, 17, 9, 64, 96, 0), (1, 8, 8, 512, 512, 0), (3, 33, 50, 32, 32, 0), (1, 64, 64, 128, 128, 0), (1, 8, 8, 512, 512, 2)])
 def test_operands_keep_24_bits(vd, shape):                            # noqa: F811
-    """A tap's sum has four truncating steps (2^-23 at most of a sum that grows to its size), each operand's remainder is below
-    2^-24, and at most 144 sums are added with rounding (2^-24 / sqrt(3) each, on a sum that grows: sqrt(144 / 2))."""
+    """A tap's sum has two truncating steps (2^-23 at most of a sum that grows to its size), a product lacks 2^-24 of itself at most,
+    the parts' sum rounds by 2^-24, and at most 26 sums and partials are added with rounding (2^-24 / sqrt(3) each, on a sum that
+    grows: sqrt(26 / 2)): two chunks of nine taps in a CTA, eight CTAs."""
     import torch
     B, H, W, Cin, Cout, up = shape
     g = torch.Generator(device="cuda").manual_seed(7)
@@ -41,10 +42,61 @@ def test_operands_keep_24_bits(vd, shape):                            # noqa: F8
     x, w = rnd(B, H, W, Cin), rnd(Cout, Cin, 3, 3) / (9 * Cin) ** 0.5
     want = exact_conv(x, w, 3, up)
     got = vd.op_conv2d(x, w, upsample=up, impl=vd.VD_IMPL_TC_F32).double()
-    bound = 4 * 2.0 ** -23 / 2 + 2.0 ** -24 + 2.0 ** -24 / 3 ** 0.5 * (144 / 2) ** 0.5
+    bound = 2 * 2.0 ** -23 / 2 + 2 * 2.0 ** -24 + 2.0 ** -24 / 3 ** 0.5 * (26 / 2) ** 0.5
     if up:
         bound += 2.0 ** -24                                           # the sums of up to four weights are rounded once
     assert float((got - want).norm() / want.norm()) <= bound
+
+
+def wide(g, lo, hi, *shape):
+    """Numbers of 24 significant bits, the last one set, of either sign and of sizes 2^lo to 2^hi."""
+    import torch
+    m = 2 * torch.randint(2 ** 22, 2 ** 23, shape, device="cuda", generator=g) + 1
+    e = torch.randint(lo, hi + 1, shape, device="cuda", generator=g)
+    sign = 2 * torch.randint(0, 2, shape, device="cuda", generator=g) - 1
+    return torch.ldexp((sign * m).double(), (e - 23).double()).float()
+
+
+@pytest.mark.parametrize("shape", [(1, 19, 21, 32, 32, 0), (1, 8, 8, 512, 512, 0), (1, 11, 5, 64, 32, 2)])
+@pytest.mark.parametrize("whole", ["activations", "weights"])
+def test_no_bit_of_an_operand_is_lost(vd, shape, whole):              # noqa: F811
+    """One tap of one input channel per output channel, times a power of two: the other operand comes back as it was,
+    sizes from 2^-110 to 2^100."""
+    import torch
+    B, H, W, Cin, Cout, up = shape
+    g = torch.Generator(device="cuda").manual_seed(11)
+    one = 2.0 ** torch.randint(-3, 4, (Cout,), device="cuda", generator=g).float()
+    src = torch.randint(0, Cin, (Cout,), device="cuda", generator=g)
+    if whole == "activations":
+        x, taps = wide(g, -110, 100, B, H, W, Cin), one
+    else:
+        x, taps = torch.ones(B, H, W, Cin, device="cuda"), wide(g, -110, 100, Cout)
+    w = torch.zeros(Cout, Cin, 3, 3, device="cuda")
+    w[torch.arange(Cout, device="cuda"), src, 1, 1] = taps
+    got = vd.op_conv2d(x, w, upsample=up, impl=vd.VD_IMPL_TC_F32)
+    want = x[..., src].double() * taps.double()
+    if up:
+        want = want.repeat_interleave(2, dim=1).repeat_interleave(2, dim=2)
+    assert torch.equal(got.double(), want)
+
+
+@pytest.mark.parametrize("terms", [1, 2, 4])
+def test_sums_of_few_products(vd, terms):                             # noqa: F811
+    """Products of 24 by 24 bits, a few per sum: each lacks at most 2^-24 of itself (the parts that are not multiplied); of the partial
+    sums, all but the smallest are exact but for truncations of 2^-23 of what they come to (the six of 2^-8 of a product, and where
+    products of other sizes meet); the sum of the parts and its addition to the running sum round by 2^-24 each."""
+    import torch
+    g = torch.Generator(device="cuda").manual_seed(12)
+    x = wide(g, -3, 3, 1, 64, 64, 32)
+    w = torch.zeros(32, 32, 9, device="cuda")
+    for o in range(32):
+        at = torch.randperm(288, device="cuda", generator=g)[:terms]
+        w[o].view(-1)[at] = wide(g, -1, 1, terms)
+    w = w.view(32, 32, 3, 3)
+    got = vd.op_conv2d(x, w, impl=vd.VD_IMPL_TC_F32).double()
+    err, size = (got - exact_conv(x, w, 3, 0)).abs(), exact_conv(x.abs(), w.abs(), 3, 0)
+    bound = 2.0 ** -24 * (1 + 2 + (2 * terms if terms > 1 else 6 * 2.0 ** -7))
+    assert float((err / size.clamp(min=1e-30)).max()) <= bound
 
 
 @pytest.mark.parametrize("B,H,W,Cin,Cout,cpg", [(2, 17, 9, 64, 128, 4), (1, 16, 16, 512, 512, 16), (1, 33, 50, 32, 64, 8)])
