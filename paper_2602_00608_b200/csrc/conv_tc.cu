@@ -659,7 +659,7 @@ conv_tc_kernel(const ConvArgs a, const __grid_constant__ CUtensorMap tmap, const
                 }
                 if (have_next) vm_next = issue(nx);              // the staging slots are free again: the next unit is on its way
                 if (cur_slot == 0) {
-                    ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bars->a_empty[stage]), phase ^ 1, abort_flag));
+                    ok = mbar_wait(smem_u32(&bars->a_empty[stage]), phase ^ 1, abort_flag);
                     if (!ok) break;
                     // a shortcut chunk: the stage will be filled by bulk tensor loads (one per tile of this CTA)
                     if (second && ptid == 0 && cur_have) mbar_expect_tx(smem_u32(&bars->a_full[stage]), (uint32_t)cur_cnt * SC_TILE_BYTES);
@@ -761,7 +761,7 @@ conv_tc_kernel(const ConvArgs a, const __grid_constant__ CUtensorMap tmap, const
                                 if (vm & (1u << u)) load_raw_at(IN_BF16, xb + goff[u], raw[u]);
                         }
                         if (slot == 0) {
-                            ok = __all_sync(0xffffffffu, mbar_wait<PH ? 256 : 0>(smem_u32(&bars->a_empty[stage]), phase ^ 1, abort_flag));
+                            ok = mbar_wait<PH ? 256 : 0>(smem_u32(&bars->a_empty[stage]), phase ^ 1, abort_flag);
                             if (!ok) break;
                             if (second && ptid == 0 && cnt > 0) mbar_expect_tx(smem_u32(&bars->a_full[stage]), (uint32_t)cnt * SC_TILE_BYTES);
                         }
