@@ -7,6 +7,9 @@
 // so a sum has two steps only, a tap of 32 channels, and the products of either size have their own: the largest, of 16 bits
 // each, mostly add up exactly, and what is cut from the others is below 2^-31.  The warps that have made the operand read the sums
 // and add them to their registers, smallest first, with rounding, while the next tap runs: two accumulators in turn.
+// An infinite operand, or one that rounds to infinity in bf16, has parts that are NaN, and so are the sums that it is in: those are
+// made anew from the operands themselves, one by one (redo_sums).  (Of the decode named below 830 -> 835 us, for the registers around
+// the call; with parts that hold no NaN and a look at every sum 897, with a look where an operand asks for it 846.)
 // Relative 2-norm error against 64 bits, FMA kernel (conv_f32.cu) / this one, normally distributed operands: 512->512 at 16x16 3.1e-7 /
 // 1.2e-7, at 24x24 4.2e-7 / 1.7e-7, 256->256 at 48x48 4.3e-7 / 1.3e-7, 128->128 at 64x64 3.1e-7 / 1.1e-7, 32->32 at 128x128 2.3e-7 / 0.9e-7;
 // sizes that spread over 2^24: 512->512 at 24x24 4.1e-7 / 1.7e-7; positive ones, whose truncations add up: 1.3e-7 / 1.0e-7 there, 0.57e-7 /
@@ -18,10 +21,10 @@
 // tap's weights are one box of 96 rows, the parts one above the other, so that x0 takes one MMA of N = 96 with all three, x1 one
 // of 64 and x2 one of 32, each added where products of that size are.  Two CTAs share an SM.  Bound by the taps' hand-over (issue,
 // sum, barrier) and by the chain of latencies around it.
-// us, launches of a decode, FMA kernel -> this one: 512->512 at 8x8 28.9 -> 26.7, at 16x16 43.4 -> 29.0, upsampling to 16x16 30.6 -> 27.5, to
-// 32x32 76.0 -> 43.8; 512->256 at 32x32 76.1 -> 45.3, 256->256 43.2 -> 28.9, 128->128 at 64x64 45.4 -> 31.0; 32->32 on four 256x256
-// frames 142 -> 109, at 128x128 45 -> 37.  Decodes: 64x64 of the full-width layout 1254 -> 831 us, sixteen 256x256 frames of the small
-// one 2770 -> 2184.
+// us, launches of a decode, FMA kernel -> this one: 512->512 at 8x8 28.9 -> 26.8, at 16x16 43.4 -> 29.0, upsampling to 16x16 30.6 -> 27.5, to
+// 32x32 76.0 -> 45.0; 512->256 at 32x32 76.1 -> 45.4, 256->256 43.2 -> 29.0, 128->128 at 64x64 45.4 -> 31.0; 32->32 on four 256x256
+// frames 142 -> 113, at 128x128 45 -> 37.  Decodes: 64x64 of the full-width layout 1252 -> 835 us, sixteen 256x256 frames of the small
+// one 2765 -> 2216.
 #include <string.h>
 
 #include <algorithm>
@@ -135,9 +138,58 @@ struct Operand {
     }
 };
 
+// Those of a thread's sixteen partial sums (one pixel, channels [16 h, 16 h + 16) of the CTA's block) that are NaN, in plain fp32.
+// It works everything out for itself: what it would be handed would be kept in registers where they are short.
+template <int KIND>
+__device__ __noinline__ void redo_sums(const ConvArgs& a, const TShape& sh, float* row, const float* s_scale, const float* s_shift) {
+    constexpr int TAPS = taps_of(KIND), COLS = KIND == K3X3 ? 3 : 2;
+    const int S = sh.splits, rank = S > 1 ? (int)cluster_ctarank() : 0;
+    const int H = KIND == KPHASE ? a.Hs : a.H, W = KIND == KPHASE ? a.Ws : a.W;
+    const int tiles_x = (W + TILE_W - 1) / TILE_W, tiles = tiles_x * ((H + TILE_H - 1) / TILE_H), nblk = a.Cout / BN;
+    int item = (int)blockIdx.x / S;
+    const int blk = item % nblk;
+    item /= nblk;
+    const int par = KIND == KPHASE ? (item & 3) : 0;
+    if (KIND == KPHASE) item >>= 2;
+    const int tile = item % tiles, frame = item / tiles;
+    const int warp = (int)threadIdx.x >> 5, lane = (int)threadIdx.x & 31, R = (warp & 3) * 32 + lane, h = (warp - kProd0) >> 2;
+    const int y = (tile / tiles_x) * TILE_H + (R >> 3), x = (tile % tiles_x) * TILE_W + (R & 7);
+    if (y >= H || x >= W) return;
+    const int kchunks = a.Cin / kChunk, k0 = rank * kchunks / S, nch = ((rank + 1) * kchunks / S - k0) * kChunk;
+    const float* image = (const float*)a.x + (size_t)frame * H * W * a.Cin + k0 * kChunk;
+    const bool prologue = a.scale != nullptr || a.in_rec != nullptr;
+    // A NaN among the operands ends it: a frame of them costs one product per sum, beginning with the tap that reads the pixel itself.
+    const int centre = KIND == KPHASE ? (par ^ 3) : 4;
+#pragma unroll 1
+    for (int o = 0; o < 16; ++o) {
+        float* at = row + exchange_piece(lane, h * 4 + (o >> 2)) * 4 + (o & 3);
+        if (!isnan(*at)) continue;
+        float sum = 0.f;
+#pragma unroll 1
+        for (int t = 0; t < TAPS && !isnan(sum); ++t) {
+            const int tap = (t + centre) % TAPS;
+            const int sy = y - 1 + (KIND == KPHASE ? par >> 1 : 0) + tap / COLS, sx = x - 1 + (KIND == KPHASE ? par & 1 : 0) + tap % COLS;
+            const bool inside = sy >= 0 && sy < H && sx >= 0 && sx < W;
+            const __nv_bfloat16* w = (const __nv_bfloat16*)a.w + (((size_t)(par * TAPS + tap) * nblk + blk) * (PARTS * BN) + h * 16 + o) * a.Cin + k0 * kChunk;
+#pragma unroll 1
+            for (int c = 0; c < nch && !isnan(sum); ++c) {
+                float v = 0.f, weight = 0.f;
+                if (inside) {
+                    v = __ldcg(image + ((size_t)sy * W + sx) * a.Cin + c);
+                    if (prologue) v = fmaf(v, s_scale[c], s_shift[c]);
+                    if (a.silu) v = v / (1.0f + expf(-v));
+                }
+                for (int p = PARTS - 1; p >= 0; --p) weight += __bfloat162float(w[(size_t)p * BN * a.Cin + c]);
+                sum = fmaf(v, weight, sum);
+            }
+        }
+        *at = sum;
+    }
+}
+
 template <int KIND>
 __global__ void __launch_bounds__(kThreads, 2)
-conv_f32_tc_kernel(const ConvArgs a, const TShape sh, const __grid_constant__ CUtensorMap tm_w, unsigned int* status) {
+conv_f32_tc_kernel(const __grid_constant__ ConvArgs a, const __grid_constant__ TShape sh, const __grid_constant__ CUtensorMap tm_w, unsigned int* status) {
     constexpr int TAPS = taps_of(KIND);
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -334,6 +386,11 @@ conv_f32_tc_kernel(const ConvArgs a, const TShape sh, const __grid_constant__ CU
             float* row = part + (R0 + lane) * BN;
 #pragma unroll
             for (int c = 0; c < 4; ++c) *(float4*)(row + exchange_piece(lane, h * 4 + c) * 4) = make_float4(v[4 * c], v[4 * c + 1], v[4 * c + 2], v[4 * c + 3]);
+            bool odd = false;
+#pragma unroll
+            for (int c = 0; c < 16; ++c) odd |= isnan(v[c]);
+            if (odd) redo_sums<KIND>(a, sh, row, s_scale, s_shift);
+            __syncwarp();
             fence_proxy_async_smem();
             named_barrier_sync(1, kProd);
             if (S > 1) {                                     // an owner's rows lie together
@@ -393,9 +450,11 @@ __global__ void pack_weight_f32_tc_kernel(const T* w, __nv_bfloat16* packed, int
             }
         const size_t row = ((size_t)tap * (Cout / BN) + o / BN) * (PARTS * BN) + o % BN;
         for (int p = 0; p < PARTS; ++p) {
-            const __nv_bfloat16 part = __float2bfloat16_rn(v);
+            // (the parts add up to the weight: an infinity is its first part, and what would round up to one is cut)
+            const bool cut = fabsf(v) >= 3.39617752e38f;     // 2^128 (1 - 2^-9)
+            const __nv_bfloat16 part = cut ? __ushort_as_bfloat16((unsigned short)(__float_as_uint(v) >> 16)) : __float2bfloat16_rn(v);
             packed[(row + p * BN) * Cin + c] = part;
-            v -= __bfloat162float(part);
+            v = isinf(v) ? 0.f : v - __bfloat162float(part);
         }
     }
 }

@@ -99,6 +99,36 @@ def test_sums_of_few_products(vd, terms):                             # noqa: F8
     assert float((err / size.clamp(min=1e-30)).max()) <= bound
 
 
+@pytest.mark.parametrize("up", [0, 2])
+@pytest.mark.parametrize("where", ["activations", "weights"])
+def test_infinities_and_the_largest_numbers(vd, where, up):           # noqa: F811
+    """Infinities, NaN and numbers that round to infinity in bf16 go through a layer as they do in 64 bits: with weights (or
+    activations) of one, two and three parts, and with zero."""
+    import torch
+    g = torch.Generator(device="cuda").manual_seed(13)
+    rnd = lambda *s: torch.randn(*s, device="cuda", generator=g)
+    x, w = rnd(1, 21, 20, 64), rnd(64, 64, 3, 3) / 40
+    inf = float("inf")
+    large = [inf, -inf, float("nan"), 3.4028234e38, -3.4028234e38, 3.3962e38, 3.3961e38, -3.39e38, 2.0 ** 127]
+    if where == "activations":
+        w[:, 5] = torch.tensor([0.5, -0.25, 1 / 3, -0.0078, 0.75390625, 0.0, 2.0 ** -20, 0.1], device="cuda")[torch.arange(64) % 8][:, None, None]
+        if up:
+            w *= 0.25                                                 # (sums of four weights stay below one)
+        for i, v in enumerate(large):
+            x[0, 2 + 7 * (i // 3), 2 + 7 * (i % 3), 5] = v
+    else:
+        x /= 8 * x.abs().max()
+        x[0, ::3, ::2, 7], x[0, 1::3, ::2, 7], x[0, 2::3, 1::2, 7] = 0.5, 1 / 3, 0.0
+        for i, v in enumerate(large):
+            w[3 * i, 7, 1, 1] = v
+    got, want = vd.op_conv2d(x, w, upsample=up, impl=vd.VD_IMPL_TC_F32), exact_conv(x, w, 3, up).float()
+    assert int(torch.isinf(want).sum()) >= 9 and int(torch.isnan(want).sum()) >= 1 and float(want[torch.isfinite(want)].abs().max()) > 1e37
+    assert torch.equal(torch.isnan(got), torch.isnan(want)) and torch.equal(torch.isinf(got), torch.isinf(want))
+    fin = torch.isfinite(want)
+    assert torch.equal(got[~fin].nan_to_num(nan=0.0), want[~fin].nan_to_num(nan=0.0))
+    assert torch.allclose(got[fin], want[fin], rtol=1e-6, atol=2e-6)  # 4 * 2^-24 of a sum's largest term; of the others, sums of 576 of size 0.025
+
+
 @pytest.mark.parametrize("B,H,W,Cin,Cout,cpg", [(2, 17, 9, 64, 128, 4), (1, 16, 16, 512, 512, 16), (1, 33, 50, 32, 64, 8)])
 def test_records_of_the_output_and_of_the_input(vd, B, H, W, Cin, Cout, cpg):      # noqa: F811
     import torch
