@@ -141,7 +141,11 @@ struct Operand {
 // Those of a thread's sixteen partial sums (one pixel, channels [16 h, 16 h + 16) of the CTA's block) that are NaN, in plain fp32.
 // It works everything out for itself: what it would be handed would be kept in registers where they are short.
 template <int KIND>
-__device__ __noinline__ void redo_sums(const ConvArgs& a, const TShape& sh, float* row, const float* s_scale, const float* s_shift) {
+__device__ __noinline__ void redo_sums(const ConvArgs& a, const TShape& sh) {
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+    const float* s_scale = (const float*)(smem + sh.tail_off);
+    const float* s_shift = s_scale + kMaxSlice;
     constexpr int TAPS = taps_of(KIND), COLS = KIND == K3X3 ? 3 : 2;
     const int S = sh.splits, rank = S > 1 ? (int)cluster_ctarank() : 0;
     const int H = KIND == KPHASE ? a.Hs : a.H, W = KIND == KPHASE ? a.Ws : a.W;
@@ -153,6 +157,7 @@ __device__ __noinline__ void redo_sums(const ConvArgs& a, const TShape& sh, floa
     if (KIND == KPHASE) item >>= 2;
     const int tile = item % tiles, frame = item / tiles;
     const int warp = (int)threadIdx.x >> 5, lane = (int)threadIdx.x & 31, R = (warp & 3) * 32 + lane, h = (warp - kProd0) >> 2;
+    float* row = (float*)smem + R * BN;
     const int y = (tile / tiles_x) * TILE_H + (R >> 3), x = (tile % tiles_x) * TILE_W + (R & 7);
     if (y >= H || x >= W) return;
     const int kchunks = a.Cin / kChunk, k0 = rank * kchunks / S, nch = ((rank + 1) * kchunks / S - k0) * kChunk;
@@ -389,7 +394,7 @@ conv_f32_tc_kernel(const __grid_constant__ ConvArgs a, const __grid_constant__ T
             bool odd = false;
 #pragma unroll
             for (int c = 0; c < 16; ++c) odd |= isnan(v[c]);
-            if (odd) redo_sums<KIND>(a, sh, row, s_scale, s_shift);
+            if (odd) redo_sums<KIND>(a, sh);
             __syncwarp();
             fence_proxy_async_smem();
             named_barrier_sync(1, kProd);
