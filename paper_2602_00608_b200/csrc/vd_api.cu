@@ -243,7 +243,7 @@ class Planner {
             f32 = conv_f32_choose(probe, &s.f32, clusters_ ? kF32MaxSplits : 1);
             if (f32 && upsample) { phase = true; a.upsample = 2; }
         }
-        const bool f32_tc = f32 && wnames.size() == 1 && conv_f32_tc_choose(probe, &s.f32_tc, clusters_ ? kF32MaxSplits : 1) && conv_f32_tc_pays(probe);
+        const bool f32_tc = f32 && !(cfg_.flags & VD_FLAG_FORCE_SIMT) && wnames.size() == 1 && conv_f32_tc_choose(probe, &s.f32_tc, clusters_ ? kF32MaxSplits : 1) && conv_f32_tc_pays(probe);
         s.f32_tc.valid = f32_tc ? 1 : 0;
         s.f32.valid = f32 && !f32_tc ? 1 : 0;
         ConvW cw = conv_weight(wnames, Cout_each, Cin, ksize * ksize, tc, phase, f32_tc);
