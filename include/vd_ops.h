@@ -127,7 +127,9 @@ VD_API vd_status vd_op_conv2d(const vd_conv_desc* d, const void* x, const void* 
                               const float* scale, const float* shift, const float* residual, void* y,
                               void* cuda_stream);
 
-/* The kernel that vd_op_conv2d launches for these arguments (host-only; no pointer is followed). */
+/* The kernel that vd_op_conv2d launches for these arguments (host-only; no pointer is followed).  The packed form of a weight
+ * belongs to `impl`, so VD_IMPL_AUTO of an fp32 layer is the FFMA kernel here; which kernel a handle's layer takes says
+ * vd_step_info. */
 typedef enum {
     VD_ROUTE_DIRECT = 0,        /* tiled FFMA kernel, scalar accesses */
     VD_ROUTE_THIN = 1,          /* first convolution (4 or 8 input channels), FFMA */

@@ -21,7 +21,7 @@ VD_FLAG_CANARY = 0x8
 VD_FLAG_FUSED_STATS = 0x10
 VD_FLAG_NO_CLUSTERS = 0x20
 VD_IMPL_AUTO, VD_IMPL_SIMT, VD_IMPL_TC, VD_IMPL_TC_SPLIT, VD_IMPL_TC_F32 = 0, 1, 2, 3, 4
-VD_ROUTE_DIRECT, VD_ROUTE_THIN, VD_ROUTE_F32, VD_ROUTE_TC, VD_ROUTE_SPLIT, VD_ROUTE_SPLIT_PAIRS = 0, 1, 2, 3, 4, 5
+VD_ROUTE_DIRECT, VD_ROUTE_THIN, VD_ROUTE_F32, VD_ROUTE_TC, VD_ROUTE_SPLIT, VD_ROUTE_SPLIT_PAIRS, VD_ROUTE_F32_TC = 0, 1, 2, 3, 4, 5, 6
 VD_STEP_INGEST, VD_STEP_GN_STATS, VD_STEP_CONV, VD_STEP_ATTENTION = 0, 1, 2, 3
 STATUS_NAMES = {0: "VD_OK", -1: "VD_ERR_INVALID_ARG", -2: "VD_ERR_UNSUPPORTED", -3: "VD_ERR_WORKSPACE",
                 -4: "VD_ERR_CUDA", -5: "VD_ERR_DEVICE_TIMEOUT"}

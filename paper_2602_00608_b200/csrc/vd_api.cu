@@ -333,7 +333,7 @@ class Planner {
         s.conv = a;
         s.use_tc = tc;
         s.has_residual = residual_off >= 0;
-        fill_info(s, name, tc, Cin, Cout, ksize, upsample, H, W, Cout, out_dtype, out_nchw, y_is_frames ? -1 : (long)y_off);
+        fill_info(s, name, tc || f32_tc, Cin, Cout, ksize, upsample, H, W, Cout, out_dtype, out_nchw, y_is_frames ? -1 : (long)y_off);
         const double P = (double)H * W;
         s.info.flops_per_frame = 2.0 * ksize * ksize * Cin * (double)Cout * P;
         s.info.out_u8 = out_u8 ? 1 : 0;

@@ -92,3 +92,16 @@ def test_views_into_larger_buffers_give_the_same_result(cin, cout, k, nchw, move
         want = want + res.double()
     # fp32 sums of at most 324 products in sequence: 2^-24 / sqrt(3) * sqrt(324 / 2)
     assert float((got.double() - want).norm() / want.norm()) <= 1e-6
+
+
+def test_the_single_precision_tensor_core_kernel_is_named():
+    for upsample in (0, 2):
+        assert vd.conv_route(desc(128, 64, upsample=upsample, impl=vd.VD_IMPL_TC_F32)) == vd.VD_ROUTE_F32_TC
+        assert vd.conv_route(desc(128, 64, upsample=upsample, impl=vd.VD_IMPL_AUTO)) == vd.VD_ROUTE_F32
+    for d in (desc(128, 64, k=1), desc(20, 64), desc(128, 48), desc(128, 64, upsample=1)):
+        d.impl = vd.VD_IMPL_TC_F32
+        with pytest.raises(vd.VdError):
+            vd.conv_route(d)
+    d = desc(128, 64, impl=vd.VD_IMPL_TC_F32)
+    with pytest.raises(vd.VdError):
+        vd.conv_route(d, w=264)                              # (a bulk copy starts on a 16-byte boundary)
