@@ -13,9 +13,10 @@
 // in memory.  Where the query tiles leave SMs idle the keys are divided too: `splits` pairs form a cluster, each takes its
 // share of the key tiles, and their outputs meet in distributed shared memory, added in a fixed order.
 // What bounds it: 256 KB of K and V come from L2 per tile and CTA for 4096 tensor cycles.  Against one CTA per 128 queries and
-// half of the channels, which computes the scores twice and reads Q anew for every key tile (us, one B200, the launches of a
-// decode): 1024 tokens 32 -> 23, 1961 54 -> 31, 5400 126 -> 73, eight times 5400 878 -> 509, two times 14400 1611 -> 806, which
-// is 1054 TFLOP/s, 64 % of the measured bf16 peak.
+// half of the channels, which computes the scores twice and reads Q anew for every key tile (us, one B200, with the transpose, the
+// same call again and again): 1024 tokens 30.8 -> 22.5, 1961 51.3 -> 28.7, 5400 117.9 -> 71.7, eight times 5400 753 -> 404, two times
+// 14400 1379 -> 724, which is 1173 TFLOP/s, 73 % of the measured bf16 peak.  Within decodes that hold the GPU at its power cap:
+// eight times 5400 878 -> 509, two times 14400 1611 -> 806.
 // Every wait is bounded (see tc_common.cuh).
 #include <algorithm>
 #include <mutex>
@@ -422,8 +423,9 @@ attn_tc_kernel(const AttnTcParams a, const __grid_constant__ CUtensorMap tm_q, c
 }
 
 // Up to 128 tokens: one tile of everything, so the kernel is a chain of latencies (loads, scores, softmax, P V, output) without
-// a loop, and a cluster's barriers would only lengthen it (64 tokens, with the transpose: 12.6 us, 16.8 on the pairs).  A CTA
-// takes all the queries and 128 channels of the output, and computes the scores for itself.
+// a loop, and a cluster's barriers would only lengthen it (with the transpose, us: 64 tokens 12.3, on a pair 16.6, on the kernel
+// before these 13.9; 128 tokens 12.4, 15.4, 14.4).  A CTA takes all the queries and 128 channels of the output, and computes the
+// scores for itself.
 constexpr int SMALL = 128, SMALL_STAGES = 5, SMALL_STAGE_BYTES = 2 * SMALL * CHUNK * 2;      // Q chunk + K chunk
 constexpr int SMALL_V_BYTES = 2 * 128 * CHUNK * 2;           // 128 channels x 2 x 64 keys
 constexpr int SMALL_SMEM = SMALL_STAGES * SMALL_STAGE_BYTES + SMALL_V_BYTES + 4 * SMALL * 4 + 256 + 1024;
@@ -660,9 +662,10 @@ int max_clusters(int splits) {
 
 // Pairs that share a query tile's keys: the fewest rounds of clusters x (key tiles of a pair + what a cluster costs besides, in
 // tiles: its fill, and the exchange where the keys are divided).  0: the device cannot hold a pair.
-// Measured with 1 / 2 / 3 / 4 pairs, us: 1024 tokens 23.4 / 21.2 / 23.2 / 22.6, 1961 35.7 / 31.6 / 33.7 / 46.0, 3600 53 / 42 / 62 / 59, 5400
-// 73 / 88 / 79 / 99, two times 5400 138 / 132 / 148 / 186, eight times 395 / 475 / 567 / 705, 14400 340 / 376 / 382 / 407, two times 714 /
-// 689 / 745 / 831: the rule takes 2, 2, 2, 1, 2, 1, 1, 2.
+// Measured with 1 / 2 / 3 / 4 pairs, us, the same call again and again (what the rule takes in brackets): 400 tokens [18.5] / 20.2, 1024
+// 22.6 / [22.5] / 22.6 / 22.6, 1537 30.0 / 27.7 / 25.8 / [25.7], 1791 32.8 / 28.7 / 28.7 / [26.7], 1961 34.9 / [28.7] / 28.7 / 43.1, 2200 36.9 / 30.8 /
+// [30.0] / 48.3, 3000 43.1 / [34.9] / 53.3 / 50.7, 3600 53.0 / [41.0] / 61.4 / 57.5, 5400 [71.7] / 86.1 / 77.9 / 96.5, two times 5400 137 / [132] / 147 /
+// 187, eight times [406] / 494 / 586 / 706, 14400 369 / [384] / 405 / 409, two times 746 / [738] / 784 / 876, four times 1024 32.3 / [34.8] / 54.3 / 59.6.
 int choose_splits(int B, int T, bool no_clusters) {
     const long long q_tiles = (long long)((T + BQ - 1) / BQ) * std::max(B, 1);
     const int ntiles = (T + BKV - 1) / BKV;
