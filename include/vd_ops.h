@@ -197,6 +197,12 @@ VD_API vd_status vd_op_gn_stats(const void* x, int32_t dtype, int32_t batch, int
                                 int32_t groups, float eps, const float* gamma, const float* beta, const float* offset,
                                 float* scale, float* shift, void* scratch, void* cuda_stream);
 
+/* The same operator on the kernels that a handle of max_batch 1 takes (vd_op_gn_stats: those of larger max_batch).  They add up in
+ * another order; what is said above holds of either. */
+VD_API vd_status vd_op_gn_stats_single(const void* x, int32_t dtype, int32_t batch, int32_t h, int32_t w, int32_t c,
+                                       int32_t groups, float eps, const float* gamma, const float* beta, const float* offset,
+                                       float* scale, float* shift, void* scratch, void* cuda_stream);
+
 /* The same operator for callers that cannot hand over (or allocate) a scratch buffer.  The paper
  * has no counterpart of this entry point; it exists for hosts where device allocation is not an
  * option at call time: frame loops that must not hit the allocator's implicit synchronisation,

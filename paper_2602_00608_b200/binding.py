@@ -29,7 +29,7 @@ STATUS_NAMES = {0: "VD_OK", -1: "VD_ERR_INVALID_ARG", -2: "VD_ERR_UNSUPPORTED", 
 EXPORTED = [
     "vd_query_workspace", "vd_create", "vd_decode", "vd_decode_extrapolated", "vd_decode_host", "vd_get_status",
     "vd_last_error", "vd_destroy", "vd_num_steps", "vd_get_step", "vd_profile", "vd_debug_stop_after",
-    "vd_conv_packed_weight_bytes", "vd_conv_pack_weight", "vd_op_conv2d", "vd_conv_route", "vd_op_conv2d_ex", "vd_conv_record_slots", "vd_op_merge_records", "vd_conv_stats_scratch_bytes", "vd_op_conv2d_stats", "vd_gn_scratch_bytes", "vd_op_gn_stats",
+    "vd_conv_packed_weight_bytes", "vd_conv_pack_weight", "vd_op_conv2d", "vd_conv_route", "vd_op_conv2d_ex", "vd_conv_record_slots", "vd_op_merge_records", "vd_conv_stats_scratch_bytes", "vd_op_conv2d_stats", "vd_gn_scratch_bytes", "vd_op_gn_stats", "vd_op_gn_stats_single",
     "vd_op_attention", "vd_attention_scratch_bytes", "vd_op_gn_stats_static", "vd_clear_status", "vd_decode_host_stream", "vd_debug_check_canaries", "vd_debug_status_offset", "vd_debug_wait_probe",
 ]
 
@@ -116,6 +116,7 @@ def lib():
         l.vd_gn_scratch_bytes.argtypes = [c_int32, c_int32]
         l.vd_gn_scratch_bytes.restype = c_size_t
         l.vd_op_gn_stats.argtypes = [vp, c_int32, c_int32, c_int32, c_int32, c_int32, c_int32, c_float, vp, vp, vp, vp, vp, vp, vp]
+        l.vd_op_gn_stats_single.argtypes = l.vd_op_gn_stats.argtypes
         l.vd_op_gn_stats_static.argtypes = [vp, c_int32, c_int32, c_int32, c_int32, c_int32, c_int32, c_float, vp, vp, vp, vp, vp]
         l.vd_op_attention.argtypes = [vp, vp, vp, vp, c_int32, c_int32, c_int32, c_int32, c_int32, c_int32, c_float, c_int32, vp, vp]
         l.vd_attention_scratch_bytes.argtypes = [c_int32, c_int32, c_int32]
@@ -415,15 +416,17 @@ def op_conv2d_stats(x_nhwc, w_oihw, gamma, beta, groups: int, eps: float, bias=N
     return y, out_scale, out_shift
 
 
-def op_gn_stats(x_nhwc, gamma, beta, groups: int, eps: float, offset=None):
-    """Per-(sample, channel) GroupNorm scale and shift of an NHWC device tensor (of x + offset[c] if given)."""
+def op_gn_stats(x_nhwc, gamma, beta, groups: int, eps: float, offset=None, single=False):
+    """Per-(sample, channel) GroupNorm scale and shift of an NHWC device tensor (of x + offset[c] if given).  single: on the kernels of
+    a handle of max_batch 1."""
     import torch
     b, h, w, c = x_nhwc.shape
     scratch = torch.empty(max(1, lib().vd_gn_scratch_bytes(max(b, 1), groups)), dtype=torch.uint8, device=x_nhwc.device)
     scale = torch.empty((b, c), dtype=torch.float32, device=x_nhwc.device)
     shift = torch.empty((b, c), dtype=torch.float32, device=x_nhwc.device)
     p = lambda t: None if t is None else c_void_p(t.data_ptr())
-    _check(lib().vd_op_gn_stats(p(x_nhwc.contiguous()), _dt(x_nhwc), b, h, w, c, groups, eps, p(gamma), p(beta), p(offset), p(scale), p(shift), p(scratch), _stream_ptr()))
+    op = lib().vd_op_gn_stats_single if single else lib().vd_op_gn_stats
+    _check(op(p(x_nhwc.contiguous()), _dt(x_nhwc), b, h, w, c, groups, eps, p(gamma), p(beta), p(offset), p(scale), p(shift), p(scratch), _stream_ptr()))
     return scale, shift
 
 

@@ -1286,9 +1286,9 @@ size_t vd_gn_scratch_bytes(int32_t batch, int32_t groups) {
     return gn_scratch_bytes(batch, groups);
 }
 
-vd_status vd_op_gn_stats(const void* x, int32_t dtype, int32_t batch, int32_t h, int32_t w, int32_t c, int32_t groups,
-                         float eps, const float* gamma, const float* beta, const float* offset, float* scale, float* shift,
-                         void* scratch, void* cuda_stream) {
+static vd_status gn_stats(bool single, const void* x, int32_t dtype, int32_t batch, int32_t h, int32_t w, int32_t c, int32_t groups,
+                          float eps, const float* gamma, const float* beta, const float* offset, float* scale, float* shift,
+                          void* scratch, void* cuda_stream) {
     if (!x || !gamma || !beta || !scale || !shift || !scratch) return fail(nullptr, VD_ERR_INVALID_ARG, "NULL pointer");
     if (dtype != VD_F32 && dtype != VD_BF16) return fail(nullptr, VD_ERR_INVALID_ARG, "bad dtype");
     if (batch < 0 || h < 1 || w < 1 || c < 1 || groups < 1 || c % groups != 0 || (c / groups) % 4 != 0 || c > 1024)
@@ -1298,9 +1298,22 @@ vd_status vd_op_gn_stats(const void* x, int32_t dtype, int32_t batch, int32_t h,
     if (batch == 0) return VD_OK;
     unsigned int* counters = (unsigned int*)((char*)scratch + gn_partial_bytes(batch, groups));
     GnArgs a{x, dtype, batch, h * w, c, groups, eps, gamma, beta, scale, shift, (float*)scratch, counters, offset};
+    a.single = single ? 1 : 0;
     cudaError_t e = cudaMemsetAsync(counters, 0, (size_t)batch * sizeof(unsigned int), (cudaStream_t)cuda_stream);
     if (e == cudaSuccess) e = launch_gn_stats(a, (cudaStream_t)cuda_stream);
     return e == cudaSuccess ? VD_OK : cuda_fail(nullptr, e, "vd_op_gn_stats");
+}
+
+vd_status vd_op_gn_stats(const void* x, int32_t dtype, int32_t batch, int32_t h, int32_t w, int32_t c, int32_t groups,
+                         float eps, const float* gamma, const float* beta, const float* offset, float* scale, float* shift,
+                         void* scratch, void* cuda_stream) {
+    return gn_stats(false, x, dtype, batch, h, w, c, groups, eps, gamma, beta, offset, scale, shift, scratch, cuda_stream);
+}
+
+vd_status vd_op_gn_stats_single(const void* x, int32_t dtype, int32_t batch, int32_t h, int32_t w, int32_t c, int32_t groups,
+                                float eps, const float* gamma, const float* beta, const float* offset, float* scale, float* shift,
+                                void* scratch, void* cuda_stream) {
+    return gn_stats(true, x, dtype, batch, h, w, c, groups, eps, gamma, beta, offset, scale, shift, scratch, cuda_stream);
 }
 
 size_t vd_attention_scratch_bytes(int32_t batch, int32_t tokens, int32_t channels) {
