@@ -1,6 +1,6 @@
 """GroupNorm statistics of single frames and of several at once are two kernels (handles of max_batch 1 and of more).  Both, against 64
 bits: each storage type, wide and narrow layers, an offset per channel, a mean far from zero, groups without variance; the same
-bits every time, alone and in a batch."""
+bits every time, alone and in a batch.  (Samples of up to 3 million elements in 16-channel columns are a third kernel's.)"""
 import pytest
 
 pytestmark = pytest.mark.gpu
@@ -22,9 +22,9 @@ def want_of(x, gamma, beta, G, eps, off):
 
 @pytest.mark.parametrize("single", [False, True])
 @pytest.mark.parametrize("B,H,W,C,G,bf16,offset,mean", [
-    (1, 77, 77, 512, 32, False, False, 0.5), (1, 77, 77, 512, 32, True, True, 0.5), (2, 67, 93, 64, 8, False, True, 0.5),
+    (1, 77, 77, 512, 32, False, False, 0.5), (1, 77, 77, 512, 32, True, True, 0.5), (2, 251, 203, 64, 8, False, True, 0.5),
     (1, 240, 360, 256, 32, False, False, 0.5), (1, 200, 131, 128, 32, True, True, 0.5), (3, 45, 61, 1000, 250, False, False, 0.5),
-    (1, 70, 71, 20, 5, False, True, 0.5), (2, 70, 71, 24, 3, True, True, 0.5), (1, 70, 71, 20, 5, True, False, 0.5), (1, 95, 97, 128, 32, False, False, 300.0),
+    (1, 70, 71, 20, 5, False, True, 0.5), (2, 70, 71, 24, 3, True, True, 0.5), (1, 70, 71, 20, 5, True, False, 0.5), (1, 160, 151, 128, 32, False, False, 300.0),
 ])
 def test_gn_stats_of_either_kernel(vd, single, B, H, W, C, G, bf16, offset, mean):
     import torch
@@ -47,7 +47,7 @@ def test_groups_without_variance(vd, single):
     import torch
     g = torch.Generator(device="cuda").manual_seed(3)
     const = torch.rand(2, 8, device="cuda", generator=g).mul_(10).sub_(5).repeat_interleave(16, dim=1)
-    x = const[:, None, None, :].expand(2, 70, 71, 128).contiguous()
+    x = const[:, None, None, :].expand(2, 160, 151, 128).contiguous()
     gamma, beta = torch.linspace(0.9, 1.1, 128, device="cuda"), torch.linspace(-0.1, 0.1, 128, device="cuda")
     sc, sh = vd.op_gn_stats(x, gamma, beta, 8, 0.25, single=single)
     assert torch.allclose(sc, (gamma * 2).expand(2, 128), rtol=1e-6, atol=0)         # 1 / sqrt(0.25)
