@@ -4,7 +4,8 @@ kernel on a small case:
     python bench_op.py gn --h 480 --w 720 --c 128 [--f32] [--iters 5]
     python bench_op.py attn --tokens 5400 --c 512 [--iters 5]
 
-gn:   GroupNorm statistics (vd_op_gn_stats) of an NHWC tensor, 32 groups; prints the mean device time and the
+gn:   GroupNorm statistics of an NHWC tensor, 32 groups, on the kernel of handles for one frame (vd_op_gn_stats_single) or, with
+      --batch, for several (vd_op_gn_stats); prints the mean device time and the
       achieved GB/s (algorithmic bytes: one read of the tensor).
 attn: single-head attention core (vd_op_attention) over `tokens` tokens; prints the mean device time and
       the achieved TFLOP/s (algorithmic flops 4*T*T*C).
@@ -54,7 +55,7 @@ def main():
         dt = torch.float32 if a.f32 else torch.bfloat16
         x = torch.randn((a.batch, a.h, a.w, a.c), generator=g, device="cuda").to(dt)
         gamma, beta = torch.ones(a.c, device="cuda"), torch.zeros(a.c, device="cuda")
-        ms = _time(lambda: vd.op_gn_stats(x, gamma, beta, 32, 1e-6), a.iters, a.warmup)
+        ms = _time(lambda: vd.op_gn_stats(x, gamma, beta, 32, 1e-6, single=a.batch == 1), a.iters, a.warmup)
         byts = x.numel() * x.element_size()
         print(json.dumps({"op": "gn_stats", "ms": ms, "gbs": byts / ms / 1e6, "mbytes": byts / 1e6, "args": vars(a)}))
     else:
