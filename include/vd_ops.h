@@ -224,7 +224,9 @@ VD_API vd_status vd_op_gn_stats_static(const void* x, int32_t dtype, int32_t bat
  * device rows of `dtype` with `ld` elements between consecutive tokens (so q, k, v may be
  * slices of one [tokens, 3C] tensor); tokens >= 1.  The tensor-core kernel needs bf16, 512
  * channels, 16-byte aligned pointers, ld multiples of 8, and `scratch`: device memory of
- * vd_attention_scratch_bytes bytes (it holds V transposed); the FFMA kernel ignores scratch. */
+ * vd_attention_scratch_bytes bytes (it holds V transposed); the FFMA kernel ignores scratch.  How it
+ * divides the keys follows from tokens and batch, so an item's bits may differ (by rounding) between
+ * calls of different batch; a handle's do not (it divides them for max_batch). */
 VD_API size_t vd_attention_scratch_bytes(int32_t batch, int32_t tokens, int32_t channels);
 VD_API vd_status vd_op_attention(const void* q, const void* k, const void* v, void* o, int32_t dtype,
                                  int32_t batch, int32_t tokens, int32_t channels, int32_t ld_qkv, int32_t ld_o,
